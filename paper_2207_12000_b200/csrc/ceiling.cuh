@@ -10,56 +10,45 @@
 // sums, no output rows, no scratch.  Their results mean nothing; their duration is the yardstick.
 #pragma once
 
-template <int G, int V, int U>
-__global__ void __launch_bounds__(kThreads, G <= 4 ? 4 : GNNPRE_SEG_MIN_BLOCKS) k_ceiling(const SegArgs a, float* __restrict__ sink) {
+template <int G>
+__global__ void __launch_bounds__(kThreads, 4) k_ceiling(const SegArgs a, float* __restrict__ sink) {
     constexpr unsigned kFull = 0xffffffffu;
+    constexpr int kChunk = G < kSegWindow ? kSegWindow : G;
+    constexpr int M = kChunk / G;
+    __shared__ __align__(16) uint32_t stages[kThreads / G][kChunk];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1);
+    uint32_t* stage = stages[threadIdx.x / G];
     const int64_t s = a.seg_lo + ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G;
-    int64_t e = 0, e_end = 0;
+    const uint32_t* entries = a.colx;
+    int left = 0;
     if (s < a.seg_hi) {
-        e = a.segs[s].start;
-        e_end = a.segs[s + 1].start;
+        entries += a.segs[s].start - a.colx_base;
+        left = (int)(a.segs[s + 1].start - a.segs[s].start);
     }
-    const float4* xlane[V];
-    const uint32_t ldx4 = (uint32_t)(a.ldx >> 2);
+    const int q0 = blockIdx.y * a.tile_f4;
+    const char* xlane = reinterpret_cast<const char*>(a.x + 4 * q0) + (gl < min(a.tile_f4, a.f4 - q0) ? 16 * gl : 0);
+    const uint32_t row_bytes = (uint32_t)a.ldx * 4u;
+    Quad acc = quad_zero();
+    while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        const int q = gl + v * G;
-        xlane[v] = reinterpret_cast<const float4*>(a.x) + (q < a.f4 ? q : 0);
-    }
-    float4 acc[V];
+        for (int m = 0; m < M; ++m)  // lanes past the end fetch row 0
+            stage[gl + m * G] = gl + m * G < left ? __ldg(entries + gl + m * G) & ~kRowEndBit : 0u;
+        const int cnt = max(0, min(left, kChunk));
+        const int cnt_max = G == 32 ? cnt : kChunk == kSegWindow ? kChunk : __reduce_max_sync(kFull, cnt);
+        __syncwarp();
+        for (int t0 = 0; t0 < cnt_max; t0 += kSegWindow) {
+            Quad x[kSegWindow];
 #pragma unroll
-    for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    while (__any_sync(kFull, e < e_end)) {
-        const int64_t left = e_end - e;
-        const int cnt = left >= G ? G : (left > 0 ? (int)left : 0);
-        uint32_t c = 0;  // lanes past the end fetch row 0
-        if (gl < cnt) c = a.colx[e + gl - a.colx_base] & ~kRowEndBit;
-        const int cnt_max = G == 32 ? cnt : __reduce_max_sync(kFull, cnt);
-        for (int t0 = 0; t0 < cnt_max; t0 += U) {
-            float4 x[U][V];
+            for (int u = 0; u < kSegWindow; ++u) x[u] = quad_gather(xlane, stage[t0 + u], row_bytes);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint64_t off = (uint64_t)__shfl_sync(kFull, c, t0 + u, G) * ldx4;
-#pragma unroll
-                for (int v = 0; v < V; ++v) x[u][v] = __ldg(xlane[v] + off);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    acc[v].x += x[u][v].x; acc[v].y += x[u][v].y;
-                    acc[v].z += x[u][v].z; acc[v].w += x[u][v].w;
-                }
-            }
+            for (int u = 0; u < kSegWindow; ++u) quad_add(acc, x[u]);
         }
-        e += G;
+        __syncwarp();
+        entries += kChunk;
+        left -= kChunk;
     }
-    float r = 0.f;
-#pragma unroll
-    for (int v = 0; v < V; ++v) r += (acc[v].x + acc[v].y) + (acc[v].z + acc[v].w);
-    if (gl == 0 && s < a.seg_hi) sink[s] = r;
+    if (gl == 0 && s < a.seg_hi) sink[s] = (acc.lo.x + acc.lo.y) + (acc.hi.x + acc.hi.y);
 }
 
 // The bulk-copy pipeline of k_segments_tma (same stages, same bounded waits, same give-up path) with the sums

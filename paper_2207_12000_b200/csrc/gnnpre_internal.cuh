@@ -153,6 +153,7 @@ struct gnnpre_plan {
     gnnpre::DevBuf<int32_t> deg;
     gnnpre::DevBuf<float> rscale, cscale;
     gnnpre::DevBuf<int32_t> nzrows;     // rows owning >= 1 edge, ascending (only when !rows_all_nonempty)
+    gnnpre::DevBuf<float> nzscale;      // their row scales, in the same order
     gnnpre::DevBuf<int32_t> emptyrows;  // rows owning no edge
     // support structure
     gnnpre::DevBuf<int64_t> rowptr_t;         // the support's row pointers

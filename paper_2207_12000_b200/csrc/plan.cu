@@ -235,10 +235,16 @@ __global__ void k_nonempty_flags(int64_t n, const int64_t* __restrict__ rowptr_t
 }
 
 __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const int32_t* __restrict__ rank,
-                             int32_t* __restrict__ nzrows, int32_t* __restrict__ emptyrows) {
+                             const float* __restrict__ rscale, int32_t* __restrict__ nzrows, float* __restrict__ nzscale,
+                             int32_t* __restrict__ emptyrows) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    if (flag[i]) nzrows[rank[i]] = (int32_t)i; else emptyrows[i - rank[i]] = (int32_t)i;
+    if (flag[i]) {
+        nzrows[rank[i]] = (int32_t)i;
+        nzscale[rank[i]] = rscale[i];
+    } else {
+        emptyrows[i - rank[i]] = (int32_t)i;
+    }
 }
 
 // ---------------------------------------------------------------- warp-level segments
@@ -365,19 +371,18 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, int nu
         while ((int64_t)p * 2 <= per_warp && p < 4096) p *= 2;
         return p;
     }
-    // about 32 Ki gathered floats per segment, but short enough that every SM's 2048 threads get a
-    // segment per lane group; a power of two between 32 and 4096 edges.  Rows wider than 256 floats
-    // get at least 128 edges per segment (256 when the graph still leaves a thousand edges per lane
-    // group): with shorter ones most rows are cut and adding up their parts costs more than the
-    // segments save (F = 602, 23 M edges: 17.0 ms per two hops at 32 edges, 13.5 ms at 256).
-    const int64_t f4 = std::min<int64_t>(std::max<int64_t>(slab_width, 4), 512) / 4;
+    // Register kernel: segments long enough that few rows are cut, short enough that every lane group an SM holds (28
+    // warps) gets two (four or eight lanes per group) or three (wider) of them, up to 256 edges.  On 169 K nodes,
+    // 2.3 M edges, us per hop at 32 / 64 / 128 / 256 edges: 16 columns, mean 32 / 32 / 34 / 52; 32 columns, GCN
+    // 47 / 44 / 49 / 69; 64 columns 80 / 69 / 71 / 82; 128 columns 133 / 109 / 105 / 114.  Beyond 256 edges, up to 1024,
+    // only while eight segments per lane group remain (23 M edges, 128 columns: 829 / 744 / 702 us at 64 / 128 / 256, as
+    // fast at 1024; 12.8 M edges: 531 at 256, 583 at 1024): what longer segments save there is tables and scratch rows.
+    const int64_t f4 = std::min<int64_t>(std::max<int64_t>(slab_width, 4), 128) / 4;
     const int64_t lanes = f4 <= 4 ? 4 : f4 <= 8 ? 8 : f4 <= 16 ? 16 : 32;
-    const int64_t groups = (int64_t)std::max(num_sms, 1) * (2048 / lanes);
-    int64_t by_width = 32768 / std::max<int64_t>(slab_width, 4);
-    if (by_width < 128) by_width = m / groups >= 1024 ? 256 : 128;
-    const int64_t L = std::min<int64_t>(by_width, m / groups);
+    const int64_t per_group = m / ((int64_t)std::max(num_sms, 1) * (28 * 32 / lanes));
+    const int64_t L = std::max(std::min<int64_t>(per_group / (lanes <= 8 ? 2 : 3), 256), per_group / 8);
     int32_t p = 32;
-    while ((int64_t)p * 2 <= L && p < 4096) p *= 2;
+    while ((int64_t)p * 2 <= L && p < 1024) p *= 2;
     return p;
 }
 
@@ -443,7 +448,7 @@ gnnpre_plan::~gnnpre_plan() {
 }
 
 int64_t gnnpre_plan::device_bytes() const {
-    size_t t = deg.bytes() + rscale.bytes() + cscale.bytes() + nzrows.bytes() + emptyrows.bytes() + rowptr_t.bytes() +
+    size_t t = deg.bytes() + rscale.bytes() + cscale.bytes() + nzrows.bytes() + nzscale.bytes() + emptyrows.bytes() + rowptr_t.bytes() +
                colx.bytes() + colx_stage[0].bytes() + colx_stage[1].bytes() + segments.bytes() + fixups.bytes() + hubs.bytes() +
                scratch.bytes() + dev_error.bytes();
     for (const auto& s : slab) t += s.bytes();
@@ -552,8 +557,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         if (P->num_empty > 0) {
             P->rows_all_nonempty = false;
             GNNPRE_TRY(P->nzrows.alloc((size_t)P->num_nonempty));
+            GNNPRE_TRY(P->nzscale.alloc((size_t)P->num_nonempty));
             GNNPRE_TRY(P->emptyrows.alloc((size_t)P->num_empty));
-            k_split_rows<<<grid_for(n, kTB), kTB, 0, st>>>(n, flag.p, rank.p, P->nzrows.p, P->emptyrows.p);
+            k_split_rows<<<grid_for(n, kTB), kTB, 0, st>>>(n, flag.p, rank.p, P->rscale.p, P->nzrows.p, P->nzscale.p, P->emptyrows.p);
             GNNPRE_CUDA(cudaGetLastError());
             GNNPRE_CUDA(cudaStreamSynchronize(st));
         } else {

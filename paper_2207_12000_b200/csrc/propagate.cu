@@ -39,16 +39,16 @@ __global__ void k_wait_that_runs_out(int* error, uint32_t polls) {
 #include "fixups.cuh"
 #include "ceiling.cuh"
 
-template <int G, int V, int U>
+template <int G>
 int launch_segments_shape(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
     const int64_t groups = a.seg_hi - a.seg_lo;
-    const unsigned grid = (unsigned)((groups * G + kThreads - 1) / kThreads);
+    const dim3 grid((unsigned)((groups * G + kSegThreads - 1) / kSegThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
     const int ep = epilogue_of(a.tp);
-#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                 \
-    do {                                                                                                    \
-        if (ep == kEpSum) k_segments<G, V, U, OP_, EMPTY_, kEpSum><<<grid, kThreads, 0, st>>>(a);           \
-        else if (ep == kEpTeleport) k_segments<G, V, U, OP_, EMPTY_, kEpTeleport><<<grid, kThreads, 0, st>>>(a); \
-        else k_segments<G, V, U, OP_, EMPTY_, kEpPlain><<<grid, kThreads, 0, st>>>(a);                      \
+#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                    \
+    do {                                                                                                       \
+        if (ep == kEpSum) k_segments<G, OP_, EMPTY_, kEpSum><<<grid, kSegThreads, 0, st>>>(a);                 \
+        else if (ep == kEpTeleport) k_segments<G, OP_, EMPTY_, kEpTeleport><<<grid, kSegThreads, 0, st>>>(a);  \
+        else k_segments<G, OP_, EMPTY_, kEpPlain><<<grid, kSegThreads, 0, st>>>(a);                            \
     } while (0)
     switch (P->op) {
     case GNNPRE_OP_GCN_SYM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GCN_SYM, false); break;
@@ -60,6 +60,21 @@ int launch_segments_shape(const gnnpre_plan* P, const SegArgs& a, cudaStream_t s
 #undef GNNPRE_LAUNCH_SEGMENTS
     GNNPRE_CUDA(cudaGetLastError());
     return GNNPRE_OK;
+}
+
+// Float4 per column tile of the register kernels: equal tiles of at most 128 columns.
+int32_t equal_tile_f4(int32_t f4) {
+    const int32_t tiles = (f4 + 31) / 32;
+    return (f4 + tiles - 1) / tiles;
+}
+
+// The register kernel on all columns of `a`, one launch.
+int launch_segments_gather(const gnnpre_plan* P, SegArgs a, cudaStream_t st) {
+    a.tile_f4 = equal_tile_f4(a.f4);
+    if (a.tile_f4 <= 4) return launch_segments_shape<4>(P, a, st);
+    if (a.tile_f4 <= 8) return launch_segments_shape<8>(P, a, st);
+    if (a.tile_f4 <= 16) return launch_segments_shape<16>(P, a, st);
+    return launch_segments_shape<32>(P, a, st);
 }
 
 // Bulk-copy variant: one persistent CTA per SM, as many warps (at most kTmaMaxWarps) as fit into the
@@ -197,36 +212,36 @@ Teleport teleport_of(const gnnpre_plan* P, const HopArgs& h, int32_t f0) {
 
 namespace {
 
-// A column tile of 68..128 columns (17..32 float4) goes through the bulk-copy kernel unless the plan says otherwise.
+int64_t l2_cache_bytes() {
+    static std::atomic<int64_t> cached{0};
+    int64_t bytes = cached.load(std::memory_order_relaxed);
+    if (bytes == 0) {
+        int dev = 0, got = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&got, cudaDevAttrL2CacheSize, dev) != cudaSuccess || got <= 0)
+            got = 126 << 20;
+        cached.store(bytes = got, std::memory_order_relaxed);
+    }
+    return bytes;
+}
+
+// A column tile of 68..128 columns goes through the bulk-copy kernel when X's tile is at least four times the L2 and
+// rows are long (mean degree >= 32).  Its rows in flight (213 KB per SM) then hide the DRAM latency that the register
+// kernel's 90 KB do not; everywhere else its copy engine, about 33 ps per row whatever the row's width, is the slower
+// path.  us per hop, bulk copy / register: 2.4 M nodes of mean degree 51, mean operator, 72 columns 3478 / 3849,
+// 100 columns 4021 / 4420, 128 columns 4631 / 4757, GCN 100 columns 5175 / 5647.  But 800 K nodes of degree 63, GCN, 100
+// columns (2.4 x L2) 1930 / 1762; 1.7 M nodes of degree 15, GCN, 128 columns (6.7 x L2) 1441 / 1200; 169 K nodes of
+// degree 15, GCN, 128 columns 155 / 121.
 bool tile_uses_bulk_copy(const gnnpre_plan* P, int32_t width) {
     const int32_t f4 = width / 4;
-    return !(P->flags & GNNPRE_FLAG_NO_BULK_COPY) && f4 > 16 && f4 <= 32 && tma_warps(f4) >= 2;
+    return !(P->flags & GNNPRE_FLAG_NO_BULK_COPY) && f4 > 16 && f4 <= 32 && P->n * (int64_t)width * 4 > 4 * l2_cache_bytes() &&
+           P->nnz_tilde >= 32 * P->n;
 }
 
-// Columns one segment launch covers.  Rows wider than 256 columns are cut into 128-column tiles for the bulk-copy
-// kernel: the register kernel holds only two such rows per lane in flight (F = 602 on 23 M edges: 8.4 TB/s of
-// gathered bytes for its 512-column tile against 11 TB/s for the copy engine on the rest of the row).
-// Rows of 132..256 columns go the same way, as two equal tiles, once a 128-column tile of X no longer fits the
-// L2 (2.4 M nodes, 124 M edges, F = 256: 11.9 ms per hop-launch on the register kernel plus 1.6 ms of fix-ups for
-// its 128-edge segments, against 2 x 4.7 ms); while it fits, the register kernel's four rows per lane are the
-// faster path (169 K nodes, F = 256: 0.25 ms against 2 x 0.15 ms).
-int64_t l2_cache_bytes() {
-    static int64_t cached = -1;
-    if (cached < 0) {
-        int dev = 0, bytes = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&bytes, cudaDevAttrL2CacheSize, dev) != cudaSuccess || bytes <= 0)
-            bytes = 126 << 20;
-        cached = bytes;
-    }
-    return cached;
-}
-
+// Columns one segment launch covers: all of them, as tiles of one launch, while a 128-column tile of X fits the L2.
+// Beyond that each tile is a launch of its own, so that only one tile's rows compete for the cache at a time.
 int32_t segment_tile_width(const gnnpre_plan* P, int32_t width) {
-    if (!tile_uses_bulk_copy(P, 128)) return kMaxTile;
-    if (width > 256) return 128;
-    if (width > 128 && P->n * 512 > l2_cache_bytes()) return 4 * ((width / 4 + 1) / 2);
-    return kMaxTile;
+    if ((P->flags & GNNPRE_FLAG_NO_BULK_COPY) || P->n * 512 <= l2_cache_bytes()) return width;
+    return 4 * equal_tile_f4(width / 4);
 }
 
 }  // namespace
@@ -256,16 +271,13 @@ int launch_segments(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int6
         a.rscale = P->rscale.p;
         a.cscale = P->cscale.p;
         a.nzrows = P->nzrows.p;
-        a.f4 = w / 4;
+        a.rank_scale = P->rows_all_nonempty ? P->rscale.p : P->nzscale.p;
+        a.num_ranks = (int32_t)P->num_nonempty;
+        a.f4 = a.tile_f4 = w / 4;
         a.diag_weight = 1.0f + P->gin_eps;
         a.tp = teleport_of(P, h, f0);
         if (tile_uses_bulk_copy(P, w)) GNNPRE_TRY(launch_segments_tma(P, a, st));
-        else if (a.f4 <= 4) GNNPRE_TRY((launch_segments_shape<4, 1, 4>(P, a, st)));
-        else if (a.f4 <= 8) GNNPRE_TRY((launch_segments_shape<8, 1, 8>(P, a, st)));
-        else if (a.f4 <= 16) GNNPRE_TRY((launch_segments_shape<16, 1, 8>(P, a, st)));
-        else if (a.f4 <= 32) GNNPRE_TRY((launch_segments_shape<32, 1, GNNPRE_SEG_U>(P, a, st)));
-        else if (a.f4 <= 64) GNNPRE_TRY((launch_segments_shape<32, 2, 4>(P, a, st)));
-        else GNNPRE_TRY((launch_segments_shape<32, 4, 2>(P, a, st)));
+        else GNNPRE_TRY(launch_segments_gather(P, a, st));
     }
     return GNNPRE_OK;
 }
@@ -331,10 +343,10 @@ int launch_ceiling_tma(const gnnpre_plan* P, const SegArgs& a, float* sink, cuda
     return GNNPRE_OK;
 }
 
-template <int G, int V, int U>
+template <int G>
 int launch_ceiling_shape(const SegArgs& a, float* sink, cudaStream_t st) {
-    const unsigned grid = (unsigned)(((a.seg_hi - a.seg_lo) * G + kThreads - 1) / kThreads);
-    k_ceiling<G, V, U><<<grid, kThreads, 0, st>>>(a, sink);
+    const dim3 grid((unsigned)(((a.seg_hi - a.seg_lo) * G + kThreads - 1) / kThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
+    k_ceiling<G><<<grid, kThreads, 0, st>>>(a, sink);
     GNNPRE_CUDA(cudaGetLastError());
     return GNNPRE_OK;
 }
@@ -358,12 +370,13 @@ int launch_ceiling(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int64
             if (a.f4 == 25) GNNPRE_TRY(launch_ceiling_tma<25>(P, a, sink, st));
             else if (a.f4 == 32) GNNPRE_TRY(launch_ceiling_tma<32>(P, a, sink, st));
             else GNNPRE_TRY(launch_ceiling_tma<0>(P, a, sink, st));
-        } else if (a.f4 <= 4) GNNPRE_TRY((launch_ceiling_shape<4, 1, 4>(a, sink, st)));
-        else if (a.f4 <= 8) GNNPRE_TRY((launch_ceiling_shape<8, 1, 8>(a, sink, st)));
-        else if (a.f4 <= 16) GNNPRE_TRY((launch_ceiling_shape<16, 1, 8>(a, sink, st)));
-        else if (a.f4 <= 32) GNNPRE_TRY((launch_ceiling_shape<32, 1, GNNPRE_SEG_U>(a, sink, st)));
-        else if (a.f4 <= 64) GNNPRE_TRY((launch_ceiling_shape<32, 2, 4>(a, sink, st)));
-        else GNNPRE_TRY((launch_ceiling_shape<32, 4, 2>(a, sink, st)));
+        } else {
+            a.tile_f4 = equal_tile_f4(a.f4);
+            if (a.tile_f4 <= 4) GNNPRE_TRY(launch_ceiling_shape<4>(a, sink, st));
+            else if (a.tile_f4 <= 8) GNNPRE_TRY(launch_ceiling_shape<8>(a, sink, st));
+            else if (a.tile_f4 <= 16) GNNPRE_TRY(launch_ceiling_shape<16>(a, sink, st));
+            else GNNPRE_TRY(launch_ceiling_shape<32>(a, sink, st));
+        }
     }
     return GNNPRE_OK;
 }

@@ -1,159 +1,203 @@
 // Register-gather segment kernel.  Included by propagate.cu inside its unnamed namespace (uses segments_common.cuh).
 #pragma once
 
-// G lanes per segment, V float4 per lane (row width <= 4*G*V floats), U rows in flight per lane.
+// A group of G lanes walks one segment of the edge list; lane q of the group owns float4 q of the column tile, so a
+// tile is at most 4 G columns wide (wider rows are cut into equal tiles, blockIdx.y).
 //
-// Accumulation: the U rows of one step are added in a short plain fp32 chain, and that partial sum
-// enters the row's running sum by a compensated (Kahan) addition, so the rounding error of a row
-// stays at a few ulps of sum_j |w_j x_j| whatever its degree, at ~2 extra instructions per edge.
-#ifndef GNNPRE_SEG_U
-#define GNNPRE_SEG_U 8
-#endif
-#ifndef GNNPRE_SEG_MIN_BLOCKS
-#define GNNPRE_SEG_MIN_BLOCKS 3
-#endif
-template <int G, int V, int U, int OP, bool HAS_EMPTY, int EP>
-__global__ void __launch_bounds__(kThreads, G <= 4 ? 4 : GNNPRE_SEG_MIN_BLOCKS) k_segments(const SegArgs a) {
+// Column entries are taken G (at least 8) at a time, fetched one chunk ahead, and the group reads them back from
+// shared memory four to a 128-bit broadcast load, weights as ready-made pairs.  Eight neighbour rows are then
+// requested back to back (a "window"), summed in a plain fp32 chain, and that sum joins the row's running sum by a
+// compensated (Kahan) addition: rounding stays at a few ulps of sum_j |w_j x_j| whatever the row's length.  Windows
+// are counted from the segment's start and a row end closes the sum inside its window, so the order of the additions
+// depends on the segment alone - not on G, the tile, the launch or the other segments of the warp.
+//
+// Where every sum of a chunk goes is worked out by the lanes side by side when the chunk is staged (RowOut): a
+// finished row goes to its output row, the first sum to a scratch row if its row began in an earlier segment, and the
+// segment's last edge always closes a sum - into a scratch row if its row continues in the next segment.  What the
+// padding behind that edge adds is therefore never stored.
+//
+// Bound by what an SM can draw from the L2 (64 bytes per cycle: a loop that only gathers takes 59 us on 169 K nodes,
+// 2.3 M edges, 128 columns) and, on short rows, by the instructions around the row ends.  On that graph, us per launch,
+// before (rows of 68..128 columns through the copy engine, one shuffle per edge and operand elsewhere) / now: 128
+// columns GCN 148 / 109, mean 123 / 77; 64 columns GCN 105 / 71, mean 75 / 51; 16 columns GCN 45 / 39, mean 35 / 29;
+// 256 columns, sum operator 223 / 186.  A persistent grid, four rows in flight at 48 registers, and 256-thread CTAs were
+// each slower.
+constexpr int kSegWindow = 8;
+
+struct __align__(16) RowOut {
+    char* dst;    // first byte of this column tile in the row the sum goes to
+    float scale;  // r_i; 1 for a scratch row
+    int row;      // output row; -1 for a scratch row (no epilogue)
+};
+
+template <int G, bool WEIGHTED>
+struct __align__(16) SegStage {  // read in 16-byte pieces
+    static constexpr int kChunk = G < kSegWindow ? kSegWindow : G;  // edges staged at a time
+    RowOut out[kChunk];
+    uint32_t col[kChunk];
+    float2 w[WEIGHTED ? kChunk : 1];
+};
+
+template <int G, int OP, bool HAS_EMPTY, int EP>
+__global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
+    constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN;
+    using Stage = SegStage<G, kWeighted>;
+    constexpr int C = Stage::kChunk;
+    constexpr int M = C / G;  // entries per lane and chunk
+    __shared__ __align__(16) Stage stages[kSegThreads / G];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1);
     const int gshift = lane & ~(G - 1);
-    const unsigned glow = G == 32 ? kFull : ((1u << G) - 1u);
-    const unsigned gmask = glow << gshift;
-    const int64_t s = a.seg_lo + ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G;
+    constexpr unsigned kGroupLow = G == 32 ? kFull : ((1u << G) - 1u);
+    Stage& stage = stages[threadIdx.x / G];
+    const int64_t s = a.seg_lo + ((int64_t)blockIdx.x * kSegThreads + threadIdx.x) / G;
 
-    int64_t e = 0, e_end = 0;
-    int rank = 0, slot_head = -1, slot_tail = -1;
+    const int q0 = blockIdx.y * a.tile_f4;
+    const bool on = gl < min(a.tile_f4, a.f4 - q0);
+    // lanes beyond the row's width re-read its first float4: every load is unconditional and in bounds
+    const char* const xlane = reinterpret_cast<const char*>(a.x) + 16 * (q0 + (on ? gl : 0));
+    const uint32_t row_bytes = (uint32_t)a.ldx * 4u;
+    const int out_off = 16 * gl;
+
+    const uint32_t* entries = a.colx;
+    int left = 0, rank = 0, slot_head = -1, slot_tail = -1;
     if (s < a.seg_hi) {
         const Segment g = a.segs[s];
-        e = g.start;
-        e_end = a.segs[s + 1].start;
+        entries += g.start - a.colx_base;
+        left = (int)(a.segs[s + 1].start - g.start);
         rank = g.rank;
         slot_head = g.slot_head;
         slot_tail = g.slot_tail;
     }
-    // Lane gl owns float4 columns gl, gl + G, ...; lanes beyond the row's width re-read column 0 so
-    // that every load is unconditional and in bounds (their sums are never stored).
-    bool on[V];
-    const float4* xlane[V];
-    const uint32_t ldx4 = (uint32_t)(a.ldx >> 2);
+    uint32_t c_cur[M], c_next[M];
+    float w[M], scale[M];
+    int row[M];
+    auto fetch_rows = [&]() {  // rows and scales of the next C sums
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        const int q = gl + v * G;
-        on[v] = q < a.f4;
-        xlane[v] = reinterpret_cast<const float4*>(a.x) + (on[v] ? q : 0);
+        for (int m = 0; m < M; ++m) {
+            const int i = min(rank + gl + m * G, a.num_ranks - 1);
+            row[m] = HAS_EMPTY ? __ldg(a.nzrows + i) : i;
+            scale[m] = OP == GNNPRE_OP_GIN_SUM ? 1.f : __ldg(a.rank_scale + i);
+        }
+    };
+#pragma unroll
+    for (int m = 0; m < M; ++m) c_cur[m] = gl + m * G < left ? __ldg(entries + gl + m * G) : 0u;
+#pragma unroll
+    for (int m = 0; m < M; ++m) c_next[m] = gl + m * G + C < left ? __ldg(entries + gl + m * G + C) : 0u;
+    fetch_rows();
+    if (OP == GNNPRE_OP_GCN_SYM) {
+#pragma unroll
+        for (int m = 0; m < M; ++m) w[m] = __ldg(a.cscale + (c_cur[m] & ~kRowEndBit));
     }
-    bool head_pending = slot_head >= 0;  // the first row began in an earlier segment
-    bool open = false;                   // the last edge seen so far did not end its row
-    float4 acc[V], tot[V], cmp[V];       // this step's plain sum; the row's running sum and its compensation
-#pragma unroll
-    for (int v = 0; v < V; ++v) acc[v] = tot[v] = cmp[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    Quad acc = quad_zero(), tot = quad_zero(), cmp = quad_zero();  // this window's plain sum; the row's running sum
 
-    while (__any_sync(kFull, e < e_end)) {
-        // ---- this chunk's edges: lane gl of the group owns edge e + gl; lanes past the end hold 0,
-        // a valid column without a row-end mark
-        const int64_t left = e_end - e;
-        const int cnt = left >= G ? G : (left > 0 ? (int)left : 0);
-        uint32_t c = 0;
-        if (gl < cnt) c = a.colx[e + gl - a.colx_base];
-        const unsigned ends = (__ballot_sync(kFull, (c & kRowEndBit) != 0) >> gshift) & glow;
-        int my_row = rank + __popc(ends & ((1u << gl) - 1u));
-        float my_r = 1.f, w = 1.f;
-        if (c & kRowEndBit) {
-            if (HAS_EMPTY) my_row = a.nzrows[my_row];
-            if (OP != GNNPRE_OP_GIN_SUM) my_r = a.rscale[my_row];
+    while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
+        // ---- stage this chunk: lanes past the end hold column 0 without a row-end mark
+        unsigned ends = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+            ends |= ((__ballot_sync(kFull, (int)c_cur[m] < 0) >> gshift) & kGroupLow) << (m * G);
+        const int rank_after = rank + __popc(ends);
+        int slot_last = -1;  // scratch row of this chunk's last sum, if its row is cut by the segment's end
+        if (left > 0 && left <= C && ((ends >> (left - 1)) & 1u) == 0) {
+            slot_last = ends == 0 && slot_head >= 0 ? slot_head : slot_tail;
+            ends |= 1u << (left - 1);
         }
-        if (OP == GNNPRE_OP_GCN_SYM) {
-            w = a.cscale[c & ~kRowEndBit];
-        } else if (OP == GNNPRE_OP_GIN_SUM) {
-            w = (int)(c & ~kRowEndBit) == my_row ? a.diag_weight : 1.f;  // every row owns its self-loop: rank == row
+        const int last = __popc(ends) - 1;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const int i = gl + m * G;
+            const uint32_t col = c_cur[m] & ~kRowEndBit;
+            stage.col[i] = col;
+            // every row owns its self-loop, so the rank of a row is its index
+            if (OP == GNNPRE_OP_GIN_SUM)
+                w[m] = (int)col == rank + __popc(ends & ((1u << i) - 1u)) ? a.diag_weight : 1.f;
+            int slot = i == 0 ? slot_head : -1;
+            if (slot_last >= 0 && i == last) slot = slot_last;
+            RowOut o;
+            o.dst = reinterpret_cast<char*>(slot >= 0 ? a.scratch + (int64_t)slot * a.scratch_ld : a.out + (int64_t)row[m] * a.ldo) + 16 * q0;
+            o.scale = slot >= 0 ? 1.f : scale[m];
+            o.row = slot >= 0 ? -1 : row[m];
+            stage.out[i] = o;
         }
-        if (cnt > 0) open = ((ends >> (cnt - 1)) & 1u) == 0;  // the chunk's last edge does not end its row
-        const int cnt_max = G == 32 ? cnt : __reduce_max_sync(kFull, cnt);
+        if (ends != 0) slot_head = -1;
+        rank = rank_after;
+        entries += C;
+        left -= C;
+        float w_next[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            c_cur[m] = c_next[m];
+            c_next[m] = gl + m * G + C < left ? __ldg(entries + gl + m * G + C) : 0u;
+            if (OP == GNNPRE_OP_GCN_SYM) w_next[m] = __ldg(a.cscale + (c_cur[m] & ~kRowEndBit));
+        }
+        fetch_rows();
+        const int here = left + C;  // edges of this group from here to the segment's end
+        const int cnt = G == 32 ? min(here, C) : C == kSegWindow ? C : __reduce_max_sync(kFull, min(here, C));
+        const unsigned ends_any = G == 32 ? ends : __reduce_or_sync(kFull, ends);
+        const RowOut* out = stage.out;
+        EpiloguePiece<EP> piece;
+        __syncwarp();
+        if (EP != kEpPlain) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
 
-        // ---- gather and accumulate, U rows in flight
-        for (int t0 = 0; t0 < cnt_max; t0 += U) {
-            float4 x[U][V];
-            uint32_t craw[U];
-            // Four-lane groups also hand every edge's row and row scale around ahead of time: with eight groups in a
-            // warp a row ends somewhere in almost every step, and the two shuffles under a partial mask that a row end
-            // otherwise costs are dearer than two plain ones per edge (measured: faster at G = 4, slower at G = 8, 16).
-            constexpr bool kRowsAhead = G == 4;
-            int rowv[U];
-            float rv[U];
-            float wv[U];  // the edges' weights, handed to the group together with their column entries (whole-warp
-                          // shuffles outside any branch: a shuffle under a partial mask inside the per-edge
-                          // condition below cost the weighted operators half again the time of the unweighted one)
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                craw[u] = __shfl_sync(kFull, c, t0 + u, G);
-                if (OP != GNNPRE_OP_SAGE_MEAN) wv[u] = __shfl_sync(kFull, w, t0 + u, G);
-                if (kRowsAhead) {
-                    rowv[u] = __shfl_sync(kFull, my_row, t0 + u, G);
-                    rv[u] = __shfl_sync(kFull, my_r, t0 + u, G);
-                }
-                const uint64_t off = (uint64_t)(craw[u] & ~kRowEndBit) * ldx4;
-#pragma unroll
-                for (int v = 0; v < V; ++v) x[u][v] = __ldg(xlane[v] + off);
+        auto flush = [&]() {  // the last edge added closes a sum
+            const RowOut o = *out++;
+            quad_kahan(tot, cmp, acc);
+            float4 v = make_float4(tot.lo.x, tot.lo.y, tot.hi.x, tot.hi.y);
+            if (on) {
+                if (EP == kEpPlain || o.row < 0) v = make_float4(v.x * o.scale, v.y * o.scale, v.z * o.scale, v.w * o.scale);
+                else v = piece.finish(v, o.scale, a.tp, o.row, 4 * q0, gl);
+                *reinterpret_cast<float4*>(o.dst + out_off) = v;
             }
+            acc = tot = cmp = quad_zero();
+            if (EP != kEpPlain && out < stage.out + C) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
+        };
+
+#pragma unroll 1
+        for (int t0 = 0; t0 < cnt; t0 += kSegWindow) {
+            Quad x[kSegWindow];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int t = t0 + u;
-                if (t < cnt) {
-                    if (OP == GNNPRE_OP_SAGE_MEAN) {
+            for (int u = 0; u < kSegWindow; u += 4) {
+                const uint4 c = *reinterpret_cast<const uint4*>(&stage.col[t0 + u]);
+                x[u] = quad_gather(xlane, c.x, row_bytes);
+                x[u + 1] = quad_gather(xlane, c.y, row_bytes);
+                x[u + 2] = quad_gather(xlane, c.z, row_bytes);
+                x[u + 3] = quad_gather(xlane, c.w, row_bytes);
+            }
+            if (kWeighted && t0 == 0) {  // the weights follow behind the chunk's first row requests
 #pragma unroll
-                        for (int v = 0; v < V; ++v) {
-                            acc[v].x += x[u][v].x; acc[v].y += x[u][v].y;
-                            acc[v].z += x[u][v].z; acc[v].w += x[u][v].w;
-                        }
+                for (int m = 0; m < M; ++m) stage.w[gl + m * G] = make_float2(w[m], w[m]);
+                __syncwarp();
+            }
+            if (((ends_any >> t0) & 0xffu) == 0) {
+#pragma unroll
+                for (int u = 0; u < kSegWindow; u += 2) {
+                    if (kWeighted) {
+                        const float4 p = *reinterpret_cast<const float4*>(&stage.w[t0 + u]);
+                        quad_fma_pair(acc, make_float2(p.x, p.y), x[u]);
+                        quad_fma_pair(acc, make_float2(p.z, p.w), x[u + 1]);
                     } else {
-                        const float ww = wv[u];
-#pragma unroll
-                        for (int v = 0; v < V; ++v) {
-                            acc[v].x = fmaf(ww, x[u][v].x, acc[v].x); acc[v].y = fmaf(ww, x[u][v].y, acc[v].y);
-                            acc[v].z = fmaf(ww, x[u][v].z, acc[v].z); acc[v].w = fmaf(ww, x[u][v].w, acc[v].w);
-                        }
+                        quad_add(acc, x[u]);
+                        quad_add(acc, x[u + 1]);
                     }
                 }
-                if (craw[u] & kRowEndBit) {
-                    // last edge of a row (never set on a padding lane): the whole group arrives here together
-                    const int row = kRowsAhead ? rowv[u] : __shfl_sync(gmask, my_row, gshift + t);
-                    const float r = kRowsAhead ? rv[u] : __shfl_sync(gmask, my_r, gshift + t);
-                    const bool partial = head_pending;  // the row began earlier: leave the sum for the fix-up
-                    head_pending = false;
-                    float* dst = partial ? a.scratch + (int64_t)slot_head * a.scratch_ld : a.out + (int64_t)row * a.ldo;
+            } else {
+                const unsigned we = ends >> t0;
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        kahan4(tot[v], cmp[v], acc[v]);
-                        if (on[v])
-                            reinterpret_cast<float4*>(dst)[gl + v * G] =
-                                partial ? tot[v] : finish_row_piece<EP>(tot[v], r, a.tp, row, gl + v * G);
-                        acc[v] = tot[v] = cmp[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
+                for (int u = 0; u < kSegWindow; ++u) {
+                    if (kWeighted) quad_fma_pair(acc, stage.w[t0 + u], x[u]);
+                    else quad_add(acc, x[u]);
+                    if ((we >> u) & 1u) flush();
                 }
             }
-            if (t0 < cnt) {  // this step's plain sum joins the row's compensated sum (never on a padding
-                             // step: the result must not depend on which segment shares the warp)
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    kahan4(tot[v], cmp[v], acc[v]);
-                    acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
+            quad_kahan(tot, cmp, acc);
+            acc = quad_zero();
         }
-        rank += __popc(ends);
-        e += G;
-    }
-
-    // ---- the row holding the last edge continues in the next segment
-    if (open) {
-        const int slot = head_pending ? slot_head : slot_tail;
-        if (slot >= 0) {
-            float* dst = a.scratch + (int64_t)slot * a.scratch_ld;
+        __syncwarp();
+        if (OP == GNNPRE_OP_GCN_SYM) {
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (on[v]) reinterpret_cast<float4*>(dst)[gl + v * G] = tot[v];
+            for (int m = 0; m < M; ++m) w[m] = w_next[m];
         }
     }
 }
-

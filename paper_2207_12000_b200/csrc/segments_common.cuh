@@ -19,32 +19,45 @@ struct Teleport {
 // optional code slowed the plain kernels down although its branches were never taken (the L2-resident workload by
 // 10 % for the teleport term and by 40 % for the sum).
 constexpr int kEpPlain = 0, kEpTeleport = 1, kEpSum = 2;
+// What the epilogue of one row reads besides its sum (column tile at f0, float4 q); loaded before the sum is complete
+// where the kernel knows the row ahead of time.
+template <int EP>
+struct EpiloguePiece {
+    float4 x0, z;
+    __device__ __forceinline__ void load(const Teleport& tp, int64_t row, int f0, int q, bool on) {
+        if (EP == kEpPlain || !on) return;
+        if (EP == kEpTeleport || tp.alpha != 0.f || tp.zsum_first)
+            x0 = __ldg(reinterpret_cast<const float4*>(tp.x0 + row * tp.ldx0 + f0) + q);
+        if (EP == kEpSum && !tp.zsum_first) z = *(reinterpret_cast<const float4*>(tp.zsum + row * tp.ldz + f0) + q);
+    }
+    // the value to store for the row; adds it to the sum of hops (every finished row piece passes here once per hop)
+    __device__ __forceinline__ float4 finish(const float4& sum, float scale, const Teleport& tp, int64_t row, int f0, int q) const {
+        float4 o = make_float4(sum.x * scale, sum.y * scale, sum.z * scale, sum.w * scale);
+        if (EP == kEpTeleport || (EP == kEpSum && tp.alpha != 0.f)) {
+            o.x = fmaf(tp.keep, o.x, tp.alpha * x0.x);
+            o.y = fmaf(tp.keep, o.y, tp.alpha * x0.y);
+            o.z = fmaf(tp.keep, o.z, tp.alpha * x0.z);
+            o.w = fmaf(tp.keep, o.w, tp.alpha * x0.w);
+        }
+        if (EP == kEpSum) {
+            float4 acc = z;
+            if (tp.zsum_first) acc = make_float4(tp.gamma0 * x0.x, tp.gamma0 * x0.y, tp.gamma0 * x0.z, tp.gamma0 * x0.w);
+            acc.x = fmaf(tp.gamma, o.x, acc.x);
+            acc.y = fmaf(tp.gamma, o.y, acc.y);
+            acc.z = fmaf(tp.gamma, o.z, acc.z);
+            acc.w = fmaf(tp.gamma, o.w, acc.w);
+            *(reinterpret_cast<float4*>(tp.zsum + row * tp.ldz + f0) + q) = acc;
+        }
+        return o;
+    }
+};
+
+// Both at once, for a row whose sum is already there.
 template <int EP>
 __device__ __forceinline__ float4 finish_row_piece(float4 sum, float scale, const Teleport& tp, int64_t row, int q) {
-    float4 o = make_float4(sum.x * scale, sum.y * scale, sum.z * scale, sum.w * scale);
-    if (EP == kEpTeleport || (EP == kEpSum && tp.alpha != 0.f)) {
-        const float4 z = __ldg(reinterpret_cast<const float4*>(tp.x0 + row * tp.ldx0) + q);
-        o.x = fmaf(tp.keep, o.x, tp.alpha * z.x);
-        o.y = fmaf(tp.keep, o.y, tp.alpha * z.y);
-        o.z = fmaf(tp.keep, o.z, tp.alpha * z.z);
-        o.w = fmaf(tp.keep, o.w, tp.alpha * z.w);
-    }
-    if (EP == kEpSum) {  // every finished row piece passes here exactly once per hop
-        float4* zp = reinterpret_cast<float4*>(tp.zsum + row * tp.ldz) + q;
-        float4 acc;
-        if (tp.zsum_first) {
-            const float4 x = __ldg(reinterpret_cast<const float4*>(tp.x0 + row * tp.ldx0) + q);
-            acc = make_float4(tp.gamma0 * x.x, tp.gamma0 * x.y, tp.gamma0 * x.z, tp.gamma0 * x.w);
-        } else {
-            acc = *zp;
-        }
-        acc.x = fmaf(tp.gamma, o.x, acc.x);
-        acc.y = fmaf(tp.gamma, o.y, acc.y);
-        acc.z = fmaf(tp.gamma, o.z, acc.z);
-        acc.w = fmaf(tp.gamma, o.w, acc.w);
-        *zp = acc;
-    }
-    return o;
+    EpiloguePiece<EP> piece;
+    piece.load(tp, row, 0, q, true);
+    return piece.finish(sum, scale, tp, row, 0, q);
 }
 
 // Which epilogue a launch needs.
@@ -63,11 +76,62 @@ struct SegArgs {
     int64_t scratch_ld;
     const float* rscale;
     const float* cscale;
+    const float* rank_scale;  // row scales in rank order: rank_scale[k] = rscale[row of rank k]
     const int32_t* nzrows;
-    int32_t f4;  // float4 per row of this column tile
+    int32_t num_ranks;  // rows that own an edge
+    int32_t f4;         // float4 per row of this launch's columns
+    int32_t tile_f4;    // float4 per row of one column tile (register kernel: tile blockIdx.y)
     float diag_weight;  // GIN: 1 + eps
     Teleport tp;
 };
+
+// A float4 handled as two packed pairs: Blackwell adds and multiplies two fp32 per instruction
+// (add/fma .f32x2).  Each lane of each pair is an ordinary IEEE operation, so results equal the scalar
+// code's bit for bit.
+struct Quad {
+    float2 lo, hi;
+};
+
+__device__ __forceinline__ Quad quad_zero() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+
+__device__ __forceinline__ Quad quad_load(const unsigned char* p) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+
+__device__ __forceinline__ void quad_add(Quad& a, const Quad& x) {
+    a.lo = __fadd2_rn(a.lo, x.lo);
+    a.hi = __fadd2_rn(a.hi, x.hi);
+}
+
+// w holds the weight twice
+__device__ __forceinline__ void quad_fma_pair(Quad& a, float2 w, const Quad& x) {
+    a.lo = __ffma2_rn(w, x.lo, a.lo);
+    a.hi = __ffma2_rn(w, x.hi, a.hi);
+}
+
+__device__ __forceinline__ void quad_fma(Quad& a, float w, const Quad& x) { quad_fma_pair(a, make_float2(w, w), x); }
+
+// float4 of row `col` through the read-only path; `base` points at this lane's piece of row 0
+__device__ __forceinline__ Quad quad_gather(const char* base, uint32_t col, uint32_t row_bytes) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(base + (uint64_t)col * row_bytes));
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+
+// Compensated addition of x into (sum, comp), as kahan1 does per component: a - b is evaluated as
+// fma(-1, b, a), which rounds the same.
+__device__ __forceinline__ void kahan_pair(float2& sum, float2& comp, const float2& x) {
+    const float2 neg = make_float2(-1.f, -1.f);
+    const float2 y = __ffma2_rn(neg, comp, x);
+    const float2 t = __fadd2_rn(sum, y);
+    comp = __ffma2_rn(neg, y, __ffma2_rn(neg, sum, t));
+    sum = t;
+}
+
+__device__ __forceinline__ void quad_kahan(Quad& sum, Quad& comp, const Quad& x) {
+    kahan_pair(sum.lo, comp.lo, x.lo);
+    kahan_pair(sum.hi, comp.hi, x.hi);
+}
 
 // Compensated (Kahan) addition of x into the pair (sum, comp): the low-order bits that the addition
 // drops are carried in comp.
@@ -86,5 +150,12 @@ __device__ __forceinline__ void kahan4(float4& sum, float4& comp, const float4& 
 }
 
 constexpr int kThreads = 256;
+// Register segment kernel: 14 CTAs of two warps per SM, i.e. 72 registers per thread.  Small CTAs, because segments
+// differ in length and a finished warp's place should not wait for seven others.
+constexpr int kSegThreads = 64;
+#ifndef GNNPRE_SEG_BLOCKS
+#define GNNPRE_SEG_BLOCKS 14
+#endif
+constexpr int kSegBlocks = GNNPRE_SEG_BLOCKS;
 constexpr int kMaxDevices = 64;
 

@@ -88,46 +88,6 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* tma
         : "memory");
 }
 
-// A float4 handled as two packed pairs: Blackwell adds and multiplies two fp32 per instruction
-// (add/fma .f32x2).  Each lane of each pair is an ordinary IEEE operation, so results equal the scalar
-// code's bit for bit.
-struct Quad {
-    float2 lo, hi;
-};
-
-__device__ __forceinline__ Quad quad_zero() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-
-__device__ __forceinline__ Quad quad_load(const unsigned char* p) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
-}
-
-__device__ __forceinline__ void quad_add(Quad& a, const Quad& x) {
-    a.lo = __fadd2_rn(a.lo, x.lo);
-    a.hi = __fadd2_rn(a.hi, x.hi);
-}
-
-__device__ __forceinline__ void quad_fma(Quad& a, float w, const Quad& x) {
-    const float2 ww = make_float2(w, w);
-    a.lo = __ffma2_rn(ww, x.lo, a.lo);
-    a.hi = __ffma2_rn(ww, x.hi, a.hi);
-}
-
-// Compensated addition of x into (sum, comp), as kahan1 does per component: a - b is evaluated as
-// fma(-1, b, a), which rounds the same.
-__device__ __forceinline__ void kahan_pair(float2& sum, float2& comp, const float2& x) {
-    const float2 neg = make_float2(-1.f, -1.f);
-    const float2 y = __ffma2_rn(neg, comp, x);
-    const float2 t = __fadd2_rn(sum, y);
-    comp = __ffma2_rn(neg, y, __ffma2_rn(neg, sum, t));
-    sum = t;
-}
-
-__device__ __forceinline__ void quad_kahan(Quad& sum, Quad& comp, const Quad& x) {
-    kahan_pair(sum.lo, comp.lo, x.lo);
-    kahan_pair(sum.hi, comp.hi, x.hi);
-}
-
 // Per-stage bookkeeping a warp keeps in registers between issuing a chunk and summing it.
 struct TmaChunk {
     uint32_t c;      // this lane's column entry (row-end mark in bit 31); 0 on padding lanes

@@ -348,6 +348,33 @@ def test_bulk_copy_kernel_matches_register_kernel_bitwise(B, op, F):
     check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), to_np(X), res[0])
 
 
+@pytest.mark.parametrize("op,F", [(0, 100), (1, 100), (1, 128), (2, 124)])
+def test_bulk_copy_kernel_on_a_dense_graph_far_larger_than_the_cache(B, op, F):
+    """The copy engine takes over when X is more than four times the L2 and rows are long; same segments, same order of
+    additions, so the register kernel must give the same bits."""
+    g = gi.rmat(1500000, 25000000, 29, directed_candidates=False, device="cuda")
+    X = gi.normal_matrix(g.n, F, 9, device="cuda")
+    res = []
+    for flags in (0, B.GNNPRE_FLAG_NO_BULK_COPY):
+        plan = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, gin_eps=EPS, force_blocks=2, segment_edges=1000, flags=flags)
+        res.append(B.gnnpre_propagate(plan, X, 1)[0][0])
+        torch.cuda.synchronize()
+        plan.close()
+    assert torch.equal(res[0], res[1])
+
+
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132, 260])
+@pytest.mark.parametrize("seg", [1, 7, 8, 9, 31, 33])
+def test_register_kernel_tile_and_segment_edges(B, op, F, seg):
+    """Widths around the lane-group and column-tile sizes, segments around the window and chunk sizes; rows of every
+    length from none to several segments, with the segment's last edge ending its row or not."""
+    n = 90
+    edges = [(i, j) for i in range(0, n, 7) for j in range(i + 1, min(n, i + 1 + 2 * i))]
+    g = gi.from_edge_list(n, edges)
+    run_case(B, g, op, F, 2, b=3, seg=seg)
+
+
 def test_two_tile_rows_on_a_graph_larger_than_the_cache(B):
     """Rows of 132..256 columns are cut into two equal tiles for the copy engine once a 128-column tile of X no
     longer fits the L2 (here 400,000 nodes: 205 MB per tile; F = 200 gives two tiles of 100 columns, F = 252 two of
