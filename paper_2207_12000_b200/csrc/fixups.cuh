@@ -1,5 +1,5 @@
-// Kernels that finish what the segment kernels leave: rows cut by segment boundaries, and rows without edges.
-// Included by propagate.cu inside its unnamed namespace (uses Teleport, finish_row_piece, kahan4, kThreads).
+// The kernel that finishes what the segment kernels leave: rows cut by segment boundaries, and rows without edges.
+// Included by propagate.cu inside its unnamed namespace (uses segments_common.cuh).
 #pragma once
 
 struct FixArgs {
@@ -8,12 +8,16 @@ struct FixArgs {
     const int32_t* hubs;     // fix-ups with more than hub_parts parts: entries [hub_lo, hub_hi) lie in [fix_lo, fix_hi)
     int64_t hub_lo, hub_hi;
     int32_t hub_parts;
+    const int32_t* emptyrows;  // rows without any edge (SAGE, D_i = 0); num_empty = 0 leaves them alone
+    int64_t num_empty;
     const float* scratch;
     int64_t scratch_ld;
     const float* rscale;
     float* out;
     int64_t ldo;
-    int32_t f4;
+    int32_t f4;       // float4 per row of this launch's columns
+    int32_t tile_f4;  // float4 per row of one column tile (tile blockIdx.y)
+    bool back_to_back;  // see launch_dependent
     Teleport tp;
 };
 
@@ -34,145 +38,131 @@ __device__ __forceinline__ void pair_add4(float4& s, float4& e, const float4& t,
     pair_add1(s.w, e.w, t.w, f.w);
 }
 
-// Adds up the parts of the cut rows.  A row's parts are P consecutive scratch rows; they are summed as a tree of
-// fixed shape, so the result is the same from run to run, and - for tiles of up to 128 columns - the same whatever
-// the tile width, so that a matrix cut into column tiles or slabs of any widths comes out bit-identical:
+// Adds up the parts of the cut rows, and writes the rows without edges.
+// A row's parts are P consecutive scratch rows; they are summed as a tree of fixed shape, so the result is the same
+// from run to run and whatever the tile width, so that a matrix cut into column tiles or slabs of any widths comes out
+// bit-identical:
 //   - chain c of C adds parts c, c + C, c + 2C, ... in that order with compensated additions, its loads issued
 //     a batch ahead of its adds; the chains' sums (compensation folded in) then meet pairwise (c with c^1, then c^2,
 //     then c^4), each carried as a value and an error term;
-//   - an ordinary row gets one warp and C = 8 chains: a group of G lanes covers the row's width, so a warp holds
-//     32 / G groups and every lane carries G / 4 chains (tiles wider than 128 columns, V > 1: one chain per warp);
+//   - an ordinary row gets one warp and C = 8 chains: a group of G lanes covers the tile's width, so a warp holds
+//     32 / G groups and every lane carries G / 4 chains;
 //   - a hub row (P > hub_parts, listed by the plan) gets a whole CTA, C = 64 chains (8 per warp): the warps'
 //     sums meet in shared memory and warp 0 adds them in warp order.
-// The first (hub_hi - hub_lo) CTAs of the grid take the hubs, the others eight ordinary rows each.
-template <int G, int V, int EP>
-__global__ void __launch_bounds__(kThreads) k_row_fixups(const FixArgs a) {
+// The first (hub_hi - hub_lo) CTAs of the grid take the hubs, the next ones eight ordinary rows each, the rest the
+// rows without edges (zero, or alpha * X_0[i] with a teleport term), kEmptyPerGroup to a lane group.
+// Bound by latency: two dependent loads per row, and most rows have two or three parts.  A lane keeps at most eight
+// parts in flight (with sixteen the kernel held 98 to 174 registers and ran narrow rows in five waves), and the row's
+// place and scale are fetched while the segment kernel still runs.  169 K nodes, 16 columns, mean operator, three
+// hops: 146 -> 100 us a call (three launches per hop before, each after the end of the one before it).
+constexpr int kEmptyPerGroup = 16;
+
+template <int G, int EP>
+__global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
     constexpr int kWarps = kThreads / 32;
-    constexpr int S = 32 / G;                  // lane groups per warp
-    constexpr int CH = V == 1 ? G / 4 : 1;     // chains per lane
-    constexpr int CW = S * CH;                 // chains per warp: 8, or 1 for wide tiles
-    constexpr int kRounds = 16 / (CH * V);     // 16 float4 of parts in flight per lane
-    __shared__ float4 meet[kWarps][2][G * V];
+    constexpr int S = 32 / G;                         // lane groups per warp
+    constexpr int CH = G / 4;                         // chains per lane
+    constexpr int CW = S * CH;                        // chains per warp
+    constexpr int kRounds = CH >= 8 ? 1 : CH >= 4 ? 2 : 4;  // parts in flight per chain
+    static_assert(CW == 8, "the tree's shape must not depend on the width");
+    __shared__ float4 meet[kWarps][2][G];
+    allow_next_kernel();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gl = lane & (G - 1), sub = lane / G;
+    const int q0 = blockIdx.y * a.tile_f4;
+    const bool on = gl < min(a.tile_f4, a.f4 - q0);
     const int64_t nhub = a.hub_hi - a.hub_lo;
+    const int64_t ordinary = (a.fix_hi - a.fix_lo + kWarps - 1) / kWarps;
+    if ((int64_t)blockIdx.x >= nhub + ordinary) {
+        const int64_t i0 = ((int64_t)blockIdx.x - nhub - ordinary) * (kThreads / G * kEmptyPerGroup) + threadIdx.x / G;
+        int row[kEmptyPerGroup];
+#pragma unroll
+        for (int k = 0; k < kEmptyPerGroup; ++k) {
+            const int64_t i = i0 + k * (kThreads / G);
+            row[k] = i < a.num_empty ? a.emptyrows[i] : -1;
+        }
+        wait_previous_kernel();
+#pragma unroll
+        for (int k = 0; k < kEmptyPerGroup; ++k)
+            if (row[k] >= 0 && on)
+                *(reinterpret_cast<float4*>(a.out + (int64_t)row[k] * a.ldo) + q0 + gl) =
+                    finish_row_piece<EP>(make_float4(0.f, 0.f, 0.f, 0.f), 0.f, a.tp, row[k], q0 + gl);
+        return;
+    }
     const bool hub_cta = (int64_t)blockIdx.x < nhub;
     const int64_t i = hub_cta ? (int64_t)a.hubs[a.hub_lo + blockIdx.x]
                               : a.fix_lo + ((int64_t)blockIdx.x - nhub) * kWarps + warp;
     const int chains = hub_cta ? CW * kWarps : CW;           // chains that share the row
     const int chain0 = (hub_cta ? warp * CW : 0) + sub * CH;  // this lane's first chain
     int parts = 0, row = 0;
-    const float* base = a.scratch;
+    float scale = 0.f;
+    const float* base = a.scratch + 4 * (q0 + (on ? gl : 0));
     if (i < a.fix_hi) {
         const RowFixup f = a.fix[i];
         parts = f.seg_last - f.seg_first + 1;
         row = f.row;
+        scale = a.rscale[row];
         base += (int64_t)f.slot0 * a.scratch_ld;
     }
     const bool mine = i < a.fix_hi && (hub_cta || parts <= a.hub_parts);  // hubs are left to their CTAs
     if (!mine) parts = 0;
-    bool on[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) on[v] = gl + v * G < a.f4;
+    wait_previous_kernel();
 
-    float4 acc[CH][V], cmp[CH][V];
+    float4 acc[CH], cmp[CH];
 #pragma unroll
-    for (int j = 0; j < CH; ++j)
-#pragma unroll
-        for (int v = 0; v < V; ++v) acc[j][v] = cmp[j][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < CH; ++j) acc[j] = cmp[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int p0 = 0; p0 < parts; p0 += chains * kRounds) {
-        float4 part[kRounds][CH][V];
+        float4 part[kRounds][CH];
 #pragma unroll
         for (int r = 0; r < kRounds; ++r) {
 #pragma unroll
             for (int j = 0; j < CH; ++j) {
                 const int p = p0 + r * chains + chain0 + j;
-                const float* src = base + (int64_t)(p < parts ? p : 0) * a.scratch_ld;
-#pragma unroll
-                for (int v = 0; v < V; ++v)
-                    part[r][j][v] = p < parts && on[v] ? *reinterpret_cast<const float4*>(src + 4 * (gl + v * G))
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+                part[r][j] = p < parts ? *reinterpret_cast<const float4*>(base + (int64_t)p * a.scratch_ld)
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
 #pragma unroll
         for (int r = 0; r < kRounds; ++r) {
 #pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                if (p0 + r * chains + chain0 + j < parts) {
-#pragma unroll
-                    for (int v = 0; v < V; ++v) kahan4(acc[j][v], cmp[j][v], part[r][j][v]);
-                }
-            }
+            for (int j = 0; j < CH; ++j)
+                if (p0 + r * chains + chain0 + j < parts) kahan4(acc[j], cmp[j], part[r][j]);
         }
     }
     // The chains meet pairwise, first inside the lane (chains chain0 .. chain0 + CH - 1), then across the lane
     // groups of the warp.  A hub's partial sums can be far larger than their total (40,000 terms of either sign), so
     // every sum travels as a pair (value, error term) and each pairwise addition keeps its exact rounding error.
-    float4 tot[V], err[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
+    for (int j = 0; j < CH; ++j)  // a compensated sum stands for acc - cmp
+        cmp[j] = make_float4(-cmp[j].x, -cmp[j].y, -cmp[j].z, -cmp[j].w);
 #pragma unroll
-        for (int j = 0; j < CH; ++j)  // a compensated sum stands for acc - cmp
-            cmp[j][v] = make_float4(-cmp[j][v].x, -cmp[j][v].y, -cmp[j][v].z, -cmp[j][v].w);
+    for (int step = 1; step < CH; step <<= 1) {
 #pragma unroll
-        for (int step = 1; step < CH; step <<= 1) {
+        for (int j = 0; j < CH; j += 2 * step) pair_add4(acc[j], cmp[j], acc[j + step], cmp[j + step]);
+    }
+    float4 tot = acc[0], err = cmp[0];
 #pragma unroll
-            for (int j = 0; j < CH; j += 2 * step) pair_add4(acc[j][v], cmp[j][v], acc[j + step][v], cmp[j + step][v]);
-        }
-        tot[v] = acc[0][v];
-        err[v] = cmp[0][v];
-#pragma unroll
-        for (int off = G; off < 32; off <<= 1) {
-            float4 os, oe;
-            os.x = __shfl_xor_sync(kFull, tot[v].x, off); os.y = __shfl_xor_sync(kFull, tot[v].y, off);
-            os.z = __shfl_xor_sync(kFull, tot[v].z, off); os.w = __shfl_xor_sync(kFull, tot[v].w, off);
-            oe.x = __shfl_xor_sync(kFull, err[v].x, off); oe.y = __shfl_xor_sync(kFull, err[v].y, off);
-            oe.z = __shfl_xor_sync(kFull, err[v].z, off); oe.w = __shfl_xor_sync(kFull, err[v].w, off);
-            pair_add4(tot[v], err[v], os, oe);
-        }
+    for (int off = G; off < 32; off <<= 1) {
+        float4 os, oe;
+        os.x = __shfl_xor_sync(kFull, tot.x, off); os.y = __shfl_xor_sync(kFull, tot.y, off);
+        os.z = __shfl_xor_sync(kFull, tot.z, off); os.w = __shfl_xor_sync(kFull, tot.w, off);
+        oe.x = __shfl_xor_sync(kFull, err.x, off); oe.y = __shfl_xor_sync(kFull, err.y, off);
+        oe.z = __shfl_xor_sync(kFull, err.z, off); oe.w = __shfl_xor_sync(kFull, err.w, off);
+        pair_add4(tot, err, os, oe);
     }
     if (hub_cta) {  // uniform over the CTA
         if (sub == 0) {
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                meet[warp][0][gl + v * G] = tot[v];
-                meet[warp][1][gl + v * G] = err[v];
-            }
+            meet[warp][0][gl] = tot;
+            meet[warp][1][gl] = err;
         }
         __syncthreads();
         if (warp != 0) return;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            tot[v] = meet[0][0][gl + v * G];
-            err[v] = meet[0][1][gl + v * G];
-            for (int w = 1; w < kWarps; ++w) pair_add4(tot[v], err[v], meet[w][0][gl + v * G], meet[w][1][gl + v * G]);
-        }
+        tot = meet[0][0][gl];
+        err = meet[0][1][gl];
+        for (int w = 1; w < kWarps; ++w) pair_add4(tot, err, meet[w][0][gl], meet[w][1][gl]);
     }
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        tot[v].x += err[v].x; tot[v].y += err[v].y; tot[v].z += err[v].z; tot[v].w += err[v].w;
-    }
-    if (mine && sub == 0) {
-        const float r = a.rscale[row];
-        float* dst = a.out + (int64_t)row * a.ldo;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const int q = gl + v * G;
-            if (on[v]) *reinterpret_cast<float4*>(dst + 4 * q) = finish_row_piece<EP>(tot[v], r, a.tp, row, q);
-        }
-    }
+    tot.x += err.x; tot.y += err.y; tot.z += err.z; tot.w += err.w;
+    if (mine && sub == 0 && on)
+        *(reinterpret_cast<float4*>(a.out + (int64_t)row * a.ldo) + q0 + gl) = finish_row_piece<EP>(tot, scale, a.tp, row, q0 + gl);
 }
-
-// Rows without any edge (SAGE, D_i = 0) are zero rows of the result.
-// (With a teleport term they keep alpha * X_0[i].)
-template <int EP>
-__global__ void k_zero_rows(const int32_t* __restrict__ rows, int64_t count, float* __restrict__ out, int64_t ldo,
-                            int32_t f4, const Teleport tp) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count * f4) return;
-    const int64_t r = rows[t / f4];
-    const int q = (int)(t % f4);
-    *reinterpret_cast<float4*>(out + r * ldo + 4 * q) = finish_row_piece<EP>(make_float4(0.f, 0.f, 0.f, 0.f), 0.f, tp, r, q);
-}
-

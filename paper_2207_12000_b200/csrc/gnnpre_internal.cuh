@@ -214,13 +214,14 @@ struct HopArgs {
     float gamma = 0.f;       // weight of the hop being computed
     float gamma0 = 0.f;      // weight of X_0
     bool zsum_first = false; // first hop: Z starts from gamma0 * X_0 instead of its old value
+    bool back_to_back = false;  // nothing but this library's kernels between this call's launches on the stream
 };
 
 // propagate.cu
 int launch_segments(const gnnpre_plan* plan, const HopArgs& a, int64_t seg_lo, int64_t seg_hi, cudaStream_t stream);
-int launch_fixups(const gnnpre_plan* plan, const HopArgs& a, int64_t fix_lo, int64_t fix_hi, int64_t hub_lo, int64_t hub_hi,
-                  cudaStream_t stream);
-int launch_zero_empty_rows(const gnnpre_plan* plan, const HopArgs& a, cudaStream_t stream);
+// The cut rows of a fix-up range and, with `empty_rows`, the rows without edges; one launch if there is anything to do.
+int launch_finish(const gnnpre_plan* plan, const HopArgs& a, int64_t fix_lo, int64_t fix_hi, int64_t hub_lo, int64_t hub_hi,
+                  bool empty_rows, int64_t* launches, cudaStream_t stream);
 struct WeightedSum {         // optional extra output of propagate_resident
     const float* gamma;      // host, K + 1 weights
     float* Z;                // device [n, ldz]

@@ -343,13 +343,10 @@ __global__ void k_hub_scatter(int64_t nfix, const int32_t* __restrict__ flag, co
     if (i < nfix && flag[i]) hubs[scan[i]] = (int32_t)i;
 }
 
-// Parts beyond which a cut row counts as a hub and gets a whole CTA of the fix-up kernel (64 chains) instead of a
-// warp (8 chains).  One value for all widths up to 128 columns, because the tree's shape decides the bits and
-// those must not depend on how a matrix is cut into column tiles; wider tiles hold fewer parts per batch of loads.
-int32_t hub_parts_for(int64_t width) {
-    const int64_t f4 = std::min<int64_t>(std::max<int64_t>(width, 4), 512) / 4;
-    return f4 <= 32 ? 64 : f4 <= 64 ? 32 : 16;
-}
+// Parts beyond which a cut row counts as a hub and gets a whole CTA of the finishing kernel (64 chains) instead of a
+// warp (8 chains).  One value for all widths, because the tree's shape decides the bits and those must not depend on
+// how a matrix is cut into column tiles.
+constexpr int32_t kHubParts = 64;
 
 __global__ void k_clear_pad(int64_t nseg, Segment* __restrict__ segs) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -722,7 +719,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     GNNPRE_CUDA(cudaMemcpy(fix_at.data(), d_fix_at.p, sizeof(int32_t) * (size_t)(b + 1), cudaMemcpyDeviceToHost));
 
     // hub rows (more parts than a warp adds quickly) are listed so that the fix-up kernel can give each a CTA
-    P->hub_parts = hub_parts_for(P->slab_width);
+    P->hub_parts = kHubParts;
     std::vector<int32_t> hub_at((size_t)b + 1, 0);
     if (n_fix > 0) {
         DevBuf<int32_t> hub_flag, hub_scan, d_hub_at;

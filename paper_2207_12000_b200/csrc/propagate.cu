@@ -9,9 +9,10 @@
 // coalesced load, then gathers the neighbours' feature rows with 128-bit loads, several rows in
 // flight per lane, and accumulates in fp32 registers.  Bit 31 of a column entry marks the last edge
 // of a row: there the group scales the sum by r_i and stores the output row.  Rows cut by a segment
-// boundary leave their partial sums in scratch rows, which k_row_fixups adds up in a fixed order.
+// boundary leave their partial sums in scratch rows, which k_finish_rows adds up in a fixed order.
 #include <algorithm>
 #include <atomic>
+#include <utility>
 
 #include "gnnpre_internal.cuh"
 
@@ -44,22 +45,21 @@ int launch_segments_shape(const gnnpre_plan* P, const SegArgs& a, cudaStream_t s
     const int64_t groups = a.seg_hi - a.seg_lo;
     const dim3 grid((unsigned)((groups * G + kSegThreads - 1) / kSegThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
     const int ep = epilogue_of(a.tp);
-#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                    \
-    do {                                                                                                       \
-        if (ep == kEpSum) k_segments<G, OP_, EMPTY_, kEpSum><<<grid, kSegThreads, 0, st>>>(a);                 \
-        else if (ep == kEpTeleport) k_segments<G, OP_, EMPTY_, kEpTeleport><<<grid, kSegThreads, 0, st>>>(a);  \
-        else k_segments<G, OP_, EMPTY_, kEpPlain><<<grid, kSegThreads, 0, st>>>(a);                            \
+#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                                    \
+    do {                                                                                                                       \
+        if (ep == kEpSum) return launch_dependent(k_segments<G, OP_, EMPTY_, kEpSum>, grid, kSegThreads, 0, a.back_to_back, st, a); \
+        if (ep == kEpTeleport)                                                                                                 \
+            return launch_dependent(k_segments<G, OP_, EMPTY_, kEpTeleport>, grid, kSegThreads, 0, a.back_to_back, st, a);     \
+        return launch_dependent(k_segments<G, OP_, EMPTY_, kEpPlain>, grid, kSegThreads, 0, a.back_to_back, st, a);            \
     } while (0)
     switch (P->op) {
-    case GNNPRE_OP_GCN_SYM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GCN_SYM, false); break;
-    case GNNPRE_OP_GIN_SUM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GIN_SUM, false); break;
+    case GNNPRE_OP_GCN_SYM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GCN_SYM, false);
+    case GNNPRE_OP_GIN_SUM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GIN_SUM, false);
     default:
         if (P->rows_all_nonempty) GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_SAGE_MEAN, false);
-        else GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_SAGE_MEAN, true);
+        GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_SAGE_MEAN, true);
     }
 #undef GNNPRE_LAUNCH_SEGMENTS
-    GNNPRE_CUDA(cudaGetLastError());
-    return GNNPRE_OK;
 }
 
 // Float4 per column tile of the register kernels: equal tiles of at most 128 columns.
@@ -154,9 +154,7 @@ int launch_segments_tma_width(const gnnpre_plan* P, const SegArgs& a, cudaStream
     }
     const int64_t nseg = a.seg_hi - a.seg_lo;
     const unsigned grid = (unsigned)std::min<int64_t>(P->num_sms, (nseg + nwarps - 1) / nwarps);
-    kernel<<<grid, nwarps * 32, smem, st>>>(a, *tmap, P->dev_error.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    return GNNPRE_OK;
+    return launch_dependent(kernel, dim3(grid), (unsigned)(nwarps * 32), smem, a.back_to_back, st, a, *tmap, P->dev_error.p);
 }
 
 // Rows (or column tiles) of 100 and of 128 columns get kernels with the row size compiled in.
@@ -180,19 +178,17 @@ int launch_segments_tma(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st)
     }
 }
 
-template <int G, int V>
-int launch_fixups_shape(const FixArgs& a, cudaStream_t st) {
-    const int64_t rows_per_cta = kThreads / 32;
-    const unsigned grid = (unsigned)((a.hub_hi - a.hub_lo) + (a.fix_hi - a.fix_lo + rows_per_cta - 1) / rows_per_cta);
+template <int G>
+int launch_finish_shape(const FixArgs& a, cudaStream_t st) {
+    const int64_t rows_per_cta = kThreads / 32, empty_per_cta = kThreads / G * kEmptyPerGroup;
+    const int64_t ctas = (a.hub_hi - a.hub_lo) + (a.fix_hi - a.fix_lo + rows_per_cta - 1) / rows_per_cta +
+                         (a.num_empty + empty_per_cta - 1) / empty_per_cta;
+    const dim3 grid((unsigned)ctas, (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
     const int ep = epilogue_of(a.tp);
-    if (ep == kEpSum) k_row_fixups<G, V, kEpSum><<<grid, kThreads, 0, st>>>(a);
-    else if (ep == kEpTeleport) k_row_fixups<G, V, kEpTeleport><<<grid, kThreads, 0, st>>>(a);
-    else k_row_fixups<G, V, kEpPlain><<<grid, kThreads, 0, st>>>(a);
-    GNNPRE_CUDA(cudaGetLastError());
-    return GNNPRE_OK;
+    if (ep == kEpSum) return launch_dependent(k_finish_rows<G, kEpSum>, grid, kThreads, 0, a.back_to_back, st, a);
+    if (ep == kEpTeleport) return launch_dependent(k_finish_rows<G, kEpTeleport>, grid, kThreads, 0, a.back_to_back, st, a);
+    return launch_dependent(k_finish_rows<G, kEpPlain>, grid, kThreads, 0, a.back_to_back, st, a);
 }
-
-constexpr int kMaxTile = 512;  // columns one launch covers (G = 32, V = 4)
 
 Teleport teleport_of(const gnnpre_plan* P, const HopArgs& h, int32_t f0) {
     Teleport tp;
@@ -276,54 +272,40 @@ int launch_segments(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int6
         a.f4 = a.tile_f4 = w / 4;
         a.diag_weight = 1.0f + P->gin_eps;
         a.tp = teleport_of(P, h, f0);
+        a.back_to_back = h.back_to_back;
         if (tile_uses_bulk_copy(P, w)) GNNPRE_TRY(launch_segments_tma(P, a, st));
         else GNNPRE_TRY(launch_segments_gather(P, a, st));
     }
     return GNNPRE_OK;
 }
 
-int launch_fixups(const gnnpre_plan* P, const HopArgs& h, int64_t fix_lo, int64_t fix_hi, int64_t hub_lo, int64_t hub_hi,
-                  cudaStream_t st) {
-    if (fix_hi <= fix_lo) return GNNPRE_OK;
-    for (int32_t f0 = 0; f0 < h.width; f0 += kMaxTile) {
-        const int32_t w = std::min<int32_t>(kMaxTile, h.width - f0);
-        FixArgs a;
-        a.fix = P->fixups.p;
-        a.fix_lo = fix_lo;
-        a.fix_hi = fix_hi;
-        a.hubs = P->hubs.p;
-        a.hub_lo = hub_lo;
-        a.hub_hi = hub_hi;
-        a.hub_parts = P->hub_parts;
-        a.scratch = P->scratch.p + f0;
-        a.scratch_ld = P->slab_width;
-        a.rscale = P->rscale.p;
-        a.out = h.xout + f0;
-        a.ldo = h.ldo;
-        a.f4 = w / 4;
-        a.tp = teleport_of(P, h, f0);
-        if (a.f4 <= 4) GNNPRE_TRY((launch_fixups_shape<4, 1>(a, st)));
-        else if (a.f4 <= 8) GNNPRE_TRY((launch_fixups_shape<8, 1>(a, st)));
-        else if (a.f4 <= 16) GNNPRE_TRY((launch_fixups_shape<16, 1>(a, st)));
-        else if (a.f4 <= 32) GNNPRE_TRY((launch_fixups_shape<32, 1>(a, st)));
-        else if (a.f4 <= 64) GNNPRE_TRY((launch_fixups_shape<32, 2>(a, st)));
-        else GNNPRE_TRY((launch_fixups_shape<32, 4>(a, st)));
-    }
-    return GNNPRE_OK;
-}
-
-int launch_zero_empty_rows(const gnnpre_plan* P, const HopArgs& h, cudaStream_t st) {
-    if (P->num_empty == 0) return GNNPRE_OK;
-    const int32_t f4 = h.width / 4;
-    const int64_t items = P->num_empty * f4;
-    const Teleport tp = teleport_of(P, h, 0);
-    const unsigned grid = (unsigned)((items + 255) / 256);
-    const int ep = epilogue_of(tp);
-    if (ep == kEpSum) k_zero_rows<kEpSum><<<grid, 256, 0, st>>>(P->emptyrows.p, P->num_empty, h.xout, h.ldo, f4, tp);
-    else if (ep == kEpTeleport) k_zero_rows<kEpTeleport><<<grid, 256, 0, st>>>(P->emptyrows.p, P->num_empty, h.xout, h.ldo, f4, tp);
-    else k_zero_rows<kEpPlain><<<grid, 256, 0, st>>>(P->emptyrows.p, P->num_empty, h.xout, h.ldo, f4, tp);
-    GNNPRE_CUDA(cudaGetLastError());
-    return GNNPRE_OK;
+int launch_finish(const gnnpre_plan* P, const HopArgs& h, int64_t fix_lo, int64_t fix_hi, int64_t hub_lo, int64_t hub_hi,
+                  bool empty_rows, int64_t* launches, cudaStream_t st) {
+    FixArgs a;
+    a.num_empty = empty_rows ? P->num_empty : 0;
+    if (fix_hi <= fix_lo && a.num_empty == 0) return GNNPRE_OK;
+    a.fix = P->fixups.p;
+    a.fix_lo = fix_lo;
+    a.fix_hi = fix_hi;
+    a.hubs = P->hubs.p;
+    a.hub_lo = hub_lo;
+    a.hub_hi = hub_hi;
+    a.hub_parts = P->hub_parts;
+    a.emptyrows = P->emptyrows.p;
+    a.scratch = P->scratch.p;
+    a.scratch_ld = P->slab_width;
+    a.rscale = P->rscale.p;
+    a.out = h.xout;
+    a.ldo = h.ldo;
+    a.f4 = h.width / 4;
+    a.tile_f4 = equal_tile_f4(a.f4);
+    a.back_to_back = h.back_to_back;
+    a.tp = teleport_of(P, h, 0);
+    ++*launches;
+    if (a.tile_f4 <= 4) return launch_finish_shape<4>(a, st);
+    if (a.tile_f4 <= 8) return launch_finish_shape<8>(a, st);
+    if (a.tile_f4 <= 16) return launch_finish_shape<16>(a, st);
+    return launch_finish_shape<32>(a, st);
 }
 
 namespace {
@@ -413,6 +395,7 @@ int propagate_resident(gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, f
             h.xout = out[k] + f_lo;
             h.ldo = ldo;
             h.width = (int32_t)std::min<int64_t>(P->slab_width, P->feat_dim - f_lo);
+            h.back_to_back = true;
             if (wsum) {
                 h.zsum = wsum->Z + f_lo;
                 h.ldz = wsum->ldz;
@@ -420,11 +403,8 @@ int propagate_resident(gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, f
                 h.gamma0 = wsum->gamma[0];
                 h.zsum_first = k == 0;
             }
-            const int tiles = (h.width + kMaxTile - 1) / kMaxTile;
             const int seg_tile = segment_tile_width(P, h.width);
             const int seg_tiles = (h.width + seg_tile - 1) / seg_tile;
-            rc = launch_zero_empty_rows(P, h, st);
-            launches += P->num_empty ? 1 : 0;
             const bool per_block = (P->flags & GNNPRE_FLAG_LAUNCH_PER_BLOCK) != 0;
             const size_t groups = per_block ? P->blocks.size() : 1;
             for (size_t j = 0; j < groups && rc == GNNPRE_OK; ++j) {
@@ -441,10 +421,7 @@ int propagate_resident(gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, f
                     launches += seg_tiles;
                     seg_launches += seg_tiles;
                 }
-                if (rc == GNNPRE_OK && fix_hi > fix_lo) {
-                    rc = launch_fixups(P, h, fix_lo, fix_hi, hub_lo, hub_hi, st);
-                    launches += tiles;
-                }
+                if (rc == GNNPRE_OK) rc = launch_finish(P, h, fix_lo, fix_hi, hub_lo, hub_hi, j == 0, &launches, st);
             }
         }
         if (rc == GNNPRE_OK) rc = mark(hop_ev);

@@ -40,6 +40,7 @@ struct __align__(16) SegStage {  // read in 16-byte pieces
 
 template <int G, int OP, bool HAS_EMPTY, int EP>
 __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
+    allow_next_kernel();
     constexpr unsigned kFull = 0xffffffffu;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN;
     using Stage = SegStage<G, kWeighted>;
@@ -91,6 +92,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
         for (int m = 0; m < M; ++m) w[m] = __ldg(a.cscale + (c_cur[m] & ~kRowEndBit));
     }
     Quad acc = quad_zero(), tot = quad_zero(), cmp = quad_zero();  // this window's plain sum; the row's running sum
+    wait_previous_kernel();
 
     while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
         // ---- stage this chunk: lanes past the end hold column 0 without a row-end mark

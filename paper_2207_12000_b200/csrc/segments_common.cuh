@@ -81,6 +81,7 @@ struct SegArgs {
     int32_t num_ranks;  // rows that own an edge
     int32_t f4;         // float4 per row of this launch's columns
     int32_t tile_f4;    // float4 per row of one column tile (register kernel: tile blockIdx.y)
+    bool back_to_back;  // see launch_dependent
     float diag_weight;  // GIN: 1 + eps
     Teleport tp;
 };
@@ -131,6 +132,32 @@ __device__ __forceinline__ void kahan_pair(float2& sum, float2& comp, const floa
 __device__ __forceinline__ void quad_kahan(Quad& sum, Quad& comp, const Quad& x) {
     kahan_pair(sum.lo, comp.lo, x.lo);
     kahan_pair(sum.hi, comp.hi, x.hi);
+}
+
+// Programmatic dependent launch: the kernels of a resident call follow one another in a stream, and each is launched
+// while the one before it still runs.  What a kernel reads of the plan's own tables it may read at once;
+// wait_previous_kernel() comes before its first access to a matrix or to scratch rows and returns when the previous
+// kernel has completed and its stores are visible; every thread of every kernel passes it, so the guarantee carries
+// over to the kernels before that one.  Both are no-ops in a kernel launched without the attribute, as the streamed
+// schedules launch theirs: there copies on other streams bring the tables and matrices in.
+__device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+int launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, bool overlap, cudaStream_t st,
+                     Args&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    GNNPRE_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+    return GNNPRE_OK;
 }
 
 // Compensated (Kahan) addition of x into the pair (sum, comp): the low-order bits that the addition

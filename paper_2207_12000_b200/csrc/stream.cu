@@ -269,14 +269,12 @@ int run_slabs(gnnpre_plan* P, const float* X, int64_t ldx, bool x_host, int32_t 
             h.width = (int32_t)width;
             h.colx = P->colx.p;
             h.colx_edge_base = 0;
-            GNNPRE_TRY(launch_zero_empty_rows(P, h, P->s_compute));
-            launches += P->num_empty ? 1 : 0;
             for (size_t j = 0; j < P->blocks.size(); ++j) {
                 const Block& B = P->blocks[j];
                 GNNPRE_TRY(stager.stage(j, &h));
                 GNNPRE_TRY(launch_segments(P, h, B.seg_lo, B.seg_hi, P->s_compute));
-                GNNPRE_TRY(launch_fixups(P, h, B.fix_lo, B.fix_hi, B.hub_lo, B.hub_hi, P->s_compute));
-                launches += (B.seg_hi > B.seg_lo) + (B.fix_hi > B.fix_lo);
+                GNNPRE_TRY(launch_finish(P, h, B.fix_lo, B.fix_hi, B.hub_lo, B.hub_hi, j == 0, &launches, P->s_compute));
+                launches += B.seg_hi > B.seg_lo;
                 cudaEvent_t done = nullptr;
                 GNNPRE_TRY(ev.record(P->s_compute, &done));
                 stager.launched(j, done);
@@ -447,17 +445,15 @@ int run_panels(gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, float* co
         h.width = job.hi - job.lo;
         h.colx = P->colx.p;
         h.colx_edge_base = 0;
-        GNNPRE_TRY(launch_zero_empty_rows(P, h, P->s_compute));
-        launches += P->num_empty ? 1 : 0;
         for (size_t j = 0; j < P->blocks.size(); ++j) {
             const Block& B = P->blocks[j];
             GNNPRE_TRY(stager.stage(j, &h));
             const int kspan = j == 0 || j + 1 == P->blocks.size()
                                   ? trace.open(P->s_compute, "hop %lld cols %lld.. block %lld", job.k, job.lo, (long long)j) : -1;
             GNNPRE_TRY(launch_segments(P, h, B.seg_lo, B.seg_hi, P->s_compute));
-            GNNPRE_TRY(launch_fixups(P, h, B.fix_lo, B.fix_hi, B.hub_lo, B.hub_hi, P->s_compute));
+            GNNPRE_TRY(launch_finish(P, h, B.fix_lo, B.fix_hi, B.hub_lo, B.hub_hi, j == 0, &launches, P->s_compute));
             trace.close(P->s_compute, kspan);
-            launches += (B.seg_hi > B.seg_lo) + (B.fix_hi > B.fix_lo);
+            launches += B.seg_hi > B.seg_lo;
             cudaEvent_t done = nullptr;
             GNNPRE_TRY(ev.record(P->s_compute, &done));
             stager.launched(j, done);
