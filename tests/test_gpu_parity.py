@@ -426,6 +426,21 @@ def test_normalized_adjacency_values_bit_exact(B, op):
             hplan.close()
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("seg", [1, 31, 33, 127, 128, 129, 300])
+def test_normalized_values_at_segment_edges(B, op, seg):
+    """The values kernel walks segments 128 edges at a time: segment lengths around its chunks, rows without edges,
+    a hub of degree 5,000, bit for bit."""
+    g = gi.from_edge_list(5200, [(0, j) for j in range(100, 5100)] + [(j, j + 3) for j in range(200, 900)])
+    want = orc.normalized_values(op, EPS, g.rowptr.numpy(), g.colidx.numpy()).astype(np.float32)
+    for b in (1, 4):
+        plan = B.gnnpre_build_plan(*dev(g), op, 16, gin_eps=EPS, force_blocks=b, segment_edges=seg)
+        got = B.gnnpre_normalize(plan)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(to_np(got).view(np.uint32), want.view(np.uint32))
+        plan.close()
+
+
 def test_a_device_wait_that_runs_out_is_reported_and_leaves_the_plan_usable(B):
     """Failure detection without a fault: a warp polls a barrier that nothing completes, gives up after its
     limit and sets the plan's error word; the host reads GNNPRE_ERR_TIMEOUT once, and the same plan then
