@@ -7,8 +7,10 @@
 //   warps 0-3  producers.  Per K-chunk of 32 features they gather the 128 batch rows of the tile straight
 //            out of the hop matrix into the 128-byte-swizzled operand layout with 16-byte asynchronous
 //            copies (cp.async: no registers, zero fill past the last feature and for rows outside the
-//            batch), keep three chunks in flight beyond the one they announce, and arrive on the stage's
-//            `full` mbarrier after a proxy fence.  (Tensor copies in tile::gather4 mode were measured
+//            batch); the copies themselves arrive on the stage's `full` mbarrier when they have landed, so all
+//            free stages are in flight.  The proxy fence is the MMA warp's: in the copying threads it waits for
+//            everything they still have in flight, whatever the depth of the ring (2.4 M rows x 3 hops, F = 100,
+//            hidden 256, random order: 2111 us with the fence there, 1905 us here).  (Tensor copies in tile::gather4 mode were measured
 //            first: at 128 bytes per gathered row the copy engine's per-row rate, about 95 rows per
 //            microsecond and SM, capped the kernel at 60 % of what the output stores alone sustain.)
 //            The weight travels by tiled tensor copies, counted in bytes on an mbarrier.
@@ -47,7 +49,6 @@ namespace {
 constexpr int kLcTileM = 128;                     // batch rows per tile = accumulator lanes
 constexpr int kLcChunk = 32;                      // features per stage: 32 fp32 = one 128-byte swizzle row
 constexpr int kLcMaxStages = 8;
-constexpr int kLcLookahead = 3;                   // chunks a producer thread keeps in flight beyond the one it announces
 constexpr int kLcPipeBytes = 192 * 1024;          // operand stages plus, when it fits, the resident weight
 constexpr int kLcResidentMax = 128 * 1024;        // largest weight kept in shared memory for the whole launch
 constexpr int kLcEpiBytes = 32 * 128;             // one [32, 32] fp32 output box
@@ -57,6 +58,12 @@ constexpr int kLcProducerWarps = 4;
 constexpr int kLcProducerThreads = 32 * kLcProducerWarps;
 constexpr int kLcMmaWarp = kLcProducerWarps;       // warps: 0-3 producers, 4 MMA, 5-12 epilogue
 constexpr int kLcThreads = 32 * (kLcProducerWarps + 1 + 8);
+constexpr int kLcX3EpilogueWarps = 4;              // split-operand kernel: four epilogue warps, 16 KB more for operands
+constexpr int kLcX3SplitWarps = 4;                 // warps that compute the low parts: 9-12
+constexpr int kLcX3SplitWarp0 = kLcProducerWarps + 1 + kLcX3EpilogueWarps;
+constexpr int kLcX3Threads = 32 * (kLcX3SplitWarp0 + kLcX3SplitWarps);
+constexpr int kLcX3MaxStages = 5;
+constexpr int kLcSmemBytes = 225 * 1024;          // operands, weight and output boxes, besides 1 KB of alignment
 constexpr int kLcMaxHops = 8;                     // hop matrices per launch
 constexpr uint32_t kLcTmemCols = 512;
 constexpr uint32_t kLcSuspendNs = 20000;          // a failed poll parks the warp for up to this long
@@ -90,7 +97,8 @@ struct LcArgs {
     int64_t ldw;
     int32_t halves;        // column parts: CTAs with blockIdx.x % halves == h compute columns [h n_half, (h + 1) n_half)
     int32_t n_half;
-    uint32_t small_off;    // offset of the low parts inside a stage
+    uint32_t small_off;    // offset of the buffers of low parts
+    int32_t low_buffers;
     // failure-detection self-test: the producers never announce a chunk, so every wait runs out
     int32_t drop_announcements;
     uint32_t spin_limit;   // polls before a wait gives up
@@ -141,6 +149,11 @@ __device__ __forceinline__ bool lc_wait(uint32_t bar, uint32_t parity, volatile 
 // read, the rest of the 16 bytes is written as zeros.
 __device__ __forceinline__ void lc_copy16(uint32_t dst, const float* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+
+// Arrives on `bar` (one of its expected arrivals) once every copy this thread has issued so far has landed.
+__device__ __forceinline__ void lc_copies_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void lc_tile_load(uint32_t dst, const CUtensorMap* tmap, int x0, int y0, uint32_t bar) {
@@ -205,14 +218,16 @@ __device__ __forceinline__ void lc_tile_store(const CUtensorMap* tmap, int x0, i
                  : "memory");
 }
 
-// Epilogue role (warps 5-12), shared by both kernels: tiles first, first + step, ...; the accumulator holds
-// n_cols columns that go to columns col0 .. col0 + n_cols of Y.  Two warps per quarter of the accumulator's
-// lanes: the first four epilogue warps take the even 32-column boxes, the last four the odd ones.
+// Epilogue role (the warps after the MMA warp), shared by both kernels: tiles first, first + step, ...; the accumulator
+// holds n_cols columns that go to columns col0 .. col0 + n_cols of Y.  WARPS / 4 warps per quarter of the accumulator's
+// lanes share its 32-column boxes in turn.
+template <int WARPS>
 __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a, uint32_t tiles0, uint32_t tmem_base,
                                             uint32_t acc_full0, uint32_t acc_empty0, volatile int* abort_flag, int first,
                                             int step, int n_cols, int col0) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ew = warp - kLcMmaWarp - 1;  // 0..7
+    constexpr int kTurn = WARPS / 4;
+    const int ew = warp - kLcMmaWarp - 1;  // 0 .. WARPS - 1
     const int q = warp & 3;                // tensor-memory lanes 32q .. 32q+31 are the ones this warp may read
     const int half = ew >> 2;
     const uint32_t box = tiles0 + a.epi_off + (uint32_t)ew * kLcEpiBytes;
@@ -227,13 +242,13 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const bool relu = (a.relu_mask >> hop) & 1u;
         const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)buf * kLcMaxHidden;
-        // the read of box i + 2 is in flight while box i is written out
+        // the read of the next box is in flight while box i is written out
         uint32_t v[2][32];
         if (half < boxes) lc_tmem_load32(taddr + 32u * half, v[0]);
 #pragma unroll 2
-        for (int i = half, u = 0; i < boxes; i += 2, u ^= 1) {
+        for (int i = half, u = 0; i < boxes; i += kTurn, u ^= 1) {
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (i + 2 < boxes) lc_tmem_load32(taddr + 32u * (i + 2), v[u ^ 1]);
+            if (i + kTurn < boxes) lc_tmem_load32(taddr + 32u * (i + kTurn), v[u ^ 1]);
             // the previous store must have read the staging box before it is overwritten
             if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncwarp();
@@ -328,8 +343,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
         const int row0 = 32 * warp + (lane >> 3);            // this thread's rows: row0 + 4 i, i < 8
         int s = 0;           // stage the next chunk goes to
         uint32_t ph = 0;
-        int s_done = 0;      // stage whose copies are announced next
-        uint32_t issued = 0, announced = 0;
+        uint32_t issued = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const int hop = t / a.tiles_m, mt = t - hop * a.tiles_m;
@@ -359,7 +373,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
                     const bool live = src_row[i] != nullptr && bytes != 0;
                     lc_copy16(dst, live ? src_row[i] + col : a.hop[hop], live ? bytes : 0u);
                 }
-                asm volatile("cp.async.commit_group;" ::: "memory");
+                if (!a.drop_announcements) lc_copies_arrive(full_bar(s));
                 if (!a.w_resident && pt == 0) {
                     lc_mbar_arrive_expect_tx(full_bar(s), w_chunk_bytes);
                     lc_tile_load(a_dst + kLcABytes, &maps.w, kc * kLcChunk, 0, full_bar(s));
@@ -369,24 +383,9 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
                     s = 0;
                     ph ^= 1u;
                 }
-                if (issued - announced > (uint32_t)kLcLookahead) {
-                    // all but the newest kLcLookahead groups have landed: hand the oldest to the MMA warp
-                    asm volatile("cp.async.wait_group %0;" ::"n"(kLcLookahead) : "memory");
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    if (!a.drop_announcements) lc_mbar_arrive(full_bar(s_done));
-                    ++announced;
-                    if (++s_done == a.stages) s_done = 0;
-                }
             }
         }
-        // the tail: everything still in flight lands, then the remaining chunks are announced
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        while (announced < issued) {
-            if (!a.drop_announcements) lc_mbar_arrive(full_bar(s_done));
-            ++announced;
-            if (++s_done == a.stages) s_done = 0;
-        }
+        asm volatile("cp.async.wait_all;" ::: "memory");  // nothing may land after this CTA has left
         // tensor copies of the weight land in this CTA's shared memory: wait for them before leaving
         if (pt == 0) {
             if (a.w_resident) {
@@ -421,6 +420,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
                         ok = false;
                         break;
                     }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies, seen by the tensor core
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t a_src = tiles0 + (uint32_t)s * a.stage_stride;
                     const uint32_t b_src = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * w_chunk_bytes : a_src + kLcABytes;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
         __syncwarp();
     } else {
         // ---------------------------------------------------------------- epilogue
-        lc_epilogue(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, blockIdx.x, gridDim.x,
+        lc_epilogue<8>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, blockIdx.x, gridDim.x,
                     a.hidden, 0);
     }
 
@@ -463,27 +463,32 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // below 2^-21 |x||w|.  Shared memory has to hold both parts of both operands, so a CTA computes at most
 // 128 output columns: with hidden > 128, even and odd CTAs take the two column halves and every batch row is
 // gathered once per part (the later reads mostly hit L2).  No tensor copies on the input side: the producer
-// threads bring rows of the hop matrix AND rows of the weight in with 16-byte asynchronous copies,
-// then read their own pieces back, split them and write the two parts (each thread touches only bytes
-// it copied itself, so the copy's wait_group is all the synchronisation the split needs).
-__device__ __forceinline__ void lc_split_piece(uint32_t big_addr, uint32_t small_addr) {
-    // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
-    // enters a product as 1), so the tile as it was copied already acts as the high part; only the low part
-    // is computed and stored.
-    uint32_t v[4];
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(big_addr) : "memory");
+// threads bring rows of the hop matrix AND rows of the weight in with 16-byte asynchronous copies; four warps of their own
+// (9-12) read each stage that has landed and write its low parts into one of two further buffers.  When the copying
+// threads did that themselves they also had to fence, and so waited for all their copies in flight: 4587 us against 3550
+// (2.4 M rows x 3 hops, F = 100, hidden 256, random order), 1540 against 908 (500 K rows x 2, F = 256).
+// K-steps of the last chunk beyond the features are neither copied nor multiplied.
+//
+// The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
+// enters a product as 1), so the tile as it was copied already acts as the high part; only the low part
+// is computed and stored.
+__device__ __forceinline__ void lc_load_piece(uint32_t (&v)[4], uint32_t addr) {
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
+}
+
+__device__ __forceinline__ void lc_store_low_part(const uint32_t (&v)[4], uint32_t addr) {
     uint32_t lo[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const uint32_t hi = v[j] & 0xffffe000u;
         lo[j] = __float_as_uint(__uint_as_float(v[j]) - __uint_as_float(hi));  // exact; read by the tensor core as tf32
     }
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(small_addr), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]) : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]) : "memory");
 }
 
-__global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __grid_constant__ LcMaps maps, const LcArgs a) {
+__global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __grid_constant__ LcMaps maps, const LcArgs a) {
     extern __shared__ unsigned char lc_smem[];
-    __shared__ __align__(8) unsigned long long bars[2 * kLcMaxStages + 6];
+    __shared__ __align__(8) unsigned long long bars[4 * kLcMaxStages + 6];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int* abort_flag = &abort_word;
@@ -492,20 +497,24 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
     const uint32_t tiles0 = (lc_smem_u32(lc_smem) + 1023u) & ~1023u;
     const uint32_t bar0 = lc_smem_u32(&bars[0]);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (kLcMaxStages + s); };
-    auto acc_full_bar = [&](int b) { return bar0 + 8u * (2 * kLcMaxStages + b); };
-    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (2 * kLcMaxStages + 2 + b); };
-    const uint32_t drain_bar = bar0 + 8u * (2 * kLcMaxStages + 4);
-    const uint32_t w_bar = bar0 + 8u * (2 * kLcMaxStages + 5);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kLcMaxStages + s); };           // a stage's copied (high) part is free
+    auto low_empty_bar = [&](int l) { return bar0 + 8u * (2 * kLcMaxStages + l); };  // a buffer of low parts is free
+    auto copied_bar = [&](int s) { return bar0 + 8u * (3 * kLcMaxStages + s); };      // a stage's copies have landed
+    auto acc_full_bar = [&](int b) { return bar0 + 8u * (4 * kLcMaxStages + b); };
+    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (4 * kLcMaxStages + 2 + b); };
+    const uint32_t drain_bar = bar0 + 8u * (4 * kLcMaxStages + 4);
+    const uint32_t w_bar = bar0 + 8u * (4 * kLcMaxStages + 5);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kLcMaxStages; ++s) {
-            lc_mbar_init(full_bar(s), kLcProducerThreads);
+            lc_mbar_init(copied_bar(s), kLcProducerThreads);
+            lc_mbar_init(full_bar(s), kLcX3SplitWarps);  // a stage's low parts are there as well
             lc_mbar_init(empty_bar(s), 1);
+            lc_mbar_init(low_empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             lc_mbar_init(acc_full_bar(b), 1);
-            lc_mbar_init(acc_empty_bar(b), 8);
+            lc_mbar_init(acc_empty_bar(b), kLcX3EpilogueWarps);
         }
         lc_mbar_init(drain_bar, 1);
         lc_mbar_init(w_bar, kLcProducerThreads);
@@ -529,10 +538,27 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
     constexpr uint32_t kPart = kLcABytes;               // bytes of one part of the rows' chunk: [128, 32] floats
     const uint32_t w_part = (uint32_t)a.n_half * 128u;  // bytes of one part of the weight's chunk: [n_half, 32] floats
 
+    const uint32_t low0 = tiles0 + a.small_off;  // buffers of low parts, as large as a stage each
+    // K-steps of 8 features in chunk kc: 16-byte pieces beyond them are neither copied nor multiplied
+    auto k_steps = [&](int kc) { return min(4, (a.feat_dim - kc * kLcChunk + 7) >> 3); };
+
+    // Eight consecutive lanes take the eight 16-byte pieces of one row's chunk; four producer or splitter warps take 32
+    // rows each, a thread eight of them (of the tile and of the weight part): row0 + 4 i.
+    const int piece = lane & 7;
+    const int row0 = 32 * (warp & 3) + (lane >> 3);
+    auto split_part = [&](int kc, uint32_t big_part, uint32_t small_part, int row_limit) {
+        if (piece >= 2 * k_steps(kc)) return;
+        uint32_t v[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (row0 + 4 * i < row_limit) lc_load_piece(v[i], big_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (row0 + 4 * i < row_limit) lc_store_low_part(v[i], small_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
+    };
+
     if (warp < kLcProducerWarps) {
         // ---------------------------------------------------------------- producers
-        const int piece = lane & 7;
-        const int row0 = 32 * warp + (lane >> 3);  // this thread's rows (of the tile and of the weight half): row0 + 4 i
         const float* w_row[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -545,6 +571,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
             const int col = kc * kLcChunk + 4 * piece;
             const int left = a.feat_dim - col;
             const uint32_t bytes = left >= 4 ? 16u : left > 0 ? 4u * left : 0u;
+            if (piece >= 2 * k_steps(kc)) return;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int row = row0 + 4 * i;
@@ -554,38 +581,19 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
                 lc_copy16(dst, live ? rows[i] + col : a.wt, live ? bytes : 0u);
             }
         };
-        auto split_part = [&](uint32_t big_part, uint32_t small_part, int row_limit) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int row = row0 + 4 * i;
-                if (row >= row_limit) continue;
-                const uint32_t off = 128u * row + ((uint32_t)(piece ^ (row & 7)) << 4);
-                lc_split_piece(big_part + off, small_part + off);
-            }
-        };
         if (a.w_resident) {  // the weight half, once: both parts stay in shared memory for every tile
             for (int kc = 0; kc < a.k_chunks; ++kc) copy_chunk(w_row, kc, tiles0 + a.w_off + (uint32_t)kc * 2u * w_part, a.n_half);
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             for (int kc = 0; kc < a.k_chunks; ++kc) {
                 const uint32_t wb = tiles0 + a.w_off + (uint32_t)kc * 2u * w_part;
-                split_part(wb, wb + w_part, a.n_half);
+                split_part(kc, wb, wb + w_part, a.n_half);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             lc_mbar_arrive(w_bar);
         }
-        const uint32_t lookahead = (uint32_t)a.stages - 1u;  // 1, 2 or 3
-        int s = 0, s_done = 0;
-        uint32_t ph = 0, issued = 0, announced = 0;
-        auto announce = [&]() {  // the oldest unannounced chunk has landed: split it and hand it to the MMA warp
-            const uint32_t base = tiles0 + (uint32_t)s_done * a.stage_stride;
-            split_part(base, base + a.small_off, kLcTileM);
-            if (!a.w_resident) split_part(base + kPart, base + a.small_off + kPart, a.n_half);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            lc_mbar_arrive(full_bar(s_done));
-            ++announced;
-            if (++s_done == a.stages) s_done = 0;
-        };
+        int s = 0;
+        uint32_t ph = 0;
         bool ok = true;
         for (int t = first; t < total_tiles && ok; t += step) {
             const int hop = t / a.tiles_m, mt = t - hop * a.tiles_m;
@@ -605,31 +613,19 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
                 const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
                 copy_chunk(src_row, kc, base, kLcTileM);
                 if (!a.w_resident) copy_chunk(w_row, kc, base + kPart, a.n_half);
-                asm volatile("cp.async.commit_group;" ::: "memory");
-                ++issued;
+                lc_copies_arrive(copied_bar(s));
                 if (++s == a.stages) {
                     s = 0;
                     ph ^= 1u;
                 }
-                if (issued - announced > lookahead) {
-                    if (lookahead == 1u) {
-                        asm volatile("cp.async.wait_group 1;" ::: "memory");
-                    } else if (lookahead == 2u) {
-                        asm volatile("cp.async.wait_group 2;" ::: "memory");
-                    } else {
-                        asm volatile("cp.async.wait_group 3;" ::: "memory");
-                    }
-                    announce();
-                }
             }
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        while (announced < issued) announce();
+        asm volatile("cp.async.wait_all;" ::: "memory");  // nothing may land after this CTA has left
     } else if (warp == kLcMmaWarp) {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
             const uint32_t idesc = lc_instr_desc(a.n_half);
-            int s = 0, it = 0;
+            int s = 0, it = 0, low = 0;
             uint32_t ph = 0;
             bool ok = !a.w_resident || lc_wait(w_bar, 0, abort_flag, a.error, a.spin_limit);
             for (int t = first; t < total_tiles && ok; t += step, ++it) {
@@ -643,20 +639,24 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
                         ok = false;
                         break;
                     }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // both parts, seen by the tensor core
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
-                    const uint32_t xh = base, xl = base + a.small_off;
+                    const uint32_t small = low0 + (uint32_t)low * a.stage_stride;
+                    const uint32_t xh = base, xl = small;
                     const uint32_t wh = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart;
-                    const uint32_t wl = a.w_resident ? wh + w_part : base + a.small_off + kPart;
-#pragma unroll
-                    for (int j = 0; j < kLcChunk / 8; ++j) {
+                    const uint32_t wl = a.w_resident ? wh + w_part : small + kPart;
+                    const int steps = k_steps(kc);
+                    for (int j = 0; j < steps; ++j) {
                         const uint32_t o = 32u * j;
                         // small terms first, the leading term last
                         lc_mma_tf32(tmem_d, lc_operand_desc(xl + o), lc_operand_desc(wh + o), idesc, (kc | j) != 0);
                         lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wl + o), idesc, 1u);
                         lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wh + o), idesc, 1u);
                     }
+                    lc_mma_commit(low_empty_bar(low));
                     lc_mma_commit(empty_bar(s));
+                    if (++low == a.low_buffers) low = 0;
                     if (++s == a.stages) {
                         s = 0;
                         ph ^= 1u;
@@ -669,8 +669,36 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer_x3(const __gri
                 if (lc_mbar_try_wait(drain_bar, 0)) break;
         }
         __syncwarp();
+    } else if (warp >= kLcX3SplitWarp0) {
+        // ---------------------------------------------------------------- splitters
+        int s = 0, low = 0;
+        uint32_t ph = 0, low_ph = 0;
+        bool ok = true;
+        for (int t = first; t < total_tiles && ok; t += step) {
+            for (int kc = 0; kc < a.k_chunks; ++kc) {
+                ok = lc_wait(copied_bar(s), ph, abort_flag, a.error, a.spin_limit) &&
+                     lc_wait(low_empty_bar(low), low_ph ^ 1u, abort_flag, a.error, a.spin_limit);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride, small = low0 + (uint32_t)low * a.stage_stride;
+                split_part(kc, base, small, kLcTileM);
+                if (!a.w_resident) split_part(kc, base + kPart, small + kPart, a.n_half);
+                __syncwarp();
+                if (lane == 0) lc_mbar_arrive(full_bar(s));
+                if (++s == a.stages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+                if (++low == a.low_buffers) {
+                    low = 0;
+                    low_ph ^= 1u;
+                }
+            }
+        }
     } else {
-        lc_epilogue(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first, step, a.n_half,
+        lc_epilogue<kLcX3EpilogueWarps>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first, step, a.n_half,
                     half * a.n_half);
     }
 
@@ -757,7 +785,7 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     const int32_t n_half = (int32_t)(hidden / halves);
     bool resident;
     uint32_t stage_stride, small_off = 0, w_off;
-    int32_t stages;
+    int32_t stages, low_buffers = 0;
     int64_t w_bytes;
     if (!x3) {
         w_bytes = (int64_t)k_chunks * hidden * 128;
@@ -765,17 +793,20 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)(kLcABytes + hidden * 128);
         stages = (int32_t)std::min<int64_t>(kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     } else {
-        // per chunk a high and a low part of the tile's rows (16 KB each) and of the weight part (n_half x 128 B each)
+        // a stage takes a chunk of the tile's rows as copied (16 KB, plus n_half x 128 B of the weight when it is streamed);
+        // buffers of the same size take low parts.  Two of those where three stages remain, else one.
         const uint32_t w_part = (uint32_t)n_half * 128u;
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
-        small_off = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + w_part;
-        stage_stride = 2u * small_off;
-        stages = (int32_t)std::min<int64_t>(4, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
+        stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + w_part;
+        const int64_t fit = (kLcSmemBytes - kLcX3EpilogueWarps * kLcEpiBytes - (resident ? w_bytes : 0)) / stage_stride;
+        low_buffers = fit >= 5 ? 2 : 1;
+        stages = (int32_t)std::min<int64_t>(kLcX3MaxStages, fit - low_buffers);
+        small_off = (uint32_t)stages * stage_stride;
     }
-    w_off = (uint32_t)stages * stage_stride;
+    w_off = (uint32_t)(stages + low_buffers) * stage_stride;
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
-    const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
+    const size_t smem = 1024 + (size_t)epi_off + (x3 ? kLcX3EpilogueWarps : 8) * kLcEpiBytes;
     auto kernel = x3 ? k_lc_first_layer_x3 : k_lc_first_layer;
     GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
 
@@ -810,11 +841,12 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.halves = halves;
         a.n_half = n_half;
         a.small_off = small_off;
+        a.low_buffers = low_buffers;
         a.drop_announcements = selftest_polls > 0 ? 1 : 0;
         a.spin_limit = selftest_polls > 0 ? selftest_polls : kLcSpinLimit;
         const int64_t total = (int64_t)kn * tiles_m;
         const unsigned grid = (unsigned)(std::min<int64_t>(num_sms / halves, total) * halves);
-        kernel<<<grid, kLcThreads, smem, st>>>(maps, a);
+        kernel<<<grid, x3 ? kLcX3Threads : kLcThreads, smem, st>>>(maps, a);
         GNNPRE_CUDA(cudaGetLastError());
     }
     return GNNPRE_OK;
