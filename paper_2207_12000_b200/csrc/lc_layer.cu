@@ -58,12 +58,11 @@ constexpr int kLcProducerWarps = 4;
 constexpr int kLcProducerThreads = 32 * kLcProducerWarps;
 constexpr int kLcMmaWarp = kLcProducerWarps;       // warps: 0-3 producers, 4 MMA, 5-12 epilogue
 constexpr int kLcThreads = 32 * (kLcProducerWarps + 1 + 8);
-constexpr int kLcX3EpilogueWarps = 4;              // split-operand kernel: four epilogue warps, 16 KB more for operands
-constexpr int kLcX3SplitWarps = 4;                 // warps that compute the low parts: 9-12
+constexpr int kLcX3EpilogueWarps = 4;              // split-operand kernel: warps 5-8, two staging boxes each
+constexpr int kLcX3SplitWarps = 4;                 // warps 9-12 compute the low parts
 constexpr int kLcX3SplitWarp0 = kLcProducerWarps + 1 + kLcX3EpilogueWarps;
 constexpr int kLcX3Threads = 32 * (kLcX3SplitWarp0 + kLcX3SplitWarps);
-constexpr int kLcX3MaxStages = 5;
-constexpr int kLcSmemBytes = 225 * 1024;          // operands, weight and output boxes, besides 1 KB of alignment
+constexpr uint32_t kLcX3MaxCols = 128;             // output columns of a CTA, columns of one accumulator buffer
 constexpr int kLcMaxHops = 8;                     // hop matrices per launch
 constexpr uint32_t kLcTmemCols = 512;
 constexpr uint32_t kLcSuspendNs = 20000;          // a failed poll parks the warp for up to this long
@@ -97,8 +96,6 @@ struct LcArgs {
     int64_t ldw;
     int32_t halves;        // column parts: CTAs with blockIdx.x % halves == h compute columns [h n_half, (h + 1) n_half)
     int32_t n_half;
-    uint32_t small_off;    // offset of the buffers of low parts
-    int32_t low_buffers;
     // failure-detection self-test: the producers never announce a chunk, so every wait runs out
     int32_t drop_announcements;
     uint32_t spin_limit;   // polls before a wait gives up
@@ -191,6 +188,17 @@ __device__ __forceinline__ void lc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uin
         : "memory");
 }
 
+// The same with A in tensor memory: row = lane, one 32-bit column per element of K.
+__device__ __forceinline__ void lc_mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
 // Makes the mbarrier track the completion of every MMA this thread has issued so far.
 __device__ __forceinline__ void lc_mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -209,6 +217,17 @@ __device__ __forceinline__ void lc_tmem_load32(uint32_t taddr, uint32_t (&v)[32]
         : "memory");
 }
 
+__device__ __forceinline__ void lc_tmem_store32(uint32_t taddr, const uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"r"(v[0]),
+        "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]),
+        "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]),
+        "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]),
+        "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(taddr)
+        : "memory");
+}
+
 // Tensor store of one [32 rows, 32 columns] box (128-byte swizzle) from shared memory; rows and
 // columns beyond the matrix are clipped by the copy engine.
 __device__ __forceinline__ void lc_tile_store(const CUtensorMap* tmap, int x0, int y0, uint32_t src) {
@@ -220,17 +239,18 @@ __device__ __forceinline__ void lc_tile_store(const CUtensorMap* tmap, int x0, i
 
 // Epilogue role (the warps after the MMA warp), shared by both kernels: tiles first, first + step, ...; the accumulator
 // holds n_cols columns that go to columns col0 .. col0 + n_cols of Y.  WARPS / 4 warps per quarter of the accumulator's
-// lanes share its 32-column boxes in turn.
-template <int WARPS>
+// lanes share its 32-column boxes in turn; a warp has BOXES staging boxes in shared memory.
+template <int WARPS, int BOXES>
 __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a, uint32_t tiles0, uint32_t tmem_base,
                                             uint32_t acc_full0, uint32_t acc_empty0, volatile int* abort_flag, int first,
-                                            int step, int n_cols, int col0) {
+                                            int step, int n_cols, int col0, uint32_t acc_stride) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int kTurn = WARPS / 4;
     const int ew = warp - kLcMmaWarp - 1;  // 0 .. WARPS - 1
     const int q = warp & 3;                // tensor-memory lanes 32q .. 32q+31 are the ones this warp may read
     const int half = ew >> 2;
-    const uint32_t box = tiles0 + a.epi_off + (uint32_t)ew * kLcEpiBytes;
+    const uint32_t box0 = tiles0 + a.epi_off + (uint32_t)(ew * BOXES) * kLcEpiBytes;
+    uint32_t box = box0;
     const int boxes = (n_cols + 31) / 32;
     const int total_tiles = a.num_hops * a.tiles_m;
     int it = 0;
@@ -241,7 +261,7 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
         if (!__all_sync(0xffffffffu, lc_wait(acc_full0 + 8u * buf, acc_ph, abort_flag, a.error, a.spin_limit))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const bool relu = (a.relu_mask >> hop) & 1u;
-        const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)buf * kLcMaxHidden;
+        const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)buf * acc_stride;
         // the read of the next box is in flight while box i is written out
         uint32_t v[2][32];
         if (half < boxes) lc_tmem_load32(taddr + 32u * half, v[0]);
@@ -249,8 +269,8 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
         for (int i = half, u = 0; i < boxes; i += kTurn, u ^= 1) {
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             if (i + kTurn < boxes) lc_tmem_load32(taddr + 32u * (i + kTurn), v[u ^ 1]);
-            // the previous store must have read the staging box before it is overwritten
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            // the last store from this staging box must have read it before it is overwritten
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BOXES - 1) : "memory");
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -273,6 +293,7 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
                 lc_tile_store(&maps.y[hop], col0 + 32 * i, mt * kLcTileM + 32 * q, box);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
+            if (BOXES == 2) box = box == box0 ? box0 + kLcEpiBytes : box0;
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -444,8 +465,8 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
         __syncwarp();
     } else {
         // ---------------------------------------------------------------- epilogue
-        lc_epilogue<8>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, blockIdx.x, gridDim.x,
-                    a.hidden, 0);
+        lc_epilogue<8, 1>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, blockIdx.x, gridDim.x,
+                          a.hidden, 0, kLcMaxHidden);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -464,9 +485,12 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // 128 output columns: with hidden > 128, even and odd CTAs take the two column halves and every batch row is
 // gathered once per part (the later reads mostly hit L2).  No tensor copies on the input side: the producer
 // threads bring rows of the hop matrix AND rows of the weight in with 16-byte asynchronous copies; four warps of their own
-// (9-12) read each stage that has landed and write its low parts into one of two further buffers.  When the copying
-// threads did that themselves they also had to fence, and so waited for all their copies in flight: 4587 us against 3550
-// (2.4 M rows x 3 hops, F = 100, hidden 256, random order), 1540 against 908 (500 K rows x 2, F = 256).
+// (9-12) read each stage that has landed and write the low parts of its rows into tensor memory, from where the tensor core
+// takes them as operand A (lane = row): beside the two 128-column accumulators there are 32 columns for each of eight
+// stages, and shared memory holds four stages of copied rows beside 128 KB of weight.  2.4 M rows x 3 hops, F = 100, hidden
+// 256, random order: 4587 us when the copying threads split into a second half of two stages (and their proxy fence waited
+// for all their copies in flight), 3550 us with splitter warps and two buffers of low parts in shared memory, 2816 us now;
+// 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the L2's and the copy path's latency over those four stages.
 // K-steps of the last chunk beyond the features are neither copied nor multiplied.
 //
 // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
@@ -476,19 +500,19 @@ __device__ __forceinline__ void lc_load_piece(uint32_t (&v)[4], uint32_t addr) {
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
 }
 
+__device__ __forceinline__ uint32_t lc_low_part(uint32_t v) {
+    return __float_as_uint(__uint_as_float(v) - __uint_as_float(v & 0xffffe000u));  // exact; read by the tensor core as tf32
+}
+
 __device__ __forceinline__ void lc_store_low_part(const uint32_t (&v)[4], uint32_t addr) {
-    uint32_t lo[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t hi = v[j] & 0xffffe000u;
-        lo[j] = __float_as_uint(__uint_as_float(v[j]) - __uint_as_float(hi));  // exact; read by the tensor core as tf32
-    }
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]) : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(lc_low_part(v[0])), "r"(lc_low_part(v[1])),
+                 "r"(lc_low_part(v[2])), "r"(lc_low_part(v[3]))
+                 : "memory");
 }
 
 __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __grid_constant__ LcMaps maps, const LcArgs a) {
     extern __shared__ unsigned char lc_smem[];
-    __shared__ __align__(8) unsigned long long bars[4 * kLcMaxStages + 6];
+    __shared__ __align__(8) unsigned long long bars[3 * kLcMaxStages + 6];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int* abort_flag = &abort_word;
@@ -497,20 +521,18 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
     const uint32_t tiles0 = (lc_smem_u32(lc_smem) + 1023u) & ~1023u;
     const uint32_t bar0 = lc_smem_u32(&bars[0]);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (kLcMaxStages + s); };           // a stage's copied (high) part is free
-    auto low_empty_bar = [&](int l) { return bar0 + 8u * (2 * kLcMaxStages + l); };  // a buffer of low parts is free
-    auto copied_bar = [&](int s) { return bar0 + 8u * (3 * kLcMaxStages + s); };      // a stage's copies have landed
-    auto acc_full_bar = [&](int b) { return bar0 + 8u * (4 * kLcMaxStages + b); };
-    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (4 * kLcMaxStages + 2 + b); };
-    const uint32_t drain_bar = bar0 + 8u * (4 * kLcMaxStages + 4);
-    const uint32_t w_bar = bar0 + 8u * (4 * kLcMaxStages + 5);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kLcMaxStages + s); };
+    auto copied_bar = [&](int s) { return bar0 + 8u * (2 * kLcMaxStages + s); };  // a stage's copies have landed
+    auto acc_full_bar = [&](int b) { return bar0 + 8u * (3 * kLcMaxStages + b); };
+    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (3 * kLcMaxStages + 2 + b); };
+    const uint32_t drain_bar = bar0 + 8u * (3 * kLcMaxStages + 4);
+    const uint32_t w_bar = bar0 + 8u * (3 * kLcMaxStages + 5);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kLcMaxStages; ++s) {
             lc_mbar_init(copied_bar(s), kLcProducerThreads);
             lc_mbar_init(full_bar(s), kLcX3SplitWarps);  // a stage's low parts are there as well
             lc_mbar_init(empty_bar(s), 1);
-            lc_mbar_init(low_empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             lc_mbar_init(acc_full_bar(b), 1);
@@ -535,10 +557,11 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
     const int total_tiles = a.num_hops * a.tiles_m;
     const int half = blockIdx.x % a.halves;
     const int first = blockIdx.x / a.halves, step = gridDim.x / a.halves;
-    constexpr uint32_t kPart = kLcABytes;               // bytes of one part of the rows' chunk: [128, 32] floats
+    constexpr uint32_t kPart = kLcABytes;               // bytes of the rows' chunk: [128, 32] floats
     const uint32_t w_part = (uint32_t)a.n_half * 128u;  // bytes of one part of the weight's chunk: [n_half, 32] floats
 
-    const uint32_t low0 = tiles0 + a.small_off;  // buffers of low parts, as large as a stage each
+    // Tensor memory: two accumulators of kLcX3MaxCols columns, then the low parts of each stage's rows, 32 columns a stage.
+    auto tmem_low = [&](int s) { return tmem_base + 2u * kLcX3MaxCols + 32u * s; };
     // K-steps of 8 features in chunk kc: 16-byte pieces beyond them are neither copied nor multiplied
     auto k_steps = [&](int kc) { return min(4, (a.feat_dim - kc * kLcChunk + 7) >> 3); };
 
@@ -546,15 +569,15 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
     // rows each, a thread eight of them (of the tile and of the weight part): row0 + 4 i.
     const int piece = lane & 7;
     const int row0 = 32 * (warp & 3) + (lane >> 3);
-    auto split_part = [&](int kc, uint32_t big_part, uint32_t small_part, int row_limit) {
+    auto split_weight = [&](int kc, uint32_t big_part, uint32_t small_part) {
         if (piece >= 2 * k_steps(kc)) return;
         uint32_t v[8][4];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (row0 + 4 * i < row_limit) lc_load_piece(v[i], big_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
+            if (row0 + 4 * i < a.n_half) lc_load_piece(v[i], big_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (row0 + 4 * i < row_limit) lc_store_low_part(v[i], small_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
+            if (row0 + 4 * i < a.n_half) lc_store_low_part(v[i], small_part + 128u * (row0 + 4 * i) + ((uint32_t)(piece ^ ((row0 + 4 * i) & 7)) << 4));
     };
 
     if (warp < kLcProducerWarps) {
@@ -587,7 +610,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             for (int kc = 0; kc < a.k_chunks; ++kc) {
                 const uint32_t wb = tiles0 + a.w_off + (uint32_t)kc * 2u * w_part;
-                split_part(kc, wb, wb + w_part, a.n_half);
+                split_weight(kc, wb, wb + w_part);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             lc_mbar_arrive(w_bar);
@@ -625,7 +648,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
             const uint32_t idesc = lc_instr_desc(a.n_half);
-            int s = 0, it = 0, low = 0;
+            int s = 0, it = 0;
             uint32_t ph = 0;
             bool ok = !a.w_resident || lc_wait(w_bar, 0, abort_flag, a.error, a.spin_limit);
             for (int t = first; t < total_tiles && ok; t += step, ++it) {
@@ -633,7 +656,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
                 const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
                 if (!lc_wait(acc_empty_bar(buf), acc_ph ^ 1u, abort_flag, a.error, a.spin_limit)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcMaxHidden;
+                const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcX3MaxCols;
                 for (int kc = 0; kc < a.k_chunks; ++kc) {
                     if (!lc_wait(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
                         ok = false;
@@ -642,21 +665,18 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // both parts, seen by the tensor core
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
-                    const uint32_t small = low0 + (uint32_t)low * a.stage_stride;
-                    const uint32_t xh = base, xl = small;
+                    const uint32_t xh = base, xl = tmem_low(s);
                     const uint32_t wh = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart;
-                    const uint32_t wl = a.w_resident ? wh + w_part : small + kPart;
+                    const uint32_t wl = wh + w_part;
                     const int steps = k_steps(kc);
                     for (int j = 0; j < steps; ++j) {
                         const uint32_t o = 32u * j;
                         // small terms first, the leading term last
-                        lc_mma_tf32(tmem_d, lc_operand_desc(xl + o), lc_operand_desc(wh + o), idesc, (kc | j) != 0);
+                        lc_mma_tf32_ta(tmem_d, xl + 8u * j, lc_operand_desc(wh + o), idesc, (kc | j) != 0);
                         lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wl + o), idesc, 1u);
                         lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wh + o), idesc, 1u);
                     }
-                    lc_mma_commit(low_empty_bar(low));
                     lc_mma_commit(empty_bar(s));
-                    if (++low == a.low_buffers) low = 0;
                     if (++s == a.stages) {
                         s = 0;
                         ph ^= 1u;
@@ -671,35 +691,40 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
         __syncwarp();
     } else if (warp >= kLcX3SplitWarp0) {
         // ---------------------------------------------------------------- splitters
-        int s = 0, low = 0;
-        uint32_t ph = 0, low_ph = 0;
+        // A thread has one row of the tile, the tensor-memory lane of the same number.
+        const int row = 32 * (warp & 3) + lane;
+        int s = 0;
+        uint32_t ph = 0;
         bool ok = true;
         for (int t = first; t < total_tiles && ok; t += step) {
             for (int kc = 0; kc < a.k_chunks; ++kc) {
-                ok = lc_wait(copied_bar(s), ph, abort_flag, a.error, a.spin_limit) &&
-                     lc_wait(low_empty_bar(low), low_ph ^ 1u, abort_flag, a.error, a.spin_limit);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride, small = low0 + (uint32_t)low * a.stage_stride;
-                split_part(kc, base, small, kLcTileM);
-                if (!a.w_resident) split_part(kc, base + kPart, small + kPart, a.n_half);
+                // (the producers refilled the stage after the tensor core had read it, low parts included)
+                ok = __all_sync(0xffffffffu, lc_wait(copied_bar(s), ph, abort_flag, a.error, a.spin_limit));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
+                uint32_t v[8][4], lo[32];
+#pragma unroll
+                for (int p = 0; p < 8; ++p) lc_load_piece(v[p], base + 128u * row + ((uint32_t)(p ^ (row & 7)) << 4));
+#pragma unroll
+                for (int p = 0; p < 8; ++p)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) lo[4 * p + j] = lc_low_part(v[p][j]);
+                lc_tmem_store32(tmem_low(s) + ((uint32_t)(32 * (warp & 3)) << 16), lo);
+                if (!a.w_resident) split_weight(kc, base + kPart, base + kPart + w_part);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) lc_mbar_arrive(full_bar(s));
                 if (++s == a.stages) {
                     s = 0;
                     ph ^= 1u;
                 }
-                if (++low == a.low_buffers) {
-                    low = 0;
-                    low_ph ^= 1u;
-                }
             }
         }
     } else {
-        lc_epilogue<kLcX3EpilogueWarps>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first, step, a.n_half,
-                    half * a.n_half);
+        lc_epilogue<kLcX3EpilogueWarps, 2>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first, step, a.n_half,
+                    half * a.n_half, kLcX3MaxCols);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -784,8 +809,8 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     const int32_t k_chunks = (int32_t)((feat_dim + kLcChunk - 1) / kLcChunk);
     const int32_t n_half = (int32_t)(hidden / halves);
     bool resident;
-    uint32_t stage_stride, small_off = 0, w_off;
-    int32_t stages, low_buffers = 0;
+    uint32_t stage_stride, w_off;
+    int32_t stages;
     int64_t w_bytes;
     if (!x3) {
         w_bytes = (int64_t)k_chunks * hidden * 128;
@@ -793,20 +818,16 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)(kLcABytes + hidden * 128);
         stages = (int32_t)std::min<int64_t>(kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     } else {
-        // a stage takes a chunk of the tile's rows as copied (16 KB, plus n_half x 128 B of the weight when it is streamed);
-        // buffers of the same size take low parts.  Two of those where three stages remain, else one.
+        // a stage takes a chunk of the tile's rows as copied (16 KB) and, when the weight is streamed, both parts of its chunk
         const uint32_t w_part = (uint32_t)n_half * 128u;
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
-        stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + w_part;
-        const int64_t fit = (kLcSmemBytes - kLcX3EpilogueWarps * kLcEpiBytes - (resident ? w_bytes : 0)) / stage_stride;
-        low_buffers = fit >= 5 ? 2 : 1;
-        stages = (int32_t)std::min<int64_t>(kLcX3MaxStages, fit - low_buffers);
-        small_off = (uint32_t)stages * stage_stride;
+        stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + 2u * w_part;
+        stages = (int32_t)std::min<int64_t>(kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     }
-    w_off = (uint32_t)(stages + low_buffers) * stage_stride;
+    w_off = (uint32_t)stages * stage_stride;
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
-    const size_t smem = 1024 + (size_t)epi_off + (x3 ? kLcX3EpilogueWarps : 8) * kLcEpiBytes;
+    const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
     auto kernel = x3 ? k_lc_first_layer_x3 : k_lc_first_layer;
     GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
 
@@ -840,8 +861,6 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.ldw = ldw;
         a.halves = halves;
         a.n_half = n_half;
-        a.small_off = small_off;
-        a.low_buffers = low_buffers;
         a.drop_announcements = selftest_polls > 0 ? 1 : 0;
         a.spin_limit = selftest_polls > 0 ? selftest_polls : kLcSpinLimit;
         const int64_t total = (int64_t)kn * tiles_m;
