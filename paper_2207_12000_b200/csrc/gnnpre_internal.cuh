@@ -34,19 +34,21 @@ void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int 
 // reported as failed.  kind 0 = device memory, 1 = page-locked host memory.
 bool injected_alloc_failure(int kind);
 
-// Device allocation that frees itself.
+// Device memory: an allocation of its own that frees itself, or a piece of another buffer (see Carve).
 template <typename T>
 struct DevBuf {
     T* p = nullptr;
     size_t count = 0;
+    bool owned = true;
     DevBuf() = default;
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
     ~DevBuf() { reset(); }
     void reset() {
-        if (p) cudaFree(p);
+        if (p && owned) cudaFree(p);
         p = nullptr;
         count = 0;
+        owned = true;
     }
     int alloc(size_t n) {
         reset();
@@ -60,6 +62,46 @@ struct DevBuf {
         return GNNPRE_OK;
     }
     size_t bytes() const { return count * sizeof(T); }
+};
+
+// Several buffers carved out of one device allocation.  An allocation or a free costs about 100 us here, whatever its
+// size, and a plan has some twenty buffers.  Failure injection counts each of them.
+class Carve {
+public:
+    template <typename T>
+    void want(DevBuf<T>& b, size_t n) {
+        b.reset();
+        if (n == 0) return;
+        if (injected_alloc_failure(0)) failed_ = true;
+        items_.push_back({reinterpret_cast<void**>(&b.p), total_});
+        b.count = n;
+        b.owned = false;
+        total_ += (n * sizeof(T) + 255) & ~(size_t)255;
+    }
+    size_t bytes() const { return total_; }
+    // places the buffers in `room`, which lives at least as long as they do
+    int place(char* room) {
+        if (failed_) {
+            set_last_cuda_error(cudaErrorMemoryAllocation, "cudaMalloc (injected failure)", __FILE__, __LINE__);
+            return GNNPRE_ERR_OOM_DEVICE;
+        }
+        for (const Item& it : items_) *it.p = room + it.offset;
+        return GNNPRE_OK;
+    }
+    // ... or in a new allocation
+    int place(DevBuf<char>& arena) {
+        if (!failed_) GNNPRE_TRY(arena.alloc(total_));
+        return place(arena.p);
+    }
+
+private:
+    struct Item {
+        void** p;
+        size_t offset;
+    };
+    std::vector<Item> items_;
+    size_t total_ = 0;
+    bool failed_ = false;
 };
 
 // Page-locked host allocation.
@@ -149,6 +191,8 @@ struct gnnpre_plan {
     bool rows_all_nonempty = true;  // every row owns an edge (always true with self-loops)
     int64_t num_nonempty = 0, num_empty = 0;
 
+    // what the buffers below (but for the streamed structure's and the streaming state's) are pieces of
+    gnnpre::DevBuf<char> arena[2];
     // per-node arrays (device)
     gnnpre::DevBuf<int32_t> deg;
     gnnpre::DevBuf<float> rscale, cscale;

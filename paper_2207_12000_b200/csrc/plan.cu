@@ -19,197 +19,256 @@ inline unsigned grid_for(int64_t items, int per_block) {
     return (unsigned)std::max<int64_t>(1, g);
 }
 
-// ---------------------------------------------------------------- validation, degrees, scales
+// ---------------------------------------------------------------- rows: pointers, degrees, scales
 
 enum : int { kErrRowptr = 1, kErrColRange = 2, kErrDiagonal = 4, kErrOrder = 8, kErrDegree = 16 };
 
-// One warp per row: checks the input contract of the CSR.
-__global__ void k_validate(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
-                           const int32_t* __restrict__ colidx, int* err) {
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const int64_t lo = rowptr[row], hi = rowptr[row + 1];
+// One thread per row.  Checks the row pointers; D_i = number of nonzeros in row i of A (Section 2) unless the caller
+// gave the degrees; A^_ij = r_i c_j: GCN r = c = (D_i + 1)^{-1/2} (Eq. 1); SAGE r = 1/D_i (0 for D_i = 0), c = 1;
+// GIN r = c = 1, evaluated in fp64 (IEEE sqrt and divide) and rounded once to fp32; the support's row pointers (with
+// self-loops row i of the support is row i of A plus one entry, so rowptr_t[i] = rowptr[i] + i); whether the row owns
+// an edge (flag may be nullptr).
+__global__ void k_rows(int op, int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ deg_in,
+                       int32_t* __restrict__ deg, float* __restrict__ rscale, float* __restrict__ cscale,
+                       int64_t* __restrict__ rowptr_t, int32_t* __restrict__ flag, int* err) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int64_t lo = rowptr[i], hi = rowptr[i + 1];
     int bad = 0;
-    if (lo < 0 || hi < lo || hi > nnz) {
-        bad |= kErrRowptr;
-    } else {
-        if (hi - lo >= 0x7fffffffLL) bad |= kErrDegree;
-        for (int64_t e = lo + lane; e < hi; e += 32) {
-            const int32_t c = colidx[e];
-            if (c < 0 || c >= n) bad |= kErrColRange;
-            if (c == row) bad |= kErrDiagonal;
-            if (e + 1 < hi && colidx[e + 1] <= c) bad |= kErrOrder;
-        }
-    }
+    if (lo < 0 || hi < lo || hi > nnz || (i == 0 && lo != 0) || (i == n - 1 && hi != nnz)) bad |= kErrRowptr;
+    else if (hi - lo >= 0x7fffffffLL) bad |= kErrDegree;
     if (bad) atomicOr(err, bad);
+    const int32_t d = deg_in ? deg_in[i] : (int32_t)(hi - lo);
+    deg[i] = d;
+    double r = 1.0, c = 1.0;
+    if (op == GNNPRE_OP_GCN_SYM) {
+        r = c = 1.0 / sqrt((double)d + 1.0);
+    } else if (op == GNNPRE_OP_SAGE_MEAN) {
+        r = d > 0 ? 1.0 / (double)d : 0.0;
+    }
+    rscale[i] = (float)r;
+    cscale[i] = (float)c;
+    const int64_t diag = op != GNNPRE_OP_SAGE_MEAN;
+    rowptr_t[i] = lo + diag * i;
+    if (i == n - 1) rowptr_t[n] = hi + diag * n;
+    if (flag) flag[i] = hi > lo;
 }
 
-// D_i = number of nonzeros in row i of A (Section 2).
 __global__ void k_degrees(int64_t n, const int64_t* __restrict__ rowptr, int32_t* __restrict__ deg) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) deg[i] = (int32_t)(rowptr[i + 1] - rowptr[i]);
 }
 
-// A^_ij = r_i c_j: GCN r = c = (D_i + 1)^{-1/2} (Eq. 1); SAGE r = 1/D_i (0 for D_i = 0), c = 1;
-// GIN r = c = 1.  Evaluated in fp64 (IEEE sqrt and divide) and rounded once to fp32.
-__global__ void k_scales(int op, int64_t n, const int32_t* __restrict__ deg, float* __restrict__ rscale,
-                         float* __restrict__ cscale) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double r = 1.0, c = 1.0;
-    if (op == GNNPRE_OP_GCN_SYM) {
-        r = c = 1.0 / sqrt((double)deg[i] + 1.0);
-    } else if (op == GNNPRE_OP_SAGE_MEAN) {
-        r = deg[i] > 0 ? 1.0 / (double)deg[i] : 0.0;
-    }
-    rscale[i] = (float)r;
-    cscale[i] = (float)c;
-}
-
 // ---------------------------------------------------------------- the support's edge list E
 
-// One warp per row.  With `diag`, row i of the support is row i of A plus the self-loop (i, i) at
-// its column-sorted position, so rowptr_t[i] = rowptr[i] + i.  The last entry of every non-empty
-// row carries kRowEndBit.
-__global__ void k_support(int diag, int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                          int64_t* __restrict__ rowptr_t, uint32_t* __restrict__ colx) {
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const int64_t lo = rowptr[row], hi = rowptr[row + 1];
-    const int64_t base = lo + (diag ? row : 0);
-    const int64_t len_t = hi - lo + (diag ? 1 : 0);
-    if (lane == 0) {
-        rowptr_t[row] = base;
-        if (row == n - 1) rowptr_t[n] = base + len_t;
+// Row holding edge e: the last i with rowptr[i] <= e (rows without edges are skipped because their successor shares
+// their start).  Stays inside [0, n) whatever rowptr holds.
+__device__ __forceinline__ int64_t row_of_edge(const int64_t* __restrict__ rowptr, int64_t n, int64_t e) {
+    int64_t lo = 0, hi = n;  // invariant: rowptr[lo] <= e < rowptr[hi]
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (rowptr[mid] <= e) lo = mid; else hi = mid;
     }
-    int64_t below = 0;  // entries of the row with column < row
-    for (int64_t e0 = lo; e0 < hi; e0 += 32) {
-        const int64_t e = e0 + lane;
-        bool lt = false;
-        if (e < hi) {
-            const int32_t c = colidx[e];
-            lt = c < row;
-            const int64_t pos = (e - lo) + ((diag && !lt) ? 1 : 0);
-            colx[base + pos] = (uint32_t)c | (pos == len_t - 1 ? kRowEndBit : 0u);
-        }
-        below += __popc(__ballot_sync(0xffffffffu, lt));
-    }
-    if (diag && lane == 0) colx[base + below] = (uint32_t)row | (below == len_t - 1 ? kRowEndBit : 0u);
+    return lo;
 }
 
-// ---------------------------------------------------------------- exclusive scan (int32)
+// The same by a whole warp, 32 probes at a time: four or five dependent loads instead of twenty.
+__device__ __forceinline__ int64_t row_of_edge_warp(const int64_t* __restrict__ rowptr, int64_t n, int64_t e, int lane) {
+    int64_t lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) >> 5;
+        const int64_t probe = lo + (lane + 1) * step;
+        const bool le = probe < hi && rowptr[probe] <= e;
+        const int k = __popc(__ballot_sync(0xffffffffu, le));  // probes are ascending: the first k hold
+        hi = min(hi, lo + (k + 1) * step);
+        lo += k * step;
+    }
+    return lo;
+}
+
+// Copies the edge list into the support: entry (row, col) with its row-end mark, self-loops (with `diag`) inserted at
+// their column-sorted position, and checks the contract of colidx on the way (`check`).  The row pointers have been
+// checked.  A warp takes `per_warp` consecutive edges whatever rows they belong to - a warp per row took 148 us for
+// 1.8 M edges because one row holds 20,000 of them, and the check a pass of its own (54 us) - and finds the rows of 32
+// edges from the next 32 row pointers.  The last blocks, one thread per row, write the self-loops of rows without edges.
+__global__ void k_support(int diag, int check, int64_t n, int64_t nnz, int64_t per_warp, int64_t edge_blocks,
+                          const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
+                          uint32_t* __restrict__ colx, int* err) {
+    constexpr unsigned kFull = 0xffffffffu;
+    if ((int64_t)blockIdx.x >= edge_blocks) {
+        const int64_t i = ((int64_t)blockIdx.x - edge_blocks) * blockDim.x + threadIdx.x;
+        if (i < n) {
+            const int64_t lo = rowptr[i];
+            if (rowptr[i + 1] == lo) colx[lo + i] = (uint32_t)i | kRowEndBit;
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int64_t e_beg = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+    const int64_t e_end = min(nnz, e_beg + per_warp);
+    if (e_beg >= e_end) return;
+    int64_t r = row_of_edge_warp(rowptr, n, e_beg, lane);  // row of the first edge of the 32
+    int bad = 0;
+    for (int64_t e0 = e_beg; e0 < e_end; e0 += 32) {
+        const int64_t e = min(e0 + lane, e_end - 1);  // lanes past the end repeat the last edge
+        const int32_t c = colidx[e];
+        int64_t row = -1;
+        for (int tries = 0; tries < 4; ++tries) {  // row = base + number of row ends at or before e among the next 32
+            const int64_t base = r + 32 * tries;
+            const int64_t end_of = rowptr[min(base + 1 + lane, n)];
+            int k = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(kFull, end_of, k + step - 1) <= e) k += step;
+            const int64_t last_end = __shfl_sync(kFull, end_of, 31);
+            if (row < 0 && !(k == 31 && last_end <= e)) row = base + k;
+            if (__all_sync(kFull, row >= 0)) break;
+        }
+        if (row < 0) row = row_of_edge(rowptr, n, e);  // a long run of rows without edges
+        row = min(row, n - 1);
+        const int64_t lo = rowptr[row], hi = rowptr[row + 1];
+        int32_t prev = __shfl_up_sync(kFull, c, 1), next = __shfl_down_sync(kFull, c, 1);
+        if (lane == 0) prev = e > 0 ? colidx[e - 1] : 0;
+        if (lane == 31 || e0 + lane + 1 >= e_end) next = e + 1 < nnz ? colidx[e + 1] : 0;
+        if (check) {
+            if (c < 0 || c >= n) bad |= kErrColRange;
+            if (c == row) bad |= kErrDiagonal;
+            if (e + 1 < hi && next <= c) bad |= kErrOrder;
+        }
+        if (e0 + lane < e_end) {
+            const bool last = e == hi - 1;
+            if (diag) {
+                const int above = c > row;  // the self-loop comes before this entry
+                colx[e + row + above] = (uint32_t)c | (last && above ? kRowEndBit : 0u);
+                if (above && (e == lo || prev < row)) colx[e + row] = (uint32_t)row;
+                if (!above && last) colx[e + row + 1] = (uint32_t)row | kRowEndBit;
+            } else {
+                colx[e] = (uint32_t)c | (last ? kRowEndBit : 0u);
+            }
+        }
+        r = __shfl_sync(kFull, row, 31);
+    }
+    if (bad) atomicOr(err, bad);
+}
+
+// ---------------------------------------------------------------- exclusive scan
 
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kTB * kScanItems;
 
-__device__ __forceinline__ int block_exclusive_scan(int v, int* total) {
-    __shared__ int warp_sums[kTB / 32];
+// Scratch rows, fix-ups and hub rows that a segment (or all segments before it) accounts for.
+struct SegCounts {
+    int32_t slots, fixups, hubs;
+};
+__device__ __forceinline__ SegCounts operator+(const SegCounts& a, const SegCounts& b) {
+    return {a.slots + b.slots, a.fixups + b.fixups, a.hubs + b.hubs};
+}
+__device__ __forceinline__ SegCounts shfl_up(const SegCounts& v, int d) {
+    return {__shfl_up_sync(0xffffffffu, v.slots, d), __shfl_up_sync(0xffffffffu, v.fixups, d),
+            __shfl_up_sync(0xffffffffu, v.hubs, d)};
+}
+__device__ __forceinline__ int32_t shfl_up(int32_t v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
+
+// Sum over the threads before this one; *total = sum over the block.
+template <typename T>
+__device__ __forceinline__ T block_exclusive_scan(const T& v, T* total) {
+    __shared__ T warp_sums[kTB / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
+    T incl = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += t;
+        const T t = shfl_up(incl, d);
+        if (lane >= d) incl = incl + t;
     }
     if (lane == 31) warp_sums[warp] = incl;
+    const T before = shfl_up(incl, 1);
     __syncthreads();
-    if (warp == 0) {
-        int w = lane < kTB / 32 ? warp_sums[lane] : 0;
-#pragma unroll
-        for (int d = 1; d < kTB / 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, w, d);
-            if (lane >= d) w += t;
-        }
-        if (lane < kTB / 32) warp_sums[lane] = w;  // inclusive over warps
+    T run{}, off{};
+    for (int w = 0; w < kTB / 32; ++w) {
+        if (w == warp) off = run;
+        run = run + warp_sums[w];
     }
+    *total = run;
     __syncthreads();
-    const int warp_off = warp > 0 ? warp_sums[warp - 1] : 0;
-    *total = warp_sums[kTB / 32 - 1];
-    const int r = warp_off + incl - v;
-    __syncthreads();
-    return r;
+    return lane > 0 ? off + before : off;
 }
 
-__global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t n, int32_t* __restrict__ sums) {
+template <typename T>
+__global__ void k_tile_sums(const T* __restrict__ in, int64_t n, T* __restrict__ sums) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    int s = 0;
+    T s{};
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k)
-        if (base + k < n) s += in[base + k];
-    int total;
+        if (base + k < n) s = s + in[base + k];
+    T total;
     block_exclusive_scan(s, &total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
 // out[i] = tile_off[tile] + exclusive prefix inside the tile; the last tile also writes out[n] = grand total.
-__global__ void k_tile_scan(const int32_t* __restrict__ in, int64_t n, const int32_t* __restrict__ tile_off,
-                            int32_t* __restrict__ out) {
+template <typename T>
+__global__ void k_tile_scan(const T* __restrict__ in, int64_t n, const T* __restrict__ tile_off, T* __restrict__ out) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    int v[kScanItems];
-    int s = 0;
+    T v[kScanItems];
+    T s{};
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        v[k] = base + k < n ? in[base + k] : 0;
-        s += v[k];
+        v[k] = base + k < n ? in[base + k] : T{};
+        s = s + v[k];
     }
-    int total;
-    int run = block_exclusive_scan(s, &total) + (tile_off ? tile_off[blockIdx.x] : 0);
+    T total;
+    T run = block_exclusive_scan(s, &total);
+    if (tile_off) run = tile_off[blockIdx.x] + run;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         if (base + k < n) out[base + k] = run;
-        run += v[k];
+        run = run + v[k];
         if (base + k == n - 1) out[n] = run;
     }
 }
 
-// out has n + 1 entries: exclusive prefix sums and the total.  `in` and `out` may not alias.
-int exclusive_scan(const int32_t* in, int64_t n, int32_t* out, cudaStream_t st) {
-    if (n == 0) {
-        GNNPRE_CUDA(cudaMemsetAsync(out, 0, sizeof(int32_t), st));
-        return GNNPRE_OK;
-    }
-    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-    if (tiles == 1) {
-        k_tile_scan<<<1, kTB, 0, st>>>(in, n, nullptr, out);
+int64_t scan_tiles(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
+
+// Items of temporary memory exclusive_scan wants.
+size_t scan_temp_items(int64_t n) {
+    size_t items = 0;
+    for (int64_t t = scan_tiles(n); t > 1; t = scan_tiles(t)) items += 2 * (size_t)t + 1;
+    return items;
+}
+
+// out has n + 1 entries (n >= 1): exclusive prefix sums and the total.  `in` and `out` may not alias.
+template <typename T>
+int exclusive_scan(const T* in, int64_t n, T* out, T* temp, cudaStream_t st) {
+    const int64_t tiles = scan_tiles(n);
+    const T* offs = nullptr;
+    if (tiles > 1) {
+        T* sums = temp;
+        T* tile_offs = temp + tiles;
+        k_tile_sums<<<(unsigned)tiles, kTB, 0, st>>>(in, n, sums);
         GNNPRE_CUDA(cudaGetLastError());
-        return GNNPRE_OK;
+        GNNPRE_TRY(exclusive_scan(sums, tiles, tile_offs, tile_offs + tiles + 1, st));
+        offs = tile_offs;
     }
-    DevBuf<int32_t> sums, offs;
-    GNNPRE_TRY(sums.alloc((size_t)tiles));
-    GNNPRE_TRY(offs.alloc((size_t)tiles + 1));
-    k_tile_sums<<<(unsigned)tiles, kTB, 0, st>>>(in, n, sums.p);
+    k_tile_scan<<<(unsigned)tiles, kTB, 0, st>>>(in, n, offs, out);
     GNNPRE_CUDA(cudaGetLastError());
-    GNNPRE_TRY(exclusive_scan(sums.p, tiles, offs.p, st));
-    k_tile_scan<<<(unsigned)tiles, kTB, 0, st>>>(in, n, offs.p, out);
-    GNNPRE_CUDA(cudaGetLastError());
-    GNNPRE_CUDA(cudaStreamSynchronize(st));  // temporaries die here
     return GNNPRE_OK;
 }
 
-// ---------------------------------------------------------------- rows of edges
-
-// Row holding edge e of the support: the last i with rowptr_t[i] <= e (rows without edges are skipped
-// because their successor shares their start).
-__device__ __forceinline__ int64_t row_of_edge(const int64_t* __restrict__ rowptr_t, int64_t n, int64_t e) {
-    int64_t lo = 0, hi = n;  // invariant: rowptr_t[lo] <= e < rowptr_t[hi]
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (rowptr_t[mid] <= e) lo = mid; else hi = mid;
-    }
-    return lo;
-}
+// ---------------------------------------------------------------- what the host has to know
 
 struct BlockRows {
     int32_t row_lo, row_hi, first_partial, last_partial;
     int64_t done_row_hi;
 };
 
-__global__ void k_block_rows(int b, const int64_t* __restrict__ e_off, const int64_t* __restrict__ rowptr_t,
-                             int64_t n, BlockRows* __restrict__ out) {
+// Thread l <= b: block l's rows (l < b), and what the segments before the block account for.
+__global__ void k_block_report(int b, const int64_t* __restrict__ e_off, const int64_t* __restrict__ seg_base,
+                               const SegCounts* __restrict__ before, const int64_t* __restrict__ rowptr_t, int64_t n,
+                               BlockRows* __restrict__ rows, SegCounts* __restrict__ at) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= b) return;
+    if (l > b) return;
+    at[l] = before[seg_base[l]];
+    if (l == b) return;
     const int64_t lo = e_off[l], hi = e_off[l + 1];
     const int64_t r0 = row_of_edge(rowptr_t, n, lo), r1 = row_of_edge(rowptr_t, n, hi - 1);
     BlockRows o;
@@ -224,15 +283,10 @@ __global__ void k_block_rows(int b, const int64_t* __restrict__ e_off, const int
         if (rowptr_t[mid + 1] <= hi) a = mid + 1; else z = mid;
     }
     o.done_row_hi = a;
-    out[l] = o;
+    rows[l] = o;
 }
 
 // ---------------------------------------------------------------- rows with and without edges
-
-__global__ void k_nonempty_flags(int64_t n, const int64_t* __restrict__ rowptr_t, int32_t* __restrict__ flag) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = rowptr_t[i + 1] > rowptr_t[i];
-}
 
 __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const int32_t* __restrict__ rank,
                              const float* __restrict__ rscale, int32_t* __restrict__ nzrows, float* __restrict__ nzscale,
@@ -252,7 +306,7 @@ __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const 
 // Segment t of block l nominally starts at e_lo(l) + t*L.  A start that falls inside a row is moved
 // forward to the next row start when that lies within `snap` edges (and inside the block), so that
 // short rows are never cut; long rows are cut and their parts summed by a fix-up.
-// Temporarily: slot_head holds the "first row began earlier" flag and pad holds the first row's index.
+// Until k_segment_finalize: slot_head holds the "first row began earlier" flag and pad the first row's index.
 __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict__ seg_base,
                                  const int64_t* __restrict__ e_off, int32_t L, int32_t snap,
                                  const int64_t* __restrict__ rowptr_t, int64_t n, const int32_t* __restrict__ rank,
@@ -292,72 +346,60 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     segs[s] = g;
 }
 
-// flags[2s] = segment s needs a head slot; flags[2s+1] = it needs a tail slot; emit[s] = the row
-// that began before segment s ends inside it (one fix-up per such row).
-__global__ void k_segment_flags(int64_t nseg, const Segment* __restrict__ segs, const int64_t* __restrict__ rowptr_t,
-                                int32_t* __restrict__ flags, int32_t* __restrict__ emit) {
+// What segment s accounts for: a scratch row if its first row began earlier (head), one if the row of its last edge
+// goes on and began in it (tail), a fix-up if the row that began earlier ends in it.  first[s] = the segment that row
+// began in.
+__global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs, const int64_t* __restrict__ rowptr_t,
+                                 int32_t hub_parts, SegCounts* __restrict__ counts, int32_t* __restrict__ first) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     const Segment g = segs[s], nx = segs[s + 1];
     const int head = g.slot_head;
     // the row holding this segment's last edge continues iff the next segment's first row began earlier
     const int tail = nx.slot_head && rowptr_t[nx.pad] >= g.start;
-    flags[2 * s] = head;
-    flags[2 * s + 1] = tail;
-    emit[s] = head && rowptr_t[(int64_t)g.pad + 1] <= nx.start;
-}
-
-__global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, const int64_t* __restrict__ rowptr_t,
-                                   const int32_t* __restrict__ flags, const int32_t* __restrict__ slot_scan,
-                                   const int32_t* __restrict__ emit, const int32_t* __restrict__ emit_scan,
-                                   RowFixup* __restrict__ fixups) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg) return;
-    const int32_t row = segs[s].pad;
-    if (emit[s]) {
-        const int64_t first_edge = rowptr_t[row];
+    const int emit = head && rowptr_t[(int64_t)g.pad + 1] <= nx.start;
+    int hub = 0;
+    if (emit) {
+        const int64_t first_edge = rowptr_t[g.pad];
         int64_t lo = 0, hi = s;  // segs[lo].start <= first_edge < segs[hi].start
         while (hi - lo > 1) {
             const int64_t mid = (lo + hi) >> 1;
             if (segs[mid].start <= first_edge) lo = mid; else hi = mid;
         }
-        RowFixup f;
-        f.row = row;
-        f.seg_first = (int32_t)lo;
-        f.seg_last = (int32_t)s;
-        f.slot0 = slot_scan[2 * lo + 1];  // the tail slot of the row's first segment; the other parts follow it
-        fixups[emit_scan[s]] = f;
+        first[s] = (int32_t)lo;
+        hub = s - lo + 1 > hub_parts;
     }
-    segs[s].slot_head = flags[2 * s] ? slot_scan[2 * s] : -1;
-    segs[s].slot_tail = flags[2 * s + 1] ? slot_scan[2 * s + 1] : -1;
+    counts[s] = {head + tail, emit, hub};
 }
 
-__global__ void k_hub_flags(int64_t nfix, const RowFixup* __restrict__ fix, int32_t hub_parts, int32_t* __restrict__ flag) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nfix) flag[i] = fix[i].seg_last - fix[i].seg_first + 1 > hub_parts;
-}
-
-__global__ void k_hub_scatter(int64_t nfix, const int32_t* __restrict__ flag, const int32_t* __restrict__ scan,
-                              int32_t* __restrict__ hubs) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nfix && flag[i]) hubs[scan[i]] = (int32_t)i;
+__global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, const SegCounts* __restrict__ counts,
+                                   const SegCounts* __restrict__ before, const int32_t* __restrict__ first,
+                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s > nseg) return;
+    if (s < nseg) {
+        const SegCounts c = counts[s], b = before[s];
+        const int head = segs[s].slot_head;
+        if (c.fixups) {
+            RowFixup f;
+            f.row = segs[s].pad;
+            f.seg_first = first[s];
+            f.seg_last = (int32_t)s;
+            // the tail slot (the last slot) of the row's first segment; the other parts follow it
+            f.slot0 = before[first[s] + 1].slots - 1;
+            fixups[b.fixups] = f;
+            if (c.hubs) hubs[b.hubs] = b.fixups;
+        }
+        segs[s].slot_head = head ? b.slots : -1;
+        segs[s].slot_tail = c.slots > head ? b.slots + head : -1;
+    }
+    segs[s].pad = 0;
 }
 
 // Parts beyond which a cut row counts as a hub and gets a whole CTA of the finishing kernel (64 chains) instead of a
 // warp (8 chains).  One value for all widths, because the tree's shape decides the bits and those must not depend on
 // how a matrix is cut into column tiles.
 constexpr int32_t kHubParts = 64;
-
-__global__ void k_clear_pad(int64_t nseg, Segment* __restrict__ segs) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s <= nseg) segs[s].pad = 0;
-}
-
-__global__ void k_gather_i32(int count, const int64_t* __restrict__ idx, const int32_t* __restrict__ src,
-                             int32_t* __restrict__ dst) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) dst[i] = src[idx[i]];
-}
 
 int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, int num_sms) {
     if (bulk_copy) {
@@ -445,9 +487,7 @@ gnnpre_plan::~gnnpre_plan() {
 }
 
 int64_t gnnpre_plan::device_bytes() const {
-    size_t t = deg.bytes() + rscale.bytes() + cscale.bytes() + nzrows.bytes() + nzscale.bytes() + emptyrows.bytes() + rowptr_t.bytes() +
-               colx.bytes() + colx_stage[0].bytes() + colx_stage[1].bytes() + segments.bytes() + fixups.bytes() + hubs.bytes() +
-               scratch.bytes() + dev_error.bytes();
+    size_t t = arena[0].bytes() + arena[1].bytes() + colx_stage[0].bytes() + colx_stage[1].bytes();
     for (const auto& s : slab) t += s.bytes();
     for (const auto& s : whole) t += s.bytes();
     return (int64_t)t;
@@ -472,97 +512,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->teleport_alpha = opts->teleport_alpha;
     P->flags = opts->flags;
     P->structure_mem = csr->mem;
+    P->hub_parts = kHubParts;
     const int64_t m = P->nnz_tilde;
-
-    // ---- the CSR on the device (a temporary copy when the caller's lives on the host)
-    DevBuf<int64_t> tmp_rowptr;
-    DevBuf<int32_t> tmp_colidx, tmp_deg;
-    const int64_t* d_rowptr = csr->rowptr;
-    const int32_t* d_colidx = csr->colidx;
-    const int32_t* d_deg_in = degrees;
-    if (csr->mem == GNNPRE_MEM_HOST) {
-        if (csr->rowptr[0] != 0 || csr->rowptr[n] != nnz) return GNNPRE_ERR_INVALID_CSR;
-        GNNPRE_TRY(tmp_rowptr.alloc((size_t)n + 1));
-        GNNPRE_TRY(tmp_colidx.alloc((size_t)nnz));
-        GNNPRE_CUDA(cudaMemcpy(tmp_rowptr.p, csr->rowptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice));
-        if (nnz) GNNPRE_CUDA(cudaMemcpy(tmp_colidx.p, csr->colidx, sizeof(int32_t) * (size_t)nnz, cudaMemcpyHostToDevice));
-        d_rowptr = tmp_rowptr.p;
-        d_colidx = tmp_colidx.p;
-        if (degrees) {
-            GNNPRE_TRY(tmp_deg.alloc((size_t)n));
-            GNNPRE_CUDA(cudaMemcpy(tmp_deg.p, degrees, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
-            d_deg_in = tmp_deg.p;
-        }
-    } else {
-        int64_t ends[2] = {-1, -1};
-        GNNPRE_CUDA(cudaMemcpy(&ends[0], csr->rowptr, sizeof(int64_t), cudaMemcpyDeviceToHost));
-        GNNPRE_CUDA(cudaMemcpy(&ends[1], csr->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost));
-        if (ends[0] != 0 || ends[1] != nnz) return GNNPRE_ERR_INVALID_CSR;
-    }
-
-    // ---- validation
-    if (!(opts->flags & GNNPRE_FLAG_SKIP_VALIDATION)) {
-        DevBuf<int> err;
-        GNNPRE_TRY(err.alloc(1));
-        GNNPRE_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
-        k_validate<<<grid_for(n * 32, kTB), kTB, 0, st>>>(n, nnz, d_rowptr, d_colidx, err.p);
-        GNNPRE_CUDA(cudaGetLastError());
-        int h = 0;
-        GNNPRE_CUDA(cudaMemcpy(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost));
-        if (h) return GNNPRE_ERR_INVALID_CSR;
-    }
-
-    // ---- degrees and scales
-    GNNPRE_TRY(P->deg.alloc((size_t)n));
-    if (d_deg_in) {
-        GNNPRE_CUDA(cudaMemcpyAsync(P->deg.p, d_deg_in, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st));
-    } else {
-        k_degrees<<<grid_for(n, kTB), kTB, 0, st>>>(n, d_rowptr, P->deg.p);
-        GNNPRE_CUDA(cudaGetLastError());
-    }
-    GNNPRE_TRY(P->rscale.alloc((size_t)n));
-    GNNPRE_TRY(P->cscale.alloc((size_t)n));
-    k_scales<<<grid_for(n, kTB), kTB, 0, st>>>(P->op, n, P->deg.p, P->rscale.p, P->cscale.p);
-    GNNPRE_CUDA(cudaGetLastError());
-
-    // ---- E, the support's edge list
-    GNNPRE_TRY(P->rowptr_t.alloc((size_t)n + 1));
-    GNNPRE_TRY(P->colx.alloc((size_t)m));
-    k_support<<<grid_for(n * 32, kTB), kTB, 0, st>>>(diag ? 1 : 0, n, d_rowptr, d_colidx, P->rowptr_t.p, P->colx.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    GNNPRE_CUDA(cudaStreamSynchronize(st));
-    tmp_colidx.reset();
-    tmp_rowptr.reset();
-    tmp_deg.reset();
-
-    // ---- rows with / without edges (only SAGE can have empty rows)
-    DevBuf<int32_t> rank;
-    P->rows_all_nonempty = true;
-    P->num_nonempty = n;
-    P->num_empty = 0;
-    if (!diag) {
-        DevBuf<int32_t> flag;
-        GNNPRE_TRY(flag.alloc((size_t)n));
-        GNNPRE_TRY(rank.alloc((size_t)n + 1));
-        k_nonempty_flags<<<grid_for(n, kTB), kTB, 0, st>>>(n, P->rowptr_t.p, flag.p);
-        GNNPRE_CUDA(cudaGetLastError());
-        GNNPRE_TRY(exclusive_scan(flag.p, n, rank.p, st));
-        int32_t nonempty = 0;
-        GNNPRE_CUDA(cudaMemcpy(&nonempty, rank.p + n, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        P->num_nonempty = nonempty;
-        P->num_empty = n - nonempty;
-        if (P->num_empty > 0) {
-            P->rows_all_nonempty = false;
-            GNNPRE_TRY(P->nzrows.alloc((size_t)P->num_nonempty));
-            GNNPRE_TRY(P->nzscale.alloc((size_t)P->num_nonempty));
-            GNNPRE_TRY(P->emptyrows.alloc((size_t)P->num_empty));
-            k_split_rows<<<grid_for(n, kTB), kTB, 0, st>>>(n, flag.p, rank.p, P->rscale.p, P->nzrows.p, P->nzscale.p, P->emptyrows.p);
-            GNNPRE_CUDA(cudaGetLastError());
-            GNNPRE_CUDA(cudaStreamSynchronize(st));
-        } else {
-            rank.reset();
-        }
-    }
+    if (csr->mem == GNNPRE_MEM_HOST && (csr->rowptr[0] != 0 || csr->rowptr[n] != nnz)) return GNNPRE_ERR_INVALID_CSR;
 
     // ---- Eq. 12: (b, c)
     const int64_t F = P->feat_dim;
@@ -573,10 +525,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->beta_X = opts->operands_mem == GNNPRE_MEM_HOST ? 4 : 2;
     P->budget_bytes = opts->budget_bytes;
     if (P->budget_bytes <= 0) {
-        size_t free_b = 0, total_b = 0;
+        size_t free_b = 0, total_b = 0;  // nothing of the plan has been allocated yet
         GNNPRE_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        // what this plan already holds counts as part of the budget it is about to be charged for
-        P->budget_bytes = (int64_t)free_b + P->device_bytes();
+        P->budget_bytes = (int64_t)free_b;
     }
     const int64_t max_c = (F + 3) / 4;
     const int64_t max_b = std::min<int64_t>(std::max<int64_t>(m, 1), 1 << 20);
@@ -654,27 +605,96 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const int64_t nseg = seg_base[(size_t)b];
     if (nseg >= 0x3fffffffLL) return GNNPRE_ERR_INVALID_ARG;
     P->num_segments = nseg;
-    GNNPRE_TRY(P->segments.alloc((size_t)nseg + 1));
-    if (m == 0) {
-        // no edges at all: every row is empty; one empty block
-        P->blocks[0] = Block{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, n};
-        Segment sentinel{0, 0, -1, -1, 0};
-        GNNPRE_CUDA(cudaMemcpy(P->segments.p, &sentinel, sizeof(Segment), cudaMemcpyHostToDevice));
-        return GNNPRE_OK;
+    const bool e_host = P->structure_mem == GNNPRE_MEM_HOST;
+
+    // ---- device memory: one allocation for what has a known size, one for what the segments turn out to need - or, if the
+    // caller set no budget, nothing is streamed and what they can need at most is small, a single one.  (An allocation of a few MB takes about
+    // 370 us and its release 300, one of 64 MB no more.)  The temporaries of the build live where E goes at the very end,
+    // if there is room.
+    struct Report {  // followed by BlockRows[b] and SegCounts[b + 1]
+        int32_t err, nonempty;
+    };
+    static_assert(sizeof(Report) == 8 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
+    const size_t report_bytes = sizeof(Report) + sizeof(BlockRows) * (size_t)b + sizeof(SegCounts) * (size_t)(b + 1);
+    DevBuf<uint32_t> e_temp;
+    DevBuf<uint32_t>& colx = e_host ? e_temp : P->colx;  // E of a host-resident structure is on the device for the build only
+    Carve fixed;
+    fixed.want(P->deg, (size_t)n);
+    fixed.want(P->rscale, (size_t)n);
+    fixed.want(P->cscale, (size_t)n);
+    fixed.want(P->rowptr_t, (size_t)n + 1);
+    fixed.want(P->segments, (size_t)nseg + 1);
+    fixed.want(P->dev_error, 1);
+    if (!e_host) fixed.want(P->colx, (size_t)m);
+    auto want_sized = [&](Carve& carve, int64_t fixups, int64_t hubs, int64_t nonempty, int64_t empty, int64_t slots) {
+        carve.want(P->fixups, (size_t)fixups);
+        carve.want(P->hubs, (size_t)hubs);
+        if (empty > 0) {
+            carve.want(P->nzrows, (size_t)nonempty);
+            carve.want(P->nzscale, (size_t)nonempty);
+            carve.want(P->emptyrows, (size_t)empty);
+        }
+        carve.want(P->scratch, (size_t)slots * (size_t)P->slab_width);
+    };
+    // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
+    const int64_t most_rows = diag ? 0 : n;
+    const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
+    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (64 << 20);
+    if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
+    GNNPRE_TRY(fixed.place(P->arena[0]));
+    if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
+    DevBuf<char> temp_arena, report;
+    DevBuf<int32_t> flag, rank, rank_temp, first;
+    DevBuf<SegCounts> counts, before, counts_temp;
+    DevBuf<int64_t> offsets;
+    Carve temps;
+    temps.want(report, report_bytes);
+    temps.want(offsets, 2 * ((size_t)b + 1));
+    if (!diag) {
+        temps.want(flag, (size_t)n);
+        temps.want(rank, (size_t)n + 1);
+        temps.want(rank_temp, scan_temp_items(n));
+    }
+    temps.want(first, (size_t)nseg);
+    temps.want(counts, (size_t)nseg);
+    temps.want(before, (size_t)nseg + 1);
+    temps.want(counts_temp, scan_temp_items(nseg));
+    if (temps.bytes() <= colx.bytes()) GNNPRE_TRY(temps.place(reinterpret_cast<char*>(colx.p)));
+    else GNNPRE_TRY(temps.place(temp_arena));
+    Report* d_report = reinterpret_cast<Report*>(report.p);
+    BlockRows* d_rows = reinterpret_cast<BlockRows*>(report.p + sizeof(Report));
+    SegCounts* d_at = reinterpret_cast<SegCounts*>(d_rows + b);
+
+    // ---- the CSR on the device (a temporary copy when the caller's lives on the host)
+    DevBuf<int64_t> tmp_rowptr;
+    DevBuf<int32_t> tmp_colidx, tmp_deg;
+    const int64_t* d_rowptr = csr->rowptr;
+    const int32_t* d_colidx = csr->colidx;
+    const int32_t* d_deg_in = degrees;
+    if (csr->mem == GNNPRE_MEM_HOST) {
+        GNNPRE_TRY(tmp_rowptr.alloc((size_t)n + 1));
+        GNNPRE_TRY(tmp_colidx.alloc((size_t)nnz));
+        GNNPRE_CUDA(cudaMemcpy(tmp_rowptr.p, csr->rowptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice));
+        if (nnz) GNNPRE_CUDA(cudaMemcpy(tmp_colidx.p, csr->colidx, sizeof(int32_t) * (size_t)nnz, cudaMemcpyHostToDevice));
+        d_rowptr = tmp_rowptr.p;
+        d_colidx = tmp_colidx.p;
+        if (degrees) {
+            GNNPRE_TRY(tmp_deg.alloc((size_t)n));
+            GNNPRE_CUDA(cudaMemcpy(tmp_deg.p, degrees, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
+            d_deg_in = tmp_deg.p;
+        }
     }
 
-    DevBuf<int64_t> d_e_off, d_seg_base;
-    GNNPRE_TRY(d_e_off.alloc((size_t)b + 1));
-    GNNPRE_TRY(d_seg_base.alloc((size_t)b + 1));
-    GNNPRE_CUDA(cudaMemcpy(d_e_off.p, e_off.data(), sizeof(int64_t) * (size_t)(b + 1), cudaMemcpyHostToDevice));
-    GNNPRE_CUDA(cudaMemcpy(d_seg_base.p, seg_base.data(), sizeof(int64_t) * (size_t)(b + 1), cudaMemcpyHostToDevice));
-
-    DevBuf<BlockRows> d_rows;
-    GNNPRE_TRY(d_rows.alloc((size_t)b));
-    k_block_rows<<<grid_for(b, kTB), kTB, 0, st>>>((int)b, d_e_off.p, P->rowptr_t.p, n, d_rows.p);
+    // ---- rows
+    GNNPRE_CUDA(cudaMemsetAsync(d_report, 0, sizeof(Report), st));
+    GNNPRE_CUDA(cudaMemsetAsync(P->dev_error.p, 0, sizeof(int), st));
+    k_rows<<<grid_for(n, kTB), kTB, 0, st>>>(P->op, n, nnz, d_rowptr, d_deg_in, P->deg.p, P->rscale.p, P->cscale.p,
+                                             P->rowptr_t.p, flag.p, &d_report->err);
     GNNPRE_CUDA(cudaGetLastError());
-    std::vector<BlockRows> h_rows((size_t)b);
-    GNNPRE_CUDA(cudaMemcpy(h_rows.data(), d_rows.p, sizeof(BlockRows) * (size_t)b, cudaMemcpyDeviceToHost));
+    if (!diag) {  // only SAGE can have rows without edges
+        GNNPRE_TRY(exclusive_scan(flag.p, n, rank.p, rank_temp.p, st));
+        GNNPRE_CUDA(cudaMemcpyAsync(&d_report->nonempty, rank.p + n, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+    }
 
     // ---- segments, scratch slots and row fix-ups
     // How far a nominal cut inside a row may move forward to the next row start.  Half a segment keeps the segments
@@ -686,67 +706,54 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const int64_t lanes = f4_slab <= 4 ? 4 : f4_slab <= 8 ? 8 : f4_slab <= 16 ? 16 : 32;
     const bool one_wave = nseg * lanes <= (int64_t)P->num_sms * 768;
     const int32_t snap = one_wave ? L - 1 : L / 2;
-    k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base.p, d_e_off.p, L, snap,
-                                                              P->rowptr_t.p, n, rank.p, P->segments.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    DevBuf<int32_t> flags, slot_scan, emit, emit_scan;
-    GNNPRE_TRY(flags.alloc((size_t)nseg * 2));
-    GNNPRE_TRY(slot_scan.alloc((size_t)nseg * 2 + 1));
-    GNNPRE_TRY(emit.alloc((size_t)nseg));
-    GNNPRE_TRY(emit_scan.alloc((size_t)nseg + 1));
-    k_segment_flags<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, flags.p, emit.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    GNNPRE_TRY(exclusive_scan(flags.p, nseg * 2, slot_scan.p, st));
-    GNNPRE_TRY(exclusive_scan(emit.p, nseg, emit_scan.p, st));
-    int32_t n_slots = 0, n_fix = 0;
-    GNNPRE_CUDA(cudaMemcpy(&n_slots, slot_scan.p + nseg * 2, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    GNNPRE_CUDA(cudaMemcpy(&n_fix, emit_scan.p + nseg, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    P->num_slots = n_slots;
-    P->num_fixups = n_fix;
-    GNNPRE_TRY(P->fixups.alloc((size_t)n_fix));
-    k_segment_finalize<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, flags.p, slot_scan.p,
-                                                            emit.p, emit_scan.p, P->fixups.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    k_clear_pad<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, P->segments.p);
-    GNNPRE_CUDA(cudaGetLastError());
-
-    // fix-up ranges per block: the scan value at each block's first segment
-    DevBuf<int32_t> d_fix_at;
-    GNNPRE_TRY(d_fix_at.alloc((size_t)b + 1));
-    k_gather_i32<<<grid_for(b + 1, kTB), kTB, 0, st>>>((int)(b + 1), d_seg_base.p, emit_scan.p, d_fix_at.p);
-    GNNPRE_CUDA(cudaGetLastError());
-    std::vector<int32_t> fix_at((size_t)b + 1);
-    GNNPRE_CUDA(cudaMemcpy(fix_at.data(), d_fix_at.p, sizeof(int32_t) * (size_t)(b + 1), cudaMemcpyDeviceToHost));
-
-    // hub rows (more parts than a warp adds quickly) are listed so that the fix-up kernel can give each a CTA
-    P->hub_parts = kHubParts;
-    std::vector<int32_t> hub_at((size_t)b + 1, 0);
-    if (n_fix > 0) {
-        DevBuf<int32_t> hub_flag, hub_scan, d_hub_at;
-        DevBuf<int64_t> d_fix_at64;
-        GNNPRE_TRY(hub_flag.alloc((size_t)n_fix));
-        GNNPRE_TRY(hub_scan.alloc((size_t)n_fix + 1));
-        k_hub_flags<<<grid_for(n_fix, kTB), kTB, 0, st>>>(n_fix, P->fixups.p, P->hub_parts, hub_flag.p);
+    if (m > 0) {
+        std::vector<int64_t> h_off(e_off);
+        h_off.insert(h_off.end(), seg_base.begin(), seg_base.end());
+        GNNPRE_CUDA(cudaMemcpyAsync(offsets.p, h_off.data(), sizeof(int64_t) * h_off.size(), cudaMemcpyHostToDevice, st));
+        const int64_t *d_e_off = offsets.p, *d_seg_base = offsets.p + b + 1;
+        // (without rows that own no edge the scan's ranks are the row numbers)
+        k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap, P->rowptr_t.p, n,
+                                                                  rank.p, P->segments.p);
         GNNPRE_CUDA(cudaGetLastError());
-        GNNPRE_TRY(exclusive_scan(hub_flag.p, n_fix, hub_scan.p, st));
-        int32_t n_hubs = 0;
-        GNNPRE_CUDA(cudaMemcpy(&n_hubs, hub_scan.p + n_fix, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        P->num_hubs = n_hubs;
-        if (n_hubs > 0) {
-            GNNPRE_TRY(P->hubs.alloc((size_t)n_hubs));
-            k_hub_scatter<<<grid_for(n_fix, kTB), kTB, 0, st>>>(n_fix, hub_flag.p, hub_scan.p, P->hubs.p);
-            GNNPRE_CUDA(cudaGetLastError());
-            std::vector<int64_t> fix_at64(fix_at.begin(), fix_at.end());
-            GNNPRE_TRY(d_fix_at64.alloc((size_t)b + 1));
-            GNNPRE_TRY(d_hub_at.alloc((size_t)b + 1));
-            GNNPRE_CUDA(cudaMemcpy(d_fix_at64.p, fix_at64.data(), sizeof(int64_t) * (size_t)(b + 1), cudaMemcpyHostToDevice));
-            k_gather_i32<<<grid_for(b + 1, kTB), kTB, 0, st>>>((int)(b + 1), d_fix_at64.p, hub_scan.p, d_hub_at.p);
-            GNNPRE_CUDA(cudaGetLastError());
-            GNNPRE_CUDA(cudaMemcpy(hub_at.data(), d_hub_at.p, sizeof(int32_t) * (size_t)(b + 1), cudaMemcpyDeviceToHost));
-        }
-        GNNPRE_CUDA(cudaStreamSynchronize(st));  // temporaries die here
+        k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);
+        GNNPRE_CUDA(cudaGetLastError());
+        GNNPRE_TRY(exclusive_scan(counts.p, nseg, before.p, counts_temp.p, st));
+        k_block_report<<<grid_for(b + 1, kTB), kTB, 0, st>>>((int)b, d_e_off, d_seg_base, before.p, P->rowptr_t.p, n, d_rows, d_at);
+        GNNPRE_CUDA(cudaGetLastError());
     }
-
+    std::vector<int64_t> h_report((report_bytes + 7) / 8);
+    GNNPRE_CUDA(cudaMemcpy(h_report.data(), report.p, report_bytes, cudaMemcpyDeviceToHost));
+    const Report* rep = reinterpret_cast<const Report*>(h_report.data());
+    const BlockRows* h_rows = reinterpret_cast<const BlockRows*>(rep + 1);
+    const SegCounts* at = reinterpret_cast<const SegCounts*>(h_rows + b);
+    if (rep->err) return GNNPRE_ERR_INVALID_CSR;
+    P->num_nonempty = diag ? n : rep->nonempty;
+    P->num_empty = n - P->num_nonempty;
+    P->rows_all_nonempty = P->num_empty == 0;
+    if (m > 0) {
+        P->num_slots = at[b].slots;
+        P->num_fixups = at[b].fixups;
+        P->num_hubs = at[b].hubs;
+    }
+    if (!one_allocation) {
+        Carve sized;
+        want_sized(sized, P->num_fixups, P->num_hubs, P->num_nonempty, P->num_empty, P->num_slots);
+        GNNPRE_TRY(sized.place(P->arena[1]));
+    }
+    if (!P->rows_all_nonempty) {
+        k_split_rows<<<grid_for(n, kTB), kTB, 0, st>>>(n, flag.p, rank.p, P->rscale.p, P->nzrows.p, P->nzscale.p, P->emptyrows.p);
+        GNNPRE_CUDA(cudaGetLastError());
+    }
+    if (m == 0) {  // no edges at all: every row is empty; one empty block
+        P->blocks[0] = Block{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, n};
+        Segment sentinel{0, 0, -1, -1, 0};
+        GNNPRE_CUDA(cudaMemcpy(P->segments.p, &sentinel, sizeof(Segment), cudaMemcpyHostToDevice));
+        GNNPRE_CUDA(cudaStreamSynchronize(st));
+        return GNNPRE_OK;
+    }
+    k_segment_finalize<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, P->segments.p, counts.p, before.p, first.p, P->fixups.p,
+                                                                P->hubs.p);
+    GNNPRE_CUDA(cudaGetLastError());
     for (int64_t l = 0; l < b; ++l) {
         Block& B = P->blocks[(size_t)l];
         const BlockRows& r = h_rows[(size_t)l];
@@ -758,29 +765,39 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         B.last_partial = r.last_partial;
         B.seg_lo = seg_base[(size_t)l];
         B.seg_hi = seg_base[(size_t)l + 1];
-        B.fix_lo = fix_at[(size_t)l];
-        B.fix_hi = fix_at[(size_t)l + 1];
-        B.hub_lo = hub_at[(size_t)l];
-        B.hub_hi = hub_at[(size_t)l + 1];
+        B.fix_lo = at[l].fixups;
+        B.fix_hi = at[l + 1].fixups;
+        B.hub_lo = at[l].hubs;
+        B.hub_hi = at[l + 1].hubs;
         B.done_row_lo = l == 0 ? 0 : h_rows[(size_t)l - 1].done_row_hi;
         B.done_row_hi = l == b - 1 ? n : r.done_row_hi;
     }
 
-    GNNPRE_TRY(P->scratch.alloc((size_t)P->num_slots * (size_t)P->slab_width));
-    GNNPRE_TRY(P->dev_error.alloc(1));
-    GNNPRE_CUDA(cudaMemset(P->dev_error.p, 0, sizeof(int)));
+
+    // ---- E, the support's edge list: overwrites the temporaries
+    {
+        const bool check = !(opts->flags & GNNPRE_FLAG_SKIP_VALIDATION);
+        // 256 edges per warp, more (up to 2048) only while every warp the device holds still gets its share
+        const int64_t per_warp = 256 * std::min<int64_t>(8, 1 + nnz / ((int64_t)P->num_sms * 64 * 512));
+        const int64_t edge_blocks = ((nnz + per_warp - 1) / per_warp + kTB / 32 - 1) / (kTB / 32);
+        const int64_t row_blocks = diag ? (n + kTB - 1) / kTB : 0;
+        k_support<<<(unsigned)(edge_blocks + row_blocks), kTB, 0, st>>>(diag ? 1 : 0, check ? 1 : 0, n, nnz, per_warp, edge_blocks,
+                                                                       d_rowptr, d_colidx, colx.p, P->dev_error.p);
+        GNNPRE_CUDA(cudaGetLastError());
+        int h = 0;
+        GNNPRE_CUDA(cudaMemcpy(&h, P->dev_error.p, sizeof(int), cudaMemcpyDeviceToHost));  // everything is in place
+        if (h) return GNNPRE_ERR_INVALID_CSR;
+    }
 
     // ---- a host-resident structure keeps E in pinned memory and streams it block by block
     if (P->structure_mem == GNNPRE_MEM_HOST) {
         GNNPRE_TRY(P->colx_host.alloc((size_t)m));
-        GNNPRE_CUDA(cudaMemcpy(P->colx_host.p, P->colx.p, sizeof(uint32_t) * (size_t)m, cudaMemcpyDeviceToHost));
-        P->colx.reset();
+        GNNPRE_CUDA(cudaMemcpy(P->colx_host.p, colx.p, sizeof(uint32_t) * (size_t)m, cudaMemcpyDeviceToHost));
         int64_t longest = 0;
         for (const Block& B : P->blocks) longest = std::max(longest, B.e_hi - B.e_lo);
         GNNPRE_TRY(P->colx_stage[0].alloc((size_t)longest));
         if (b > 1) GNNPRE_TRY(P->colx_stage[1].alloc((size_t)longest));
     }
-    GNNPRE_CUDA(cudaStreamSynchronize(st));
     return GNNPRE_OK;
 }
 

@@ -98,6 +98,33 @@ def test_plan_with_caller_degrees_and_budget_search(B):
     assert ei.value.status == -6
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("nnz_half", [15, 16, 17, 127, 128, 129, 700])
+def test_support_across_warp_boundaries_and_runs_of_empty_rows(B, op, nnz_half):
+    """The support's edge list is built 256 edges to a warp, 32 at a time: edge counts around those sizes, a hub, runs of
+    31 to 5,000 rows without edges, self-loops before, inside and behind a row's columns; and each kind of violation of
+    the column contract is found wherever it sits."""
+    n = 9000
+    far = [40, 72, 105, 400, 5400, 8999]
+    edges = [(far[i % 6] - i // 6 % 30 - 1, far[(i + 1 + i // 180) % 6] - i // 6 % 30 - 1) for i in range(nnz_half // 2)]
+    edges += [(2000, 2001 + j) for j in range(nnz_half - len(edges))]
+    g = gi.from_edge_list(n, edges)
+    rp, ci = g.rowptr.numpy(), g.colidx.numpy()
+    rp_t, ci_t = orc.support(op, rp, ci)
+    plan = B.gnnpre_build_plan(*dev(g), op, 16)
+    srp, sci = B.gnnpre_plan_support(plan)
+    np.testing.assert_array_equal(srp.numpy(), rp_t)
+    np.testing.assert_array_equal(sci.numpy(), ci_t)
+    plan.close()
+    for at in (0, g.nnz // 2, g.nnz - 1):
+        for value in (n, -1, int(np.searchsorted(rp, at, side="right")) - 1):  # out of range twice, on the diagonal
+            bad = g.colidx.clone()
+            bad[at] = value
+            with pytest.raises(B.GnnpreError) as ei:
+                B.gnnpre_build_plan(g.rowptr.cuda(), bad.cuda(), op, 16)
+            assert ei.value.status == -2
+
+
 # ------------------------------------------------------------------ propagation parity
 
 def run_case(B, g, op, F, K, *, b=1, c=1, seg=0, flags=0, ldx=None, ldo=None, seed=1):
