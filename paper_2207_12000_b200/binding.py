@@ -127,10 +127,18 @@ def _csr(rowptr: torch.Tensor, colidx: torch.Tensor) -> gnnpre_csr_t:
     return gnnpre_csr_t(rowptr.numel() - 1, colidx.numel(), rowptr.data_ptr(), colidx.data_ptr(), _mem_of(rowptr))
 
 
+# The current stream's handle without building a torch.cuda.Stream around it (3.2 us a call).
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream
+
+
+def _pointers(tensors):
+    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
 
 
 def gnnpre_degrees(rowptr: torch.Tensor, colidx: torch.Tensor, stream=None) -> torch.Tensor:
@@ -216,23 +224,28 @@ def gnnpre_propagate(plan: Plan, X: torch.Tensor, K: int, out: Sequence[torch.Te
                      stream=None, want_stats: bool = False):
     """out[k-1] = A^ applied k times to X.  X and out are fp32 row-major views (stride(1) == 1) on the
     device, or host tensors (preferably pinned) for the streamed path.  Returns (out, stats-or-None)."""
-    assert X.dtype == torch.float32 and X.dim() == 2 and X.stride(1) == 1
-    n, F = X.shape
+    shape, xs = X.shape, X.stride()
+    assert X.dtype is torch.float32 and len(shape) == 2 and xs[1] == 1
+    n, F = shape
+    on_device = X.is_cuda
     if out is None:
         Fp = (F + 3) // 4 * 4  # the library works on whole groups of 4 columns
-        if X.is_cuda:
+        if on_device:
             out = [torch.empty((n, Fp), dtype=torch.float32, device=X.device)[:, :F] for _ in range(K)]
         else:
             out = [torch.empty((n, Fp), dtype=torch.float32, pin_memory=True)[:, :F] for _ in range(K)]
     assert len(out) == K
-    ldo = out[0].stride(0) if K > 0 else F
-    for o in out:
-        assert o.dtype == torch.float32 and o.shape == (n, F) and o.stride(1) == 1 and o.stride(0) == ldo
-        assert o.is_cuda == out[0].is_cuda
-    ptrs = (ctypes.c_void_p * max(K, 1))(*[o.data_ptr() for o in out])
+    ldo, out_device = F, on_device
+    if K > 0:
+        os, out_device = out[0].stride(), out[0].is_cuda
+        ldo = os[0]
+        assert os[1] == 1
+        for o in out:
+            assert o.dtype is torch.float32 and o.shape == shape and o.stride() == os and o.is_cuda == out_device
     stats = gnnpre_stats_t() if want_stats else None
-    _check(_lib.gnnpre_propagate(plan.handle, X.data_ptr(), X.stride(0), _mem_of(X), K, ptrs, ldo,
-                                 _mem_of(out[0]) if K > 0 else _mem_of(X),
+    _check(_lib.gnnpre_propagate(plan.handle, X.data_ptr(), xs[0], GNNPRE_MEM_DEVICE if on_device else GNNPRE_MEM_HOST, K,
+                                 _pointers(out) if K > 0 else (ctypes.c_void_p * 1)(), ldo,
+                                 GNNPRE_MEM_DEVICE if out_device else GNNPRE_MEM_HOST,
                                  _stream_ptr(stream), ctypes.byref(stats) if want_stats else None),
            "gnnpre_propagate")
     return list(out), stats
@@ -276,7 +289,7 @@ def gnnpre_propagate_weighted(plan: Plan, X: torch.Tensor, gamma, *, out=None, Z
     for o in list(out) + [Z]:
         assert o.is_cuda and o.dtype == torch.float32 and o.shape == (n, F) and o.stride(1) == 1
     assert all(o.stride(0) == out[0].stride(0) for o in out)
-    ptrs = (ctypes.c_void_p * K)(*[o.data_ptr() for o in out])
+    ptrs = _pointers(out)
     g = (ctypes.c_float * (K + 1))(*[float(v) for v in gamma])
     _check(_lib.gnnpre_propagate_weighted(plan.handle, X.data_ptr(), X.stride(0), K, ptrs, out[0].stride(0), g,
                                           Z.data_ptr(), Z.stride(0), _stream_ptr(stream)), "gnnpre_propagate_weighted")
@@ -296,30 +309,31 @@ def gnnpre_lc_first_layer(hops, batch, Wt: torch.Tensor, *, relu_mask: int = 0, 
     precision: GNNPRE_LC_TF32 (tf32 operands) or GNNPRE_LC_TF32X3 (split operands, fp32-like accuracy).
     With check=True the call synchronises and raises if a device-side wait ran out."""
     K = len(hops)
-    n, F = hops[0].shape
+    shape, hs = hops[0].shape, hops[0].stride()
+    n, F = shape
+    assert hs[1] == 1
     for h in hops:
-        assert h.is_cuda and h.dtype == torch.float32 and h.shape == (n, F) and h.stride(1) == 1
-        assert h.stride(0) == hops[0].stride(0)
-    assert Wt.is_cuda and Wt.dtype == torch.float32 and Wt.dim() == 2 and Wt.shape[1] == F and Wt.stride(1) == 1
-    H = Wt.shape[0]
+        assert h.is_cuda and h.dtype is torch.float32 and h.shape == shape and h.stride() == hs
+    H, ws = Wt.shape[0], Wt.stride()
+    assert Wt.is_cuda and Wt.dtype is torch.float32 and Wt.shape == (H, F) and ws[1] == 1
     if batch is None:
         B, bptr = n, None
     else:
-        if batch.dtype == torch.int64:  # the default index type of the host framework; the library takes int32
+        if batch.dtype is torch.int64:  # the default index type of the host framework; the library takes int32
             batch = batch.to(torch.int32)
-        assert batch.is_cuda and batch.dtype == torch.int32 and batch.dim() == 1 and batch.is_contiguous()
-        B, bptr = batch.numel(), batch.data_ptr()
+        assert batch.is_cuda and batch.dtype is torch.int32 and batch.dim() == 1 and batch.is_contiguous()
+        B, bptr = batch.shape[0], batch.data_ptr()
     if out is None:
         out = torch.empty((B, K * H) if concat else (K, B, H), dtype=torch.float32, device=Wt.device)
+    os = out.stride()
     if concat:
-        assert out.shape == (B, K * H) and out.stride(1) == 1
-        ldy, hop_stride = out.stride(0), H
+        assert out.shape == (B, K * H) and os[1] == 1
+        ldy, hop_stride = os[0], H
     else:
-        assert out.shape == (K, B, H) and out.stride(2) == 1
-        ldy, hop_stride = (out.stride(1), out.stride(0)) if B > 0 else (H, 0)
+        assert out.shape == (K, B, H) and os[2] == 1
+        ldy, hop_stride = (os[1], os[0]) if B > 0 else (H, 0)
     flag = torch.zeros(1, dtype=torch.int32, device=Wt.device) if check else None
-    ptrs = (ctypes.c_void_p * K)(*[h.data_ptr() for h in hops])
-    _check(_lib.gnnpre_lc_first_layer(ptrs, K, n, F, hops[0].stride(0), bptr, B, Wt.data_ptr(), H, Wt.stride(0),
+    _check(_lib.gnnpre_lc_first_layer(_pointers(hops), K, n, F, hs[0], bptr, B, Wt.data_ptr(), H, ws[0],
                                       relu_mask, precision, out.data_ptr(), ldy, hop_stride,
                                       flag.data_ptr() if check else None, _stream_ptr(stream)), "gnnpre_lc_first_layer")
     if check and int(flag.item()) != 0:

@@ -37,6 +37,7 @@
 // word; every role then leaves its loop, the producers wait for the copies they still have in
 // flight, the MMA lane waits (bounded) for the tensor core to drain, and tensor memory is freed.
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include <cuda.h>
@@ -63,6 +64,7 @@ constexpr int kLcX3SplitWarps = 4;                 // warps 9-12 compute the low
 constexpr int kLcX3SplitWarp0 = kLcProducerWarps + 1 + kLcX3EpilogueWarps;
 constexpr int kLcX3Threads = 32 * (kLcX3SplitWarp0 + kLcX3SplitWarps);
 constexpr uint32_t kLcX3MaxCols = 128;             // output columns of a CTA, columns of one accumulator buffer
+constexpr int kLcMaxDevices = 64;
 constexpr int kLcMaxHops = 8;                     // hop matrices per launch
 constexpr uint32_t kLcTmemCols = 512;
 constexpr uint32_t kLcSuspendNs = 20000;          // a failed poll parks the warp for up to this long
@@ -829,7 +831,13 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
     const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
     auto kernel = x3 ? k_lc_first_layer_x3 : k_lc_first_layer;
-    GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the opt-in to large dynamic shared memory, per kernel and device: always the most a launch can want, so once is enough
+    constexpr int kMostSmem = 1024 + kLcPipeBytes + 8 * kLcEpiBytes;
+    static std::atomic<bool> opted_in[2][kLcMaxDevices];
+    if (dev >= kLcMaxDevices || !opted_in[x3][dev].load(std::memory_order_relaxed)) {
+        GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
+        if (dev < kLcMaxDevices) opted_in[x3][dev].store(true, std::memory_order_relaxed);
+    }
 
     LcMaps maps;
     GNNPRE_TRY(encode_map_2d(Wt, feat_dim, hidden, ldw, kLcChunk, (int)hidden, &maps.w));
@@ -839,7 +847,7 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         for (int32_t k = 0; k < kLcMaxHops; ++k) {
             const int32_t kk = k0 + std::min(k, kn - 1);
             a.hop[k] = hops[kk];
-            GNNPRE_TRY(encode_map_2d(Y + (int64_t)kk * y_hop_stride, hidden, batch_size, ldy, 32, 32, &maps.y[k]));
+            if (k < kn) GNNPRE_TRY(encode_map_2d(Y + (int64_t)kk * y_hop_stride, hidden, batch_size, ldy, 32, 32, &maps.y[k]));
         }
         a.ldh = ldh;
         a.n = n;
