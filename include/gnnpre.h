@@ -262,8 +262,7 @@ int gnnpre_selftest_wait_timeout(gnnpre_plan_t* plan, uint32_t polls, void* stre
  */
 int gnnpre_inject_alloc_failure(int64_t device_countdown, int64_t host_countdown);
 
-/* Waits for the plan's own streams and for the last device-resident call that used it (not for the whole
- * device), then frees everything the plan owns. */
+/* Waits for the device (as freeing device memory does), then frees everything the plan owns. */
 void gnnpre_plan_destroy(gnnpre_plan_t* plan);
 
 /*

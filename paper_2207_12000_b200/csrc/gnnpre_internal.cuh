@@ -230,9 +230,6 @@ struct gnnpre_plan {
     bool col_slabs_forced = false;             // c was given by the caller: the slab loop is then kept as asked
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr, s_compute = nullptr, s_struct = nullptr;
     int busy = 0;
-    // recorded on the caller's stream after the last work of every device-resident call: what
-    // gnnpre_plan_destroy waits for instead of the whole device
-    cudaEvent_t last_use = nullptr;
 
     ~gnnpre_plan();
     int64_t device_bytes() const;

@@ -27,13 +27,15 @@ enum : int { kErrRowptr = 1, kErrColRange = 2, kErrDiagonal = 4, kErrOrder = 8, 
 // gave the degrees; A^_ij = r_i c_j: GCN r = c = (D_i + 1)^{-1/2} (Eq. 1); SAGE r = 1/D_i (0 for D_i = 0), c = 1;
 // GIN r = c = 1, evaluated in fp64 (IEEE sqrt and divide) and rounded once to fp32; the support's row pointers (with
 // self-loops row i of the support is row i of A plus one entry, so rowptr_t[i] = rowptr[i] + i); whether the row owns
-// an edge (flag may be nullptr).
+// an edge (flag may be nullptr); the length of A's longest row.
 __global__ void k_rows(int op, int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ deg_in,
                        int32_t* __restrict__ deg, float* __restrict__ rscale, float* __restrict__ cscale,
-                       int64_t* __restrict__ rowptr_t, int32_t* __restrict__ flag, int* err) {
+                       int64_t* __restrict__ rowptr_t, int32_t* __restrict__ flag, int* err, int* longest) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t lo = i < n ? rowptr[i] : 0, hi = i < n ? rowptr[i + 1] : 0;
+    const int most = __reduce_max_sync(0xffffffffu, (int)min(hi - lo, (int64_t)INT32_MAX));
+    if ((threadIdx.x & 31) == 0 && most > 0) atomicMax(longest, most);
     if (i >= n) return;
-    const int64_t lo = rowptr[i], hi = rowptr[i + 1];
     int bad = 0;
     if (lo < 0 || hi < lo || hi > nnz || (i == 0 && lo != 0) || (i == n - 1 && hi != nnz)) bad |= kErrRowptr;
     else if (hi - lo >= 0x7fffffffLL) bad |= kErrDegree;
@@ -305,10 +307,13 @@ __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const 
 
 // Segment t of block l nominally starts at e_lo(l) + t*L.  A start that falls inside a row is moved
 // forward to the next row start when that lies within `snap` edges (and inside the block), so that
-// short rows are never cut; long rows are cut and their parts summed by a fix-up.
+// short rows are never cut; long rows are cut and their parts summed by a fix-up.  Where no row of the graph is longer
+// than three segments the start always moves (two may then meet: an empty segment), and nothing is left for the
+// finishing launch: 4,096 nodes of degree 16, 64 columns, two hops 13.7 us at segments of 32, 11.1 at 16 and none cut.
+// Graphs with longer rows have that launch anyway and are better off balanced (5,000 nodes, R-MAT, 16.7 us against 19.5).
 // Until k_segment_finalize: slot_head holds the "first row began earlier" flag and pad the first row's index.
 __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict__ seg_base,
-                                 const int64_t* __restrict__ e_off, int32_t L, int32_t snap,
+                                 const int64_t* __restrict__ e_off, int32_t L, int32_t snap, const int* __restrict__ longest,
                                  const int64_t* __restrict__ rowptr_t, int64_t n, const int32_t* __restrict__ rank,
                                  Segment* __restrict__ segs) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -333,7 +338,7 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     int64_t row = row_of_edge(rowptr_t, n, start);
     if (t > 0 && rowptr_t[row] < start) {
         const int64_t next = rowptr_t[row + 1];
-        if (next - start <= snap && next < e_off[lo + 1]) {
+        if ((next - start <= snap || *longest < 3 * (int64_t)L) && next < e_off[lo + 1]) {
             start = next;
             row = row_of_edge(rowptr_t, n, start);
         }
@@ -401,7 +406,7 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
 // how a matrix is cut into column tiles.
 constexpr int32_t kHubParts = 64;
 
-int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, int num_sms) {
+int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool whole_hops, int num_sms) {
     if (bulk_copy) {
         // persistent warps walk whole segments with a two-stage pipeline that drains at every segment
         // end: long segments, but at least ~4 per resident warp so the tail stays short
@@ -420,7 +425,8 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, int nu
     const int64_t lanes = f4 <= 4 ? 4 : f4 <= 8 ? 8 : f4 <= 16 ? 16 : 32;
     const int64_t per_group = m / ((int64_t)std::max(num_sms, 1) * (28 * 32 / lanes));
     const int64_t L = std::max(std::min<int64_t>(per_group / (lanes <= 8 ? 2 : 3), 256), per_group / 8);
-    int32_t p = 32;
+    // (a resident graph so small that segments of 16 all run at once gets those: its hop is a chain of latencies)
+    int32_t p = whole_hops && (m / 16) * lanes <= (int64_t)num_sms * 768 ? 16 : 32;
     while ((int64_t)p * 2 <= L && p < 1024) p *= 2;
     return p;
 }
@@ -483,7 +489,6 @@ gnnpre_plan::~gnnpre_plan() {
     if (s_d2h) cudaStreamDestroy(s_d2h);
     if (s_compute) cudaStreamDestroy(s_compute);
     if (s_struct) cudaStreamDestroy(s_struct);
-    if (last_use) cudaEventDestroy(last_use);
 }
 
 int64_t gnnpre_plan::device_bytes() const {
@@ -588,7 +593,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->segment_edges = opts->segment_edges > 0
                            ? opts->segment_edges
                            : auto_segment_edges(P->slab_width, m_launch, uses_bulk_copy(P, (int32_t)P->slab_width),
-                                                P->num_sms);
+                                                !per_block, P->num_sms);
     if (P->segment_edges < 1) return GNNPRE_ERR_INVALID_ARG;
 
     // ---- block table: block l = edges [floor(l m / b), floor((l+1) m / b))
@@ -612,9 +617,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // 370 us and its release 300, one of 64 MB no more.)  The temporaries of the build live where E goes at the very end,
     // if there is room.
     struct Report {  // followed by BlockRows[b] and SegCounts[b + 1]
-        int32_t err, nonempty;
+        int32_t err, nonempty, longest_row, unused;
     };
-    static_assert(sizeof(Report) == 8 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
+    static_assert(sizeof(Report) == 16 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
     const size_t report_bytes = sizeof(Report) + sizeof(BlockRows) * (size_t)b + sizeof(SegCounts) * (size_t)(b + 1);
     DevBuf<uint32_t> e_temp;
     DevBuf<uint32_t>& colx = e_host ? e_temp : P->colx;  // E of a host-resident structure is on the device for the build only
@@ -689,7 +694,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     GNNPRE_CUDA(cudaMemsetAsync(d_report, 0, sizeof(Report), st));
     GNNPRE_CUDA(cudaMemsetAsync(P->dev_error.p, 0, sizeof(int), st));
     k_rows<<<grid_for(n, kTB), kTB, 0, st>>>(P->op, n, nnz, d_rowptr, d_deg_in, P->deg.p, P->rscale.p, P->cscale.p,
-                                             P->rowptr_t.p, flag.p, &d_report->err);
+                                             P->rowptr_t.p, flag.p, &d_report->err, &d_report->longest_row);
     GNNPRE_CUDA(cudaGetLastError());
     if (!diag) {  // only SAGE can have rows without edges
         GNNPRE_TRY(exclusive_scan(flag.p, n, rank.p, rank_temp.p, st));
@@ -699,9 +704,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // ---- segments, scratch slots and row fix-ups
     // How far a nominal cut inside a row may move forward to the next row start.  Half a segment keeps the segments
     // balanced (moving by up to a whole one cost 3-15 % on every larger workload).  A launch so small that all its
-    // segments are resident at once is bound by latency, not balance: there the cut may move by up to L - 1 edges,
-    // which leaves a graph of short rows without any cut row and so without the fix-up launch (4,096 nodes of
-    // degree 16: two launches per step of two hops instead of four, 39 -> 31 us).
+    // segments are resident at once is bound by latency, not balance: there the cut may move by up to L - 1 edges.
     const int64_t f4_slab = std::min<int64_t>(P->slab_width, 512) / 4;
     const int64_t lanes = f4_slab <= 4 ? 4 : f4_slab <= 8 ? 8 : f4_slab <= 16 ? 16 : 32;
     const bool one_wave = nseg * lanes <= (int64_t)P->num_sms * 768;
@@ -712,8 +715,8 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         GNNPRE_CUDA(cudaMemcpyAsync(offsets.p, h_off.data(), sizeof(int64_t) * h_off.size(), cudaMemcpyHostToDevice, st));
         const int64_t *d_e_off = offsets.p, *d_seg_base = offsets.p + b + 1;
         // (without rows that own no edge the scan's ranks are the row numbers)
-        k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap, P->rowptr_t.p, n,
-                                                                  rank.p, P->segments.p);
+        k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap,
+                                                                  &d_report->longest_row, P->rowptr_t.p, n, rank.p, P->segments.p);
         GNNPRE_CUDA(cudaGetLastError());
         k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);
         GNNPRE_CUDA(cudaGetLastError());
@@ -916,17 +919,9 @@ extern "C" int gnnpre_plan_support(const gnnpre_plan_t* P, int64_t* rowptr_out, 
 
 extern "C" void gnnpre_plan_destroy(gnnpre_plan_t* P) {
     if (!P) return;
-    // Wait for the work that still uses the plan's memory - the last device-resident call (an event on the
-    // caller's stream) and the plan's own streams - not for the whole device.
-    // (an event last recorded inside a stream capture cannot be waited for: then wait for the device)
-    if (P->last_use && cudaEventSynchronize(P->last_use) != cudaSuccess) {
-        (void)cudaGetLastError();
-        cudaDeviceSynchronize();
-    }
-    if (P->s_h2d) cudaStreamSynchronize(P->s_h2d);
-    if (P->s_compute) cudaStreamSynchronize(P->s_compute);
-    if (P->s_d2h) cudaStreamSynchronize(P->s_d2h);
-    if (P->s_struct) cudaStreamSynchronize(P->s_struct);
+    // Work on the caller's streams may still use the plan's memory.  Freeing it waits for the device in any case; an event
+    // recorded after every call, to wait for instead, stood between that call and the next one's first kernel (3 us).
+    cudaDeviceSynchronize();
     (void)cudaGetLastError();
     delete P;
 }

@@ -426,8 +426,6 @@ int propagate_resident(gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, f
         }
         if (rc == GNNPRE_OK) rc = mark(hop_ev);
     }
-    if (!P->last_use) GNNPRE_CUDA(cudaEventCreateWithFlags(&P->last_use, cudaEventDisableTiming));
-    GNNPRE_CUDA(cudaEventRecord(P->last_use, st));  // the plan's scratch is in use until here
     if (stats) {
         if (rc == GNNPRE_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = GNNPRE_ERR_CUDA;
         if (rc == GNNPRE_OK) rc = check_device_error(P);
