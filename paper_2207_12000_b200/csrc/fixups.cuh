@@ -67,7 +67,6 @@ __global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
     constexpr int kRounds = CH >= 8 ? 1 : CH >= 4 ? 2 : 4;  // parts in flight per chain
     static_assert(CW == 8, "the tree's shape must not depend on the width");
     __shared__ float4 meet[kWarps][2][G];
-    allow_next_kernel();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gl = lane & (G - 1), sub = lane / G;
     const int q0 = blockIdx.y * a.tile_f4;

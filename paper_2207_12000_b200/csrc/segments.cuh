@@ -40,7 +40,6 @@ struct __align__(16) SegStage {  // read in 16-byte pieces
 
 template <int G, int OP, bool HAS_EMPTY, int EP>
 __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
-    allow_next_kernel();
     constexpr unsigned kFull = 0xffffffffu;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN;
     using Stage = SegStage<G, kWeighted>;

@@ -118,7 +118,6 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
-    allow_next_kernel();
     wait_previous_kernel();
 
     uint32_t phase[kTmaStages];
