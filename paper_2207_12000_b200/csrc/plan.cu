@@ -613,8 +613,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const bool e_host = P->structure_mem == GNNPRE_MEM_HOST;
 
     // ---- device memory: one allocation for what has a known size, one for what the segments turn out to need - or, if the
-    // caller set no budget, nothing is streamed and what they can need at most is small, a single one.  (An allocation of a few MB takes about
-    // 370 us and its release 300, one of 64 MB no more.)  The temporaries of the build live where E goes at the very end,
+    // caller set no budget, nothing is streamed and what they can need at most is small, a single one.  (An allocation of a
+    // few MB takes 370 to 1600 us and its release 300, one of 64 MB no more; one of up to 1 MB, a piece of a page the
+    // driver mostly has at hand, about 1 us.)  The temporaries of the build live where E goes at the very end,
     // if there is room.
     struct Report {  // followed by BlockRows[b] and SegCounts[b + 1]
         int32_t err, nonempty, longest_row, unused;
@@ -644,7 +645,8 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
     const int64_t most_rows = diag ? 0 : n;
     const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
-    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (64 << 20);
+    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (64 << 20) &&
+                                fixed.bytes() > (1 << 20);
     if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
     GNNPRE_TRY(fixed.place(P->arena[0]));
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
