@@ -408,6 +408,11 @@ def gnnpre_inject_alloc_failure(device_countdown: int = -1, host_countdown: int 
     _check(_lib.gnnpre_inject_alloc_failure(device_countdown, host_countdown), "gnnpre_inject_alloc_failure")
 
 
+def gnnpre_release_cached_memory() -> None:
+    """Frees the device memory that a closed plan left for the next one (at most 128 MB per device)."""
+    _check(_lib.gnnpre_release_cached_memory(), "gnnpre_release_cached_memory")
+
+
 def gnnpre_solve_budget(B_S, B_X, B_fixed, beta_S, beta_X, B_GPU, max_b, max_c):
     b, c = ctypes.c_int64(), ctypes.c_int64()
     rc = _lib.gnnpre_solve_budget(B_S, B_X, B_fixed, beta_S, beta_X, B_GPU, max_b, max_c, ctypes.byref(b),
@@ -426,5 +431,5 @@ def exported_symbols():
     return ["gnnpre_degrees", "gnnpre_build_plan", "gnnpre_plan_info", "gnnpre_plan_block", "gnnpre_plan_scales",
             "gnnpre_plan_support", "gnnpre_propagate", "gnnpre_propagate_weighted", "gnnpre_hop_static", "gnnpre_lc_first_layer", "gnnpre_lc_selftest_wait_timeout", "gnnpre_normalize",
             "gnnpre_solve_normalisation_blocks", "gnnpre_selftest_wait_timeout", "gnnpre_selftest_wait_timeout_async",
-            "gnnpre_plan_status", "gnnpre_inject_alloc_failure", "gnnpre_gather_ceiling", "gnnpre_describe_panels", "gnnpre_plan_destroy", "gnnpre_solve_budget",
+            "gnnpre_plan_status", "gnnpre_inject_alloc_failure", "gnnpre_gather_ceiling", "gnnpre_describe_panels", "gnnpre_plan_destroy", "gnnpre_release_cached_memory", "gnnpre_solve_budget",
             "gnnpre_status_string", "gnnpre_last_cuda_error"]

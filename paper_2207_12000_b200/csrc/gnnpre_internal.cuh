@@ -34,6 +34,9 @@ void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int 
 // reported as failed.  kind 0 = device memory, 1 = page-locked host memory.
 bool injected_alloc_failure(int kind);
 
+// Frees the block of device memory that the current device's cache keeps (see plan.cu); false if there is none.
+bool release_cached_block();
+
 // Device memory: an allocation of its own that frees itself, or a piece of another buffer (see Carve).
 template <typename T>
 struct DevBuf {
@@ -57,7 +60,13 @@ struct DevBuf {
             set_last_cuda_error(cudaErrorMemoryAllocation, "cudaMalloc (injected failure)", __FILE__, __LINE__);
             return GNNPRE_ERR_OOM_DEVICE;
         }
-        GNNPRE_CUDA(cudaMalloc(reinterpret_cast<void**>(&p), n * sizeof(T)));
+        cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&p), n * sizeof(T));
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            if (release_cached_block()) e = cudaMalloc(reinterpret_cast<void**>(&p), n * sizeof(T));
+        }
+        if (e != cudaSuccess) p = nullptr;
+        GNNPRE_CUDA(e);
         count = n;
         return GNNPRE_OK;
     }
@@ -193,6 +202,7 @@ struct gnnpre_plan {
 
     // what the buffers below (but for the streamed structure's and the streaming state's) are pieces of
     gnnpre::DevBuf<char> arena[2];
+    bool arena_cached = false;  // arena[0] goes back to the cache instead of being freed
     // per-node arrays (device)
     gnnpre::DevBuf<int32_t> deg;
     gnnpre::DevBuf<float> rscale, cscale;

@@ -4,7 +4,9 @@
 // O(b) block arithmetic and the Eq. 12 search.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
+#include <utility>
 
 #include "gnnpre_internal.cuh"
 
@@ -484,7 +486,59 @@ int check_device() {
 
 using namespace gnnpre;
 
+namespace {
+
+// One block of device memory per device outlives the plan that used it, so that a program that makes plan after plan (one
+// per dataset, or per operator) does not pay 0.7 to 8 ms for an allocation and its release each time.  At most
+// kMostCached bytes; only plans for resident operands without a memory budget use it; it is given back when an
+// allocation of the library fails and by gnnpre_release_cached_memory.  A block enters it when the device is idle.
+constexpr size_t kMostCached = 128u << 20, kCachedGrain = 2u << 20;
+constexpr int kCacheDevices = 64;
+
+struct CachedBlock {
+    char* p = nullptr;
+    size_t bytes = 0;
+};
+std::mutex g_cache_mutex;
+CachedBlock g_cache[kCacheDevices];
+
+CachedBlock take_cached(int device, size_t bytes) {
+    std::lock_guard<std::mutex> lock(g_cache_mutex);
+    CachedBlock b;
+    if (device < kCacheDevices && g_cache[device].bytes >= bytes) std::swap(b, g_cache[device]);
+    return b;
+}
+
+// keeps the larger of `b` and what the cache holds, frees the other
+void give_cached(int device, CachedBlock b) {
+    {
+        std::lock_guard<std::mutex> lock(g_cache_mutex);
+        if (device < kCacheDevices && g_cache[device].bytes < b.bytes) std::swap(b, g_cache[device]);
+    }
+    if (b.p) cudaFree(b.p);
+}
+
+}  // namespace
+
+bool gnnpre::release_cached_block() {
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    const CachedBlock b = take_cached(device, 1);
+    if (b.p) cudaFree(b.p);
+    return b.p != nullptr;
+}
+
+extern "C" int gnnpre_release_cached_memory(void) {
+    (void)release_cached_block();
+    return GNNPRE_OK;
+}
+
 gnnpre_plan::~gnnpre_plan() {
+    if (arena_cached && arena[0].p) {  // (a build that failed may still have kernels in flight)
+        cudaDeviceSynchronize();
+        give_cached(device, {arena[0].p, arena[0].count});
+        arena[0].owned = false;
+    }
     if (s_h2d) cudaStreamDestroy(s_h2d);
     if (s_d2h) cudaStreamDestroy(s_d2h);
     if (s_compute) cudaStreamDestroy(s_compute);
@@ -645,10 +699,20 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
     const int64_t most_rows = diag ? 0 : n;
     const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
-    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (64 << 20) &&
+    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
                                 fixed.bytes() > (1 << 20);
     if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
-    GNNPRE_TRY(fixed.place(P->arena[0]));
+    if (one_allocation && fixed.bytes() <= kMostCached - kCachedGrain) {  // in whole grains, so that the next plan's may fit
+        const size_t bytes = (fixed.bytes() + kCachedGrain - 1) / kCachedGrain * kCachedGrain;
+        const CachedBlock block = take_cached(P->device, bytes);
+        P->arena_cached = true;
+        P->arena[0].p = block.p;
+        P->arena[0].count = block.bytes;
+        if (!block.p) GNNPRE_TRY(P->arena[0].alloc(bytes));
+        GNNPRE_TRY(fixed.place(P->arena[0].p));
+    } else {
+        GNNPRE_TRY(fixed.place(P->arena[0]));
+    }
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
     DevBuf<char> temp_arena, report;
     DevBuf<int32_t> flag, rank, rank_temp, first;

@@ -193,6 +193,43 @@ def test_injected_allocation_failures_leave_nothing_behind(B):
     assert torch.cuda.mem_get_info()[0] == free0
 
 
+def test_cached_block_is_reused_bounded_and_given_back(B):
+    """Device memory of a closed resident plan is kept for the next one (one block), plans that live at the same time have
+    blocks of their own and equal results, and the release call gives the memory back."""
+    B.gnnpre_release_cached_memory()
+    free0 = torch.cuda.mem_get_info()[0]
+    g, small = gi.rmat(30000, 300000, 61, directed_candidates=True), gi.rmat(20000, 150000, 62, directed_candidates=True)
+    X, Xs = gi.normal_matrix(g.n, 64, 1, device="cuda"), gi.normal_matrix(small.n, 64, 2, device="cuda")
+    torch.cuda.synchronize()
+    d, ds = dev(g), dev(small)
+
+    def hop(plan, x):
+        r = B.gnnpre_propagate(plan, x, 1)[0][0].clone()
+        torch.cuda.synchronize()
+        return r
+
+    want, wants = [], []
+    for order in range(3):
+        a = B.gnnpre_build_plan(*d, order, 64)
+        b = B.gnnpre_build_plan(*ds, order, 64)
+        want.append(hop(a, X))
+        wants.append(hop(b, Xs))
+        a.close()
+        c = B.gnnpre_build_plan(*ds, order, 64)  # takes the block a left while b lives
+        assert torch.equal(hop(c, Xs), wants[-1]) and torch.equal(hop(b, Xs), wants[-1])
+        b.close()
+        a = B.gnnpre_build_plan(*d, order, 64)
+        assert torch.equal(hop(a, X), want[-1]) and torch.equal(hop(c, Xs), wants[-1])
+        a.close()
+        c.close()
+    del want, wants, X, Xs, a, b, c, d, ds
+    torch.cuda.empty_cache()
+    held = free0 - torch.cuda.mem_get_info()[0]
+    assert held <= 128 << 20
+    B.gnnpre_release_cached_memory()
+    assert torch.cuda.mem_get_info()[0] >= free0
+
+
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
     """X, out[] and Z are checked for shared elements, not only for equal base pointers; the hops of one call
     may be column views of one wide buffer (concatenated hops, as JKNet's COMB wants them)."""
