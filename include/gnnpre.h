@@ -80,7 +80,8 @@ typedef struct {
     int64_t feat_dim;        /* F: columns of X.  Work is done on whole groups of 4 columns: with F % 4 != 0 the
                                 1..3 pad columns up to the next multiple of 4 (which ldx, ldo >= that multiple
                                 make room for) are read from X and written to out[] with unspecified values */
-    int64_t budget_bytes;    /* B_GPU of Eq. 12; 0 = the device's free memory at plan time */
+    int64_t budget_bytes;    /* B_GPU of Eq. 12; 0 = the device's free memory at plan time (taken to suffice, without asking
+                                the driver, for a resident plan whose volumes are at most 1/16 of the device) */
     int32_t force_blocks;    /* b; 0 = solve Eq. 12 */
     int32_t force_col_slabs; /* c; 0 = solve Eq. 12 */
     int32_t segment_edges;   /* edges per warp-level segment; 0 = chosen from F */

@@ -151,9 +151,9 @@ def gnnpre_degrees(rowptr: torch.Tensor, colidx: torch.Tensor, stream=None) -> t
 class Plan:
     """Owns a gnnpre_plan_t*; destroyed with the object."""
 
-    def __init__(self, handle: int, keepalive):
+    def __init__(self, handle: int, nnz_tilde: int):
         self._h = ctypes.c_void_p(handle)
-        self._keepalive = keepalive
+        self.nnz_tilde = nnz_tilde  # edges of the operator's support
 
     @property
     def handle(self):
@@ -186,7 +186,7 @@ def gnnpre_build_plan(rowptr: torch.Tensor, colidx: torch.Tensor, op: int, feat_
     out = ctypes.c_void_p()
     _check(_lib.gnnpre_build_plan(ctypes.byref(csr), degrees.data_ptr() if degrees is not None else None,
                                   ctypes.byref(opts), ctypes.byref(out)), "gnnpre_build_plan")
-    return Plan(out.value, None)
+    return Plan(out.value, csr.nnz + (0 if op == GNNPRE_OP_SAGE_MEAN else csr.n))
 
 
 def gnnpre_plan_info(plan: Plan) -> dict:
@@ -343,7 +343,7 @@ def gnnpre_lc_first_layer(hops, batch, Wt: torch.Tensor, *, relu_mask: int = 0, 
 
 def gnnpre_normalize(plan: Plan, out: torch.Tensor | None = None, *, host: bool = False, stream=None) -> torch.Tensor:
     """fp32 value of every edge of the support (order of gnnpre_plan_support), on the device or in host memory."""
-    m = gnnpre_plan_info(plan)["nnz_tilde"]
+    m = plan.nnz_tilde
     if out is None:
         out = torch.empty(m, dtype=torch.float32, pin_memory=True) if host else torch.empty(
             m, dtype=torch.float32, device="cuda")

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "gnnpre.h"
@@ -193,7 +194,8 @@ struct gnnpre_plan {
     float teleport_alpha = 0.f;
     int32_t b = 1, c = 1;
     int64_t slab_width = 0;
-    int64_t B_S = 0, B_X = 0, B_fixed = 0, beta_S = 1, beta_X = 2, budget_bytes = 0;
+    int64_t B_S = 0, B_X = 0, B_fixed = 0, beta_S = 1, beta_X = 2;
+    mutable std::atomic<int64_t> budget_bytes{0};  // 0 = not asked for yet (see plan_budget)
     int32_t segment_edges = 0;
     uint32_t flags = 0;
     int32_t structure_mem = GNNPRE_MEM_DEVICE;
@@ -292,5 +294,6 @@ int solve_budget(int64_t B_S, int64_t B_X, int64_t B_fixed, int64_t beta_S, int6
 int check_device();
 int check_device_error(gnnpre_plan* plan);  // synchronous read of plan->dev_error: GNNPRE_ERR_TIMEOUT if set
 bool uses_bulk_copy(const gnnpre_plan* plan, int32_t width);
+int64_t plan_budget(const gnnpre_plan* plan);
 
 }  // namespace gnnpre

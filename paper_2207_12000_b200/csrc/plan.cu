@@ -3,6 +3,7 @@
 // warp-level segment tables the propagation kernels walk.  All of it runs on the GPU except the
 // O(b) block arithmetic and the Eq. 12 search.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -488,12 +489,45 @@ using namespace gnnpre;
 
 namespace {
 
+constexpr int kCacheDevices = 64;
+
+int64_t device_memory_bytes(int device) {
+    static std::atomic<int64_t> known[kCacheDevices];
+    int64_t bytes = device < kCacheDevices ? known[device].load(std::memory_order_relaxed) : 0;
+    if (bytes == 0) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
+        bytes = (int64_t)total_b;
+        if (device < kCacheDevices) known[device].store(bytes, std::memory_order_relaxed);
+    }
+    return bytes;
+}
+
+}  // namespace
+
+// B_GPU of Eq. 12: what the caller set, else the device's free memory when the plan was built or, if nobody asked then,
+// when somebody first does.
+int64_t gnnpre::plan_budget(const gnnpre_plan* P) {
+    int64_t budget = P->budget_bytes.load(std::memory_order_relaxed);
+    if (budget <= 0) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        budget = (int64_t)free_b + P->device_bytes();
+        P->budget_bytes.store(budget, std::memory_order_relaxed);
+    }
+    return budget;
+}
+
+namespace {
+
 // One block of device memory per device outlives the plan that used it, so that a program that makes plan after plan (one
 // per dataset, or per operator) does not pay 0.7 to 8 ms for an allocation and its release each time.  At most
 // kMostCached bytes; only plans for resident operands without a memory budget use it; it is given back when an
 // allocation of the library fails and by gnnpre_release_cached_memory.  A block enters it when the device is idle.
 constexpr size_t kMostCached = 128u << 20, kCachedGrain = 2u << 20;
-constexpr int kCacheDevices = 64;
 
 struct CachedBlock {
     char* p = nullptr;
@@ -583,10 +617,21 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->beta_S = csr->mem == GNNPRE_MEM_HOST ? 2 : 1;
     P->beta_X = opts->operands_mem == GNNPRE_MEM_HOST ? 4 : 2;
     P->budget_bytes = opts->budget_bytes;
-    if (P->budget_bytes <= 0) {
-        size_t free_b = 0, total_b = 0;  // nothing of the plan has been allocated yet
-        GNNPRE_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        P->budget_bytes = (int64_t)free_b;
+    const bool resident = opts->operands_mem == GNNPRE_MEM_DEVICE && csr->mem == GNNPRE_MEM_DEVICE;
+    int64_t budget = P->budget_bytes;
+    if (budget <= 0) {
+        // The free memory, but for the question: on a busy machine the driver takes 0.06 to 100 ms to answer it (median 0.4),
+        // longer than everything else a small plan needs.  A resident plan whose volumes are a sixteenth of the device at
+        // most is not asked about; gnnpre_plan_info asks when it is called.
+        const int64_t device_bytes = device_memory_bytes(P->device);
+        if (resident && P->B_S + P->beta_X * P->B_X + P->B_fixed <= device_bytes / 16) {
+            budget = device_bytes;
+        } else {
+            size_t free_b = 0, total_b = 0;  // nothing of the plan has been allocated yet
+            GNNPRE_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            budget = (int64_t)free_b;
+            P->budget_bytes = budget;
+        }
     }
     const int64_t max_c = (F + 3) / 4;
     const int64_t max_b = std::min<int64_t>(std::max<int64_t>(m, 1), 1 << 20);
@@ -603,7 +648,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
             int64_t tb = 0, tc = 0;
             // restrict the search to this c by scaling: solve with max_c = 1 on B_X / cc
             const int64_t x_part = (P->beta_X * P->B_X + cc - 1) / cc;
-            int rc = solve_budget(P->B_S, 0, P->B_fixed + x_part, P->beta_S, 1, P->budget_bytes, max_b, 1, &tb, &tc);
+            int rc = solve_budget(P->B_S, 0, P->B_fixed + x_part, P->beta_S, 1, budget, max_b, 1, &tb, &tc);
             if (rc != GNNPRE_OK) continue;
             if (b > 0) {
                 if (tb > b) continue;  // the forced b is too small for this c
@@ -935,7 +980,7 @@ extern "C" int gnnpre_plan_info(const gnnpre_plan_t* P, gnnpre_plan_info_t* o) {
     o->B_fixed = P->B_fixed;
     o->beta_S = P->beta_S;
     o->beta_X = P->beta_X;
-    o->budget_bytes = P->budget_bytes;
+    o->budget_bytes = plan_budget(P);
     o->device_bytes = P->device_bytes();
     o->host_bytes = P->host_bytes();
     o->num_segments = P->num_segments;

@@ -382,7 +382,7 @@ bool panels_apply(const gnnpre_plan* P, const float* X, int64_t ldx, int32_t K, 
     int64_t held = P->device_bytes();
     for (const auto& w : P->whole) held -= (int64_t)w.bytes();
     const int64_t need = (int64_t)(K + 1) * P->n * F * (int64_t)sizeof(float);
-    return held + need <= P->budget_bytes;
+    return held + need <= plan_budget(P);
 }
 
 // GNNPRE_ERR_OOM_DEVICE (with the buffers released) when the device cannot hold the K + 1 matrices after all.
