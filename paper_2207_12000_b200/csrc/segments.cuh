@@ -19,8 +19,8 @@
 // Bound by what an SM can draw from the L2 (64 bytes per cycle: a loop that only gathers takes 59 us on 169 K nodes,
 // 2.3 M edges, 128 columns) and, on short rows, by the instructions around the row ends.  On that graph, us per launch,
 // before (rows of 68..128 columns through the copy engine, one shuffle per edge and operand elsewhere) / now: 128
-// columns GCN 148 / 109, mean 123 / 77; 64 columns GCN 105 / 71, mean 75 / 51; 16 columns GCN 45 / 39, mean 35 / 29;
-// 256 columns, sum operator 223 / 186.  A persistent grid, four rows in flight at 48 registers, and 256-thread CTAs were
+// columns GCN 148 / 97, mean 123 / 77; 64 columns GCN 105 / 66, mean 75 / 51; 16 columns GCN 45 / 39, mean 35 / 29;
+// 256 columns, sum operator 223 / 173.  A persistent grid, four rows in flight at 48 registers, and 256-thread CTAs were
 // each slower.
 constexpr int kSegWindow = 8;
 
@@ -30,18 +30,52 @@ struct __align__(16) RowOut {
     int row;      // output row; -1 for a scratch row (no epilogue)
 };
 
+// A shared-memory load returns its bytes to every lane, 128 bytes per cycle and SM, as a row's 512 do: entry and weight of
+// an edge cost a cycle each beside the row's four.  Groups of 32 lanes therefore keep weights as single floats (169 K nodes,
+// GCN, 128 columns: 102.7 us per launch with weights stored twice, 97.3 so); narrower groups, where the instructions
+// count, as pairs ready for the packed multiply-add (64 columns: 66.0 us, 72.8 with single floats).
 template <int G, bool WEIGHTED>
 struct __align__(16) SegStage {  // read in 16-byte pieces
     static constexpr int kChunk = G < kSegWindow ? kSegWindow : G;  // edges staged at a time
+    static constexpr bool kPairs = G < 32;
+    using Weight = std::conditional_t<kPairs, float2, float>;
     RowOut out[kChunk];
     uint32_t col[kChunk];
-    float2 w[WEIGHTED ? kChunk : 1];
+    Weight w[WEIGHTED ? kChunk : 1];
+
+    __device__ __forceinline__ void set_weight(int i, float v) {
+        if constexpr (kPairs) w[i] = make_float2(v, v);
+        else w[i] = v;
+    }
+    __device__ __forceinline__ void add_weighted(Quad& acc, int i, const Quad& x) const {
+        if constexpr (kPairs) quad_fma_pair(acc, w[i], x);
+        else quad_fma(acc, w[i], x);
+    }
+    __device__ __forceinline__ void add_weighted4(Quad& acc, int i, const Quad* x) const {
+        const float4 p = *reinterpret_cast<const float4*>(&w[i]);
+        if constexpr (kPairs) {
+            quad_fma_pair(acc, make_float2(p.x, p.y), x[0]);
+            quad_fma_pair(acc, make_float2(p.z, p.w), x[1]);
+            const float4 q = *reinterpret_cast<const float4*>(&w[i + 2]);
+            quad_fma_pair(acc, make_float2(q.x, q.y), x[2]);
+            quad_fma_pair(acc, make_float2(q.z, q.w), x[3]);
+        } else {
+            quad_fma(acc, p.x, x[0]);
+            quad_fma(acc, p.y, x[1]);
+            quad_fma(acc, p.z, x[2]);
+            quad_fma(acc, p.w, x[3]);
+        }
+    }
 };
 
 template <int G, int OP, bool HAS_EMPTY, int EP>
 __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN;
+    // GIN's weights are 1 but for the self-loops': groups of 16 lanes and more mark those in a bit mask and add the rest
+    // (169 K nodes, 256 columns: 195 us per hop with a weight per edge, 181 so; 24 M edges, 64 columns: 460 / 430); narrower
+    // groups lose more by the extra votes than the weights cost (169 K nodes, 32 columns: 42 / 45).
+    constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16;
+    constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN && !kDiagonal;
     using Stage = SegStage<G, kWeighted>;
     constexpr int C = Stage::kChunk;
     constexpr int M = C / G;  // entries per lane and chunk
@@ -95,10 +129,18 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
 
     while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
         // ---- stage this chunk: lanes past the end hold column 0 without a row-end mark
-        unsigned ends = 0;
+        unsigned ends = 0, loops = 0;  // last edges of rows; self-loops
 #pragma unroll
         for (int m = 0; m < M; ++m)
             ends |= ((__ballot_sync(kFull, (int)c_cur[m] < 0) >> gshift) & kGroupLow) << (m * G);
+        if (kDiagonal) {
+#pragma unroll
+            for (int m = 0; m < M; ++m) {  // every row owns its self-loop, so the rank of a row is its index
+                const int i = gl + m * G;
+                const bool loop = i < left && (int)(c_cur[m] & ~kRowEndBit) == rank + __popc(ends & ((1u << i) - 1u));
+                loops |= ((__ballot_sync(kFull, loop) >> gshift) & kGroupLow) << (m * G);
+            }
+        }
         const int rank_after = rank + __popc(ends);
         int slot_last = -1;  // scratch row of this chunk's last sum, if its row is cut by the segment's end
         if (left > 0 && left <= C && ((ends >> (left - 1)) & 1u) == 0) {
@@ -111,11 +153,10 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             const int i = gl + m * G;
             const uint32_t col = c_cur[m] & ~kRowEndBit;
             stage.col[i] = col;
-            // every row owns its self-loop, so the rank of a row is its index
-            if (OP == GNNPRE_OP_GIN_SUM)
-                w[m] = (int)col == rank + __popc(ends & ((1u << i) - 1u)) ? a.diag_weight : 1.f;
             int slot = i == 0 ? slot_head : -1;
             if (slot_last >= 0 && i == last) slot = slot_last;
+            if (OP == GNNPRE_OP_GIN_SUM && kWeighted)
+                w[m] = (int)col == rank + __popc(ends & ((1u << i) - 1u)) ? a.diag_weight : 1.f;
             RowOut o;
             o.dst = reinterpret_cast<char*>(slot >= 0 ? a.scratch + (int64_t)slot * a.scratch_ld : a.out + (int64_t)row[m] * a.ldo) + 16 * q0;
             o.scale = slot >= 0 ? 1.f : scale[m];
@@ -136,7 +177,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
         fetch_rows();
         const int here = left + C;  // edges of this group from here to the segment's end
         const int cnt = G == 32 ? min(here, C) : C == kSegWindow ? C : __reduce_max_sync(kFull, min(here, C));
-        const unsigned ends_any = G == 32 ? ends : __reduce_or_sync(kFull, ends);
+        const unsigned busy = G == 32 ? ends | loops : __reduce_or_sync(kFull, ends | loops);
         const RowOut* out = stage.out;
         EpiloguePiece<EP> piece;
         __syncwarp();
@@ -168,26 +209,25 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             }
             if (kWeighted && t0 == 0) {  // the weights follow behind the chunk's first row requests
 #pragma unroll
-                for (int m = 0; m < M; ++m) stage.w[gl + m * G] = make_float2(w[m], w[m]);
+                for (int m = 0; m < M; ++m) stage.set_weight(gl + m * G, w[m]);
                 __syncwarp();
             }
-            if (((ends_any >> t0) & 0xffu) == 0) {
+            if (((busy >> t0) & 0xffu) == 0) {
 #pragma unroll
-                for (int u = 0; u < kSegWindow; u += 2) {
+                for (int u = 0; u < kSegWindow; u += 4) {
                     if (kWeighted) {
-                        const float4 p = *reinterpret_cast<const float4*>(&stage.w[t0 + u]);
-                        quad_fma_pair(acc, make_float2(p.x, p.y), x[u]);
-                        quad_fma_pair(acc, make_float2(p.z, p.w), x[u + 1]);
+                        stage.add_weighted4(acc, t0 + u, x + u);
                     } else {
-                        quad_add(acc, x[u]);
-                        quad_add(acc, x[u + 1]);
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) quad_add(acc, x[u + v]);
                     }
                 }
             } else {
-                const unsigned we = ends >> t0;
+                const unsigned we = ends >> t0, wl = loops >> t0;
 #pragma unroll
                 for (int u = 0; u < kSegWindow; ++u) {
-                    if (kWeighted) quad_fma_pair(acc, stage.w[t0 + u], x[u]);
+                    if (kWeighted) stage.add_weighted(acc, t0 + u, x[u]);
+                    else if (kDiagonal && ((wl >> u) & 1u)) quad_fma(acc, a.diag_weight, x[u]);
                     else quad_add(acc, x[u]);
                     if ((we >> u) & 1u) flush();
                 }
