@@ -228,14 +228,6 @@ struct gnnpre_plan {
     gnnpre::DevBuf<float> scratch;  // num_slots rows of slab_width floats
     gnnpre::DevBuf<int> dev_error;  // set by a kernel whose bounded wait ran out
     int num_sms = 0;
-    // tensor maps of the matrices the bulk-copy kernel has been launched on (a cache: not part of the plan's meaning)
-    struct TensorMapEntry {
-        const float* x;
-        int64_t ldx;
-        int32_t f4;
-        CUtensorMap map;
-    };
-    mutable std::vector<TensorMapEntry> tmaps;
     // streaming state
     gnnpre::DevBuf<float> slab[4];
     std::vector<gnnpre::DevBuf<float>> whole;  // panel schedule: X_0 .. X_K, each [n, feat_dim], grown on demand

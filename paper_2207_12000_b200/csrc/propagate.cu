@@ -118,33 +118,13 @@ int make_row_tensor_map(const float* x, int64_t n, int32_t width, int64_t ldx, C
     return GNNPRE_OK;
 }
 
-// The plan remembers the tensor maps of the matrices it has met (a K-hop call alternates between a few), so a
-// launch in steady state encodes nothing.
-int cached_tensor_map(const gnnpre_plan* P, const SegArgs& a, const CUtensorMap** out) {
-    for (const auto& c : P->tmaps) {
-        if (c.x == a.x && c.ldx == a.ldx && c.f4 == a.f4) {
-            *out = &c.map;
-            return GNNPRE_OK;
-        }
-    }
-    if (P->tmaps.size() >= 32) P->tmaps.erase(P->tmaps.begin());
-    gnnpre_plan::TensorMapEntry entry;
-    entry.x = a.x;
-    entry.ldx = a.ldx;
-    entry.f4 = a.f4;
-    GNNPRE_TRY(make_row_tensor_map(a.x, P->n, 4 * a.f4, a.ldx, &entry.map));
-    P->tmaps.push_back(entry);
-    *out = &P->tmaps.back().map;
-    return GNNPRE_OK;
-}
-
-template <int OP, bool HAS_EMPTY, int F4C, int EP>
+template <bool HAS_EMPTY, int F4C, int EP>
 int launch_segments_tma_width(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
     const int nwarps = tma_warps(a.f4);
     const size_t smem = (size_t)nwarps * kTmaStages * tma_stage_bytes(a.f4);
-    const CUtensorMap* tmap = nullptr;
-    GNNPRE_TRY(cached_tensor_map(P, a, &tmap));
-    auto kernel = k_segments_tma<OP, HAS_EMPTY, F4C, EP>;
+    CUtensorMap tmap;
+    GNNPRE_TRY(make_row_tensor_map(a.x, P->n, 4 * a.f4, a.ldx, &tmap));
+    auto kernel = k_segments_tma<HAS_EMPTY, F4C, EP>;
     // the opt-in to large dynamic shared memory is per kernel and device: once, and again only if a launch needs more
     static std::atomic<int> smem_set[kMaxDevices];
     const int dev = P->device < kMaxDevices ? P->device : 0;
@@ -154,28 +134,21 @@ int launch_segments_tma_width(const gnnpre_plan* P, const SegArgs& a, cudaStream
     }
     const int64_t nseg = a.seg_hi - a.seg_lo;
     const unsigned grid = (unsigned)std::min<int64_t>(P->num_sms, (nseg + nwarps - 1) / nwarps);
-    return launch_dependent(kernel, dim3(grid), (unsigned)(nwarps * 32), smem, a.back_to_back, st, a, *tmap, P->dev_error.p);
+    return launch_dependent(kernel, dim3(grid), (unsigned)(nwarps * 32), smem, a.back_to_back, st, a, tmap, P->dev_error.p);
 }
 
-// Rows (or column tiles) of 100 and of 128 columns get kernels with the row size compiled in.
-template <int OP, bool HAS_EMPTY>
-int launch_segments_tma_op(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
+// Rows (or column tiles) of 100 columns get kernels with the row size compiled in.
+template <bool HAS_EMPTY>
+int launch_segments_tma_rows(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
     const int ep = epilogue_of(a.tp);
-    if (ep == kEpSum) return launch_segments_tma_width<OP, HAS_EMPTY, 0, kEpSum>(P, a, st);
-    if (ep == kEpTeleport) return launch_segments_tma_width<OP, HAS_EMPTY, 0, kEpTeleport>(P, a, st);
-    if (a.f4 == 25) return launch_segments_tma_width<OP, HAS_EMPTY, 25, kEpPlain>(P, a, st);
-    if (a.f4 == 32) return launch_segments_tma_width<OP, HAS_EMPTY, 32, kEpPlain>(P, a, st);
-    return launch_segments_tma_width<OP, HAS_EMPTY, 0, kEpPlain>(P, a, st);
+    if (ep == kEpSum) return launch_segments_tma_width<HAS_EMPTY, 0, kEpSum>(P, a, st);
+    if (ep == kEpTeleport) return launch_segments_tma_width<HAS_EMPTY, 0, kEpTeleport>(P, a, st);
+    if (a.f4 == 25) return launch_segments_tma_width<HAS_EMPTY, 25, kEpPlain>(P, a, st);
+    return launch_segments_tma_width<HAS_EMPTY, 0, kEpPlain>(P, a, st);
 }
 
 int launch_segments_tma(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
-    switch (P->op) {
-    case GNNPRE_OP_GCN_SYM: return launch_segments_tma_op<GNNPRE_OP_GCN_SYM, false>(P, a, st);
-    case GNNPRE_OP_GIN_SUM: return launch_segments_tma_op<GNNPRE_OP_GIN_SUM, false>(P, a, st);
-    default:
-        return P->rows_all_nonempty ? launch_segments_tma_op<GNNPRE_OP_SAGE_MEAN, false>(P, a, st)
-                                    : launch_segments_tma_op<GNNPRE_OP_SAGE_MEAN, true>(P, a, st);
-    }
+    return P->rows_all_nonempty ? launch_segments_tma_rows<false>(P, a, st) : launch_segments_tma_rows<true>(P, a, st);
 }
 
 template <int G>
@@ -220,17 +193,18 @@ int64_t l2_cache_bytes() {
     return bytes;
 }
 
-// A column tile of 68..128 columns goes through the bulk-copy kernel when X's tile is at least four times the L2 and
-// rows are long (mean degree >= 32).  Its rows in flight (213 KB per SM) then hide the DRAM latency that the register
-// kernel's 90 KB do not; everywhere else its copy engine, about 33 ps per row whatever the row's width, is the slower
-// path.  us per hop, bulk copy / register: 2.4 M nodes of mean degree 51, mean operator, 72 columns 3478 / 3849,
-// 100 columns 4021 / 4420, 128 columns 4631 / 4757, GCN 100 columns 5175 / 5647.  But 800 K nodes of degree 63, GCN, 100
-// columns (2.4 x L2) 1930 / 1762; 1.7 M nodes of degree 15, GCN, 128 columns (6.7 x L2) 1441 / 1200; 169 K nodes of
-// degree 15, GCN, 128 columns 155 / 121.
+// The mean operator's column tiles of 68..124 columns go through the bulk-copy kernel when X's tile is at least four times
+// the L2 and rows are long (mean degree >= 32).  Its rows in flight (213 KB per SM) then hide the DRAM latency that the
+// register kernel's 90 KB do not; everywhere else its copy engine, about 33 ps per row whatever the row's width, is the
+// slower path.  us per hop, bulk copy / register: 2.4 M nodes of mean degree 51, mean operator, 72 columns 3634 / 3845,
+// 100 columns 4085 / 4509, 124 columns 4670 / 5150, but 128 columns, rows of whole cache lines, 4641 / 4461; degree 34,
+// 100 columns 3187 / 3368.  With a weight per edge the rows wait for their weights instead: GCN, degree 51, 72 / 100 / 128
+// columns 4583 / 4243, 4971 / 4927, 5519 / 4792; GIN, whose few weighted edges are marked, 4010 / 3951, 4495 / 4599,
+// 5137 / 4658.  800 K nodes of degree 63, mean, 100 columns (2.4 x L2): register; 1.7 M nodes of degree 15 as well.
 bool tile_uses_bulk_copy(const gnnpre_plan* P, int32_t width) {
     const int32_t f4 = width / 4;
-    return !(P->flags & GNNPRE_FLAG_NO_BULK_COPY) && f4 > 16 && f4 <= 32 && P->n * (int64_t)width * 4 > 4 * l2_cache_bytes() &&
-           P->nnz_tilde >= 32 * P->n;
+    return P->op == GNNPRE_OP_SAGE_MEAN && !(P->flags & GNNPRE_FLAG_NO_BULK_COPY) && f4 > 16 && f4 < 32 &&
+           P->n * (int64_t)width * 4 > 4 * l2_cache_bytes() && P->nnz_tilde >= 32 * P->n;
 }
 
 // Columns one segment launch covers: all of them, as tiles of one launch, while a 128-column tile of X fits the L2.
@@ -314,13 +288,13 @@ template <int F4C>
 int launch_ceiling_tma(const gnnpre_plan* P, const SegArgs& a, float* sink, cudaStream_t st) {
     const int nwarps = tma_warps(a.f4);
     const size_t smem = (size_t)nwarps * kTmaStages * tma_stage_bytes(a.f4);
-    const CUtensorMap* tmap = nullptr;
-    GNNPRE_TRY(cached_tensor_map(P, a, &tmap));
+    CUtensorMap tmap;
+    GNNPRE_TRY(make_row_tensor_map(a.x, P->n, 4 * a.f4, a.ldx, &tmap));
     auto kernel = k_ceiling_tma<F4C>;
     GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t nseg = a.seg_hi - a.seg_lo;
     const unsigned grid = (unsigned)std::min<int64_t>(P->num_sms, (nseg + nwarps - 1) / nwarps);
-    kernel<<<grid, nwarps * 32, smem, st>>>(a, *tmap, sink, P->dev_error.p);
+    kernel<<<grid, nwarps * 32, smem, st>>>(a, tmap, sink, P->dev_error.p);
     GNNPRE_CUDA(cudaGetLastError());
     return GNNPRE_OK;
 }
@@ -350,7 +324,6 @@ int launch_ceiling(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int64
         a.f4 = w / 4;
         if (tile_uses_bulk_copy(P, w)) {
             if (a.f4 == 25) GNNPRE_TRY(launch_ceiling_tma<25>(P, a, sink, st));
-            else if (a.f4 == 32) GNNPRE_TRY(launch_ceiling_tma<32>(P, a, sink, st));
             else GNNPRE_TRY(launch_ceiling_tma<0>(P, a, sink, st));
         } else {
             a.tile_f4 = equal_tile_f4(a.f4);

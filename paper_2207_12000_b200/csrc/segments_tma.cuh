@@ -1,4 +1,4 @@
-// Segment kernel with the gathered rows staged through shared memory by the bulk-copy (TMA) engine.
+// Segment kernel of the mean operator with the gathered rows staged through shared memory by the bulk-copy (TMA) engine.
 // Included by propagate.cu inside its unnamed namespace (uses SegArgs, Segment, kRowEndBit).
 //
 // Why: the register kernel k_segments keeps at most (warps per SM) x 8 rows in flight, bounded by
@@ -93,12 +93,12 @@ struct TmaChunk {
     uint32_t c;      // this lane's column entry (row-end mark in bit 31); 0 on padding lanes
     unsigned ends;   // row-end marks of the chunk, bit t = edge t
     int cnt;         // edges in the chunk
-    int row;         // row of this lane's edge (valid where it ends a row; everywhere for GIN)
-    float r, w;      // row scale of that row; weight of this lane's edge
+    int row;         // row of this lane's edge (valid where it ends a row)
+    float r;         // row scale of that row
 };
 
 // F4C: the row width in float4 when known at compile time (shared-memory offsets become immediates), else 0.
-template <int OP, bool HAS_EMPTY, int F4C, int EP>
+template <bool HAS_EMPTY, int F4C, int EP>
 __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
     k_segments_tma(const SegArgs a, const __grid_constant__ CUtensorMap tmap, int* error) {
     constexpr unsigned kFull = 0xffffffffu;
@@ -162,15 +162,9 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
             m.ends = __ballot_sync(kFull, (c & kRowEndBit) != 0);
             int row = rank_issue + __popc(m.ends & lt_mask);
             m.r = 1.f;
-            m.w = 1.f;
             if (c & kRowEndBit) {
                 if (HAS_EMPTY) row = a.nzrows[row];
-                if (OP != GNNPRE_OP_GIN_SUM) m.r = a.rscale[row];
-            }
-            if (OP == GNNPRE_OP_GCN_SYM) {
-                m.w = a.cscale[c & ~kRowEndBit];
-            } else if (OP == GNNPRE_OP_GIN_SUM) {
-                m.w = (int)(c & ~kRowEndBit) == row ? a.diag_weight : 1.f;
+                m.r = a.rscale[row];
             }
             m.row = row;
             rank_issue += __popc(m.ends);
@@ -228,13 +222,8 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        if (OP == GNNPRE_OP_SAGE_MEAN) {
-                            quad_add(acc, xa[u]);
-                            quad_add(acc2, xb[u]);
-                        } else {
-                            quad_fma(acc, __shfl_sync(kFull, m.w, h + u), xa[u]);
-                            quad_fma(acc2, __shfl_sync(kFull, m.w, kTmaStep + h + u), xb[u]);
-                        }
+                        quad_add(acc, xa[u]);
+                        quad_add(acc2, xb[u]);
                     }
                 }
                 quad_kahan(tot, cmp, acc);
@@ -252,17 +241,13 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
                 const unsigned step_ends = (m.ends >> t0) & ((1u << kTmaStep) - 1u);
                 if (step_ends == 0 && t0 + kTmaStep <= m.cnt) {  // no row ends here: a straight run of adds
 #pragma unroll
-                    for (int u = 0; u < kTmaStep; ++u) {
-                        if (OP == GNNPRE_OP_SAGE_MEAN) quad_add(acc, x[u]);
-                        else quad_fma(acc, __shfl_sync(kFull, m.w, t0 + u), x[u]);
-                    }
+                    for (int u = 0; u < kTmaStep; ++u) quad_add(acc, x[u]);
                 } else {
 #pragma unroll
                     for (int u = 0; u < kTmaStep; ++u) {
                         const int t = t0 + u;
                         if (t < m.cnt) {
-                            if (OP == GNNPRE_OP_SAGE_MEAN) quad_add(acc, x[u]);
-                            else quad_fma(acc, __shfl_sync(kFull, m.w, t), x[u]);
+                            quad_add(acc, x[u]);
                             if ((m.ends >> t) & 1u) flush(t, m);
                         }
                     }
