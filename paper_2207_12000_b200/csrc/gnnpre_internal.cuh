@@ -253,12 +253,15 @@ struct HopArgs {
     int32_t width;           // columns of this slab (multiple of 4)
     const float* x0;         // [n, ldx0] the slab of X_0, read only when the plan has a teleport term or zsum starts
     int64_t ldx0;
-    // fixed-weight sum of hops, Z = gamma_0 X_0 + sum_k gamma_k X_k (nullptr = none): this hop adds gamma * X_k
+    // fixed-weight sum of hops, Z = gamma_0 X_0 + sum_k gamma_k X_k (nullptr = not in this hop): this hop adds gamma * X_k,
+    // and gamma_prev * X_{k-1} first if the hop before it did not (zsum_prev)
     float* zsum = nullptr;   // [n, ldz], offset to the slab's first column
     int64_t ldz = 0;
     float gamma = 0.f;       // weight of the hop being computed
+    float gamma_prev = 0.f;
+    bool zsum_prev = false;
     float gamma0 = 0.f;      // weight of X_0
-    bool zsum_first = false; // first hop: Z starts from gamma0 * X_0 instead of its old value
+    bool zsum_first = false; // first hop that adds to Z: it starts from gamma0 * X_0 instead of its old value
     bool back_to_back = false;  // nothing but this library's kernels between this call's launches on the stream
 };
 

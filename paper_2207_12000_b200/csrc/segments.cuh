@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     constexpr int C = Stage::kChunk;
     constexpr int M = C / G;  // entries per lane and chunk
     __shared__ __align__(16) Stage stages[kSegThreads / G];
+    __shared__ EpiloguePiece<EP> pieces[EP == kEpSum ? kSegThreads : 1];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1);
     const int gshift = lane & ~(G - 1);
@@ -125,6 +126,10 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
         for (int m = 0; m < M; ++m) w[m] = __ldg(a.cscale + (c_cur[m] & ~kRowEndBit));
     }
     Quad acc = quad_zero(), tot = quad_zero(), cmp = quad_zero();  // this window's plain sum; the row's running sum
+    using Piece = std::conditional_t<EP == kEpSum, EpilogueAhead<EP>, EpiloguePiece<EP>>;
+    Piece piece;
+    if constexpr (EP == kEpSum) piece.at = &pieces[threadIdx.x];
+    bool asked = false;  // the operands of the next row's epilogue are on their way
     wait_previous_kernel();
 
     while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
@@ -179,9 +184,9 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
         const int cnt = G == 32 ? min(here, C) : C == kSegWindow ? C : __reduce_max_sync(kFull, min(here, C));
         const unsigned busy = G == 32 ? ends | loops : __reduce_or_sync(kFull, ends | loops);
         const RowOut* out = stage.out;
-        EpiloguePiece<EP> piece;
         __syncwarp();
-        if (EP != kEpPlain) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
+        if (EP != kEpPlain && !asked) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
+        asked = true;
 
         auto flush = [&]() {  // the last edge added closes a sum
             const RowOut o = *out++;
@@ -193,7 +198,8 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
                 *reinterpret_cast<float4*>(o.dst + out_off) = v;
             }
             acc = tot = cmp = quad_zero();
-            if (EP != kEpPlain && out < stage.out + C) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
+            asked = out < stage.out + C;
+            if (EP != kEpPlain && asked) piece.load(a.tp, max(out->row, 0), 4 * q0, gl, on);
         };
 
 #pragma unroll 1
@@ -241,4 +247,5 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             for (int m = 0; m < M; ++m) w[m] = w_next[m];
         }
     }
+    if (EP == kEpSum) asm volatile("cp.async.wait_all;" ::: "memory");  // the row after the segment's last was asked for too
 }

@@ -7,10 +7,13 @@ struct Teleport {
     const float* x0;
     int64_t ldx0;
     float alpha, keep;  // keep = 1 - alpha
-    // fixed-weight sum of hops (zsum == nullptr: none): Z += gamma * (the value stored for this hop)
+    // fixed-weight sum of hops (zsum == nullptr: this hop leaves Z alone): Z += gamma * (the value stored for this hop),
+    // after gamma_prev * (the hop before it, xprev) if that one left Z alone (xprev == nullptr: it did not)
     float* zsum;
     int64_t ldz;
-    float gamma, gamma0;
+    const float* xprev;
+    int64_t ldp;
+    float gamma, gamma_prev, gamma0;
     int zsum_first;
 };
 
@@ -23,12 +26,14 @@ constexpr int kEpPlain = 0, kEpTeleport = 1, kEpSum = 2;
 // where the kernel knows the row ahead of time.
 template <int EP>
 struct EpiloguePiece {
-    float4 x0, z;
+    float4 x0;
+    float4 z[EP == kEpSum ? 2 : 1];  // Z, X_{k-1}
     __device__ __forceinline__ void load(const Teleport& tp, int64_t row, int f0, int q, bool on) {
         if (EP == kEpPlain || !on) return;
         if (EP == kEpTeleport || tp.alpha != 0.f || tp.zsum_first)
             x0 = __ldg(reinterpret_cast<const float4*>(tp.x0 + row * tp.ldx0 + f0) + q);
-        if (EP == kEpSum && !tp.zsum_first) z = *(reinterpret_cast<const float4*>(tp.zsum + row * tp.ldz + f0) + q);
+        if (EP == kEpSum && !tp.zsum_first) z[0] = *(reinterpret_cast<const float4*>(tp.zsum + row * tp.ldz + f0) + q);
+        if (EP == kEpSum && tp.xprev) z[1] = __ldg(reinterpret_cast<const float4*>(tp.xprev + row * tp.ldp + f0) + q);
     }
     // the value to store for the row; adds it to the sum of hops (every finished row piece passes here once per hop)
     __device__ __forceinline__ float4 finish(const float4& sum, float scale, const Teleport& tp, int64_t row, int f0, int q) const {
@@ -40,8 +45,14 @@ struct EpiloguePiece {
             o.w = fmaf(tp.keep, o.w, tp.alpha * x0.w);
         }
         if (EP == kEpSum) {
-            float4 acc = z;
+            float4 acc = z[0];
             if (tp.zsum_first) acc = make_float4(tp.gamma0 * x0.x, tp.gamma0 * x0.y, tp.gamma0 * x0.z, tp.gamma0 * x0.w);
+            if (tp.xprev) {
+                acc.x = fmaf(tp.gamma_prev, z[1].x, acc.x);
+                acc.y = fmaf(tp.gamma_prev, z[1].y, acc.y);
+                acc.z = fmaf(tp.gamma_prev, z[1].z, acc.z);
+                acc.w = fmaf(tp.gamma_prev, z[1].w, acc.w);
+            }
             acc.x = fmaf(tp.gamma, o.x, acc.x);
             acc.y = fmaf(tp.gamma, o.y, acc.y);
             acc.z = fmaf(tp.gamma, o.z, acc.z);
@@ -49,6 +60,31 @@ struct EpiloguePiece {
             *(reinterpret_cast<float4*>(tp.zsum + row * tp.ldz + f0) + q) = acc;
         }
         return o;
+    }
+};
+
+__device__ __forceinline__ void copy_ahead(float4* dst, const float4* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// The same, its operands copied to shared memory meanwhile: held in registers beside the eight rows in flight, the twelve
+// floats of a sum of hops were spilled, which waits for them at once.  Copies through the L1 (.ca), where the halves of a
+// line that neighbouring rows share meet.  24 M edges, ten hops with a teleport term, us per hop, registers / shared memory:
+// 16 columns 283 / 254, 64 columns 659 / 598, 128 columns 978 / 920.  The teleport term alone stays in registers (64 columns
+// 586 / 608).
+template <int EP>
+struct EpilogueAhead {
+    EpiloguePiece<EP>* at;  // this lane's own
+    __device__ __forceinline__ void load(const Teleport& tp, int64_t row, int f0, int q, bool on) const {
+        if (EP == kEpPlain || !on) return;
+        if (EP == kEpTeleport || tp.alpha != 0.f || tp.zsum_first)
+            copy_ahead(&at->x0, reinterpret_cast<const float4*>(tp.x0 + row * tp.ldx0 + f0) + q);
+        if (EP == kEpSum && !tp.zsum_first) copy_ahead(&at->z[0], reinterpret_cast<const float4*>(tp.zsum + row * tp.ldz + f0) + q);
+        if (EP == kEpSum && tp.xprev) copy_ahead(&at->z[1], reinterpret_cast<const float4*>(tp.xprev + row * tp.ldp + f0) + q);
+    }
+    __device__ __forceinline__ float4 finish(const float4& sum, float scale, const Teleport& tp, int64_t row, int f0, int q) const {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return at->finish(sum, scale, tp, row, f0, q);
     }
 };
 

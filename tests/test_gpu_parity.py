@@ -516,6 +516,29 @@ def test_teleport_filter_matches_oracle(B, op, alpha):
         B.gnnpre_build_plan(drp, dci, op, 16, teleport_alpha=1.5)
 
 
+@pytest.mark.parametrize("alpha", [0.0, 0.15])
+@pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132])
+def test_weighted_hop_sum_adds_every_hop_once(B, F, alpha):
+    """Z takes its hops two at a time, so odd and even K, K = 1 and 2, on segments that cut rows, rows that span chunks
+    and rows without edges.  Against the fp64 sum of the hops the same call returned: each of the K + 1 fused
+    multiply-adds rounds once, by at most 2^-24 of a partial sum, itself at most sum_k |gamma_k X_k|."""
+    n = 90
+    g = gi.from_edge_list(n, [(i, j) for i in range(0, n, 7) for j in range(i + 1, min(n, i + 1 + 2 * i))])
+    drp, dci = dev(g)
+    X = gi.normal_matrix(n, F, 31, device="cuda")
+    for op in OPS:
+        for seg in (7, 33, 300):
+            for K in (1, 2, 3, 4, 5):
+                gamma = [0.3, -0.7, 1.1, 0.4, -0.2, 0.9][: K + 1]
+                plan = B.gnnpre_build_plan(drp, dci, op, F, gin_eps=EPS, segment_edges=seg, teleport_alpha=alpha)
+                hops, Z = B.gnnpre_propagate_weighted(plan, X, gamma)
+                torch.cuda.synchronize()
+                plan.close()
+                terms = [gk * m.double() for gk, m in zip(np.float32(gamma).astype(np.float64).tolist(), [X, *hops])]
+                bound = (K + 1) * 2.0**-24 * sum(t.abs() for t in terms)
+                assert bool(((Z.double() - sum(terms)).abs() <= bound).all()), (op, seg, K)
+
+
 @pytest.mark.parametrize("op", OPS)
 def test_weighted_hop_sum_matches_oracle(B, op):
     """Z = gamma_0 X_0 + sum_k gamma_k X_k accumulated in the kernels' epilogues: every kernel shape, blocks and
