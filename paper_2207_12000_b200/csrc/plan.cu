@@ -311,8 +311,8 @@ __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const 
 // Segment t of block l nominally starts at e_lo(l) + t*L.  A start that falls inside a row is moved
 // forward to the next row start when that lies within `snap` edges (and inside the block), so that
 // short rows are never cut; long rows are cut and their parts summed by a fix-up.  Where no row of the graph is longer
-// than three segments the start always moves (two may then meet: an empty segment), and nothing is left for the
-// finishing launch: 4,096 nodes of degree 16, 64 columns, two hops 13.7 us at segments of 32, 11.1 at 16 and none cut.
+// than three segments the start always moves (two may then meet, or one the block's end: an empty segment), and nothing
+// is left for the finishing launch: 4,096 nodes of degree 16, 64 columns, two hops 13.7 us at segments of 32, 10.4 at 16 and none cut.
 // Graphs with longer rows have that launch anyway and are better off balanced (5,000 nodes, R-MAT, 16.7 us against 19.5).
 // Until k_segment_finalize: slot_head holds the "first row began earlier" flag and pad the first row's index.
 __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict__ seg_base,
@@ -341,14 +341,14 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     int64_t row = row_of_edge(rowptr_t, n, start);
     if (t > 0 && rowptr_t[row] < start) {
         const int64_t next = rowptr_t[row + 1];
-        if ((next - start <= snap || *longest < 3 * (int64_t)L) && next < e_off[lo + 1]) {
+        if ((next - start <= snap || *longest < 3 * (int64_t)L) && next <= e_off[lo + 1]) {
             start = next;
-            row = row_of_edge(rowptr_t, n, start);
+            row = start < e_off[b] ? row_of_edge(rowptr_t, n, start) : n;  // at the very end: empty, as the sentinel
         }
     }
     g.start = start;
-    g.rank = rank ? rank[row] : (int32_t)row;
-    g.slot_head = rowptr_t[row] < start;
+    g.rank = row == n ? 0 : rank ? rank[row] : (int32_t)row;
+    g.slot_head = row < n && rowptr_t[row] < start;
     g.slot_tail = -1;
     g.pad = (int32_t)row;
     segs[s] = g;

@@ -402,6 +402,23 @@ def test_register_kernel_tile_and_segment_edges(B, op, F, seg):
     run_case(B, g, op, F, 2, b=3, seg=seg)
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("tail", [1, 15, 16, 17, 31, 40])
+def test_last_row_of_a_block_is_not_cut(B, op, flags, tail):
+    """Segments of 16 on a graph whose longest row has fewer than 48 entries: a segment that would start inside the last row
+    moves to the block's end and is empty; one block (nothing is cut) and several (only rows that a block's end cuts)."""
+    n = 60
+    g = gi.from_edge_list(n, [(i, i + 1) for i in range(n - 1)] + [(n - 1, j) for j in range(tail)])
+    for b in (1, 2, 3, 5):
+        run_case(B, g, op, 64, 2, b=b, seg=16, flags=flags)
+    drp, dci = dev(g)
+    plan = B.gnnpre_build_plan(drp, dci, op, 64, gin_eps=EPS, force_blocks=1, segment_edges=16, flags=flags)
+    fixups = plan.info()["num_row_fixups"]
+    plan.close()
+    assert fixups == 0
+
+
 def test_two_tile_rows_on_a_graph_larger_than_the_cache(B):
     """Rows of 132..256 columns are cut into two equal tiles for the copy engine once a 128-column tile of X no
     longer fits the L2 (here 400,000 nodes: 205 MB per tile; F = 200 gives two tiles of 100 columns, F = 252 two of
