@@ -698,8 +698,9 @@ def main():
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "frac_basis": basis, "peak_kind": f"{peak_kind} copy bandwidth (burst)", "traffic": traffic,
                 "traffic_source": traffic_source,
-                "kernel": "k_segments_tma (bulk-copy segment kernel)" if 68 <= F <= 128 and not args.no_bulk_copy
-                          else "segment kernel (k_segments / k_segments_tma by tile width)",
+                "kernel": "k_segments_tma (bulk-copy segment kernel)" if w.op == gi.OP_SAGE and 68 <= F < 128
+                          and g.n * F * 4 > 4 * getattr(torch.cuda.get_device_properties(0), "L2_cache_size", 126 << 20)
+                          and g.nnz >= 32 * g.n and not args.no_bulk_copy else "segment kernel (k_segments / k_segments_tma by the library's dispatch)",
                 "kernel_ms_per_launch": seg_launch_ms, "launches_per_hop": launches_per_hop,
                 "algorithmic_bytes_per_launch": gather_b / launches_per_hop,
                 "gather_model_gbs": gather_b / launches_per_hop / secs / 1e9,
