@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             quad_kahan(tot, cmp, acc);
             float4 v = make_float4(tot.lo.x, tot.lo.y, tot.hi.x, tot.hi.y);
             if (on) {
+                if (EP == kEpSum && o.row < 0) wait_copies_ahead();  // no epilogue, but the next row's copies go to the same place
                 if (EP == kEpPlain || o.row < 0) v = make_float4(v.x * o.scale, v.y * o.scale, v.z * o.scale, v.w * o.scale);
                 else v = piece.finish(v, o.scale, a.tp, o.row, 4 * q0, gl);
                 *reinterpret_cast<float4*>(o.dst + out_off) = v;
@@ -247,5 +248,5 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             for (int m = 0; m < M; ++m) w[m] = w_next[m];
         }
     }
-    if (EP == kEpSum) asm volatile("cp.async.wait_all;" ::: "memory");  // the row after the segment's last was asked for too
+    if (EP == kEpSum) wait_copies_ahead();  // the row after the segment's last was asked for too
 }

@@ -67,7 +67,10 @@ __device__ __forceinline__ void copy_ahead(float4* dst, const float4* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
-// The same, its operands copied to shared memory meanwhile: held in registers beside the eight rows in flight, the twelve
+__device__ __forceinline__ void wait_copies_ahead() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The same, its operands copied to shared memory meanwhile (copies are not ordered among themselves: those of one sum are
+// waited for before the next sum's are issued, whether or not they were wanted): held in registers beside the eight rows in flight, the twelve
 // floats of a sum of hops were spilled, which waits for them at once.  Copies through the L1 (.ca), where the halves of a
 // line that neighbouring rows share meet.  24 M edges, ten hops with a teleport term, us per hop, registers / shared memory:
 // 16 columns 283 / 254, 64 columns 659 / 598, 128 columns 978 / 920.  The teleport term alone stays in registers (64 columns
@@ -83,7 +86,7 @@ struct EpilogueAhead {
         if (EP == kEpSum && tp.xprev) copy_ahead(&at->z[1], reinterpret_cast<const float4*>(tp.xprev + row * tp.ldp + f0) + q);
     }
     __device__ __forceinline__ float4 finish(const float4& sum, float scale, const Teleport& tp, int64_t row, int f0, int q) const {
-        asm volatile("cp.async.wait_all;" ::: "memory");
+        wait_copies_ahead();
         return at->finish(sum, scale, tp, row, f0, q);
     }
 };

@@ -556,6 +556,32 @@ def test_weighted_hop_sum_adds_every_hop_once(B, F, alpha):
                 assert bool(((Z.double() - sum(terms)).abs() <= bound).all()), (op, seg, K)
 
 
+@pytest.mark.parametrize("alpha", [0.0, 0.15])
+@pytest.mark.parametrize("F", [16, 32, 64, 128])
+def test_weighted_hop_sum_behind_cut_rows_takes_its_own_operands(B, F, alpha):
+    """What the sum of hops adds to a row is fetched ahead, into one place per lane; a segment that begins inside a row has a
+    sum without such operands first.  Row 0, the row such a sum would name, is huge and has no neighbours: a trace of it in
+    any other row is far outside the bound (as in test_weighted_hop_sum_adds_every_hop_once)."""
+    n = 4000
+    g = gi.from_edge_list(n, [(i, 1 + (i * 7 + j * j) % (n - 1)) for i in range(1, n, 5) for j in range(i % 40)
+                              if i != 1 + (i * 7 + j * j) % (n - 1)] + [(2, 1000 + j) for j in range(900)])
+    X = gi.normal_matrix(n, F, 32, device="cuda")
+    X[0] = 1e30
+    drp, dci = dev(g)
+    for op in OPS:
+        for seg in (5, 16, 40):
+            gamma = [0.3, -0.7, 1.1, 0.4]
+            plan = B.gnnpre_build_plan(drp, dci, op, F, gin_eps=EPS, segment_edges=seg, teleport_alpha=alpha)
+            assert plan.info()["num_row_fixups"] > 0
+            hops, Z = B.gnnpre_propagate_weighted(plan, X, gamma)
+            torch.cuda.synchronize()
+            plan.close()
+            terms = [gk * m.double() for gk, m in zip(np.float32(gamma).astype(np.float64).tolist(), [X, *hops])]
+            bound = len(gamma) * 2.0**-24 * sum(t.abs() for t in terms)
+            assert bool(((Z.double() - sum(terms)).abs() <= bound).all()), (op, seg)
+            assert bool((hops[-1][1:].abs() < 1e20).all())
+
+
 @pytest.mark.parametrize("op", OPS)
 def test_weighted_hop_sum_matches_oracle(B, op):
     """Z = gamma_0 X_0 + sum_k gamma_k X_k accumulated in the kernels' epilogues: every kernel shape, blocks and
