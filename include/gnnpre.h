@@ -264,13 +264,14 @@ int gnnpre_selftest_wait_timeout(gnnpre_plan_t* plan, uint32_t polls, void* stre
  */
 int gnnpre_inject_alloc_failure(int64_t device_countdown, int64_t host_countdown);
 
-/* Waits for the device (as freeing device memory does), then frees everything the plan owns - except that of the plans for
- * device-resident operands without a memory budget one allocation of at most 128 MB per device is kept for the next such
- * plan (its release and a new one take 0.7 to 8 ms).  It is given back when an allocation of the library fails, and by
- * gnnpre_release_cached_memory, which frees the current device's. */
-int gnnpre_release_cached_memory(void);
-
+/* Waits for the plan's device, whichever is current (as freeing device memory does; a stream capture that is going on is not
+ * disturbed), then frees everything the plan owns - except that of the plans for device-resident operands without a memory
+ * budget one allocation of at most 128 MB per device is kept for the next such plan (its release and a new one take 0.7 to
+ * 8 ms).  It is given back when an allocation of the library fails, and by gnnpre_release_cached_memory. */
 void gnnpre_plan_destroy(gnnpre_plan_t* plan);
+
+/* Frees what plans of the current device have left for the next one. */
+int gnnpre_release_cached_memory(void);
 
 /*
  * One hop without any allocation:  out <- A^ X  computed directly from the caller's CSR.

@@ -526,7 +526,7 @@ namespace {
 // One block of device memory per device outlives the plan that used it, so that a program that makes plan after plan (one
 // per dataset, or per operator) does not pay 0.7 to 8 ms for an allocation and its release each time.  At most
 // kMostCached bytes; only plans for resident operands without a memory budget use it; it is given back when an
-// allocation of the library fails and by gnnpre_release_cached_memory.  A block enters it when the device is idle.
+// allocation of the library fails and by gnnpre_release_cached_memory.  A block enters it when its device's streams are done.
 constexpr size_t kMostCached = 128u << 20, kCachedGrain = 2u << 20;
 
 struct CachedBlock {
@@ -535,12 +535,25 @@ struct CachedBlock {
 };
 std::mutex g_cache_mutex;
 CachedBlock g_cache[kCacheDevices];
+void* g_small_page[kCacheDevices];  // four bytes that keep the driver's page of small allocations (see streams_done)
 
 CachedBlock take_cached(int device, size_t bytes) {
     std::lock_guard<std::mutex> lock(g_cache_mutex);
     CachedBlock b;
     if (device < kCacheDevices && g_cache[device].bytes >= bytes) std::swap(b, g_cache[device]);
     return b;
+}
+
+// Waits for all streams of the current device; false if that failed.  Freeing device memory does so, be it four bytes - and,
+// unlike cudaDeviceSynchronize, it does not invalidate the stream captures in the process.  5 us with the allocation while
+// the driver has its page of small allocations, 320 if that came and went with these four bytes.
+bool streams_done(int device) {
+    if (device < kCacheDevices) {
+        std::lock_guard<std::mutex> lock(g_cache_mutex);
+        if (!g_small_page[device]) (void)cudaMalloc(&g_small_page[device], 4);
+    }
+    void* p = nullptr;
+    return cudaMalloc(&p, 4) == cudaSuccess && cudaFree(p) == cudaSuccess;
 }
 
 // keeps the larger of `b` and what the cache holds, frees the other
@@ -558,7 +571,13 @@ bool gnnpre::release_cached_block() {
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) return false;
     const CachedBlock b = take_cached(device, 1);
+    void* page = nullptr;
+    if (device < kCacheDevices) {
+        std::lock_guard<std::mutex> lock(g_cache_mutex);
+        std::swap(page, g_small_page[device]);
+    }
     if (b.p) cudaFree(b.p);
+    if (page) cudaFree(page);
     return b.p != nullptr;
 }
 
@@ -568,15 +587,16 @@ extern "C" int gnnpre_release_cached_memory(void) {
 }
 
 gnnpre_plan::~gnnpre_plan() {
-    if (arena_cached && arena[0].p) {  // (a build that failed may still have kernels in flight)
-        cudaDeviceSynchronize();
-        give_cached(device, {arena[0].p, arena[0].count});
-        arena[0].owned = false;
-    }
     if (s_h2d) cudaStreamDestroy(s_h2d);
     if (s_d2h) cudaStreamDestroy(s_d2h);
     if (s_compute) cudaStreamDestroy(s_compute);
     if (s_struct) cudaStreamDestroy(s_struct);
+    // kernels on the caller's streams (or of a build that failed) may still use the block: the next plan may have it when they
+    // have ended, else it is freed
+    if (arena_cached && arena[0].p && streams_done(device)) {
+        give_cached(device, {arena[0].p, arena[0].count});
+        arena[0].owned = false;
+    }
 }
 
 int64_t gnnpre_plan::device_bytes() const {
@@ -589,6 +609,19 @@ int64_t gnnpre_plan::device_bytes() const {
 int64_t gnnpre_plan::host_bytes() const { return (int64_t)colx_host.bytes(); }
 
 namespace {
+
+// Destroys the plan with its device current, whichever the caller's is, and in the capture mode in which releases of memory
+// neither fail nor disturb captures on the caller's streams (a plan may be collected at any time).
+void destroy_plan(gnnpre_plan* P) {
+    int device = 0;
+    const bool other = cudaGetDevice(&device) == cudaSuccess && device != P->device && cudaSetDevice(P->device) == cudaSuccess;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    delete P;
+    if (swapped) cudaThreadExchangeStreamCaptureMode(&mode);
+    if (other) cudaSetDevice(device);
+    (void)cudaGetLastError();
+}
 
 int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpre_plan_opts_t* opts,
                     gnnpre_plan* P) {
@@ -957,7 +990,7 @@ extern "C" int gnnpre_build_plan(const gnnpre_csr_t* csr, const int32_t* degrees
     if (!P) return GNNPRE_ERR_OOM_HOST;
     int rc = build_plan_impl(csr, degrees, opts, P);
     if (rc != GNNPRE_OK) {
-        delete P;
+        destroy_plan(P);
         return rc;
     }
     *plan_out = P;
@@ -1029,12 +1062,7 @@ extern "C" int gnnpre_plan_support(const gnnpre_plan_t* P, int64_t* rowptr_out, 
 }
 
 extern "C" void gnnpre_plan_destroy(gnnpre_plan_t* P) {
-    if (!P) return;
-    // Work on the caller's streams may still use the plan's memory.  Freeing it waits for the device in any case; an event
-    // recorded after every call, to wait for instead, stood between that call and the next one's first kernel (3 us).
-    cudaDeviceSynchronize();
-    (void)cudaGetLastError();
-    delete P;
+    if (P) destroy_plan(P);
 }
 
 extern "C" int gnnpre_solve_budget(int64_t B_S, int64_t B_X, int64_t B_fixed, int64_t beta_S, int64_t beta_X,

@@ -1,6 +1,8 @@
 """GPU tests of the host-operand pipeline's second schedule (whole hop matrices on the device, narrow-first
 column panels), of the status query for asynchronous calls, of host-side allocation-failure injection and of
 the operand-overlap checks.  Nothing here faults, traps or hangs a device."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -228,6 +230,46 @@ def test_cached_block_is_reused_bounded_and_given_back(B):
     assert held <= 128 << 20
     B.gnnpre_release_cached_memory()
     assert torch.cuda.mem_get_info()[0] >= free0
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("thread", [False, True])
+def test_plan_closed_while_its_hops_run_and_a_stream_is_captured(B, mode, thread):
+    """Closing a plan waits for its work on any stream before its memory goes to the next plan, also while another stream is
+    being captured - which the wait must leave alone: the capture ends well and its graph replays."""
+    g, other = gi.rmat(30000, 300000, 61, directed_candidates=True), gi.rmat(30000, 300000, 63, directed_candidates=True)
+    d, do = dev(g), dev(other)
+    X = gi.normal_matrix(g.n, 64, 1, device="cuda")
+
+    def hop(structure, x):
+        plan = B.gnnpre_build_plan(*structure, 0, 64)
+        r = B.gnnpre_propagate(plan, x, 1)[0][0].clone()
+        torch.cuda.synchronize()
+        plan.close()
+        return r
+
+    want, want_other = hop(d, X), hop(do, X)
+    out, a, side, done = torch.empty_like(X), torch.zeros(8, device="cuda"), torch.cuda.Stream(), torch.cuda.Event()
+    plan = B.gnnpre_build_plan(*d, 0, 64)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode=mode):
+        with torch.cuda.stream(side):  # not part of the capture
+            torch.cuda._sleep(200_000_000)  # about 0.1 s
+            B.gnnpre_propagate(plan, X, 1, out=[out], stream=side)
+            done.record(side)
+        if thread:
+            t = threading.Thread(target=plan.close)
+            t.start()
+            t.join()
+        else:
+            plan.close()
+        a += 1
+    assert done.query()
+    assert torch.equal(hop(do, X), want_other) and torch.equal(out, want)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool((a == 1).all())
 
 
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
