@@ -10,7 +10,7 @@
 // sums, no output rows, no scratch.  Their results mean nothing; their duration is the yardstick.
 #pragma once
 
-template <int G>
+template <int G, bool FAR>
 __global__ void __launch_bounds__(kThreads, 4) k_ceiling(const SegArgs a, float* __restrict__ sink) {
     constexpr unsigned kFull = 0xffffffffu;
     constexpr int kChunk = G < kSegWindow ? kSegWindow : G;
@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_ceiling(const SegArgs a, float*
     }
     const int q0 = blockIdx.y * a.tile_f4;
     const char* xlane = reinterpret_cast<const char*>(a.x + 4 * q0) + (gl < min(a.tile_f4, a.f4 - q0) ? 16 * gl : 0);
-    const uint32_t row_bytes = (uint32_t)a.ldx * 4u;
+    const RowStride<FAR> row_bytes = (RowStride<FAR>)a.ldx * 4u;
     Quad acc = quad_zero();
     while (G == 32 ? left > 0 : __any_sync(kFull, left > 0)) {
 #pragma unroll

@@ -41,17 +41,17 @@ __global__ void k_wait_that_runs_out(int* error, uint32_t polls) {
 #include "fixups.cuh"
 #include "ceiling.cuh"
 
-template <int G>
+template <int G, bool FAR = false>
 int launch_segments_shape(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
     const int64_t groups = a.seg_hi - a.seg_lo;
     const dim3 grid((unsigned)((groups * G + kSegThreads - 1) / kSegThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
     const int ep = epilogue_of(a.tp);
 #define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                                    \
     do {                                                                                                                       \
-        if (ep == kEpSum) return launch_dependent(k_segments<G, OP_, EMPTY_, kEpSum>, grid, kSegThreads, 0, a.back_to_back, st, a); \
+        if (ep == kEpSum) return launch_dependent(k_segments<G, OP_, EMPTY_, kEpSum, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a); \
         if (ep == kEpTeleport)                                                                                                 \
-            return launch_dependent(k_segments<G, OP_, EMPTY_, kEpTeleport>, grid, kSegThreads, 0, a.back_to_back, st, a);     \
-        return launch_dependent(k_segments<G, OP_, EMPTY_, kEpPlain>, grid, kSegThreads, 0, a.back_to_back, st, a);            \
+            return launch_dependent(k_segments<G, OP_, EMPTY_, kEpTeleport, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a);     \
+        return launch_dependent(k_segments<G, OP_, EMPTY_, kEpPlain, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a);            \
     } while (0)
     switch (P->op) {
     case GNNPRE_OP_GCN_SYM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GCN_SYM, false);
@@ -72,6 +72,7 @@ int32_t equal_tile_f4(int32_t f4) {
 // The register kernel on all columns of `a`, one launch.
 int launch_segments_gather(const gnnpre_plan* P, SegArgs a, cudaStream_t st) {
     a.tile_f4 = equal_tile_f4(a.f4);
+    if (far_rows(a.ldx)) return launch_segments_shape<32, true>(P, a, st);
     if (a.tile_f4 <= 4) return launch_segments_shape<4>(P, a, st);
     if (a.tile_f4 <= 8) return launch_segments_shape<8>(P, a, st);
     if (a.tile_f4 <= 16) return launch_segments_shape<16>(P, a, st);
@@ -303,10 +304,10 @@ int launch_ceiling_tma(const gnnpre_plan* P, const SegArgs& a, float* sink, cuda
     return GNNPRE_OK;
 }
 
-template <int G>
+template <int G, bool FAR = false>
 int launch_ceiling_shape(const SegArgs& a, float* sink, cudaStream_t st) {
     const dim3 grid((unsigned)(((a.seg_hi - a.seg_lo) * G + kThreads - 1) / kThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
-    k_ceiling<G><<<grid, kThreads, 0, st>>>(a, sink);
+    k_ceiling<G, FAR><<<grid, kThreads, 0, st>>>(a, sink);
     GNNPRE_CUDA(cudaGetLastError());
     return GNNPRE_OK;
 }
@@ -331,7 +332,8 @@ int launch_ceiling(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int64
             else GNNPRE_TRY(launch_ceiling_tma<0>(P, a, sink, st));
         } else {
             a.tile_f4 = equal_tile_f4(a.f4);
-            if (a.tile_f4 <= 4) GNNPRE_TRY(launch_ceiling_shape<4>(a, sink, st));
+            if (far_rows(a.ldx)) GNNPRE_TRY((launch_ceiling_shape<32, true>(a, sink, st)));
+            else if (a.tile_f4 <= 4) GNNPRE_TRY(launch_ceiling_shape<4>(a, sink, st));
             else if (a.tile_f4 <= 8) GNNPRE_TRY(launch_ceiling_shape<8>(a, sink, st));
             else if (a.tile_f4 <= 16) GNNPRE_TRY(launch_ceiling_shape<16>(a, sink, st));
             else GNNPRE_TRY(launch_ceiling_shape<32>(a, sink, st));

@@ -68,7 +68,7 @@ struct __align__(16) SegStage {  // read in 16-byte pieces
     }
 };
 
-template <int G, int OP, bool HAS_EMPTY, int EP>
+template <int G, int OP, bool HAS_EMPTY, int EP, bool FAR>
 __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
     // GIN's weights are 1 but for the self-loops': groups of 16 lanes and more mark those in a bit mask and add the rest
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     const bool on = gl < min(a.tile_f4, a.f4 - q0);
     // lanes beyond the row's width re-read its first float4: every load is unconditional and in bounds
     const char* const xlane = reinterpret_cast<const char*>(a.x) + 16 * (q0 + (on ? gl : 0));
-    const uint32_t row_bytes = (uint32_t)a.ldx * 4u;
+    const RowStride<FAR> row_bytes = (RowStride<FAR>)a.ldx * 4u;
     const int out_off = 16 * gl;
 
     const uint32_t* entries = a.colx;

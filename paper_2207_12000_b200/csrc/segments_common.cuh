@@ -152,8 +152,15 @@ __device__ __forceinline__ void quad_fma_pair(Quad& a, float2 w, const Quad& x) 
 
 __device__ __forceinline__ void quad_fma(Quad& a, float w, const Quad& x) { quad_fma_pair(a, make_float2(w, w), x); }
 
+// Bytes from one row to the next.  FAR: from 4 GB on (a narrow view of few, very long rows), where a gather needs more than
+// one 32-bit multiply-add; those take kernels of their own, compiled for whole warps only.
+template <bool FAR>
+using RowStride = std::conditional_t<FAR, uint64_t, uint32_t>;
+inline bool far_rows(int64_t ldx) { return ldx >= (int64_t)1 << 30; }
+
 // float4 of row `col` through the read-only path; `base` points at this lane's piece of row 0
-__device__ __forceinline__ Quad quad_gather(const char* base, uint32_t col, uint32_t row_bytes) {
+template <typename Stride>
+__device__ __forceinline__ Quad quad_gather(const char* base, uint32_t col, Stride row_bytes) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(base + (uint64_t)col * row_bytes));
     return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }

@@ -419,6 +419,32 @@ def test_last_row_of_a_block_is_not_cut(B, op, flags, tail):
     assert fixups == 0
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("F", [16, 100, 132])
+def test_rows_four_gigabytes_apart(B, op, F):
+    """A narrow view of few, very long rows: at a leading dimension of 2^30 floats a row is 2^32 bytes from the next.  Same
+    bits as on rows side by side, plain, with a teleport term and with the sum of hops; and the fetch-only yardstick."""
+    n, ld = 4, (1 << 30) + 4
+    g = gi.from_edge_list(n, [(0, 1), (1, 2), (0, 2)])
+    X = gi.normal_matrix(n, F, 3, device="cuda")
+    buf = torch.empty((n - 1) * ld + F, device="cuda")
+    far = torch.as_strided(buf, (n, F), (ld, 1))
+    far.copy_(X)
+    drp, dci = dev(g)
+    for alpha in (0.0, 0.2):
+        plan = B.gnnpre_build_plan(drp, dci, op, F, gin_eps=EPS, segment_edges=2, teleport_alpha=alpha)
+        want, got = B.gnnpre_propagate(plan, X, 2)[0], B.gnnpre_propagate(plan, far, 2)[0]
+        zw, zg = (B.gnnpre_propagate_weighted(plan, x, [0.5, 0.25, 2.0])[1] for x in (X, far))
+        sinks = [torch.empty(plan.info()["num_segments"], device="cuda") for _ in range(2)]
+        for x, sink in zip((X, far), sinks):
+            B.gnnpre_gather_ceiling(plan, x, sink)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, got)) and torch.equal(zw, zg)
+        if F == 100:  # one column tile and whole warps in both (what lane groups add for empty segments means nothing)
+            assert torch.equal(*sinks)
+        plan.close()
+
+
 def test_two_tile_rows_on_a_graph_larger_than_the_cache(B):
     """Rows of 132..256 columns are cut into two equal tiles for the copy engine once a 128-column tile of X no
     longer fits the L2 (here 400,000 nodes: 205 MB per tile; F = 200 gives two tiles of 100 columns, F = 252 two of
