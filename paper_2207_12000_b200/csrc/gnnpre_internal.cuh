@@ -199,6 +199,7 @@ struct gnnpre_plan {
     int32_t segment_edges = 0;
     uint32_t flags = 0;
     int32_t structure_mem = GNNPRE_MEM_DEVICE;
+    bool degrees_given = false;     // by the caller, so not necessarily the rows' lengths
     bool rows_all_nonempty = true;  // every row owns an edge (always true with self-loops)
     int64_t num_nonempty = 0, num_empty = 0;
 

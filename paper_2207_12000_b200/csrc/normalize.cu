@@ -18,6 +18,7 @@ struct ValArgs {
     int64_t colx_base;
     const int32_t* deg;
     const float* rank_scale;   // scales of the rows that own an edge, in rank order
+    const int32_t* nzrows;     // those rows (nullptr: every row owns one)
     float* out;                // value of edge e goes to out[e - out_base]
     int64_t out_base;
     float diag_weight;         // GIN: 1 + eps, rounded once
@@ -27,7 +28,7 @@ struct ValArgs {
 // reciprocal root, one third-order step in fp64, then the square root and its reciprocal corrected by their exact
 // residuals (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
 // Dev. 34, 1990).  Eleven fp64 operations instead of a general square root and a general division; compared with those
-// for every d in [0, 2^31 - 2], bit for bit.
+// for every d in [0, 2^31 - 1], bit for bit; NaN below.
 __device__ __forceinline__ double inverse_sqrt_degree(int32_t d) {
     const double x = (double)d + 1.0;
     const double y0 = (double)rsqrtf((float)x);
@@ -38,13 +39,19 @@ __device__ __forceinline__ double inverse_sqrt_degree(int32_t d) {
     return fma(fma(-s, y, 1.0), y, y);
 }
 
+// What the formula gives for degrees that a caller got wrong: 1 / sqrt(0) is infinite (-1), the root of less NaN.
+__device__ float value_of_no_degree(int32_t di, int32_t dj) {
+    return (float)((1.0 / sqrt((double)di + 1.0)) * (1.0 / sqrt((double)dj + 1.0)));
+}
+
 // One warp per segment of the edge list, 32 edges at a time, kValChunks chunks of loads in flight: entries are read and
 // values written in whole lines whatever the rows' lengths, and the row of an edge follows from the row-end marks.
 // Bound by the gather of one degree per edge (a 32-byte sector each) from the L2.  54 M edges, GCN: 2307 us with one
 // warp per row (mean degree 15) and a general square root and division per edge, 235 us now.
+// GIVEN: the degrees are the caller's, so any integer; looking for what no degree is costs 2 %.
 constexpr int kValChunks = 4;
 
-template <int OP>
+template <int OP, bool GIVEN>
 __global__ void __launch_bounds__(256) k_edge_values(const ValArgs a) {
     const int64_t sg = a.seg_lo + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (sg >= a.seg_hi) return;
@@ -75,9 +82,12 @@ __global__ void __launch_bounds__(256) k_edge_values(const ValArgs a) {
             const int32_t col = (int32_t)(c[k] & ~kRowEndBit);
             float v;
             if (OP == GNNPRE_OP_GCN_SYM) {
-                v = (float)(inverse_sqrt_degree(__ldg(a.deg + row[k])) * inverse_sqrt_degree(__ldg(a.deg + col)));
+                const int32_t di = __ldg(a.deg + row[k]), dj = __ldg(a.deg + col);
+                v = (float)(inverse_sqrt_degree(di) * inverse_sqrt_degree(dj));
+                if (GIVEN && v != v) v = value_of_no_degree(di, dj);
             } else if (OP == GNNPRE_OP_SAGE_MEAN) {
-                v = __ldg(a.rank_scale + row[k]);  // 1 / D_i in fp64, rounded once
+                v = __ldg(a.rank_scale + row[k]);  // 1 / D_i in fp64, rounded once; 0 stands for a caller's degree below 1
+                if (GIVEN && v == 0.f) v = (float)(1.0 / (double)a.deg[a.nzrows ? a.nzrows[row[k]] : row[k]]);
             } else {
                 v = col == row[k] ? a.diag_weight : 1.f;  // every row owns its self-loop: rank == row
             }
@@ -89,9 +99,12 @@ __global__ void __launch_bounds__(256) k_edge_values(const ValArgs a) {
 int launch_values(const gnnpre_plan* P, const ValArgs& a, cudaStream_t st) {
     if (a.seg_hi <= a.seg_lo) return GNNPRE_OK;
     const unsigned grid = (unsigned)(((a.seg_hi - a.seg_lo) * 32 + 255) / 256);
-    if (P->op == GNNPRE_OP_GCN_SYM) k_edge_values<GNNPRE_OP_GCN_SYM><<<grid, 256, 0, st>>>(a);
-    else if (P->op == GNNPRE_OP_SAGE_MEAN) k_edge_values<GNNPRE_OP_SAGE_MEAN><<<grid, 256, 0, st>>>(a);
-    else k_edge_values<GNNPRE_OP_GIN_SUM><<<grid, 256, 0, st>>>(a);
+    const bool given = P->degrees_given;
+    if (P->op == GNNPRE_OP_GIN_SUM) k_edge_values<GNNPRE_OP_GIN_SUM, false><<<grid, 256, 0, st>>>(a);
+    else if (P->op == GNNPRE_OP_GCN_SYM && !given) k_edge_values<GNNPRE_OP_GCN_SYM, false><<<grid, 256, 0, st>>>(a);
+    else if (P->op == GNNPRE_OP_GCN_SYM) k_edge_values<GNNPRE_OP_GCN_SYM, true><<<grid, 256, 0, st>>>(a);
+    else if (!given) k_edge_values<GNNPRE_OP_SAGE_MEAN, false><<<grid, 256, 0, st>>>(a);
+    else k_edge_values<GNNPRE_OP_SAGE_MEAN, true><<<grid, 256, 0, st>>>(a);
     GNNPRE_CUDA(cudaGetLastError());
     return GNNPRE_OK;
 }
@@ -111,6 +124,7 @@ extern "C" int gnnpre_normalize(gnnpre_plan_t* P, float* vals_out, int32_t vals_
     a.segs = P->segments.p;
     a.deg = P->deg.p;
     a.rank_scale = P->rows_all_nonempty ? P->rscale.p : P->nzscale.p;
+    a.nzrows = P->rows_all_nonempty ? nullptr : P->nzrows.p;
     a.diag_weight = (float)(1.0 + (double)P->gin_eps);
     const bool e_host = P->structure_mem == GNNPRE_MEM_HOST;
     if (!e_host && vals_mem == GNNPRE_MEM_DEVICE) {  // everything resident: all blocks in one launch

@@ -638,6 +638,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->teleport_alpha = opts->teleport_alpha;
     P->flags = opts->flags;
     P->structure_mem = csr->mem;
+    P->degrees_given = degrees != nullptr;
     P->hub_parts = kHubParts;
     const int64_t m = P->nnz_tilde;
     if (csr->mem == GNNPRE_MEM_HOST && (csr->rowptr[0] != 0 || csr->rowptr[n] != nnz)) return GNNPRE_ERR_INVALID_CSR;

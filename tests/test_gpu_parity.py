@@ -511,6 +511,36 @@ def test_normalized_values_at_segment_edges(B, op, seg):
         plan.close()
 
 
+@pytest.mark.parametrize("op", (0, 1))
+@pytest.mark.parametrize("isolated", [False, True])
+def test_normalized_values_of_any_degree_the_caller_gives(B, op, isolated):
+    """Bit for bit, the IEEE square root and division of every degree: 0..5000, squares and powers of two and their
+    neighbours, random ones up to the largest, whose conversion to single precision rounds - and what no degree is: a row
+    with edges given as 0, -1 or less keeps the infinity, NaN or negative value the formula gives."""
+    rng = np.random.default_rng(5)
+    k = np.arange(2, 46340, 7, dtype=np.int64)
+    p = 2 ** np.arange(1, 32, dtype=np.int64)
+    d = np.concatenate([np.arange(5000), k * k - 2, k * k - 1, k * k, p - 2, p - 1, p, rng.integers(1 << 24, (1 << 31) - 1, 30000),
+                        rng.integers(1, 1 << 24, 20000), [(1 << 31) - 1, (1 << 31) - 2, -1, -2, -7]])
+    d = d[d < (1 << 31)].astype(np.int32)
+    n = len(d)
+    i = torch.arange(n - 1, dtype=torch.int64)
+    if isolated:
+        i = i[i % 5 != 0]  # 0 and a few more rows stay alone or have one neighbour
+    g = gi.from_edge_list(n, torch.stack([i, (i * 7 + 3) % (n - 1) + 1], 1)[(i * 7 + 3) % (n - 1) + 1 != i].tolist())
+    plan = B.gnnpre_build_plan(*dev(g), op, 16, degrees=torch.from_numpy(d).cuda())
+    got = to_np(B.gnnpre_normalize(plan))
+    torch.cuda.synchronize()
+    plan.close()
+    rp_t, ci_t = orc.support(op, g.rowptr.numpy(), g.colidx.numpy())
+    row = np.repeat(np.arange(n), np.diff(rp_t))
+    x = d.astype(np.float64)
+    with np.errstate(all="ignore"):
+        want = 1.0 / np.sqrt(x + 1.0)
+        want = (want[row] * want[ci_t] if op == 0 else 1.0 / x[row]).astype(np.float32)
+    np.testing.assert_array_equal(got, want)  # (equal NaN are equal)
+
+
 def test_a_device_wait_that_runs_out_is_reported_and_leaves_the_plan_usable(B):
     """Failure detection without a fault: a warp polls a barrier that nothing completes, gives up after its
     limit and sets the plan's error word; the host reads GNNPRE_ERR_TIMEOUT once, and the same plan then
