@@ -311,12 +311,11 @@ __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const 
 // Segment t of block l nominally starts at e_lo(l) + t*L.  A start that falls inside a row is moved
 // forward to the next row start when that lies within `snap` edges (and inside the block), so that
 // short rows are never cut; long rows are cut and their parts summed by a fix-up.  Where no row of the graph is longer
-// than three segments the start always moves (two may then meet, or one the block's end: an empty segment), and nothing
-// is left for the finishing launch: 4,096 nodes of degree 16, 64 columns, two hops 13.7 us at segments of 32, 10.4 at 16 and none cut.
-// Graphs with longer rows have that launch anyway and are better off balanced (5,000 nodes, R-MAT, 16.7 us against 19.5).
+// than `uncut` edges the start always moves (two may then meet, or one the block's end: an empty segment), and nothing is
+// left for the finishing launch (see longest_uncut_row).
 // Until k_segment_finalize: slot_head holds the "first row began earlier" flag and pad the first row's index.
 __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict__ seg_base,
-                                 const int64_t* __restrict__ e_off, int32_t L, int32_t snap, const int* __restrict__ longest,
+                                 const int64_t* __restrict__ e_off, int32_t L, int32_t snap, int64_t uncut, const int* __restrict__ longest,
                                  const int64_t* __restrict__ rowptr_t, int64_t n, const int32_t* __restrict__ rank,
                                  Segment* __restrict__ segs) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -341,7 +340,7 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     int64_t row = row_of_edge(rowptr_t, n, start);
     if (t > 0 && rowptr_t[row] < start) {
         const int64_t next = rowptr_t[row + 1];
-        if ((next - start <= snap || *longest < 3 * (int64_t)L) && next <= e_off[lo + 1]) {
+        if ((next - start <= snap || *longest < uncut) && next <= e_off[lo + 1]) {
             start = next;
             row = start < e_off[b] ? row_of_edge(rowptr_t, n, start) : n;  // at the very end: empty, as the sentinel
         }
@@ -432,6 +431,24 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool w
     int32_t p = whole_hops && (m / 16) * lanes <= (int64_t)num_sms * 768 ? 16 : 32;
     while ((int64_t)p * 2 <= L && p < 1024) p *= 2;
     return p;
+}
+
+// The longest row (edges) of a graph in which no row is cut, so that segments end with rows and the finishing launch has
+// nothing to do, at the price of uneven and empty segments.  The launch costs the same whatever the graph, the unevenness
+// grows with it; groups of fewer than 32 lanes also wait for the longest segment of their warp.  Mean operator, rows of
+// equal length, us per hop never cut / cut:
+//   all segments at once (4,096 nodes of degree 16, 64 columns, two hops): 10.4 / 13.7, and no worse up to three segments
+//   800,000 edges, L = 32:   32 columns, rows of 1.5 L 25 / 29, 1.8 L 27 / 31, 2 L 29 / 26, 2.4 L 32 / 28; 64 columns
+//                            31 / 36, 38 / 38, 40 / 34, 40 / 36; 128 columns 36 / 43, 37 / 49, 42 / 45, 36 / 45
+//   4 million, L = 64:       16 columns, 1.6 L 51 / 64, 2 L 60 / 51; 32 columns, 1.6 L 69 / 77, 1.8 L 76 / 72; 64 columns,
+//                            1.5 L 99 / 104, 1.8 L 128 / 104; 128 columns, 1.8 L 126 / 151, 2 L 155 / 143, 2.4 L 127 / 142
+//   20 million, L = 256:     16 columns, 1.25 L 177 / 185, 1.5 L 233 / 219, 2 L 290 / 160; 64 columns, 1.25 L 325 / 332,
+//                            1.4 L 391 / 365, 2 L 645 / 302; 128 columns, 1.8 L 529 / 566, 2 L 694 / 538, 2.9 L 549 / 536
+int64_t longest_uncut_row(int64_t m, int64_t lanes, int64_t L, bool one_wave) {
+    const int64_t work = m * lanes;
+    if (one_wave) return 3 * L;
+    if (lanes == 32) return work <= (1 << 28) ? 3 * L : 2 * L;
+    return work <= (1 << 25) ? 2 * L : work <= (1 << 26) ? 3 * L / 2 : 5 * L / 4;
 }
 
 }  // namespace
@@ -854,13 +871,14 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const int64_t lanes = f4_slab <= 4 ? 4 : f4_slab <= 8 ? 8 : f4_slab <= 16 ? 16 : 32;
     const bool one_wave = nseg * lanes <= (int64_t)P->num_sms * 768;
     const int32_t snap = one_wave ? L - 1 : L / 2;
+    const int64_t uncut = longest_uncut_row(m_launch, lanes, L, one_wave);
     if (m > 0) {
         std::vector<int64_t> h_off(e_off);
         h_off.insert(h_off.end(), seg_base.begin(), seg_base.end());
         GNNPRE_CUDA(cudaMemcpyAsync(offsets.p, h_off.data(), sizeof(int64_t) * h_off.size(), cudaMemcpyHostToDevice, st));
         const int64_t *d_e_off = offsets.p, *d_seg_base = offsets.p + b + 1;
         // (without rows that own no edge the scan's ranks are the row numbers)
-        k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap,
+        k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap, uncut,
                                                                   &d_report->longest_row, P->rowptr_t.p, n, rank.p, P->segments.p);
         GNNPRE_CUDA(cudaGetLastError());
         k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);

@@ -445,6 +445,19 @@ def test_rows_four_gigabytes_apart(B, op, F):
         plan.close()
 
 
+@pytest.mark.parametrize("op", OPS)
+def test_rows_of_more_than_two_segments_are_cut_where_segments_run_in_waves(B, op):
+    """Rows of 40 entries and segments of 16, 75,000 of them: far more than run at once, so a segment takes its own 16 edges
+    and not a whole row's."""
+    n = 30000
+    g = gi.from_edge_list(n, [(i, (i + j * j) % n) for i in range(n) for j in range(1, 21)])
+    run_case(B, g, op, 64, 1, seg=16)
+    plan = B.gnnpre_build_plan(*dev(g), op, 64, gin_eps=EPS, segment_edges=16)
+    fixups = plan.info()["num_row_fixups"]
+    plan.close()
+    assert fixups > n // 2
+
+
 def test_two_tile_rows_on_a_graph_larger_than_the_cache(B):
     """Rows of 132..256 columns are cut into two equal tiles for the copy engine once a 128-column tile of X no
     longer fits the L2 (here 400,000 nodes: 205 MB per tile; F = 200 gives two tiles of 100 columns, F = 252 two of
