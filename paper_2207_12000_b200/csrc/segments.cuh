@@ -73,8 +73,11 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     constexpr unsigned kFull = 0xffffffffu;
     // GIN's weights are 1 but for the self-loops': groups of 16 lanes and more mark those in a bit mask and add the rest
     // (169 K nodes, 256 columns: 195 us per hop with a weight per edge, 181 so; 24 M edges, 64 columns: 460 / 430); narrower
-    // groups lose more by the extra votes than the weights cost (169 K nodes, 32 columns: 42 / 45).
-    constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16;
+    // groups lose more by the extra votes than the weights cost (169 K nodes, 32 columns: 42 / 45).  Beside the masks the
+    // teleport term's X_0 piece is spilled, that is, waited for as soon as it is asked for: with that term every edge has its
+    // weight (1 M nodes of degree 50, 100 columns: 3131 us per hop, 3966 with masks; 169 K nodes, 64 columns: 92 / 102; masks
+    // and the piece in shared memory: 3144, 100).
+    constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16 && EP != kEpTeleport;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN && !kDiagonal;
     using Stage = SegStage<G, kWeighted>;
     constexpr int C = Stage::kChunk;
