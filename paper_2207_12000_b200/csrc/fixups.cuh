@@ -55,7 +55,9 @@ __device__ __forceinline__ void pair_add4(float4& s, float4& e, const float4& t,
 // parts in flight (with sixteen the kernel held 98 to 174 registers and ran narrow rows in five waves), and the row's
 // place and scale are fetched while the segment kernel still runs.  169 K nodes, 16 columns, mean operator, three
 // hops: 146 -> 100 us a call (three launches per hop before, each after the end of the one before it).
-constexpr int kEmptyPerGroup = 16;
+// With a teleport term rows without edges read X_0, four rows ahead of their stores (2.4 M nodes, 100 columns, mean operator:
+// 174 us for all that follows a hop's segments, 291 a row at a time; 1.7 M nodes of degree 15 171 / 286).
+constexpr int kEmptyPerGroup = 16, kEmptyAhead = 4;
 
 template <int G, int EP>
 __global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
@@ -83,10 +85,16 @@ __global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
         }
         wait_previous_kernel();
 #pragma unroll
-        for (int k = 0; k < kEmptyPerGroup; ++k)
-            if (row[k] >= 0 && on)
-                *(reinterpret_cast<float4*>(a.out + (int64_t)row[k] * a.ldo) + q0 + gl) =
-                    finish_row_piece<EP>(make_float4(0.f, 0.f, 0.f, 0.f), 0.f, a.tp, row[k], q0 + gl);
+        for (int k0 = 0; k0 < kEmptyPerGroup; k0 += kEmptyAhead) {
+            EpiloguePiece<EP> piece[kEmptyAhead];
+#pragma unroll
+            for (int k = 0; k < kEmptyAhead; ++k) piece[k].load(a.tp, max(row[k0 + k], 0), 0, q0 + gl, on && row[k0 + k] >= 0);
+#pragma unroll
+            for (int k = 0; k < kEmptyAhead; ++k)
+                if (on && row[k0 + k] >= 0)
+                    *(reinterpret_cast<float4*>(a.out + (int64_t)row[k0 + k] * a.ldo) + q0 + gl) =
+                        piece[k].finish(make_float4(0.f, 0.f, 0.f, 0.f), 0.f, a.tp, row[k0 + k], 0, q0 + gl);
+        }
         return;
     }
     const bool hub_cta = (int64_t)blockIdx.x < nhub;
