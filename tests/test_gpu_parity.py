@@ -602,6 +602,31 @@ def test_teleport_filter_matches_oracle(B, op, alpha):
         B.gnnpre_build_plan(drp, dci, op, 16, teleport_alpha=1.5)
 
 
+@pytest.mark.parametrize("F", [72, 100, 200])
+def test_weighted_hop_sum_on_a_graph_of_the_copy_engine(B, F):
+    """Where the plain hops of the mean operator go through the bulk-copy kernel: the hops, with and without a sum, have the
+    register kernel's bits, and Z is their sum (the bound of test_weighted_hop_sum_adds_every_hop_once)."""
+    g = gi.rmat(2000000, 33000000, 29, directed_candidates=False, device="cuda")
+    X = gi.normal_matrix(g.n, F, 9, device="cuda")
+    gamma = [0.3, -0.7, 1.1, 0.4]
+    for alpha in (0.0, 0.15):
+        res = []
+        for flags in (0, B.GNNPRE_FLAG_NO_BULK_COPY):
+            plan = B.gnnpre_build_plan(g.rowptr, g.colidx, 1, F, teleport_alpha=alpha, segment_edges=700, flags=flags)
+            res.append((B.gnnpre_propagate_weighted(plan, X, gamma), B.gnnpre_propagate(plan, X, 3)[0]))
+            torch.cuda.synchronize()
+            plan.close()
+        (hops, Z), plain = res[0]
+        for a, b, c, d in zip(hops, plain, res[1][0][0], res[1][1]):
+            assert torch.equal(a, b) and torch.equal(a, c) and torch.equal(a, d)
+        assert torch.equal(Z, res[1][0][1])
+        terms = [(gk, m) for gk, m in zip(np.float32(gamma).astype(np.float64).tolist(), [X, *hops])]
+        for r0 in range(0, g.n, 250000):
+            want = sum(gk * m[r0:r0 + 250000].double() for gk, m in terms)
+            size = sum(abs(gk) * m[r0:r0 + 250000].abs().double() for gk, m in terms)
+            assert bool(((Z[r0:r0 + 250000].double() - want).abs() <= len(gamma) * 2.0**-24 * size).all())
+
+
 @pytest.mark.parametrize("alpha", [0.0, 0.15])
 @pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132])
 def test_weighted_hop_sum_adds_every_hop_once(B, F, alpha):
