@@ -41,6 +41,11 @@ bool injected_alloc_failure(int kind) {
     return false;
 }
 
+int64_t& refused_allocations() {
+    thread_local int64_t count = 0;
+    return count;
+}
+
 void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int line) {
     const char* base = std::strrchr(file, '/');
     std::snprintf(g_last_error, sizeof(g_last_error), "%s: %s (%s:%d)", cudaGetErrorName(e), what,

@@ -35,6 +35,9 @@ void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int 
 // reported as failed.  kind 0 = device memory, 1 = page-locked host memory.
 bool injected_alloc_failure(int kind);
 
+// How many device allocations of this thread the driver has refused for want of memory (injected failures do not count).
+int64_t& refused_allocations();
+
 // Frees the block of device memory that the current device's cache keeps (see plan.cu); false if there is none.
 bool release_cached_block();
 
@@ -66,6 +69,7 @@ struct DevBuf {
             (void)cudaGetLastError();
             if (release_cached_block()) e = cudaMalloc(reinterpret_cast<void**>(&p), n * sizeof(T));
         }
+        if (e == cudaErrorMemoryAllocation) ++refused_allocations();
         if (e != cudaSuccess) p = nullptr;
         GNNPRE_CUDA(e);
         count = n;

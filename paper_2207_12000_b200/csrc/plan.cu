@@ -774,14 +774,17 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const size_t report_bytes = sizeof(Report) + sizeof(BlockRows) * (size_t)b + sizeof(SegCounts) * (size_t)(b + 1);
     DevBuf<uint32_t> e_temp;
     DevBuf<uint32_t>& colx = e_host ? e_temp : P->colx;  // E of a host-resident structure is on the device for the build only
+    auto want_fixed = [&](Carve& carve) {
+        carve.want(P->deg, (size_t)n);
+        carve.want(P->rscale, (size_t)n);
+        carve.want(P->cscale, (size_t)n);
+        carve.want(P->rowptr_t, (size_t)n + 1);
+        carve.want(P->segments, (size_t)nseg + 1);
+        carve.want(P->dev_error, 1);
+        if (!e_host) carve.want(P->colx, (size_t)m);
+    };
     Carve fixed;
-    fixed.want(P->deg, (size_t)n);
-    fixed.want(P->rscale, (size_t)n);
-    fixed.want(P->cscale, (size_t)n);
-    fixed.want(P->rowptr_t, (size_t)n + 1);
-    fixed.want(P->segments, (size_t)nseg + 1);
-    fixed.want(P->dev_error, 1);
-    if (!e_host) fixed.want(P->colx, (size_t)m);
+    want_fixed(fixed);
     auto want_sized = [&](Carve& carve, int64_t fixups, int64_t hubs, int64_t nonempty, int64_t empty, int64_t slots) {
         carve.want(P->fixups, (size_t)fixups);
         carve.want(P->hubs, (size_t)hubs);
@@ -795,20 +798,29 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
     const int64_t most_rows = diag ? 0 : n;
     const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
-    const bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
-                                fixed.bytes() > (1 << 20);
+    bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
+                          fixed.bytes() > (1 << 20);
     if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
+    const int64_t refused = refused_allocations();
+    int placed;
     if (one_allocation && fixed.bytes() <= kMostCached - kCachedGrain) {  // in whole grains, so that the next plan's may fit
         const size_t bytes = (fixed.bytes() + kCachedGrain - 1) / kCachedGrain * kCachedGrain;
         const CachedBlock block = take_cached(P->device, bytes);
         P->arena_cached = true;
         P->arena[0].p = block.p;
         P->arena[0].count = block.bytes;
-        if (!block.p) GNNPRE_TRY(P->arena[0].alloc(bytes));
-        GNNPRE_TRY(fixed.place(P->arena[0].p));
+        placed = block.p ? GNNPRE_OK : P->arena[0].alloc(bytes);
+        if (placed == GNNPRE_OK) placed = fixed.place(P->arena[0].p);
     } else {
-        GNNPRE_TRY(fixed.place(P->arena[0]));
+        placed = fixed.place(P->arena[0]);
     }
+    if (placed != GNNPRE_OK && one_allocation && refused_allocations() > refused) {  // no room for the most: what is needed, then
+        one_allocation = P->arena_cached = false;
+        Carve exact;
+        want_fixed(exact);
+        placed = exact.place(P->arena[0]);
+    }
+    GNNPRE_TRY(placed);
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
     DevBuf<char> temp_arena, report;
     DevBuf<int32_t> flag, rank, rank_temp, first;

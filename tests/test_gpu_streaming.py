@@ -272,6 +272,36 @@ def test_plan_closed_while_its_hops_run_and_a_stream_is_captured(B, mode, thread
     assert bool((a == 1).all())
 
 
+@pytest.mark.parametrize("op", OPS)
+def test_plan_on_a_device_with_little_room_left(B, op):
+    """A small plan takes one block for the most that its segments can need; where that has no room, the plan is built with
+    what they do need."""
+    g = gi.rmat(60000, 500000, 64, directed_candidates=True)
+    d = dev(g)
+    F = 512
+    X, out = gi.normal_matrix(g.n, F, 1, device="cuda"), torch.empty((g.n, F), device="cuda")
+    B.gnnpre_release_cached_memory()
+    plan = B.gnnpre_build_plan(*d, op, F)
+    held = plan.info()["device_bytes"]
+    want = B.gnnpre_propagate(plan, X, 1)[0][0]
+    torch.cuda.synchronize()
+    plan.close()
+    B.gnnpre_release_cached_memory()
+    torch.cuda.empty_cache()
+    assert held > 60 << 20
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (held - (20 << 20)), dtype=torch.uint8, device="cuda")
+    try:
+        plan = B.gnnpre_build_plan(*d, op, F)
+        assert plan.info()["device_bytes"] < held - (20 << 20)
+        B.gnnpre_propagate(plan, X, 1, out=[out])
+        torch.cuda.synchronize()
+        plan.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert torch.equal(out, want)
+
+
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
     """X, out[] and Z are checked for shared elements, not only for equal base pointers; the hops of one call
     may be column views of one wide buffer (concatenated hops, as JKNet's COMB wants them)."""
