@@ -81,8 +81,8 @@ typedef struct {
     int64_t feat_dim;        /* F: columns of X.  Work is done on whole groups of 4 columns: with F % 4 != 0 the
                                 1..3 pad columns up to the next multiple of 4 (which ldx, ldo >= that multiple
                                 make room for) are read from X and written to out[] with unspecified values */
-    int64_t budget_bytes;    /* B_GPU of Eq. 12; 0 = the device's free memory at plan time (taken to suffice, without asking
-                                the driver, for a resident plan whose volumes are at most 1/16 of the device) */
+    int64_t budget_bytes;    /* B_GPU of Eq. 12; 0 = the device's free memory at plan time (for a resident plan whose volumes
+                                are at most 1/16 of the device the driver is not asked unless the plan does not fit) */
     int32_t force_blocks;    /* b; 0 = solve Eq. 12 */
     int32_t force_col_slabs; /* c; 0 = solve Eq. 12 */
     int32_t segment_edges;   /* edges per warp-level segment; 0 = chosen from F */
@@ -106,7 +106,8 @@ typedef struct {
     int64_t slab_width;        /* columns per slab: 4 * ceil(F / (4c)) */
     int64_t B_S, B_X, B_fixed; /* Eq. 12's volumes in bytes: 4*nnz_tilde + 8*(n+1); 4*n*F; 16*n (per-node arrays) */
     int64_t beta_S, beta_X;    /* Eq. 12's coefficients as this library sets them */
-    int64_t budget_bytes;
+    int64_t budget_bytes;      /* B_GPU that (b, c) were solved with: the caller's, else the device's free memory when the plan
+                                  was built or, where the driver was not asked, all of its memory */
     int64_t device_bytes;      /* device memory the plan holds */
     int64_t host_bytes;        /* pinned host memory the plan holds */
     int64_t num_segments;      /* warp-level edge segments over all blocks */

@@ -199,6 +199,7 @@ struct gnnpre_plan {
     int32_t b = 1, c = 1;
     int64_t slab_width = 0;
     int64_t B_S = 0, B_X = 0, B_fixed = 0, beta_S = 1, beta_X = 2;
+    int64_t solved_budget = 0;                     // what Eq. 12 was solved with
     mutable std::atomic<int64_t> budget_bytes{0};  // 0 = not asked for yet (see plan_budget)
     int32_t segment_edges = 0;
     uint32_t flags = 0;

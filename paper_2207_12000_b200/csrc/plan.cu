@@ -522,8 +522,8 @@ int64_t device_memory_bytes(int device) {
 
 }  // namespace
 
-// B_GPU of Eq. 12: what the caller set, else the device's free memory when the plan was built or, if nobody asked then,
-// when somebody first does.
+// Device memory that calls on the plan may count on: what the caller set, else the device's free memory when the plan was
+// built or, if nobody asked then, when somebody first does.
 int64_t gnnpre::plan_budget(const gnnpre_plan* P) {
     int64_t budget = P->budget_bytes.load(std::memory_order_relaxed);
     if (budget <= 0) {
@@ -640,7 +640,8 @@ void destroy_plan(gnnpre_plan* P) {
     (void)cudaGetLastError();
 }
 
-int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpre_plan_opts_t* opts,
+// ask: the free memory is asked for whatever the plan's size.
+int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpre_plan_opts_t* opts, bool ask,
                     gnnpre_plan* P) {
     const int64_t n = csr->n, nnz = csr->nnz;
     const bool diag = opts->op != GNNPRE_OP_SAGE_MEAN;
@@ -673,9 +674,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     if (budget <= 0) {
         // The free memory, but for the question: on a busy machine the driver takes 0.06 to 100 ms to answer it (median 0.4),
         // longer than everything else a small plan needs.  A resident plan whose volumes are a sixteenth of the device at
-        // most is not asked about; gnnpre_plan_info asks when it is called.
+        // most is not asked about (unless it turns out not to fit: gnnpre_build_plan).
         const int64_t device_bytes = device_memory_bytes(P->device);
-        if (resident && P->B_S + P->beta_X * P->B_X + P->B_fixed <= device_bytes / 16) {
+        if (resident && !ask && P->B_S + P->beta_X * P->B_X + P->B_fixed <= device_bytes / 16) {
             budget = device_bytes;
         } else {
             size_t free_b = 0, total_b = 0;  // nothing of the plan has been allocated yet
@@ -684,6 +685,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
             P->budget_bytes = budget;
         }
     }
+    P->solved_budget = budget;
     const int64_t max_c = (F + 3) / 4;
     const int64_t max_b = std::min<int64_t>(std::max<int64_t>(m, 1), 1 << 20);
     int64_t b = opts->force_blocks, c = opts->force_col_slabs;
@@ -798,7 +800,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
     const int64_t most_rows = diag ? 0 : n;
     const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
-    bool one_allocation = opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
+    bool one_allocation = !ask && opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
                           fixed.bytes() > (1 << 20);
     if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
     const int64_t refused = refused_allocations();
@@ -1017,9 +1019,17 @@ extern "C" int gnnpre_build_plan(const gnnpre_csr_t* csr, const int32_t* degrees
     if (opts->feat_dim < 1) return GNNPRE_ERR_INVALID_ARG;
     if (opts->segment_edges < 0 || opts->segment_edges > (1 << 20)) return GNNPRE_ERR_INVALID_ARG;
     GNNPRE_TRY(check_device());
+    const int64_t refused = refused_allocations();
     gnnpre_plan* P = new (std::nothrow) gnnpre_plan();
     if (!P) return GNNPRE_ERR_OOM_HOST;
-    int rc = build_plan_impl(csr, degrees, opts, P);
+    int rc = build_plan_impl(csr, degrees, opts, false, P);
+    if (rc == GNNPRE_ERR_OOM_DEVICE && P->budget_bytes <= 0 && refused_allocations() > refused) {
+        // (b, c) were solved for a device that holds the plan easily, but there is no room: for what is free, then
+        destroy_plan(P);
+        P = new (std::nothrow) gnnpre_plan();
+        if (!P) return GNNPRE_ERR_OOM_HOST;
+        rc = build_plan_impl(csr, degrees, opts, true, P);
+    }
     if (rc != GNNPRE_OK) {
         destroy_plan(P);
         return rc;
@@ -1044,7 +1054,7 @@ extern "C" int gnnpre_plan_info(const gnnpre_plan_t* P, gnnpre_plan_info_t* o) {
     o->B_fixed = P->B_fixed;
     o->beta_S = P->beta_S;
     o->beta_X = P->beta_X;
-    o->budget_bytes = plan_budget(P);
+    o->budget_bytes = P->solved_budget;
     o->device_bytes = P->device_bytes();
     o->host_bytes = P->host_bytes();
     o->num_segments = P->num_segments;

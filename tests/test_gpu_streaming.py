@@ -302,6 +302,44 @@ def test_plan_on_a_device_with_little_room_left(B, op):
     assert torch.equal(out, want)
 
 
+def test_budget_reported_is_the_one_the_block_counts_were_solved_with(B):
+    """gnnpre_plan_info's budget solves to the plan's own (b, c), whatever is free by the time somebody asks; and a plan that
+    has no room at (1, 1) is solved again for what is free."""
+    g = gi.erdos_renyi(200000, 2000000, 5, device="cuda")
+    d = g.rowptr, g.colidx
+    F = 512
+
+    def solved(info):
+        return B.gnnpre_solve_budget(info["B_S"], info["B_X"], info["B_fixed"], info["beta_S"], info["beta_X"],
+                                     info["budget_bytes"], 1 << 20, F // 4)
+
+    X, out = gi.normal_matrix(g.n, F, 1, device="cuda"), torch.empty((g.n, F), device="cuda")
+    plan = B.gnnpre_build_plan(*d, 0, F, segment_edges=12)
+    first = plan.info()
+    assert solved(first) == (first["b"], first["c"]) == (1, 1) and first["device_bytes"] > 350 << 20
+    want = B.gnnpre_propagate(plan, X, 1)[0][0]
+    torch.cuda.synchronize()
+    B.gnnpre_build_plan(*d, 0, F // 8).close()  # (its kernels are loaded)
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (60 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        again = plan.info()
+        assert again["budget_bytes"] == first["budget_bytes"] and again["device_bytes"] == first["device_bytes"]
+        plan.close()
+        B.gnnpre_release_cached_memory()
+        more = torch.empty(torch.cuda.mem_get_info()[0] - (250 << 20), dtype=torch.uint8, device="cuda")
+        plan = B.gnnpre_build_plan(*d, 0, F, segment_edges=12)
+        info = plan.info()
+        assert info["c"] > 1 and info["budget_bytes"] < 300 << 20 and solved(info) == (info["b"], info["c"])
+        B.gnnpre_propagate(plan, X, 1, out=[out])
+        torch.cuda.synchronize()
+        plan.close()
+    finally:
+        fill = more = None
+        torch.cuda.empty_cache()
+    torch.testing.assert_close(out, want, rtol=1e-5, atol=1e-5)
+
+
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
     """X, out[] and Z are checked for shared elements, not only for equal base pointers; the hops of one call
     may be column views of one wide buffer (concatenated hops, as JKNet's COMB wants them)."""
