@@ -975,6 +975,12 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         GNNPRE_CUDA(cudaMemcpy(P->colx_host.p, colx.p, sizeof(uint32_t) * (size_t)m, cudaMemcpyDeviceToHost));
         int64_t longest = 0;
         for (const Block& B : P->blocks) longest = std::max(longest, B.e_hi - B.e_lo);
+        // (the build's copies make room for the staging buffers: a structure kept on the host may be one that hardly fits)
+        tmp_rowptr.reset();
+        tmp_colidx.reset();
+        tmp_deg.reset();
+        temp_arena.reset();
+        e_temp.reset();
         GNNPRE_TRY(P->colx_stage[0].alloc((size_t)longest));
         if (b > 1) GNNPRE_TRY(P->colx_stage[1].alloc((size_t)longest));
     }

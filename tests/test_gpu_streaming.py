@@ -340,6 +340,31 @@ def test_budget_reported_is_the_one_the_block_counts_were_solved_with(B):
     torch.testing.assert_close(out, want, rtol=1e-5, atol=1e-5)
 
 
+def test_host_structure_builds_in_the_memory_of_its_copies(B):
+    """A structure that stays on the host: its staging buffers take the place of the build's copies, so the build never holds
+    more than the CSR, E once and the tables."""
+    g = gi.erdos_renyi(200000, 20000000, 5, device="cuda")
+    rp, ci = g.rowptr.cpu().pin_memory(), g.colidx.cpu().pin_memory()
+    build = dict(force_blocks=2, budget_bytes=1 << 32, operands_mem=B.GNNPRE_MEM_HOST)
+    plan = B.gnnpre_build_plan(rp, ci, 0, 16, **build)
+    stages = 4 * (g.nnz + g.n)
+    tables = plan.info()["device_bytes"] - stages
+    plan.close()
+    n, nnz = g.n, g.nnz
+    del g
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    B.gnnpre_release_cached_memory()
+    room = (4 * nnz + 8 * n) + 4 * (nnz + n) + tables + (30 << 20)
+    assert stages > 2 * (30 << 20)
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    try:
+        B.gnnpre_build_plan(rp, ci, 0, 16, **build).close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+
+
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
     """X, out[] and Z are checked for shared elements, not only for equal base pointers; the hops of one call
     may be column views of one wide buffer (concatenated hops, as JKNet's COMB wants them)."""
