@@ -151,9 +151,17 @@ def gnnpre_degrees(rowptr: torch.Tensor, colidx: torch.Tensor, stream=None) -> t
 class Plan:
     """Owns a gnnpre_plan_t*; destroyed with the object."""
 
-    def __init__(self, handle: int, nnz_tilde: int):
+    def __init__(self, handle: int, keepalive=None, nnz_tilde: int | None = None):
         self._h = ctypes.c_void_p(handle)
-        self.nnz_tilde = nnz_tilde  # edges of the operator's support
+        self._keepalive = keepalive
+        self._nnz_tilde = nnz_tilde
+
+    @property
+    def nnz_tilde(self) -> int:
+        """Edges of the operator's support."""
+        if self._nnz_tilde is None:
+            self._nnz_tilde = gnnpre_plan_info(self)["nnz_tilde"]
+        return self._nnz_tilde
 
     @property
     def handle(self):
@@ -186,7 +194,7 @@ def gnnpre_build_plan(rowptr: torch.Tensor, colidx: torch.Tensor, op: int, feat_
     out = ctypes.c_void_p()
     _check(_lib.gnnpre_build_plan(ctypes.byref(csr), degrees.data_ptr() if degrees is not None else None,
                                   ctypes.byref(opts), ctypes.byref(out)), "gnnpre_build_plan")
-    return Plan(out.value, csr.nnz + (0 if op == GNNPRE_OP_SAGE_MEAN else csr.n))
+    return Plan(out.value, nnz_tilde=csr.nnz + (0 if op == GNNPRE_OP_SAGE_MEAN else csr.n))
 
 
 def gnnpre_plan_info(plan: Plan) -> dict:

@@ -365,6 +365,18 @@ def test_host_structure_builds_in_the_memory_of_its_copies(B):
         torch.cuda.empty_cache()
 
 
+def test_plan_object_around_a_bare_handle(B):
+    """A Plan made from a handle, as before it carried the support's size."""
+    g = gi.rmat(3000, 20000, 65, directed_candidates=True)
+    plan = B.gnnpre_build_plan(*dev(g), 0, 16)
+    want = to_np(B.gnnpre_normalize(plan))
+    bare = B.Plan(plan.handle.value, None)
+    got = to_np(B.gnnpre_normalize(bare))
+    bare._h = None  # the first object owns the plan
+    np.testing.assert_array_equal(got, want)
+    plan.close()
+
+
 def test_overlapping_operands_are_rejected_and_column_views_accepted(B):
     """X, out[] and Z are checked for shared elements, not only for equal base pointers; the hops of one call
     may be column views of one wide buffer (concatenated hops, as JKNet's COMB wants them)."""
