@@ -74,6 +74,7 @@ typedef struct {
 #define GNNPRE_FLAG_NO_BULK_COPY 4u     /* gather into registers for every width (default: the mean operator's rows
                                            of 68..124 columns are staged through shared memory by the bulk-copy
                                            engine on dense graphs several times the L2); same bits */
+#define GNNPRE_FLAG_BULK_COPY 8u        /* ... on any graph (for tests and measurements); same bits */
 
 typedef struct {
     int32_t op;              /* gnnpre_op_t */

@@ -17,6 +17,7 @@ from . import build as _build
 GNNPRE_OP_GCN_SYM, GNNPRE_OP_SAGE_MEAN, GNNPRE_OP_GIN_SUM = 0, 1, 2
 GNNPRE_MEM_DEVICE, GNNPRE_MEM_HOST = 0, 1
 GNNPRE_FLAG_LAUNCH_PER_BLOCK, GNNPRE_FLAG_SKIP_VALIDATION, GNNPRE_FLAG_NO_BULK_COPY = 1, 2, 4
+GNNPRE_FLAG_BULK_COPY = 8
 GNNPRE_MAX_HOPS = 64
 GNNPRE_SCHEDULE_RESIDENT, GNNPRE_SCHEDULE_SLABS, GNNPRE_SCHEDULE_PANELS = 0, 1, 2
 

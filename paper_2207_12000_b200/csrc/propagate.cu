@@ -207,14 +207,15 @@ int64_t l2_cache_bytes() {
 // 5137 / 4658.  800 K nodes of degree 63, mean, 100 columns (2.4 x L2): register; 1.7 M nodes of degree 15 as well.
 bool tile_uses_bulk_copy(const gnnpre_plan* P, int32_t width) {
     const int32_t f4 = width / 4;
-    return P->op == GNNPRE_OP_SAGE_MEAN && !(P->flags & GNNPRE_FLAG_NO_BULK_COPY) && f4 > 16 && f4 < 32 &&
-           P->n * (int64_t)width * 4 > 4 * l2_cache_bytes() && P->nnz_tilde >= 32 * P->n;
+    if (P->op != GNNPRE_OP_SAGE_MEAN || (P->flags & GNNPRE_FLAG_NO_BULK_COPY) || f4 <= 16 || f4 >= 32) return false;
+    return (P->flags & GNNPRE_FLAG_BULK_COPY) || (P->n * (int64_t)width * 4 > 4 * l2_cache_bytes() && P->nnz_tilde >= 32 * P->n);
 }
 
 // Columns one segment launch covers: all of them, as tiles of one launch, while a 128-column tile of X fits the L2.
 // Beyond that each tile is a launch of its own, so that only one tile's rows compete for the cache at a time.
 int32_t segment_tile_width(const gnnpre_plan* P, int32_t width) {
-    if ((P->flags & GNNPRE_FLAG_NO_BULK_COPY) || P->n * 512 <= l2_cache_bytes()) return width;
+    const bool one_launch = (P->flags & GNNPRE_FLAG_NO_BULK_COPY) || P->n * 512 <= l2_cache_bytes();
+    if (one_launch && !(P->flags & GNNPRE_FLAG_BULK_COPY)) return width;
     return 4 * equal_tile_f4(width / 4);
 }
 

@@ -350,32 +350,29 @@ def test_streamed_pageable_host_memory_and_check_against_oracle(B):
 @pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("F", [68, 100, 128, 300, 516])
 def test_bulk_copy_kernel_matches_register_kernel_bitwise(B, op, F):
-    """Rows of 68..128 columns are staged through shared memory by the copy engine; the summation order is that
-    of the register kernel for such rows (plain sums over steps of 8 edges), so the two agree bit for bit (and both
-    agree with the oracle).  Rows wider than 256 columns are cut into 128-column tiles for the copy engine
-    (300 = 128 + 128 + a 44-column tile left to the register kernel; 516 = four tiles + 4 columns); the register
-    kernel for rows that wide sums over steps of 2 edges, so there the two paths agree to rounding only and each
-    is checked against the oracle."""
+    """The mean operator's rows of 68..124 columns are staged through shared memory by the copy engine on large graphs, here
+    asked for; wider ones are cut into equal tiles (300 = three of 100, 516 = five of at most 104).  The summation order is
+    the register kernel's (plain sums over steps of 8 edges), so the two agree bit for bit and both agree with the oracle.
+    The other operators and 128 columns take the register kernel either way."""
     g = gi.rmat(30000, 400000, 17, directed_candidates=True)
     drp, dci = dev(g)
     X = gi.normal_matrix(g.n, F, 9, device="cuda")
     for b, seg in ((1, 256), (3, 64), (2, 1000)):  # same segment length for both: same summation order
         res = []
-        for flags in (0, B.GNNPRE_FLAG_NO_BULK_COPY):
+        for flags in (B.GNNPRE_FLAG_BULK_COPY, B.GNNPRE_FLAG_NO_BULK_COPY):
             plan = B.gnnpre_build_plan(drp, dci, op, F, gin_eps=EPS, force_blocks=b, segment_edges=seg, flags=flags)
             outs, st = B.gnnpre_propagate(plan, X, 2, want_stats=True)
             res.append(outs)
             plan.close()
         for k in range(2):
-            if F <= 128:
-                assert torch.equal(res[0][k], res[1][k]), (b, seg, k)
+            assert torch.equal(res[0][k], res[1][k]), (b, seg, k)
         if F > 128:
             check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), to_np(X), res[1])
             check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), to_np(X), res[0])
     check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), to_np(X), res[0])
 
 
-@pytest.mark.parametrize("op,F", [(1, 92), (1, 100), (1, 124), (1, 200), (2, 124)])
+@pytest.mark.parametrize("op,F", [(1, 92), (1, 100), (1, 124), (1, 200)])
 def test_bulk_copy_kernel_on_a_dense_graph_far_larger_than_the_cache(B, op, F):
     """The copy engine takes over when X is more than four times the L2 and rows are long; same segments, same order of
     additions, so the register kernel must give the same bits."""
@@ -458,10 +455,38 @@ def test_rows_of_more_than_two_segments_are_cut_where_segments_run_in_waves(B, o
     assert fixups > n // 2
 
 
+@pytest.mark.parametrize("F", [68, 72, 100, 124, 200])
+@pytest.mark.parametrize("seg", [1, 7, 16, 17, 300])
+@pytest.mark.parametrize("isolated", [False, True])
+def test_bulk_copy_kernel_at_segment_edges(B, F, seg, isolated):
+    """The bulk-copy kernel on short, cut and empty segments: segments around its chunks of 16 edges, rows of every length
+    from none to several segments, rows that end with their segment or not; plain, with a teleport term, one launch per block,
+    and hops with a sum.  The register kernel's bits throughout, and the oracle's hops."""
+    n = 300 if isolated else 90
+    edges = [(i, j) for i in range(0, 90, 7) for j in range(i + 1, min(90, i + 1 + 2 * i))] + [(i, i + 1) for i in range(89)]
+    g = gi.from_edge_list(n, edges)
+    drp, dci = dev(g)
+    X = gi.normal_matrix(n, F, 9, device="cuda")
+    for alpha in (0.0, 0.15):
+        for extra in (0, B.GNNPRE_FLAG_LAUNCH_PER_BLOCK):
+            res = []
+            for flags in (B.GNNPRE_FLAG_BULK_COPY, B.GNNPRE_FLAG_NO_BULK_COPY):
+                plan = B.gnnpre_build_plan(drp, dci, 1, F, force_blocks=3, segment_edges=seg, flags=flags | extra, teleport_alpha=alpha)
+                hops = B.gnnpre_propagate(plan, X, 2)[0]
+                whops, Z = B.gnnpre_propagate_weighted(plan, X, [0.5, 0.25, -2.0])
+                torch.cuda.synchronize()
+                res.append([*hops, *whops, Z])
+                plan.close()
+            assert all(torch.equal(a, b) for a, b in zip(*res)), (alpha, extra)
+            assert torch.equal(res[0][0], res[0][2]) and torch.equal(res[0][1], res[0][3])
+        if alpha == 0.0:
+            check_all_hops(1, EPS, g.rowptr.numpy(), g.colidx.numpy(), to_np(X), res[0][:2])
+
+
 def test_two_tile_rows_on_a_graph_larger_than_the_cache(B):
-    """Rows of 132..256 columns are cut into two equal tiles for the copy engine once a 128-column tile of X no
+    """Rows of 132..256 columns are cut into two equal tiles, each a launch of its own, once a 128-column tile of X no
     longer fits the L2 (here 400,000 nodes: 205 MB per tile; F = 200 gives two tiles of 100 columns, F = 252 two of
-    128 and 124).  Checked against the oracle, and against the register kernel to rounding."""
+    128 and 124).  Checked against the oracle, and against one launch over both tiles."""
     g = gi.rmat(400000, 3000000, 23, directed_candidates=True)
     drp, dci = dev(g)
     rp, ci = g.rowptr.numpy(), g.colidx.numpy()
@@ -801,14 +826,15 @@ def test_resuming_from_a_finished_hop_gives_the_same_bits(B):
 
 @pytest.mark.parametrize("op", OPS)
 def test_streamed_slabs_through_the_bulk_copy_kernel(B, op):
-    """Column slabs of 100 columns (F = 200, c = 2) and a 128-column tail tile (F = 640): the tensor map of the
-    bulk-copy kernel starts at a column offset, in dense slab buffers and in the caller's strided matrix."""
+    """Column slabs of 100 columns (F = 200, c = 2) and tiles of 80 and 128 columns (F = 160, 640): the tensor map of the
+    bulk-copy kernel (asked for; the mean operator has it) starts at a column offset, in dense slab buffers and in the
+    caller's strided matrix."""
     g = gi.rmat(12000, 150000, 31, directed_candidates=True)
     rp, ci = g.rowptr.numpy(), g.colidx.numpy()
-    for F, c in ((200, 2), (640, 1)):
+    for F, c in ((200, 2), (160, 1), (640, 1)):
         X = gi.normal_matrix(g.n, F, 8, device="cuda")
         plan = B.gnnpre_build_plan(*dev(g), op, F, gin_eps=EPS, force_blocks=3, force_col_slabs=c,
-                                   operands_mem=B.GNNPRE_MEM_HOST)
+                                   operands_mem=B.GNNPRE_MEM_HOST, flags=B.GNNPRE_FLAG_BULK_COPY)
         houts = [torch.empty(g.n, F).pin_memory() for _ in range(2)]
         B.gnnpre_propagate(plan, X.cpu().pin_memory(), 2, houts)
         check_all_hops(op, EPS, rp, ci, to_np(X), houts)
