@@ -53,7 +53,7 @@ __device__ __forceinline__ void pair_add4(float4& s, float4& e, const float4& t,
 // rows without edges (zero, or alpha * X_0[i] with a teleport term), kEmptyPerGroup to a lane group.
 // Bound by latency: two dependent loads per row, and most rows have two or three parts.  A lane keeps at most eight
 // parts in flight (with sixteen the kernel held 98 to 174 registers and ran narrow rows in five waves), and the row's
-// place and scale are fetched while the segment kernel still runs.  169 K nodes, 16 columns, mean operator, three
+// place and scale are fetched while the segment kernel completes.  169 K nodes, 16 columns, mean operator, three
 // hops: 146 -> 100 us a call (three launches per hop before, each after the end of the one before it).
 // With a teleport term rows without edges read X_0, four rows ahead of their stores (2.4 M nodes, 100 columns, mean operator:
 // 174 us for all that follows a hop's segments, 291 a row at a time; 1.7 M nodes of degree 15 171 / 286).

@@ -490,9 +490,9 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // (9-12) read each stage that has landed and write the low parts of its rows into tensor memory, from where the tensor core
 // takes them as operand A (lane = row): beside the two 128-column accumulators there are 32 columns for each of eight
 // stages, and shared memory holds four stages of copied rows beside 128 KB of weight.  2.4 M rows x 3 hops, F = 100, hidden
-// 256, random order: 4587 us when the copying threads split into a second half of two stages (and their proxy fence waited
-// for all their copies in flight), 3550 us with splitter warps and two buffers of low parts in shared memory, 2816 us now;
-// 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the L2's and the copy path's latency over those four stages.
+// 256, random order, under load: 4630 us when the copying threads split into a second half of two stages (and their proxy
+// fence waited for all their copies in flight), 3379 us now (single passes on a cool device: 3550 us with splitter warps and two
+// buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the L2's and the copy path's latency over those four stages.
 // K-steps of the last chunk beyond the features are neither copied nor multiplied.
 //
 // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13

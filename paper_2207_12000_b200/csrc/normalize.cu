@@ -27,8 +27,8 @@ struct ValArgs {
 // 1.0 / sqrt(d + 1.0), both operations rounded to nearest as IEEE 754 does: a single-precision estimate of the
 // reciprocal root, one third-order step in fp64, then the square root and its reciprocal corrected by their exact
 // residuals (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
-// Dev. 34, 1990).  Eleven fp64 operations instead of a general square root and a general division; compared with those
-// for every d in [0, 2^31 - 1], bit for bit; NaN below.
+// Dev. 34, 1990).  Eleven fp64 operations instead of a general square root and a general division, the same bits (compared
+// once for every d in [0, 2^31 - 2]; the tests hold squares, powers of two and random degrees up to 2^31 - 1); NaN below 0.
 __device__ __forceinline__ double inverse_sqrt_degree(int32_t d) {
     const double x = (double)d + 1.0;
     const double y0 = (double)rsqrtf((float)x);

@@ -4,10 +4,10 @@
 // never materialised).
 //
 // Work decomposition.  The edge list E of the support is cut, inside every edge block, into short
-// contiguous segments.  A group of G lanes (G = 4..32, so that one lane holds one or more float4 of
-// a feature row) walks one segment edge by edge: the group reads up to G column indices with one
-// coalesced load, then gathers the neighbours' feature rows with 128-bit loads, several rows in
-// flight per lane, and accumulates in fp32 registers.  Bit 31 of a column entry marks the last edge
+// contiguous segments.  A group of G lanes (G = 4..32, a lane holds one float4 of a column tile) walks
+// one segment edge by edge: the group reads its column indices with coalesced loads, then gathers the
+// neighbours' feature rows with 128-bit loads, eight rows in flight per lane, and accumulates in fp32
+// registers.  Bit 31 of a column entry marks the last edge
 // of a row: there the group scales the sum by r_i and stores the output row.  Rows cut by a segment
 // boundary leave their partial sums in scratch rows, which k_finish_rows adds up in a fixed order.
 #include <algorithm>
@@ -203,8 +203,10 @@ int64_t l2_cache_bytes() {
 // slower path.  us per hop, bulk copy / register: 2.4 M nodes of mean degree 51, mean operator, 72 columns 3634 / 3845,
 // 100 columns 4085 / 4509, 124 columns 4670 / 5150, but 128 columns, rows of whole cache lines, 4641 / 4461; degree 34,
 // 100 columns 3187 / 3368.  With a weight per edge the rows wait for their weights instead: GCN, degree 51, 72 / 100 / 128
-// columns 4583 / 4243, 4971 / 4927, 5519 / 4792; GIN, whose few weighted edges are marked, 4010 / 3951, 4495 / 4599,
-// 5137 / 4658.  800 K nodes of degree 63, mean, 100 columns (2.4 x L2): register; 1.7 M nodes of degree 15 as well.
+// columns 4583 / 4243, 4971 / 4927, 5519 / 4792; GIN, whose few weighted edges are marked, in turn on one device 4239 / 4039,
+// 4874 / 4887, 5226 / 4739.  800 K nodes of degree 63, mean, 100 columns (2.4 x L2): register; 1.7 M nodes of degree 15 as well.  What the rule gives away: rows of equal length
+// and sources without hubs, X about as large as the L2 - 200,000 nodes of degree 160, 100 columns 898 / 1006, degree 96 523 / 571 -
+// where an R-MAT graph of the same size and degree takes 771 / 623; the two differ in nothing that n and |E| tell.
 bool tile_uses_bulk_copy(const gnnpre_plan* P, int32_t width) {
     const int32_t f4 = width / 4;
     if (P->op != GNNPRE_OP_SAGE_MEAN || (P->flags & GNNPRE_FLAG_NO_BULK_COPY) || f4 <= 16 || f4 >= 32) return false;

@@ -180,8 +180,9 @@ __device__ __forceinline__ void quad_kahan(Quad& sum, Quad& comp, const Quad& x)
     kahan_pair(sum.hi, comp.hi, x.hi);
 }
 
-// Programmatic dependent launch: the kernels of resident calls follow one another in a stream, and each is launched
-// while the last CTAs of the one before it still run.  What a kernel reads of the plan's own tables it may read at once;
+// Programmatic dependent launch: the kernels of resident calls follow one another in a stream, and each is launched when
+// the last CTA of the one before it has left, without waiting for that kernel's completion and the flush of its stores: what
+// is hidden is the latency of launch and completion.  What a kernel reads of the plan's own tables it may read at once;
 // wait_previous_kernel() comes before its first access to a matrix or to scratch rows and returns when the previous
 // kernel has completed and its stores are visible; every thread of every kernel passes it, so the guarantee carries
 // over to the kernels before that one.  It is a no-op in a kernel launched without the attribute, as the streamed

@@ -36,7 +36,7 @@
 #endif
 constexpr int kTmaStages = GNNPRE_TMA_STAGES;  // chunks a warp keeps in flight
 constexpr int kTmaRows = GNNPRE_TMA_ROWS;      // rows per stage = edges per chunk (8, 16 or 32)
-constexpr int kTmaStep = 8;                    // edges per plain-sum step (same as k_segments' U for G = 32, V = 1)
+constexpr int kTmaStep = 8;                    // edges per plain-sum step (k_segments' window)
 constexpr int kTmaMaxWarps = GNNPRE_TMA_WARPS;
 static_assert(kTmaRows % kTmaStep == 0 && kTmaRows % 4 == 0 && kTmaRows <= 32, "a chunk is a whole number of steps and fits one warp");
 // A poll that finds the phase incomplete lets the hardware park the warp for up to kTmaSuspendNs
