@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_ceiling(const SegArgs a, float*
     int left = 0;
     if (s < a.seg_hi) {
         entries += a.segs[s].start - a.colx_base;
-        left = (int)(a.segs[s + 1].start - a.segs[s].start);
+        left = a.segs[s].len;
     }
     const int q0 = blockIdx.y * a.tile_f4;
     const char* xlane = reinterpret_cast<const char*>(a.x + 4 * q0) + (gl < min(a.tile_f4, a.f4 - q0) ? 16 * gl : 0);
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
 
     const int64_t W = (int64_t)gridDim.x * nwarps;
     for (int64_t s = a.seg_lo + (int64_t)blockIdx.x * nwarps + warp; s < a.seg_hi && !failed; s += W) {
-        const int64_t e_beg = a.segs[s].start, e_end = a.segs[s + 1].start;
+        const int64_t e_beg = a.segs[s].start, e_end = e_beg + a.segs[s].len;
         const int nchunks = (int)((e_end - e_beg + kTmaRows - 1) / kTmaRows);
         uint32_t c_next = 0;
         if (lane < kTmaRows && e_beg + lane < e_end) c_next = a.colx[e_beg + lane - a.colx_base];

@@ -153,7 +153,7 @@ struct PinnedBuf {
 // Bit 31 of an entry of the plan's column array marks the last edge of its row.
 constexpr uint32_t kRowEndBit = 0x80000000u;
 
-// One warp-level segment: edges [start, next segment's start).  A segment never crosses an
+// One warp-level segment: `len` edges from `start` on, up to the next segment's start.  A segment never crosses an
 // edge-block boundary.  `rank` is the index, among rows that own at least one edge, of the row
 // holding the segment's first edge.  slot_head >= 0: that row began in an earlier segment, and
 // the part of it inside this segment goes to scratch row slot_head.  slot_tail >= 0: the row
@@ -164,7 +164,7 @@ struct Segment {
     int32_t rank;
     int32_t slot_head;
     int32_t slot_tail;
-    int32_t pad;
+    int32_t len;
 };
 
 // A row whose edges span segments seg_first..seg_last: its result is
@@ -226,6 +226,8 @@ struct gnnpre_plan {
     // decomposition
     std::vector<gnnpre::Block> blocks;
     gnnpre::DevBuf<gnnpre::Segment> segments;  // num_segments + 1 (the sentinel carries the end edge)
+    gnnpre::DevBuf<gnnpre::Segment> by_source;  // the same in the order a whole hop takes them; nullptr: as they are
+    gnnpre::DevBuf<int32_t> by_source_counts;
     gnnpre::DevBuf<gnnpre::RowFixup> fixups;
     gnnpre::DevBuf<int32_t> hubs;      // indices of the fix-ups with more than hub_parts parts, ascending
     int64_t num_hubs = 0;
@@ -295,6 +297,7 @@ int solve_budget(int64_t B_S, int64_t B_X, int64_t B_fixed, int64_t beta_S, int6
 int check_device();
 int check_device_error(gnnpre_plan* plan);  // synchronous read of plan->dev_error: GNNPRE_ERR_TIMEOUT if set
 bool uses_bulk_copy(const gnnpre_plan* plan, int32_t width);
+bool beyond_cache(const gnnpre_plan* plan, int32_t width);
 int64_t plan_budget(const gnnpre_plan* plan);
 
 }  // namespace gnnpre

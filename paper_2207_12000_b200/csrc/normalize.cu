@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) k_edge_values(const ValArgs a) {
     if (sg >= a.seg_hi) return;
     const int lane = threadIdx.x & 31;
     const int64_t start = a.segs[sg].start;
-    const int len = (int)(a.segs[sg + 1].start - start);
+    const int len = a.segs[sg].len;
     const uint32_t* entries = a.colx + (start - a.colx_base);
     float* out = a.out + (start - a.out_base);
     int rank = a.segs[sg].rank;

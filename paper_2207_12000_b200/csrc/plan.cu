@@ -313,7 +313,7 @@ __global__ void k_split_rows(int64_t n, const int32_t* __restrict__ flag, const 
 // short rows are never cut; long rows are cut and their parts summed by a fix-up.  Where no row of the graph is longer
 // than `uncut` edges the start always moves (two may then meet, or one the block's end: an empty segment), and nothing is
 // left for the finishing launch (see longest_uncut_row).
-// Until k_segment_finalize: slot_head holds the "first row began earlier" flag and pad the first row's index.
+// Until k_segment_finalize: slot_head holds the "first row began earlier" flag and len the first row's index.
 __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict__ seg_base,
                                  const int64_t* __restrict__ e_off, int32_t L, int32_t snap, int64_t uncut, const int* __restrict__ longest,
                                  const int64_t* __restrict__ rowptr_t, int64_t n, const int32_t* __restrict__ rank,
@@ -326,7 +326,7 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
         g.rank = 0;
         g.slot_head = 0;
         g.slot_tail = -1;
-        g.pad = (int32_t)n;
+        g.len = (int32_t)n;
         segs[s] = g;
         return;
     }
@@ -349,7 +349,7 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     g.rank = row == n ? 0 : rank ? rank[row] : (int32_t)row;
     g.slot_head = row < n && rowptr_t[row] < start;
     g.slot_tail = -1;
-    g.pad = (int32_t)row;
+    g.len = (int32_t)row;
     segs[s] = g;
 }
 
@@ -363,11 +363,11 @@ __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs,
     const Segment g = segs[s], nx = segs[s + 1];
     const int head = g.slot_head;
     // the row holding this segment's last edge continues iff the next segment's first row began earlier
-    const int tail = nx.slot_head && rowptr_t[nx.pad] >= g.start;
-    const int emit = head && rowptr_t[(int64_t)g.pad + 1] <= nx.start;
+    const int tail = nx.slot_head && rowptr_t[nx.len] >= g.start;
+    const int emit = head && rowptr_t[(int64_t)g.len + 1] <= nx.start;
     int hub = 0;
     if (emit) {
-        const int64_t first_edge = rowptr_t[g.pad];
+        const int64_t first_edge = rowptr_t[g.len];
         int64_t lo = 0, hi = s;  // segs[lo].start <= first_edge < segs[hi].start
         while (hi - lo > 1) {
             const int64_t mid = (lo + hi) >> 1;
@@ -389,7 +389,7 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
         const int head = segs[s].slot_head;
         if (c.fixups) {
             RowFixup f;
-            f.row = segs[s].pad;
+            f.row = segs[s].len;
             f.seg_first = first[s];
             f.seg_last = (int32_t)s;
             // the tail slot (the last slot) of the row's first segment; the other parts follow it
@@ -400,7 +400,43 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
         segs[s].slot_head = head ? b.slots : -1;
         segs[s].slot_tail = c.slots > head ? b.slots + head : -1;
     }
-    segs[s].pad = 0;
+    segs[s].len = s < nseg ? (int32_t)(segs[s + 1].start - segs[s].start) : 0;
+}
+
+// ---------------------------------------------------------------- the order in which a hop takes its segments
+
+// A hop over a matrix beyond the L2 reads most rows from memory, and in the order of the edge list every segment reads from all
+// of it.  But a row's columns ascend, so a segment that lies inside one row reads from a part of the matrix, the narrower the
+// longer the row - and most edges belong to long rows.  Taken in the order of their middle columns those segments sweep over
+// the matrix together, and the rows that they share are in the L2; the segments of several rows come last.  Every segment does
+// what it did, so the bits are the same.  us per hop, edge order / this: 2.4 M nodes, 124 M edges, mean operator, 100 columns
+// 3871 / 3637 (bulk copy), 4366 / 3870 (registers); GCN, 128 columns 4971 / 4295; sum, 64 columns 2417 / 2247; 16 columns
+// 1386 / 1378; 1 M nodes, 30 M edges, GCN, 128 columns 1072 / 1029; 400 K nodes, 40 M edges, sum, 256 columns 2200 / 2090;
+// about the L2's size: 300 K nodes, 40 M edges, GCN, 128 columns 1115 / 1068, 96 columns 997 / 990; well inside it: 169 K
+// nodes, 2.5 M edges, GCN, 128 columns 99 / 102.  Four or eight coarse ranges of columns instead: 3 to 6 % slower.
+constexpr int kOrderBuckets = 1024;  // by the middle column; one more for the segments of several rows and the empty ones
+
+__device__ __forceinline__ int order_bucket(const Segment* __restrict__ segs, int64_t s, int64_t nseg,
+                                            const uint32_t* __restrict__ colx, int64_t n) {
+    if (s + 1 >= nseg) return kOrderBuckets;
+    const Segment g = segs[s], nx = segs[s + 1];
+    const bool one_row = nx.rank == g.rank || (nx.rank == g.rank + 1 && nx.slot_head < 0);
+    if (g.len == 0 || !one_row) return kOrderBuckets;
+    return (int)((int64_t)(colx[g.start + g.len / 2] & ~kRowEndBit) * kOrderBuckets / n);
+}
+
+// SCATTER false: counts[b] = segments of bucket b.  true: counts[b] holds where the bucket begins; copies the segments there.
+template <bool SCATTER>
+__global__ void k_segment_order(int64_t nseg, const Segment* __restrict__ segs, const uint32_t* __restrict__ colx, int64_t n,
+                                int32_t* __restrict__ counts, Segment* __restrict__ ordered) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int bucket = s < nseg ? order_bucket(segs, s, nseg, colx, n) : -1;
+    const unsigned same = __match_any_sync(0xffffffffu, bucket);  // one addition per bucket and warp
+    const int lane = threadIdx.x & 31, first = __ffs(same) - 1;
+    int at = 0;
+    if (lane == first && bucket >= 0) at = atomicAdd(&counts[bucket], __popc(same));
+    at = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
+    if (SCATTER && bucket >= 0) ordered[at] = segs[s];
 }
 
 // Parts beyond which a cut row counts as a hub and gets a whole CTA of the finishing kernel (64 chains) instead of a
@@ -408,28 +444,30 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
 // how a matrix is cut into column tiles.
 constexpr int32_t kHubParts = 64;
 
-int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool whole_hops, int num_sms) {
+int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool beyond, bool whole_hops, int num_sms) {
     if (bulk_copy) {
-        // persistent warps walk whole segments with a two-stage pipeline that drains at every segment
-        // end: long segments, but at least ~4 per resident warp so the tail stays short
+        // persistent warps walk whole segments with a two-stage pipeline that drains at every segment end: long segments, but
+        // at least ~4 per resident warp so the tail stays short, and short enough that half the edges lie in segments of a
+        // single row (k_segment_order; 124 M edges, 100 columns, us per hop at 256 / 512 / 1024 / 2048 edges
+        // 3843 / 3651 / 3637 / 3745)
         const int64_t per_warp = m / ((int64_t)std::max(num_sms, 1) * 16 * 4);
         int32_t p = 256;
-        while ((int64_t)p * 2 <= per_warp && p < 4096) p *= 2;
+        while ((int64_t)p * 2 <= per_warp && p < 1024) p *= 2;
         return p;
     }
-    // Register kernel: segments long enough that few rows are cut, short enough that every lane group an SM holds (28
-    // warps) gets two (four or eight lanes per group) or three (wider) of them, up to 256 edges.  On 169 K nodes,
-    // 2.3 M edges, us per hop at 32 / 64 / 128 / 256 edges: 16 columns, mean 32 / 32 / 34 / 52; 32 columns, GCN
-    // 47 / 44 / 49 / 69; 64 columns 80 / 69 / 71 / 82; 128 columns 133 / 109 / 105 / 114.  Beyond 256 edges, up to 1024,
-    // only while eight segments per lane group remain (23 M edges, 128 columns: 829 / 744 / 702 us at 64 / 128 / 256, as
-    // fast at 1024; 12.8 M edges: 531 at 256, 583 at 1024): what longer segments save there is tables and scratch rows.
     const int64_t f4 = std::min<int64_t>(std::max<int64_t>(slab_width, 4), 128) / 4;
     const int64_t lanes = f4 <= 4 ? 4 : f4 <= 8 ? 8 : f4 <= 16 ? 16 : 32;
-    const int64_t per_group = m / ((int64_t)std::max(num_sms, 1) * (28 * 32 / lanes));
+    const int64_t per_group = m / ((int64_t)std::max(num_sms, 1) * (28 * 32 / lanes));  // lane groups the device holds at a time
+    // Register kernel: segments long enough that few rows are cut, short enough that every lane group gets two (four or eight lanes per
+    // group) or three (wider) of them, up to 256 edges.  Beyond 256 edges, up to 1024, only while eight segments per lane
+    // group remain (23 M edges, 128 columns: 829 / 744 / 702 us at 64 / 128 / 256, as fast at 1024; 12.8 M edges: 531 at 256,
+    // 583 at 1024): what longer segments save there is tables and scratch rows.  Up to 512 for a matrix beyond the L2, where
+    // segments of a single row are the better ones (124 M edges, 100 columns, at 128 / 256 / 512 / 1024 edges
+    // 4008 / 3898 / 3870 / 3950; GCN, 128 columns 4434 / 4331 / 4295).
     const int64_t L = std::max(std::min<int64_t>(per_group / (lanes <= 8 ? 2 : 3), 256), per_group / 8);
     // (a resident graph so small that segments of 16 all run at once gets those: its hop is a chain of latencies)
     int32_t p = whole_hops && (m / 16) * lanes <= (int64_t)num_sms * 768 ? 16 : 32;
-    while ((int64_t)p * 2 <= L && p < 1024) p *= 2;
+    while ((int64_t)p * 2 <= L && p < (beyond ? 512 : 1024)) p *= 2;
     return p;
 }
 
@@ -745,7 +783,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     P->segment_edges = opts->segment_edges > 0
                            ? opts->segment_edges
                            : auto_segment_edges(P->slab_width, m_launch, uses_bulk_copy(P, (int32_t)P->slab_width),
-                                                !per_block, P->num_sms);
+                                                beyond_cache(P, (int32_t)P->slab_width), !per_block, P->num_sms);
     if (P->segment_edges < 1) return GNNPRE_ERR_INVALID_ARG;
 
     // ---- block table: block l = edges [floor(l m / b), floor((l+1) m / b))
@@ -763,6 +801,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     if (nseg >= 0x3fffffffLL) return GNNPRE_ERR_INVALID_ARG;
     P->num_segments = nseg;
     const bool e_host = P->structure_mem == GNNPRE_MEM_HOST;
+    const bool by_source = !per_block && beyond_cache(P, (int32_t)P->slab_width);
 
     // ---- device memory: one allocation for what has a known size, one for what the segments turn out to need - or, if the
     // caller set no budget, nothing is streamed and what they can need at most is small, a single one.  (An allocation of a
@@ -783,6 +822,10 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         carve.want(P->rowptr_t, (size_t)n + 1);
         carve.want(P->segments, (size_t)nseg + 1);
         carve.want(P->dev_error, 1);
+        if (by_source) {
+            carve.want(P->by_source, (size_t)nseg);
+            carve.want(P->by_source_counts, 2 * (kOrderBuckets + 1) + 1);
+        }
         if (!e_host) carve.want(P->colx, (size_t)m);
     };
     Carve fixed;
@@ -967,6 +1010,17 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         int h = 0;
         GNNPRE_CUDA(cudaMemcpy(&h, P->dev_error.p, sizeof(int), cudaMemcpyDeviceToHost));  // everything is in place
         if (h) return GNNPRE_ERR_INVALID_CSR;
+    }
+    if (by_source) {
+        int32_t *counts = P->by_source_counts.p, *begins = counts + kOrderBuckets + 1;
+        GNNPRE_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * (kOrderBuckets + 1), st));
+        k_segment_order<false><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, n, counts, nullptr);
+        GNNPRE_CUDA(cudaGetLastError());
+        static_assert(kOrderBuckets + 1 <= kScanTile, "the scan needs no temporary memory");
+        GNNPRE_TRY(exclusive_scan<int32_t>(counts, kOrderBuckets + 1, begins, nullptr, st));
+        k_segment_order<true><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, n, begins, P->by_source.p);
+        GNNPRE_CUDA(cudaGetLastError());
+        GNNPRE_CUDA(cudaStreamSynchronize(st));
     }
 
     // ---- a host-resident structure keeps E in pinned memory and streams it block by block

@@ -223,6 +223,13 @@ int32_t segment_tile_width(const gnnpre_plan* P, int32_t width) {
 
 }  // namespace
 
+// Whether the rows that one segment launch over a slab of this width gathers from are more than the L2 holds (from some four
+// fifths of its size on it misses: see k_segment_order).
+bool beyond_cache(const gnnpre_plan* P, int32_t width) {
+    if (P->n * 512 <= l2_cache_bytes() * 4 / 5) return false;
+    return P->n * 4 * (int64_t)std::min(width, segment_tile_width(P, width)) > l2_cache_bytes() * 4 / 5;
+}
+
 // Whether a slab of this width is (mostly) summed by the bulk-copy kernel; the plan sizes its segments for it.
 bool uses_bulk_copy(const gnnpre_plan* P, int32_t width) {
     return tile_uses_bulk_copy(P, std::min(width, segment_tile_width(P, width)));
@@ -234,7 +241,7 @@ int launch_segments(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int6
     for (int32_t f0 = 0; f0 < h.width; f0 += tile) {
         const int32_t w = std::min<int32_t>(tile, h.width - f0);
         SegArgs a;
-        a.segs = P->segments.p;
+        a.segs = P->by_source.p && seg_hi - seg_lo == P->num_segments ? P->by_source.p : P->segments.p;
         a.seg_lo = seg_lo;
         a.seg_hi = seg_hi;
         a.colx = h.colx;
@@ -325,7 +332,7 @@ int launch_ceiling(const gnnpre_plan* P, const HopArgs& h, int64_t seg_lo, int64
     for (int32_t f0 = 0; f0 < h.width; f0 += tile) {
         const int32_t w = std::min<int32_t>(tile, h.width - f0);
         SegArgs a{};
-        a.segs = P->segments.p;
+        a.segs = P->by_source.p ? P->by_source.p : P->segments.p;
         a.seg_lo = seg_lo;
         a.seg_hi = seg_hi;
         a.colx = h.colx;

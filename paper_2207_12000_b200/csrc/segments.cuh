@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     if (s < a.seg_hi) {
         const Segment g = a.segs[s];
         entries += g.start - a.colx_base;
-        left = (int)(a.segs[s + 1].start - g.start);
+        left = g.len;
         rank = g.rank;
         slot_head = g.slot_head;
         slot_tail = g.slot_tail;

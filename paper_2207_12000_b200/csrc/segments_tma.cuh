@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kTmaMaxWarps * 32, 1)
     const int64_t W = (int64_t)gridDim.x * nwarps;
     for (int64_t s = a.seg_lo + (int64_t)blockIdx.x * nwarps + warp; s < a.seg_hi && !failed; s += W) {
         const Segment g = a.segs[s];
-        const int64_t e_beg = g.start, e_end = a.segs[s + 1].start;
+        const int64_t e_beg = g.start, e_end = g.start + g.len;
         const int nchunks = (int)((e_end - e_beg + kTmaRows - 1) / kTmaRows);
         int rank_issue = g.rank;
         // column entries of the chunk that will be issued next, fetched one chunk ahead

@@ -388,6 +388,26 @@ def test_bulk_copy_kernel_on_a_dense_graph_far_larger_than_the_cache(B, op, F):
 
 
 @pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("graph", ["hubs", "no hubs", "one row"])
+@pytest.mark.parametrize("F,seg", [(128, 32), (200, 200)])
+def test_segments_in_the_order_of_their_sources_give_the_same_bits(B, op, graph, F, seg):
+    """A whole hop over a matrix beyond the L2 takes its segments in the order of their columns, hops launched block by block in
+    that of the edge list: segments of one row, of several, empty ones, one segment only (the star's centre has all edges)."""
+    n = 300000
+    g = {"hubs": lambda: gi.rmat(n, 900000, 41, directed_candidates=False, device="cuda"), "no hubs": lambda: gi.erdos_renyi(n, 700000, 42, device="cuda"),
+         "one row": lambda: gi.from_edge_list(n, [(3, j) for j in range(5, 405)], device="cuda")}[graph]()
+    X = gi.normal_matrix(n, F, 43, device="cuda")
+    kw = dict(gin_eps=EPS, segment_edges=seg, force_blocks=1, force_col_slabs=1)
+    a = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, **kw)
+    b = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, flags=B.GNNPRE_FLAG_LAUNCH_PER_BLOCK, **kw)
+    assert a.info()["num_segments"] == b.info()["num_segments"] and a.info()["device_bytes"] > b.info()["device_bytes"]
+    for x, y in zip(B.gnnpre_propagate(a, X, 2)[0], B.gnnpre_propagate(b, X, 2)[0]):
+        assert torch.equal(x, y)
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132, 260])
 @pytest.mark.parametrize("seg", [1, 7, 8, 9, 31, 33])
 def test_register_kernel_tile_and_segment_edges(B, op, F, seg):
