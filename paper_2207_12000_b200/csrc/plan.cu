@@ -457,16 +457,29 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool b
     }
     const int64_t f4 = std::min<int64_t>(std::max<int64_t>(slab_width, 4), 128) / 4;
     const int64_t lanes = f4 <= 4 ? 4 : f4 <= 8 ? 8 : f4 <= 16 ? 16 : 32;
-    const int64_t per_group = m / ((int64_t)std::max(num_sms, 1) * (28 * 32 / lanes));  // lane groups the device holds at a time
-    // Register kernel: segments long enough that few rows are cut, short enough that every lane group gets two (four or eight lanes per
+    const int64_t groups = (int64_t)std::max(num_sms, 1) * (28 * 32 / lanes);  // lane groups the device holds at a time
+    const int64_t per_group = m / groups;
+    // Register kernel, a hop of few waves over a matrix that the L2 holds: a last wave that is nearly empty costs as much as a
+    // full one, so segments are as long as makes the waves whole - one wave while that leaves them even enough.  us per hop at
+    // segments of a power of two (two or three per group) / so, R-MAT graphs, mean operator: 600,000 edges, 16 columns
+    // 12.4 / 12.2, 32 15.4 / 13.6, 64 20.7 / 17.7, 128 31.1 / 24.7; 1.2 M 20.8 / 18.2, 24.2 / 21.3, 34.8 / 31.2, 47.9 / 45.0;
+    // 2.4 M, 16 columns 34.2 / 31.0, 32 39.4 / 36.1, 64 61.0 / 59.5; 4.8 M 58.2 / 52.5, 71.0 / 64.4; 10 M 108.0 / 102.6 (two
+    // waves; 105.4 in one), 132.3 / 126.3; 24 M, 16 columns 209 / 198 (four).  64 columns stay at 96 edges: beside the rows of
+    // a sum of hops long segments are uneven (2.4 M edges, ten hops 1155 at 80 edges, 1241 in one wave), and 128 columns of
+    // 2.4 M edges in four waves take 1 % less, but 1.5 % more with a teleport term.
+    if (whole_hops && !beyond && slab_width <= 128) {
+        const int64_t most = lanes == 4 ? 192 : lanes == 16 ? 96 : 320, waves = per_group / most + 1;
+        const int64_t whole = waves <= (lanes == 32 ? 1 : lanes == 8 ? 2 : 4) ? waves : 0;
+        if (whole > 0) return (int32_t)std::max<int64_t>(16, (m / (groups * whole) + 8) / 8 * 8);
+    }
+    // Else segments long enough that few rows are cut, short enough that every lane group gets two (four or eight lanes per
     // group) or three (wider) of them, up to 256 edges.  Beyond 256 edges, up to 1024, only while eight segments per lane
     // group remain (23 M edges, 128 columns: 829 / 744 / 702 us at 64 / 128 / 256, as fast at 1024; 12.8 M edges: 531 at 256,
     // 583 at 1024): what longer segments save there is tables and scratch rows.  Up to 512 for a matrix beyond the L2, where
     // segments of a single row are the better ones (124 M edges, 100 columns, at 128 / 256 / 512 / 1024 edges
     // 4008 / 3898 / 3870 / 3950; GCN, 128 columns 4434 / 4331 / 4295).
     const int64_t L = std::max(std::min<int64_t>(per_group / (lanes <= 8 ? 2 : 3), 256), per_group / 8);
-    // (a resident graph so small that segments of 16 all run at once gets those: its hop is a chain of latencies)
-    int32_t p = whole_hops && (m / 16) * lanes <= (int64_t)num_sms * 768 ? 16 : 32;
+    int32_t p = 32;
     while ((int64_t)p * 2 <= L && p < (beyond ? 512 : 1024)) p *= 2;
     return p;
 }
@@ -480,13 +493,16 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool b
 //                            31 / 36, 38 / 38, 40 / 34, 40 / 36; 128 columns 36 / 43, 37 / 49, 42 / 45, 36 / 45
 //   4 million, L = 64:       16 columns, 1.6 L 51 / 64, 2 L 60 / 51; 32 columns, 1.6 L 69 / 77, 1.8 L 76 / 72; 64 columns,
 //                            1.5 L 99 / 104, 1.8 L 128 / 104; 128 columns, 1.8 L 126 / 151, 2 L 155 / 143, 2.4 L 127 / 142
+//   whole waves:             16 columns, 2.4 M edges, L = 80, 1.8 L 26 / 30, 2.2 L 30 / 28; 4.8 M, L = 152, 1.5 L 42 / 48,
+//                            1.8 L 50 / 51; 32 columns, 1.2 M, L = 80, 1.8 L 19 / 21, 2.2 L 22 / 19; 2.4 M, L = 152,
+//                            1.5 L 31 / 35, 1.8 L 37 / 34; 64 columns, 600,000, L = 80, 1.5 L 15 / 17, 1.8 L 19 / 16
 //   20 million, L = 256:     16 columns, 1.25 L 177 / 185, 1.5 L 233 / 219, 2 L 290 / 160; 64 columns, 1.25 L 325 / 332,
 //                            1.4 L 391 / 365, 2 L 645 / 302; 128 columns, 1.8 L 529 / 566, 2 L 694 / 538, 2.9 L 549 / 536
 int64_t longest_uncut_row(int64_t m, int64_t lanes, int64_t L, bool one_wave) {
     const int64_t work = m * lanes;
     if (one_wave) return 3 * L;
     if (lanes == 32) return work <= (1 << 28) ? 3 * L : 2 * L;
-    return work <= (1 << 25) ? 2 * L : work <= (1 << 26) ? 3 * L / 2 : 5 * L / 4;
+    return work <= (lanes == 16 ? 1 << 23 : 1 << 24) ? 2 * L : work <= (1 << 26) ? 3 * L / 2 : 5 * L / 4;
 }
 
 }  // namespace

@@ -408,6 +408,23 @@ def test_segments_in_the_order_of_their_sources_give_the_same_bits(B, op, graph,
 
 
 @pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("F", [16, 32, 64, 128])
+@pytest.mark.parametrize("m", [3000, 80000, 330000])
+def test_segments_of_a_small_graph_fill_whole_waves(B, op, F, m):
+    g = gi.rmat(m // 8, m, 44, directed_candidates=True)
+    X = gi.normal_matrix(g.n, F, 45)
+    plan = B.gnnpre_build_plan(*dev(g), op, F, gin_eps=EPS)
+    info = plan.info()
+    groups = torch.cuda.get_device_properties(0).multi_processor_count * 28 * 32 // max(4, F // 4)
+    waves = -(-info["num_segments"] // groups)
+    # the next shorter segments (of whole windows of 8 edges) would need another wave, or are below the least
+    assert info["segment_edges"] == 16 or info["nnz_tilde"] > groups * waves * (info["segment_edges"] - 8)
+    outs, _ = B.gnnpre_propagate(plan, X.cuda(), 2)
+    check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), X.numpy(), outs, single_hop=single_hop_of(B, plan))
+    plan.close()
+
+
+@pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132, 260])
 @pytest.mark.parametrize("seg", [1, 7, 8, 9, 31, 33])
 def test_register_kernel_tile_and_segment_edges(B, op, F, seg):
