@@ -462,14 +462,14 @@ int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool b
     // Register kernel, a hop of few waves over a matrix that the L2 holds: a last wave that is nearly empty costs as much as a
     // full one, so segments are as long as makes the waves whole - one wave while that leaves them even enough.  us per hop at
     // segments of a power of two (two or three per group) / so, R-MAT graphs, mean operator: 600,000 edges, 16 columns
-    // 12.4 / 12.2, 32 15.4 / 13.6, 64 20.7 / 17.7, 128 31.1 / 24.7; 1.2 M 20.8 / 18.2, 24.2 / 21.3, 34.8 / 31.2, 47.9 / 45.0;
-    // 2.4 M, 16 columns 34.2 / 31.0, 32 39.4 / 36.1, 64 61.0 / 59.5; 4.8 M 58.2 / 52.5, 71.0 / 64.4; 10 M 108.0 / 102.6 (two
-    // waves; 105.4 in one), 132.3 / 126.3; 24 M, 16 columns 209 / 198 (four).  64 columns stay at 96 edges: beside the rows of
-    // a sum of hops long segments are uneven (2.4 M edges, ten hops 1155 at 80 edges, 1241 in one wave), and 128 columns of
-    // 2.4 M edges in four waves take 1 % less, but 1.5 % more with a teleport term.
+    // 12.4 / 12.2, 32 15.4 / 13.6, 64 20.7 / 17.7, 128 31.1 / 24.7; 1.2 M 20.8 / 18.2, 24.2 / 21.3, 34.8 / 31.2; 2.4 M
+    // 34.2 / 31.0, 39.4 / 36.1, 61.0 / 59.5; 4.8 M, 16 columns 58.2 / 52.5, 32 71.0 / 67.6 (two waves); 10 M 108.0 / 102.6 (two),
+    // 132.3 / 125.8 (four); 24 M, 16 columns 209 / 198 (four).  Where the epilogue reads rows too, long segments are uneven: 64
+    // columns, 2.4 M edges, ten hops with a teleport term and their sum 1155 at 80 edges, 1241 in one wave; 128 columns, 1.2 M
+    // edges 843 at 64, 888 at 160, and without the epilogue 170 / 162; so those stay at 96 edges, and at one wave of 160.
     if (whole_hops && !beyond && slab_width <= 128) {
-        const int64_t most = lanes == 4 ? 192 : lanes == 16 ? 96 : 320, waves = per_group / most + 1;
-        const int64_t whole = waves <= (lanes == 32 ? 1 : lanes == 8 ? 2 : 4) ? waves : 0;
+        const int64_t most = lanes == 4 ? 192 : lanes == 16 ? 96 : 160, waves = per_group / most + 1;
+        const int64_t whole = waves <= (lanes == 32 ? 1 : 4) ? waves : 0;
         if (whole > 0) return (int32_t)std::max<int64_t>(16, (m / (groups * whole) + 8) / 8 * 8);
     }
     // Else segments long enough that few rows are cut, short enough that every lane group gets two (four or eight lanes per
