@@ -24,17 +24,27 @@
 // each slower.
 constexpr int kSegWindow = 8;
 
-struct __align__(16) RowOut {
+// What a sum needs when its row ends.  Shared memory is set aside in steps of 8, 16, 32, 64 KB an SM and the L1 gets the rest of
+// 256: with 8 bytes a row instead of 16 the plain kernels of whole warps stay within 32 KB, and those of four lanes store less
+// per chunk; the address is worked out at the row's end instead.  us a call, 16 / 8 bytes: 233 K nodes, 602 columns, GCN
+// 7613 / 7447; 89 K nodes, 500 columns, with its plan 692 / 680; 169 K nodes, GCN, 128 columns 311.4 / 308.2, 16 columns
+// 113.8 / 108.5, mean operator, 100 columns 253.8 / 249.8, 16 columns 88.3 / 85.9.  Groups of 8 and 16 lanes and the wide
+// kernels with an epilogue have no registers left for that (GCN, 64 columns 210 / 225).
+struct __align__(16) RowOutLong {
     char* dst;    // first byte of this column tile in the row the sum goes to
     float scale;  // r_i; 1 for a scratch row
     int row;      // output row; -1 for a scratch row (no epilogue)
+};
+struct __align__(8) RowOutShort {
+    float scale;
+    int row;  // output row; ~slot for scratch row `slot`
 };
 
 // A shared-memory load returns its bytes to every lane, 128 bytes per cycle and SM, as a row's 512 do: entry and weight of
 // an edge cost a cycle each beside the row's four.  Groups of 32 lanes therefore keep weights as single floats (169 K nodes,
 // GCN, 128 columns: 102.7 us per launch with weights stored twice, 97.3 so); narrower groups, where the instructions
 // count, as pairs ready for the packed multiply-add (64 columns: 66.0 us, 72.8 with single floats).
-template <int G, bool WEIGHTED>
+template <int G, bool WEIGHTED, typename RowOut>
 struct __align__(16) SegStage {  // read in 16-byte pieces
     static constexpr int kChunk = G < kSegWindow ? kSegWindow : G;  // edges staged at a time
     static constexpr bool kPairs = G < 32;
@@ -79,7 +89,9 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     // and the piece in shared memory: 3144, 100).
     constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16 && EP != kEpTeleport;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN && !kDiagonal;
-    using Stage = SegStage<G, kWeighted>;
+    constexpr bool kShort = G == 4 || (G == 32 && EP == kEpPlain);
+    using RowOut = std::conditional_t<kShort, RowOutShort, RowOutLong>;
+    using Stage = SegStage<G, kWeighted, RowOut>;
     constexpr int C = Stage::kChunk;
     constexpr int M = C / G;  // entries per lane and chunk
     __shared__ __align__(16) Stage stages[kSegThreads / G];
@@ -166,9 +178,11 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             if (OP == GNNPRE_OP_GIN_SUM && kWeighted)
                 w[m] = (int)col == rank + __popc(ends & ((1u << i) - 1u)) ? a.diag_weight : 1.f;
             RowOut o;
-            o.dst = reinterpret_cast<char*>(slot >= 0 ? a.scratch + (int64_t)slot * a.scratch_ld : a.out + (int64_t)row[m] * a.ldo) + 16 * q0;
+            if constexpr (!kShort)
+                o.dst = reinterpret_cast<char*>(slot >= 0 ? a.scratch + (int64_t)slot * a.scratch_ld : a.out + (int64_t)row[m] * a.ldo) + 16 * q0;
             o.scale = slot >= 0 ? 1.f : scale[m];
-            o.row = slot >= 0 ? -1 : row[m];
+            if constexpr (kShort) o.row = slot >= 0 ? ~slot : row[m];
+            else o.row = slot >= 0 ? -1 : row[m];
             stage.out[i] = o;
         }
         if (ends != 0) slot_head = -1;
@@ -199,7 +213,13 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
                 if (EP == kEpSum && o.row < 0) wait_copies_ahead();  // no epilogue, but the next row's copies go to the same place
                 if (EP == kEpPlain || o.row < 0) v = make_float4(v.x * o.scale, v.y * o.scale, v.z * o.scale, v.w * o.scale);
                 else v = piece.finish(v, o.scale, a.tp, o.row, 4 * q0, gl);
-                *reinterpret_cast<float4*>(o.dst + out_off) = v;
+                if constexpr (kShort) {
+                    char* const dst = o.row >= 0 ? reinterpret_cast<char*>(a.out + (int64_t)o.row * a.ldo) + 16 * q0
+                                                 : reinterpret_cast<char*>(a.scratch + (int64_t)~o.row * a.scratch_ld) + 16 * q0;
+                    *reinterpret_cast<float4*>(dst + out_off) = v;
+                } else {
+                    *reinterpret_cast<float4*>(o.dst + out_off) = v;
+                }
             }
             acc = tot = cmp = quad_zero();
             asked = out < stage.out + C;
