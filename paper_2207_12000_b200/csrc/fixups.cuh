@@ -51,7 +51,11 @@ __device__ __forceinline__ void pair_add4(float4& s, float4& e, const float4& t,
 //     sums meet in shared memory and warp 0 adds them in warp order.
 // The first (hub_hi - hub_lo) CTAs of the grid take the hubs, the next ones eight ordinary rows each, the rest the
 // rows without edges (zero, or alpha * X_0[i] with a teleport term), kEmptyPerGroup to a lane group.
-// Bound by latency: two dependent loads per row, and most rows have two or three parts.  A lane keeps at most eight
+// Bound by latency: two dependent loads per row, and most rows have two or three parts.  So a row whose chains have one part
+// each skips the compensated sums (of one part they are that part), and the longer ones are summed four chains at a time: what
+// a lane holds stays small, three CTAs an SM for 64 columns instead of two (169 K nodes, us a call before / now: GCN, three
+// hops 210.3 / 205.6; ten hops with a teleport term and their sum 1146 / 1124; 89 K nodes, 500 columns, with its plan 692 / 687;
+// 128 columns alike: a third CTA spills there and gains nothing, 253.8 / 255.0 for 100 columns).  A lane keeps at most eight
 // parts in flight (with sixteen the kernel held 98 to 174 registers and ran narrow rows in five waves), and the row's
 // place and scale are fetched while the segment kernel completes.  169 K nodes, 16 columns, mean operator, three
 // hops: 146 -> 100 us a call (three launches per hop before, each after the end of the one before it).
@@ -60,13 +64,16 @@ __device__ __forceinline__ void pair_add4(float4& s, float4& e, const float4& t,
 constexpr int kEmptyPerGroup = 16, kEmptyAhead = 4;
 
 template <int G, int EP>
-__global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
+constexpr int kFinishBlocks = G == 32 ? 2 : G == 16 || EP == kEpSum ? 3 : 4;
+
+template <int G, int EP>
+__global__ void __launch_bounds__(kThreads, kFinishBlocks<G, EP>) k_finish_rows(const FixArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
     constexpr int kWarps = kThreads / 32;
     constexpr int S = 32 / G;                         // lane groups per warp
     constexpr int CH = G / 4;                         // chains per lane
     constexpr int CW = S * CH;                        // chains per warp
-    constexpr int kRounds = CH >= 8 ? 1 : CH >= 4 ? 2 : 4;  // parts in flight per chain
+    constexpr int kAtOnce = CH < 4 ? CH : 4, kRounds = CH >= 4 ? 2 : 4;  // chains summed at a time, parts in flight of each
     static_assert(CW == 8, "the tree's shape must not depend on the width");
     __shared__ float4 meet[kWarps][2][G];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -116,39 +123,62 @@ __global__ void __launch_bounds__(kThreads) k_finish_rows(const FixArgs a) {
     if (!mine) parts = 0;
     wait_previous_kernel();
 
-    float4 acc[CH], cmp[CH];
-#pragma unroll
-    for (int j = 0; j < CH; ++j) acc[j] = cmp[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int p0 = 0; p0 < parts; p0 += chains * kRounds) {
-        float4 part[kRounds][CH];
-#pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const int p = p0 + r * chains + chain0 + j;
-                part[r][j] = p < parts ? *reinterpret_cast<const float4*>(base + (int64_t)p * a.scratch_ld)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-#pragma unroll
-            for (int j = 0; j < CH; ++j)
-                if (p0 + r * chains + chain0 + j < parts) kahan4(acc[j], cmp[j], part[r][j]);
-        }
-    }
+    auto part_at = [&](int p) {
+        return p < parts ? *reinterpret_cast<const float4*>(base + (int64_t)p * a.scratch_ld) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
     // The chains meet pairwise, first inside the lane (chains chain0 .. chain0 + CH - 1), then across the lane
     // groups of the warp.  A hub's partial sums can be far larger than their total (40,000 terms of either sign), so
     // every sum travels as a pair (value, error term) and each pairwise addition keeps its exact rounding error.
+    float4 tot, err;
+    if (parts <= chains) {  // most rows: no chain has more than one part
+        float4 one[CH], none[CH];
 #pragma unroll
-    for (int j = 0; j < CH; ++j)  // a compensated sum stands for acc - cmp
-        cmp[j] = make_float4(-cmp[j].x, -cmp[j].y, -cmp[j].z, -cmp[j].w);
+        for (int j = 0; j < CH; ++j) one[j] = part_at(chain0 + j);
 #pragma unroll
-    for (int step = 1; step < CH; step <<= 1) {
+        for (int j = 0; j < CH; ++j) none[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < CH; j += 2 * step) pair_add4(acc[j], cmp[j], acc[j + step], cmp[j + step]);
+        for (int step = 1; step < CH; step <<= 1) {
+#pragma unroll
+            for (int j = 0; j < CH; j += 2 * step) pair_add4(one[j], none[j], one[j + step], none[j + step]);
+        }
+        tot = one[0];
+        err = none[0];
+    } else {
+#pragma unroll 1
+        for (int j0 = 0; j0 < CH; j0 += kAtOnce) {
+            float4 acc[kAtOnce], cmp[kAtOnce];
+#pragma unroll
+            for (int j = 0; j < kAtOnce; ++j) acc[j] = cmp[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int p0 = chain0 + j0; p0 < parts; p0 += chains * kRounds) {
+                float4 part[kRounds][kAtOnce];
+#pragma unroll
+                for (int r = 0; r < kRounds; ++r) {
+#pragma unroll
+                    for (int j = 0; j < kAtOnce; ++j) part[r][j] = part_at(p0 + r * chains + j);
+                }
+#pragma unroll
+                for (int r = 0; r < kRounds; ++r) {
+#pragma unroll
+                    for (int j = 0; j < kAtOnce; ++j)
+                        if (p0 + r * chains + j < parts) kahan4(acc[j], cmp[j], part[r][j]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kAtOnce; ++j)  // a compensated sum stands for acc - cmp
+                cmp[j] = make_float4(-cmp[j].x, -cmp[j].y, -cmp[j].z, -cmp[j].w);
+#pragma unroll
+            for (int step = 1; step < kAtOnce; step <<= 1) {
+#pragma unroll
+                for (int j = 0; j < kAtOnce; j += 2 * step) pair_add4(acc[j], cmp[j], acc[j + step], cmp[j + step]);
+            }
+            if (j0 == 0) {
+                tot = acc[0];
+                err = cmp[0];
+            } else {
+                pair_add4(tot, err, acc[0], cmp[0]);
+            }
+        }
     }
-    float4 tot = acc[0], err = cmp[0];
 #pragma unroll
     for (int off = G; off < 32; off <<= 1) {
         float4 os, oe;
