@@ -24,7 +24,7 @@ inline unsigned grid_for(int64_t items, int per_block) {
 
 // ---------------------------------------------------------------- rows: pointers, degrees, scales
 
-enum : int { kErrRowptr = 1, kErrColRange = 2, kErrDiagonal = 4, kErrOrder = 8, kErrDegree = 16 };
+enum : int { kErrRowptr = 1, kErrColRange = 2, kErrDiagonal = 4, kErrOrder = 8, kErrDegree = 16, kErrRows = kErrRowptr | kErrDegree };
 
 // One thread per row.  Checks the row pointers; D_i = number of nonzeros in row i of A (Section 2) unless the caller
 // gave the degrees; A^_ij = r_i c_j: GCN r = c = (D_i + 1)^{-1/2} (Eq. 1); SAGE r = 1/D_i (0 for D_i = 0), c = 1;
@@ -92,14 +92,15 @@ __device__ __forceinline__ int64_t row_of_edge_warp(const int64_t* __restrict__ 
 }
 
 // Copies the edge list into the support: entry (row, col) with its row-end mark, self-loops (with `diag`) inserted at
-// their column-sorted position, and checks the contract of colidx on the way (`check`).  The row pointers have been
-// checked.  A warp takes `per_warp` consecutive edges whatever rows they belong to - a warp per row took 148 us for
+// their column-sorted position, and checks the contract of colidx on the way (`check`).  Row pointers that k_rows found
+// bad (*err) are left alone.  A warp takes `per_warp` consecutive edges whatever rows they belong to - a warp per row took 148 us for
 // 1.8 M edges because one row holds 20,000 of them, and the check a pass of its own (54 us) - and finds the rows of 32
 // edges from the next 32 row pointers.  The last blocks, one thread per row, write the self-loops of rows without edges.
 __global__ void k_support(int diag, int check, int64_t n, int64_t nnz, int64_t per_warp, int64_t edge_blocks,
                           const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
                           uint32_t* __restrict__ colx, int* err) {
     constexpr unsigned kFull = 0xffffffffu;
+    if (*(volatile int*)err & kErrRows) return;
     if ((int64_t)blockIdx.x >= edge_blocks) {
         const int64_t i = ((int64_t)blockIdx.x - edge_blocks) * blockDim.x + threadIdx.x;
         if (i < n) {
@@ -266,29 +267,25 @@ struct BlockRows {
     int64_t done_row_hi;
 };
 
-// Thread l <= b: block l's rows (l < b), and what the segments before the block account for.
+// Warp l <= b: block l's rows (l < b), and what the segments before the block account for.
 __global__ void k_block_report(int b, const int64_t* __restrict__ e_off, const int64_t* __restrict__ seg_base,
                                const SegCounts* __restrict__ before, const int64_t* __restrict__ rowptr_t, int64_t n,
                                BlockRows* __restrict__ rows, SegCounts* __restrict__ at) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (l > b) return;
-    at[l] = before[seg_base[l]];
+    if (lane == 0) at[l] = before[seg_base[l]];
     if (l == b) return;
     const int64_t lo = e_off[l], hi = e_off[l + 1];
-    const int64_t r0 = row_of_edge(rowptr_t, n, lo), r1 = row_of_edge(rowptr_t, n, hi - 1);
+    const int64_t r0 = row_of_edge_warp(rowptr_t, n, lo, lane), r1 = row_of_edge_warp(rowptr_t, n, hi - 1, lane);
     BlockRows o;
     o.row_lo = (int32_t)r0;
     o.row_hi = (int32_t)r1;
     o.first_partial = rowptr_t[r0] < lo;
     o.last_partial = rowptr_t[r1 + 1] > hi;
-    // rows complete after this block: every row whose end offset is <= hi
-    int64_t a = 0, z = n;  // count of i in [0, n) with rowptr_t[i + 1] <= hi
-    while (a < z) {
-        const int64_t mid = (a + z) >> 1;
-        if (rowptr_t[mid + 1] <= hi) a = mid + 1; else z = mid;
-    }
-    o.done_row_hi = a;
-    rows[l] = o;
+    // rows complete after this block, i.e. whose end offset is <= hi: those before the row of the next block's first edge
+    // (all but those behind the last edge are found so; the last block is the host's)
+    o.done_row_hi = hi < rowptr_t[n] ? row_of_edge_warp(rowptr_t, n, hi, lane) : n;
+    if (lane == 0) rows[l] = o;
 }
 
 // ---------------------------------------------------------------- rows with and without edges
@@ -342,7 +339,8 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
         const int64_t next = rowptr_t[row + 1];
         if ((next - start <= snap || *longest < uncut) && next <= e_off[lo + 1]) {
             start = next;
-            row = start < e_off[b] ? row_of_edge(rowptr_t, n, start) : n;  // at the very end: empty, as the sentinel
+            // at the very end: empty, as the sentinel
+            row = start >= e_off[b] ? n : row + 2 <= n && rowptr_t[row + 2] > start ? row + 1 : row_of_edge(rowptr_t, n, start);
         }
     }
     g.start = start;
@@ -368,7 +366,11 @@ __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs,
     int hub = 0;
     if (emit) {
         const int64_t first_edge = rowptr_t[g.len];
-        int64_t lo = 0, hi = s;  // segs[lo].start <= first_edge < segs[hi].start
+        int64_t lo = max(s - 1, (int64_t)0), hi = s;  // segs[lo].start <= first_edge < segs[hi].start, most often the segment before
+        for (int64_t back = 2; lo > 0 && segs[lo].start > first_edge; back *= 2) {
+            hi = lo;
+            lo = max(lo - back, (int64_t)0);
+        }
         while (hi - lo > 1) {
             const int64_t mid = (lo + hi) >> 1;
             if (segs[mid].start <= first_edge) lo = mid; else hi = mid;
@@ -381,9 +383,9 @@ __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs,
 
 __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, const SegCounts* __restrict__ counts,
                                    const SegCounts* __restrict__ before, const int32_t* __restrict__ first,
-                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs) {
+                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs, const int* err) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s > nseg) return;
+    if (s > nseg || *err) return;
     if (s < nseg) {
         const SegCounts c = counts[s], b = before[s];
         const int head = segs[s].slot_head;
@@ -828,9 +830,12 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         int32_t err, nonempty, longest_row, unused;
     };
     static_assert(sizeof(Report) == 16 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
+    // (the report has a place of its own: E overwrites the temporaries before the host reads it)
+    DevBuf<char> report;
     const size_t report_bytes = sizeof(Report) + sizeof(BlockRows) * (size_t)b + sizeof(SegCounts) * (size_t)(b + 1);
     DevBuf<uint32_t> e_temp;
     DevBuf<uint32_t>& colx = e_host ? e_temp : P->colx;  // E of a host-resident structure is on the device for the build only
+    const bool small_report = b <= 4096;
     auto want_fixed = [&](Carve& carve) {
         carve.want(P->deg, (size_t)n);
         carve.want(P->rscale, (size_t)n);
@@ -838,6 +843,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         carve.want(P->rowptr_t, (size_t)n + 1);
         carve.want(P->segments, (size_t)nseg + 1);
         carve.want(P->dev_error, 1);
+        if (small_report) carve.want(report, report_bytes);
         if (by_source) {
             carve.want(P->by_source, (size_t)nseg);
             carve.want(P->by_source_counts, 2 * (kOrderBuckets + 1) + 1);
@@ -883,12 +889,12 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     }
     GNNPRE_TRY(placed);
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
-    DevBuf<char> temp_arena, report;
+    DevBuf<char> temp_arena;
+    if (!small_report) GNNPRE_TRY(report.alloc(report_bytes));
     DevBuf<int32_t> flag, rank, rank_temp, first;
     DevBuf<SegCounts> counts, before, counts_temp;
     DevBuf<int64_t> offsets;
     Carve temps;
-    temps.want(report, report_bytes);
     temps.want(offsets, 2 * ((size_t)b + 1));
     if (!diag) {
         temps.want(flag, (size_t)n);
@@ -957,29 +963,39 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);
         GNNPRE_CUDA(cudaGetLastError());
         GNNPRE_TRY(exclusive_scan(counts.p, nseg, before.p, counts_temp.p, st));
-        k_block_report<<<grid_for(b + 1, kTB), kTB, 0, st>>>((int)b, d_e_off, d_seg_base, before.p, P->rowptr_t.p, n, d_rows, d_at);
+        k_block_report<<<grid_for(b + 1, kTB / 32), kTB, 0, st>>>((int)b, d_e_off, d_seg_base, before.p, P->rowptr_t.p, n, d_rows, d_at);
         GNNPRE_CUDA(cudaGetLastError());
     }
+    // What follows needs nothing that only the device knows yet if all tables have room for the most: then the host looks once,
+    // at the end, instead of waiting here as well (with the searches above by warps and by short steps, us for plan, hops and
+    // release, before / now: 89 K nodes, 1.9 M edges, 500 columns, GCN, two hops 680 / 651; 64 columns, mean operator 241 / 213).
     std::vector<int64_t> h_report((report_bytes + 7) / 8);
-    GNNPRE_CUDA(cudaMemcpy(h_report.data(), report.p, report_bytes, cudaMemcpyDeviceToHost));
     const Report* rep = reinterpret_cast<const Report*>(h_report.data());
     const BlockRows* h_rows = reinterpret_cast<const BlockRows*>(rep + 1);
     const SegCounts* at = reinterpret_cast<const SegCounts*>(h_rows + b);
-    if (rep->err) return GNNPRE_ERR_INVALID_CSR;
-    P->num_nonempty = diag ? n : rep->nonempty;
-    P->num_empty = n - P->num_nonempty;
-    P->rows_all_nonempty = P->num_empty == 0;
-    if (m > 0) {
-        P->num_slots = at[b].slots;
-        P->num_fixups = at[b].fixups;
-        P->num_hubs = at[b].hubs;
+    auto read_report = [&]() -> int {
+        GNNPRE_CUDA(cudaMemcpy(h_report.data(), report.p, report_bytes, cudaMemcpyDeviceToHost));
+        if (rep->err) return GNNPRE_ERR_INVALID_CSR;
+        P->num_nonempty = diag ? n : rep->nonempty;
+        P->num_empty = n - P->num_nonempty;
+        P->rows_all_nonempty = P->num_empty == 0;
+        if (m > 0) {
+            P->num_slots = at[b].slots;
+            P->num_fixups = at[b].fixups;
+            P->num_hubs = at[b].hubs;
+        }
+        return GNNPRE_OK;
+    };
+    const bool look_once = one_allocation && m > 0;
+    if (!look_once) {
+        GNNPRE_TRY(read_report());
+        if (!one_allocation) {
+            Carve sized;
+            want_sized(sized, P->num_fixups, P->num_hubs, P->num_nonempty, P->num_empty, P->num_slots);
+            GNNPRE_TRY(sized.place(P->arena[1]));
+        }
     }
-    if (!one_allocation) {
-        Carve sized;
-        want_sized(sized, P->num_fixups, P->num_hubs, P->num_nonempty, P->num_empty, P->num_slots);
-        GNNPRE_TRY(sized.place(P->arena[1]));
-    }
-    if (!P->rows_all_nonempty) {
+    if (look_once ? !diag : !P->rows_all_nonempty) {
         k_split_rows<<<grid_for(n, kTB), kTB, 0, st>>>(n, flag.p, rank.p, P->rscale.p, P->nzrows.p, P->nzscale.p, P->emptyrows.p);
         GNNPRE_CUDA(cudaGetLastError());
     }
@@ -991,8 +1007,21 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         return GNNPRE_OK;
     }
     k_segment_finalize<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, P->segments.p, counts.p, before.p, first.p, P->fixups.p,
-                                                                P->hubs.p);
+                                                                P->hubs.p, &d_report->err);
     GNNPRE_CUDA(cudaGetLastError());
+
+    // ---- E, the support's edge list: overwrites the temporaries
+    {
+        const bool check = !(opts->flags & GNNPRE_FLAG_SKIP_VALIDATION);
+        // 256 edges per warp, more (up to 2048) only while every warp the device holds still gets its share
+        const int64_t per_warp = 256 * std::min<int64_t>(8, 1 + nnz / ((int64_t)P->num_sms * 64 * 512));
+        const int64_t edge_blocks = ((nnz + per_warp - 1) / per_warp + kTB / 32 - 1) / (kTB / 32);
+        const int64_t row_blocks = diag ? (n + kTB - 1) / kTB : 0;
+        k_support<<<(unsigned)(edge_blocks + row_blocks), kTB, 0, st>>>(diag ? 1 : 0, check ? 1 : 0, n, nnz, per_warp, edge_blocks,
+                                                                       d_rowptr, d_colidx, colx.p, &d_report->err);
+        GNNPRE_CUDA(cudaGetLastError());
+    }
+    GNNPRE_TRY(read_report());  // everything is in place
     for (int64_t l = 0; l < b; ++l) {
         Block& B = P->blocks[(size_t)l];
         const BlockRows& r = h_rows[(size_t)l];
@@ -1010,22 +1039,6 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         B.hub_hi = at[l + 1].hubs;
         B.done_row_lo = l == 0 ? 0 : h_rows[(size_t)l - 1].done_row_hi;
         B.done_row_hi = l == b - 1 ? n : r.done_row_hi;
-    }
-
-
-    // ---- E, the support's edge list: overwrites the temporaries
-    {
-        const bool check = !(opts->flags & GNNPRE_FLAG_SKIP_VALIDATION);
-        // 256 edges per warp, more (up to 2048) only while every warp the device holds still gets its share
-        const int64_t per_warp = 256 * std::min<int64_t>(8, 1 + nnz / ((int64_t)P->num_sms * 64 * 512));
-        const int64_t edge_blocks = ((nnz + per_warp - 1) / per_warp + kTB / 32 - 1) / (kTB / 32);
-        const int64_t row_blocks = diag ? (n + kTB - 1) / kTB : 0;
-        k_support<<<(unsigned)(edge_blocks + row_blocks), kTB, 0, st>>>(diag ? 1 : 0, check ? 1 : 0, n, nnz, per_warp, edge_blocks,
-                                                                       d_rowptr, d_colidx, colx.p, P->dev_error.p);
-        GNNPRE_CUDA(cudaGetLastError());
-        int h = 0;
-        GNNPRE_CUDA(cudaMemcpy(&h, P->dev_error.p, sizeof(int), cudaMemcpyDeviceToHost));  // everything is in place
-        if (h) return GNNPRE_ERR_INVALID_CSR;
     }
     if (by_source) {
         int32_t *counts = P->by_source_counts.p, *begins = counts + kOrderBuckets + 1;

@@ -277,6 +277,34 @@ def test_invalid_inputs_are_rejected(B):
     plan.close()
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("fault", ["descending", "negative", "beyond", "short", "column", "diagonal", "order"])
+def test_invalid_graphs_are_rejected_by_a_build_that_looks_once(B, op, fault):
+    """Graphs of more than 1 MB of tables: the build launches everything before the host reads what the device found."""
+    g = gi.rmat(60000, 400000, 47, directed_candidates=True)
+    rp, ci = dev(g)
+    row = int((g.rowptr[1:] - g.rowptr[:-1] >= 3).nonzero()[1000])
+    lo = int(g.rowptr[row])
+    if fault == "descending":
+        rp[row + 1] = lo - 2
+    elif fault == "negative":
+        rp[row + 1] = -5
+    elif fault == "beyond":
+        rp[row + 1] = g.nnz + 7
+    elif fault == "short":
+        rp[-1] = g.nnz - 1
+    else:
+        ci[lo + 1] = {"column": g.n, "diagonal": row, "order": int(ci[lo])}[fault]
+    with pytest.raises(B.GnnpreError) as ei:
+        B.gnnpre_build_plan(rp, ci, op, 64)
+    assert ei.value.status == -2
+    plan = B.gnnpre_build_plan(*dev(g), op, 64, gin_eps=EPS)  # and the next one is as good as ever
+    X = gi.normal_matrix(g.n, 64, 48)
+    outs, _ = B.gnnpre_propagate(plan, X.cuda(), 1)
+    check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), X.numpy(), outs)
+    plan.close()
+
+
 def test_graph_without_edges(B):
     g = gi.from_edge_list(6, [])
     drp, dci = dev(g)
