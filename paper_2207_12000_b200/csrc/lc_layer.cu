@@ -64,6 +64,7 @@ constexpr int kLcX3SplitWarps = 4;                 // warps 9-12 compute the low
 constexpr int kLcX3SplitWarp0 = kLcProducerWarps + 1 + kLcX3EpilogueWarps;
 constexpr int kLcX3Threads = 32 * (kLcX3SplitWarp0 + kLcX3SplitWarps);
 constexpr uint32_t kLcX3MaxCols = 128;             // output columns of a CTA, columns of one accumulator buffer
+constexpr int kLcPairStages = 4;                   // pairs of CTAs: what tensor memory holds low parts of beside three accumulators
 constexpr int kLcMaxDevices = 64;
 constexpr int kLcMaxHops = 8;                     // hop matrices per launch
 constexpr uint32_t kLcTmemCols = 512;
@@ -131,12 +132,45 @@ __device__ __forceinline__ bool lc_mbar_try_wait(uint32_t bar, uint32_t parity) 
     return done != 0;
 }
 
+// The same for a barrier on which the other CTA of a pair arrives too.
+__device__ __forceinline__ bool lc_mbar_try_wait_pair(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity), "r"(kLcSuspendNs)
+        : "memory");
+    return done != 0;
+}
+
+// Arrives on the barrier at this address of the leading CTA (rank 0) of the pair.
+__device__ __forceinline__ void lc_mbar_arrive_leader(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .b32 remote;\n\t"
+        "mapa.shared::cluster.u32 remote, %0, 0;\n\t"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ uint32_t lc_pair_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void lc_pair_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Bounded wait.  False when the limit ran out (the abort flag and the error word are then set) or
 // when another role has already given up.
+template <bool PAIR = false>
 __device__ __forceinline__ bool lc_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* error,
                                         uint32_t limit = kLcSpinLimit) {
     for (uint32_t i = 0; i < limit; ++i) {
-        if (lc_mbar_try_wait(bar, parity)) return true;
+        if (PAIR ? lc_mbar_try_wait_pair(bar, parity) : lc_mbar_try_wait(bar, parity)) return true;
         if (*abort_flag) return false;
     }
     *abort_flag = 1;
@@ -175,35 +209,82 @@ __device__ __forceinline__ uint64_t lc_operand_desc(uint32_t addr) {
     return d;
 }
 
-// Instruction descriptor: fp32 accumulator, tf32 A and B, both K-major, M = 128, N = hidden.
-__device__ __forceinline__ uint32_t lc_instr_desc(int n) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kLcTileM >> 4) << 24);
+// Instruction descriptor: fp32 accumulator, tf32 A and B, both K-major, M rows (128, or 256 for a pair of CTAs), N = n.
+__device__ __forceinline__ uint32_t lc_instr_desc(int n, int m = kLcTileM) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// PAIR: both CTAs' rows (their own operand A) by both CTAs' columns (half of operand B each); either CTA's tensor memory gets
+// its own rows of D.  Shared and tensor memory addresses mean the same place in both.
+template <bool PAIR = false>
 __device__ __forceinline__ void lc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                             uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
 }
 
 // The same with A in tensor memory: row = lane, one 32-bit column per element of K.
+template <bool PAIR = false>
 __device__ __forceinline__ void lc_mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
                                                uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
 }
 
-// Makes the mbarrier track the completion of every MMA this thread has issued so far.
+// Makes the mbarrier (PAIR: the one at this address in both CTAs) track the completion of every MMA this thread has issued
+// so far.
+template <bool PAIR = false>
 __device__ __forceinline__ void lc_mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    if constexpr (PAIR)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                     "h"((uint16_t)3)
+                     : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// All of the tensor memory, by one warp of each CTA.
+template <bool PAIR = false>
+__device__ __forceinline__ void lc_tmem_alloc(uint32_t slot) {
+    if constexpr (PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(kLcTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(kLcTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+}
+
+template <bool PAIR = false>
+__device__ __forceinline__ void lc_tmem_free(uint32_t tmem_base) {
+    if constexpr (PAIR)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLcTmemCols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLcTmemCols) : "memory");
 }
 
 // 32 consecutive accumulator columns of this thread's tensor-memory lane.
@@ -239,13 +320,16 @@ __device__ __forceinline__ void lc_tile_store(const CUtensorMap* tmap, int x0, i
                  : "memory");
 }
 
-// Epilogue role (the warps after the MMA warp), shared by both kernels: tiles first, first + step, ...; the accumulator
+// Epilogue role (the warps after the MMA warp), shared by all kernels: tiles first, first + step, ...; an accumulator
 // holds n_cols columns that go to columns col0 .. col0 + n_cols of Y.  WARPS / 4 warps per quarter of the accumulator's
-// lanes share its 32-column boxes in turn; a warp has BOXES staging boxes in shared memory.
-template <int WARPS, int BOXES>
+// lanes share its 32-column boxes in turn; a warp has BOXES staging boxes in shared memory.  Two accumulators take turns.
+// PAIR: a tile has rows of both CTAs, this one's from row0 on, and two accumulators, the second for the next n_cols columns;
+// three take turns, and it is the leading CTA that hears of free ones.
+template <int WARPS, int BOXES, bool PAIR = false>
 __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a, uint32_t tiles0, uint32_t tmem_base,
                                             uint32_t acc_full0, uint32_t acc_empty0, volatile int* abort_flag, int first,
-                                            int step, int n_cols, int col0, uint32_t acc_stride) {
+                                            int step, int n_cols, int col0, uint32_t acc_stride, int row0 = 0) {
+    constexpr int kParts = PAIR ? 2 : 1, kAccs = PAIR ? 3 : 2, kRows = PAIR ? 2 * kLcTileM : kLcTileM;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int kTurn = WARPS / 4;
     const int ew = warp - kLcMmaWarp - 1;  // 0 .. WARPS - 1
@@ -255,11 +339,11 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
     uint32_t box = box0;
     const int boxes = (n_cols + 31) / 32;
     const int total_tiles = a.num_hops * a.tiles_m;
-    int it = 0;
-    for (int t = first; t < total_tiles; t += step, ++it) {
+    int it = 0;  // accumulators taken so far
+    for (int t = first, part = 0; t < total_tiles; ++it) {
         const int hop = t / a.tiles_m, mt = t - hop * a.tiles_m;
-        const int buf = it & 1;
-        const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
+        const int buf = it % kAccs;
+        const uint32_t acc_ph = (uint32_t)(it / kAccs) & 1u;
         if (!__all_sync(0xffffffffu, lc_wait(acc_full0 + 8u * buf, acc_ph, abort_flag, a.error, a.spin_limit))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const bool relu = (a.relu_mask >> hop) & 1u;
@@ -292,14 +376,21 @@ __device__ __forceinline__ void lc_epilogue(const LcMaps& maps, const LcArgs& a,
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
-                lc_tile_store(&maps.y[hop], col0 + 32 * i, mt * kLcTileM + 32 * q, box);
+                lc_tile_store(&maps.y[hop], col0 + part * n_cols + 32 * i, mt * kRows + row0 + 32 * q, box);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
             if (BOXES == 2) box = box == box0 ? box0 + kLcEpiBytes : box0;
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) lc_mbar_arrive(acc_empty0 + 8u * buf);
+        if (lane == 0) {
+            if (PAIR) lc_mbar_arrive_leader(acc_empty0 + 8u * buf);
+            else lc_mbar_arrive(acc_empty0 + 8u * buf);
+        }
+        if (++part == kParts) {
+            part = 0;
+            t += step;
+        }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     __syncwarp();
@@ -339,10 +430,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kLcMmaWarp) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(lc_smem_u32(&tmem_slot)),
-                     "r"(kLcTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        lc_tmem_alloc(lc_smem_u32(&tmem_slot));
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -475,7 +563,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
     __syncthreads();
     if (warp == kLcMmaWarp) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLcTmemCols) : "memory");
+        lc_tmem_free(tmem_base);
     }
 }
 
@@ -484,15 +572,21 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // that tf32 holds exactly (low 13 mantissa bits cleared) and a low part (the exact remainder, which the
 // tensor core again reads as tf32), and  x w  ~=  xh wh + xl wh + xh wl  with fp32 accumulation; the dropped terms are
 // below 2^-21 |x||w|.  Shared memory has to hold both parts of both operands, so a CTA computes at most
-// 128 output columns: with hidden > 128, even and odd CTAs take the two column halves and every batch row is
-// gathered once per part (the later reads mostly hit L2).  No tensor copies on the input side: the producer
-// threads bring rows of the hop matrix AND rows of the weight in with 16-byte asynchronous copies; four warps of their own
-// (9-12) read each stage that has landed and write the low parts of its rows into tensor memory, from where the tensor core
+// 128 weight rows.  With hidden > 128 few tiles are computed by even and odd CTAs that take a column half each and both gather
+// every batch row; many by pairs of CTAs (PAIR, a cluster of two): a tile has 256 rows, each CTA gathers its own 128 and holds half
+// of the weight, and the leading CTA's MMA warp multiplies both CTAs' rows by all columns (cta_group::2, M = 256).  Beside the low
+// parts of four stages tensor memory then holds three accumulators of 128 columns, of which a tile takes two in turn.
+// No tensor copies on the input side: the producer
+// threads bring rows of the hop matrix AND rows of the weight in with 16-byte asynchronous copies; the last four warps
+// read each stage that has landed and write the low parts of its rows into tensor memory, from where the tensor core
 // takes them as operand A (lane = row): beside the two 128-column accumulators there are 32 columns for each of eight
 // stages, and shared memory holds four stages of copied rows beside 128 KB of weight.  2.4 M rows x 3 hops, F = 100, hidden
 // 256, random order, under load: 4630 us when the copying threads split into a second half of two stages (and their proxy
 // fence waited for all their copies in flight), 3379 us now (single passes on a cool device: 3550 us with splitter warps and two
-// buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the L2's and the copy path's latency over those four stages.
+// buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the latency of a
+// tile's chain over those four stages and, in long runs, by the power that all its parts draw: pairs of CTAs 3250 -> 3130 us,
+// F = 256 990 -> 882; of those, without two of the three products 2450 us, without the stores 2545, without the copies 2640,
+// without the low parts 3050.
 // K-steps of the last chunk beyond the features are neither copied nor multiplied.
 //
 // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
@@ -512,9 +606,11 @@ __device__ __forceinline__ void lc_store_low_part(const uint32_t (&v)[4], uint32
                  : "memory");
 }
 
+template <bool PAIR>
 __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __grid_constant__ LcMaps maps, const LcArgs a) {
     extern __shared__ unsigned char lc_smem[];
-    __shared__ __align__(8) unsigned long long bars[3 * kLcMaxStages + 6];
+    __shared__ __align__(8) unsigned long long bars[3 * kLcMaxStages + 8];
+    constexpr int kCtas = PAIR ? 2 : 1, kAccs = PAIR ? 3 : 2;  // CTAs that share a tile; accumulators that take turns
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int* abort_flag = &abort_word;
@@ -526,44 +622,57 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
     auto empty_bar = [&](int s) { return bar0 + 8u * (kLcMaxStages + s); };
     auto copied_bar = [&](int s) { return bar0 + 8u * (2 * kLcMaxStages + s); };  // a stage's copies have landed
     auto acc_full_bar = [&](int b) { return bar0 + 8u * (3 * kLcMaxStages + b); };
-    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (3 * kLcMaxStages + 2 + b); };
-    const uint32_t drain_bar = bar0 + 8u * (3 * kLcMaxStages + 4);
-    const uint32_t w_bar = bar0 + 8u * (3 * kLcMaxStages + 5);
+    auto acc_empty_bar = [&](int b) { return bar0 + 8u * (3 * kLcMaxStages + 3 + b); };
+    const uint32_t drain_bar = bar0 + 8u * (3 * kLcMaxStages + 6);
+    const uint32_t w_bar = bar0 + 8u * (3 * kLcMaxStages + 7);
+    // what the MMA warp of the leading CTA waits for
+    auto arrive_for_mma = [&](uint32_t bar) {
+        if (PAIR) lc_mbar_arrive_leader(bar);
+        else lc_mbar_arrive(bar);
+    };
+    const int rank = PAIR ? (int)lc_pair_rank() : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kLcMaxStages; ++s) {
             lc_mbar_init(copied_bar(s), kLcProducerThreads);
-            lc_mbar_init(full_bar(s), kLcX3SplitWarps);  // a stage's low parts are there as well
+            lc_mbar_init(full_bar(s), kCtas * kLcX3SplitWarps);  // a stage's low parts are there as well
             lc_mbar_init(empty_bar(s), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kAccs; ++b) {
             lc_mbar_init(acc_full_bar(b), 1);
-            lc_mbar_init(acc_empty_bar(b), kLcX3EpilogueWarps);
+            lc_mbar_init(acc_empty_bar(b), kCtas * kLcX3EpilogueWarps);
         }
         lc_mbar_init(drain_bar, 1);
-        lc_mbar_init(w_bar, kLcProducerThreads);
+        lc_mbar_init(w_bar, kCtas * kLcProducerThreads);
         abort_word = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kLcMmaWarp) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(lc_smem_u32(&tmem_slot)),
-                     "r"(kLcTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        lc_tmem_alloc<PAIR>(lc_smem_u32(&tmem_slot));
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) lc_pair_sync();  // the other CTA's barriers are there, and both CTAs' tensor memory
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_slot;
 
     const int total_tiles = a.num_hops * a.tiles_m;
-    const int half = blockIdx.x % a.halves;
+    const int half = PAIR ? 0 : blockIdx.x % a.halves;
     const int first = blockIdx.x / a.halves, step = gridDim.x / a.halves;
+    const int64_t tile_rows = kCtas * kLcTileM, rank_row = rank * kLcTileM;  // batch rows of a tile; where this CTA's begin
+    // the output column of row r of this CTA's part of the weight: a pair's two accumulators take n_half columns each, and of
+    // those either CTA holds half
+    auto weight_row = [&](int r) {
+        if (!PAIR) return half * a.n_half + r;
+        const int quarter = a.n_half / 2, part = r >= quarter;
+        return part * a.n_half + rank * quarter + r - part * quarter;
+    };
     constexpr uint32_t kPart = kLcABytes;               // bytes of the rows' chunk: [128, 32] floats
     const uint32_t w_part = (uint32_t)a.n_half * 128u;  // bytes of one part of the weight's chunk: [n_half, 32] floats
 
-    // Tensor memory: two accumulators of kLcX3MaxCols columns, then the low parts of each stage's rows, 32 columns a stage.
-    auto tmem_low = [&](int s) { return tmem_base + 2u * kLcX3MaxCols + 32u * s; };
+    // Tensor memory: two accumulators (a pair: three) of kLcX3MaxCols columns, then the low parts of each stage's rows, 32
+    // columns a stage.
+    auto tmem_low = [&](int s) { return tmem_base + (uint32_t)kAccs * kLcX3MaxCols + 32u * s; };
     // K-steps of 8 features in chunk kc: 16-byte pieces beyond them are neither copied nor multiplied
     auto k_steps = [&](int kc) { return min(4, (a.feat_dim - kc * kLcChunk + 7) >> 3); };
 
@@ -588,7 +697,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int r = row0 + 4 * i;
-            w_row[i] = r < a.n_half ? a.wt + (int64_t)(half * a.n_half + r) * a.ldw : nullptr;
+            w_row[i] = r < a.n_half ? a.wt + (int64_t)weight_row(r) * a.ldw : nullptr;
         }
         // copy this thread's pieces of chunk kc of `rows` (hop rows or weight rows) to `dst_part`
         // (a part holds row_limit rows: 128 for the tile, n_half for the weight; rows beyond it do not exist)
@@ -615,7 +724,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
                 split_weight(kc, wb, wb + w_part);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            lc_mbar_arrive(w_bar);
+            arrive_for_mma(w_bar);
         }
         int s = 0;
         uint32_t ph = 0;
@@ -625,7 +734,7 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
             const float* src_row[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const int64_t pos = (int64_t)mt * kLcTileM + row0 + 4 * i;
+                const int64_t pos = mt * tile_rows + rank_row + row0 + 4 * i;
                 int64_t r = -1;
                 if (pos < a.batch_size) r = a.batch ? (int64_t)__ldg(a.batch + pos) : pos;
                 src_row[i] = (r >= 0 && r < a.n) ? a.hop[hop] + r * a.ldh : nullptr;
@@ -648,45 +757,53 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
         asm volatile("cp.async.wait_all;" ::: "memory");  // nothing may land after this CTA has left
     } else if (warp == kLcMmaWarp) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = lc_instr_desc(a.n_half);
-            int s = 0, it = 0;
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = lc_instr_desc(a.n_half, (int)tile_rows);
+            const uint32_t quarter = (uint32_t)(a.n_half / 2) * 128u;  // a pair: from the first accumulator's weight rows to the second's
+            int s = 0, it = 0;  // it: accumulators taken so far
             uint32_t ph = 0;
-            bool ok = !a.w_resident || lc_wait(w_bar, 0, abort_flag, a.error, a.spin_limit);
-            for (int t = first; t < total_tiles && ok; t += step, ++it) {
-                const int buf = it & 1;
-                const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
-                if (!lc_wait(acc_empty_bar(buf), acc_ph ^ 1u, abort_flag, a.error, a.spin_limit)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcX3MaxCols;
-                for (int kc = 0; kc < a.k_chunks; ++kc) {
-                    if (!lc_wait(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
+            bool ok = !a.w_resident || lc_wait<PAIR>(w_bar, 0, abort_flag, a.error, a.spin_limit);
+            for (int t = first; t < total_tiles && ok; t += step, it += kCtas) {
+                for (int kc = 0; kc < a.k_chunks && ok; ++kc) {
+                    if (!lc_wait<PAIR>(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
                         ok = false;
                         break;
                     }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // both parts, seen by the tensor core
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    // the copies, seen by the tensor core (a pair: either CTA's splitters have seen to that)
+                    if (!PAIR) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
                     const uint32_t xh = base, xl = tmem_low(s);
-                    const uint32_t wh = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart;
-                    const uint32_t wl = wh + w_part;
                     const int steps = k_steps(kc);
-                    for (int j = 0; j < steps; ++j) {
-                        const uint32_t o = 32u * j;
-                        // small terms first, the leading term last
-                        lc_mma_tf32_ta(tmem_d, xl + 8u * j, lc_operand_desc(wh + o), idesc, (kc | j) != 0);
-                        lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wl + o), idesc, 1u);
-                        lc_mma_tf32(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wh + o), idesc, 1u);
+#pragma unroll
+                    for (int part = 0; part < kCtas; ++part) {
+                        const int buf = (it + part) % kAccs;
+                        if (kc == 0 && !lc_wait<PAIR>(acc_empty_bar(buf), ((uint32_t)((it + part) / kAccs) & 1u) ^ 1u, abort_flag,
+                                                      a.error, a.spin_limit)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcX3MaxCols;
+                        const uint32_t wh = (a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart) + part * quarter;
+                        const uint32_t wl = wh + w_part;
+                        for (int j = 0; j < steps; ++j) {
+                            const uint32_t o = 32u * j;
+                            // small terms first, the leading term last
+                            lc_mma_tf32_ta<PAIR>(tmem_d, xl + 8u * j, lc_operand_desc(wh + o), idesc, (kc | j) != 0);
+                            lc_mma_tf32<PAIR>(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wl + o), idesc, 1u);
+                            lc_mma_tf32<PAIR>(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wh + o), idesc, 1u);
+                        }
+                        if (kc == a.k_chunks - 1) lc_mma_commit<PAIR>(acc_full_bar(buf));
                     }
-                    lc_mma_commit(empty_bar(s));
+                    if (!ok) break;
+                    lc_mma_commit<PAIR>(empty_bar(s));
                     if (++s == a.stages) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
-                if (ok) lc_mma_commit(acc_full_bar(buf));
             }
-            lc_mma_commit(drain_bar);
+            lc_mma_commit<PAIR>(drain_bar);
             for (uint32_t i = 0; i < kLcSpinLimit; ++i)
                 if (lc_mbar_try_wait(drain_bar, 0)) break;
         }
@@ -715,9 +832,10 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
                 lc_tmem_store32(tmem_low(s) + ((uint32_t)(32 * (warp & 3)) << 16), lo);
                 if (!a.w_resident) split_weight(kc, base + kPart, base + kPart + w_part);
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (PAIR) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies, seen by the tensor core
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) lc_mbar_arrive(full_bar(s));
+                if (lane == 0) arrive_for_mma(full_bar(s));
                 if (++s == a.stages) {
                     s = 0;
                     ph ^= 1u;
@@ -725,15 +843,23 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
             }
         }
     } else {
-        lc_epilogue<kLcX3EpilogueWarps, 2>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first, step, a.n_half,
-                    half * a.n_half, kLcX3MaxCols);
+        lc_epilogue<kLcX3EpilogueWarps, 2, PAIR>(maps, a, tiles0, tmem_base, acc_full_bar(0), acc_empty_bar(0), abort_flag, first,
+                                                 step, a.n_half, half * a.n_half, kLcX3MaxCols, (int)rank_row);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) {
+        // the tensor core's last arrivals are in (the leading CTA sends them to both), and nobody needs this CTA's memory any more
+        if (threadIdx.x == 0)
+            for (uint32_t i = 0; i < kLcSpinLimit; ++i)
+                if (lc_mbar_try_wait(drain_bar, 0)) break;
+        __syncwarp();
+        lc_pair_sync();
+    }
     if (warp == kLcMmaWarp) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kLcTmemCols) : "memory");
+        lc_tmem_free<PAIR>(tmem_base);
     }
 }
 
@@ -814,6 +940,7 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     uint32_t stage_stride, w_off;
     int32_t stages;
     int64_t w_bytes;
+    bool pair = false;
     if (!x3) {
         w_bytes = (int64_t)k_chunks * hidden * 128;
         resident = w_bytes <= kLcResidentMax;
@@ -824,19 +951,25 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         const uint32_t w_part = (uint32_t)n_half * 128u;
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
+        // Hidden > 128, many tiles: pairs of CTAs that gather each row once (and stream the weight half as often) instead of CTAs
+        // that take a column half each.  A tile of a pair takes longer, so a few tiles are slower.  us, halves / pairs: F = 100
+        // (resident weight), hidden 256, tiles of 128 rows x hops 1250 75 / 78, 4692 265 / 255, 13596 752 / 722, 57408
+        // 3265 / 3130; F = 160 (streamed) 626 57 / 59, 1250 105 / 100, 4692 388 / 355; F = 256 157 32 / 39, 626 82 / 82, 1250
+        // 157 / 146, 4692 587 / 516; F = 602 1250 373 / 329, 4692 1378 / 1172.
+        pair = halves == 2 && std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m >= (resident ? 28 : 8) * (int64_t)num_sms;
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + 2u * w_part;
-        stages = (int32_t)std::min<int64_t>(kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
+        stages = (int32_t)std::min<int64_t>(pair ? kLcPairStages : kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     }
     w_off = (uint32_t)stages * stage_stride;
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
     const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
-    auto kernel = x3 ? k_lc_first_layer_x3 : k_lc_first_layer;
+    auto kernel = pair ? k_lc_first_layer_x3<true> : x3 ? k_lc_first_layer_x3<false> : k_lc_first_layer;
     // the opt-in to large dynamic shared memory, per kernel and device: always the most a launch can want, so once is enough
     constexpr int kMostSmem = 1024 + kLcPipeBytes + 8 * kLcEpiBytes;
-    static std::atomic<bool> opted_in[2][kLcMaxDevices];
-    if (dev >= kLcMaxDevices || !opted_in[x3][dev].load(std::memory_order_relaxed)) {
+    static std::atomic<bool> opted_in[3][kLcMaxDevices];
+    if (dev >= kLcMaxDevices || !opted_in[x3 + pair][dev].load(std::memory_order_relaxed)) {
         GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
-        if (dev < kLcMaxDevices) opted_in[x3][dev].store(true, std::memory_order_relaxed);
+        if (dev < kLcMaxDevices) opted_in[x3 + pair][dev].store(true, std::memory_order_relaxed);
     }
 
     LcMaps maps;
@@ -855,7 +988,7 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.batch = batch;
         a.batch_size = batch_size;
         a.num_hops = kn;
-        a.tiles_m = (int32_t)tiles_m;
+        a.tiles_m = (int32_t)(pair ? (tiles_m + 1) / 2 : tiles_m);
         a.k_chunks = k_chunks;
         a.hidden = (int32_t)hidden;
         a.relu_mask = relu_mask >> k0;
@@ -871,10 +1004,20 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.n_half = n_half;
         a.drop_announcements = selftest_polls > 0 ? 1 : 0;
         a.spin_limit = selftest_polls > 0 ? selftest_polls : kLcSpinLimit;
-        const int64_t total = (int64_t)kn * tiles_m;
+        const int64_t total = (int64_t)kn * a.tiles_m;
         const unsigned grid = (unsigned)(std::min<int64_t>(num_sms / halves, total) * halves);
-        kernel<<<grid, x3 ? kLcX3Threads : kLcThreads, smem, st>>>(maps, a);
-        GNNPRE_CUDA(cudaGetLastError());
+        cudaLaunchAttribute two{};
+        two.id = cudaLaunchAttributeClusterDimension;
+        two.val.clusterDim.x = 2;
+        two.val.clusterDim.y = two.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(x3 ? kLcX3Threads : kLcThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = &two;
+        cfg.numAttrs = pair ? 1 : 0;
+        GNNPRE_CUDA(cudaLaunchKernelEx(&cfg, kernel, maps, a));
     }
     return GNNPRE_OK;
 }

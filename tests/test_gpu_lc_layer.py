@@ -102,6 +102,37 @@ def test_normal_inputs_within_the_bound_of_the_precision(B, n, F, H, bs, K, prec
         assert np.abs(got - want).max() < 0.01 * np.abs(want).max()
 
 
+PAIR_SHAPES = [  # split operands, hidden > 128, enough tiles of 128 rows (8 times the SMs, 28 times with a resident weight) for pairs of CTAs
+    (3000, 200, 192, 592 * 128 + 1, 2),  # accumulators of 96 columns; the last tile has one row, its second CTA none
+    (900, 300, 256, 50600, 3),           # the second CTA of the last tile has 40 rows
+    (66400, 104, 256, None, 8),          # no batch; resident weight
+    (3000, 33, 192, 518 * 128 + 1, 8),   # resident weight, a last chunk of one feature
+]
+
+
+@pytest.mark.parametrize("n,F,H,bs,K", PAIR_SHAPES)
+def test_pairs_of_ctas_on_one_tile(B, n, F, H, bs, K):
+    """Exact on integers (every hop against plain tf32, which is exact there too, two against the oracle), and the bound of the
+    precision on normal inputs (as above)."""
+    rng = np.random.default_rng(n + F)
+    rows = n if bs is None else bs
+    assert K * -(-rows // 128) >= (28 if F <= 128 else 8) * torch.cuda.get_device_properties(0).multi_processor_count
+    batch_np = None if bs is None else rng.integers(0, n, size=bs)
+    batch = None if bs is None else torch.from_numpy(batch_np.astype(np.int32)).cuda()
+    hops_np, Wt_np = [integer_matrix(n, F, 500 + k, -7, 7) for k in range(K)], integer_matrix(H, F, 17, -5, 5)
+    hops, Wt = [padded_cuda(h, 2) for h in hops_np], padded_cuda(Wt_np, 5)
+    Y = B.gnnpre_lc_first_layer(hops, batch, Wt, relu_mask=0b10, precision=1)
+    assert torch.equal(Y, B.gnnpre_lc_first_layer(hops, batch, Wt, relu_mask=0b10, precision=0))
+    for k in (0, 1):
+        want = orc.lc_first_layer(hops_np[k], batch_np, Wt_np, relu=k == 1)
+        assert np.array_equal(to_np(Y[k]).astype(np.float64), want)
+    hops_np[K - 1], Wt_np = gi.normal_matrix(n, F, 600).numpy(), gi.normal_matrix(H, F, 19).numpy()
+    hops[K - 1], Wt = padded_cuda(hops_np[K - 1], 2), padded_cuda(Wt_np, 5)
+    Y = B.gnnpre_lc_first_layer(hops, batch, Wt, precision=1)
+    want, scale = orc.lc_first_layer(hops_np[K - 1], batch_np, Wt_np, relu=False, want_abs=True)
+    assert (np.abs(to_np(Y[K - 1]).astype(np.float64) - want) <= (2.0 ** -20 + F * 2.0 ** -23) * scale).all()
+
+
 def test_concatenated_layout_strided_output_and_untouched_padding(B):
     n, F, H, bs, K = 1500, 100, 32, 700, 3
     hops_np = [integer_matrix(n, F, 300 + k, -6, 6) for k in range(K)]
