@@ -164,6 +164,18 @@ int launch_finish_shape(const FixArgs& a, cudaStream_t st) {
     return launch_dependent(k_finish_rows<G, kEpPlain>, grid, kThreads, 0, a.back_to_back, st, a);
 }
 
+int64_t l2_cache_bytes() {
+    static std::atomic<int64_t> cached{0};
+    int64_t bytes = cached.load(std::memory_order_relaxed);
+    if (bytes == 0) {
+        int dev = 0, got = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&got, cudaDevAttrL2CacheSize, dev) != cudaSuccess || got <= 0)
+            got = 126 << 20;
+        cached.store(bytes = got, std::memory_order_relaxed);
+    }
+    return bytes;
+}
+
 Teleport teleport_of(const gnnpre_plan* P, const HopArgs& h, int32_t f0) {
     Teleport tp;
     tp.x0 = h.x0 ? h.x0 + f0 : nullptr;
@@ -178,24 +190,15 @@ Teleport teleport_of(const gnnpre_plan* P, const HopArgs& h, int32_t f0) {
     tp.gamma_prev = h.gamma_prev;
     tp.gamma0 = h.gamma0;
     tp.zsum_first = h.zsum_first ? 1 : 0;
+    // with X_0 and Z a hop has three to five matrices; tiles of more than 64 columns that exceed the L2 alone gain nothing
+    // (600 K nodes, 128 columns: 10.3 ms without, 10.5 with; 1 M nodes, 64 columns 6.1 / 5.8)
+    tp.ahead = P->n * h.width * 16 > l2_cache_bytes() && (h.width <= 64 || !beyond_cache(P, h.width));
     return tp;
 }
 
 }  // namespace
 
 namespace {
-
-int64_t l2_cache_bytes() {
-    static std::atomic<int64_t> cached{0};
-    int64_t bytes = cached.load(std::memory_order_relaxed);
-    if (bytes == 0) {
-        int dev = 0, got = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&got, cudaDevAttrL2CacheSize, dev) != cudaSuccess || got <= 0)
-            got = 126 << 20;
-        cached.store(bytes = got, std::memory_order_relaxed);
-    }
-    return bytes;
-}
 
 // The mean operator's column tiles of 68..124 columns go through the bulk-copy kernel when X's tile is at least four times
 // the L2 and rows are long (mean degree >= 32).  Its rows in flight (213 KB per SM) then hide the DRAM latency that the

@@ -89,6 +89,12 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     // and the piece in shared memory: 3144, 100).
     constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16 && EP != kEpTeleport;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN && !kDiagonal;
+    // Epilogue operands come from memory where the hop's matrices together exceed the L2, and one row ahead is too late for that:
+    // each lane asks for the pieces that belong to its row end when the chunk is staged.  169 K nodes, without / with, us a
+    // call: teleport term, three hops, GCN, 64 columns 302 / 270, 128 394 / 385, sum operator, 100 columns 386 / 359; with
+    // the sum of ten hops GCN, 64 columns 1125 / 1035, 100 1517 / 1458, sum operator, 64 columns 1042 / 996, mean, 128
+    // 1315 / 1283.  Not the mean operator's 64 columns (889 / 918) nor narrower rows (16 columns 15 % slower).
+    constexpr bool kAhead = EP != kEpPlain && (G == 32 || (G == 16 && OP != GNNPRE_OP_SAGE_MEAN));
     constexpr bool kShort = G == 4 || (G == 32 && EP == kEpPlain);
     using RowOut = std::conditional_t<kShort, RowOutShort, RowOutLong>;
     using Stage = SegStage<G, kWeighted, RowOut>;
@@ -184,6 +190,16 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             if constexpr (kShort) o.row = slot >= 0 ? ~slot : row[m];
             else o.row = slot >= 0 ? -1 : row[m];
             stage.out[i] = o;
+            if constexpr (kAhead) {
+                if (a.tp.ahead && i <= last && slot < 0) {
+                    constexpr int kLines = G / 8;
+                    const int tile_w = min(a.tile_f4, a.f4 - q0);
+                    if (EP == kEpTeleport || a.tp.alpha != 0.f || a.tp.zsum_first)
+                        prefetch_piece<kLines>(a.tp.x0 + (int64_t)row[m] * a.tp.ldx0 + 4 * q0, tile_w);
+                    if (EP == kEpSum && !a.tp.zsum_first) prefetch_piece<kLines>(a.tp.zsum + (int64_t)row[m] * a.tp.ldz + 4 * q0, tile_w);
+                    if (EP == kEpSum && a.tp.xprev) prefetch_piece<kLines>(a.tp.xprev + (int64_t)row[m] * a.tp.ldp + 4 * q0, tile_w);
+                }
+            }
         }
         if (ends != 0) slot_head = -1;
         rank = rank_after;

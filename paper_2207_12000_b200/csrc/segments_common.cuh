@@ -15,6 +15,7 @@ struct Teleport {
     int64_t ldp;
     float gamma, gamma_prev, gamma0;
     int zsum_first;
+    int ahead;  // fetch the rows that the epilogues read into the L2 ahead of time
 };
 
 // EP, the epilogue of a finished row: 0 = scale only; 1 = scale and teleport term; 2 = the launch also accumulates the
@@ -62,6 +63,14 @@ struct EpiloguePiece {
         return o;
     }
 };
+
+// Asks for the row piece of f4 float4 (at most 8 * LINES) at p to be brought into the L2.
+template <int LINES>
+__device__ __forceinline__ void prefetch_piece(const float* p, int f4) {
+#pragma unroll
+    for (int i = 0; i < LINES; ++i)
+        if (8 * i < f4) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32 * i));
+}
 
 __device__ __forceinline__ void copy_ahead(float4* dst, const float4* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
