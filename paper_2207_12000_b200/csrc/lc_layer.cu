@@ -178,6 +178,12 @@ __device__ __forceinline__ bool lc_wait(uint32_t bar, uint32_t parity, volatile 
     return false;
 }
 
+// The same by a whole warp, which goes on converged.
+template <bool PAIR = false>
+__device__ __forceinline__ bool lc_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* error, uint32_t limit) {
+    return __all_sync(0xffffffffu, lc_wait<PAIR>(bar, parity, abort_flag, error, limit));
+}
+
 // 16 bytes global -> shared without passing through registers; only the first src_bytes (0..16) are
 // read, the rest of the 16 bytes is written as zeros.
 __device__ __forceinline__ void lc_copy16(uint32_t dst, const float* src, uint32_t src_bytes) {
@@ -214,6 +220,9 @@ __device__ __forceinline__ uint32_t lc_instr_desc(int n, int m = kLcTileM) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// MMAs and commits are called by the whole MMA warp and issued by one elected lane (always the same): in code that all lanes
+// share the compiler keeps descriptors and addresses in uniform registers, which is where the instruction wants them; in a branch
+// of one lane it moved each of them there, MMA by MMA.
 // PAIR: both CTAs' rows (their own operand A) by both CTAs' columns (half of operand B each); either CTA's tensor memory gets
 // its own rows of D.  Shared and tensor memory addresses mean the same place in both.
 template <bool PAIR = false>
@@ -221,16 +230,18 @@ __device__ __forceinline__ void lc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uin
                                             uint32_t accumulate) {
     if constexpr (PAIR)
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
             "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
             "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
 }
@@ -241,16 +252,18 @@ __device__ __forceinline__ void lc_mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a,
                                                uint32_t accumulate) {
     if constexpr (PAIR)
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
             "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
             "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
 }
@@ -260,11 +273,14 @@ __device__ __forceinline__ void lc_mma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a,
 template <bool PAIR = false>
 __device__ __forceinline__ void lc_mma_commit(uint32_t bar) {
     if constexpr (PAIR)
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                     "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(bar),
                      "h"((uint16_t)3)
                      : "memory");
     else
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+        asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                     "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+                     : "memory");
 }
 
 // All of the tensor memory, by one warp of each CTA.
@@ -515,43 +531,41 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
         }
     } else if (warp == kLcMmaWarp) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = lc_instr_desc(a.hidden);
-            int s = 0, it = 0;
-            uint32_t ph = 0;
-            bool ok = !a.w_resident || lc_wait(w_bar, 0, abort_flag, a.error, a.spin_limit);
-            for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++it) {
-                const int buf = it & 1;
-                const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
-                if (!lc_wait(acc_empty_bar(buf), acc_ph ^ 1u, abort_flag, a.error, a.spin_limit)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcMaxHidden;
-                for (int kc = 0; kc < a.k_chunks; ++kc) {
-                    if (!lc_wait(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies, seen by the tensor core
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_src = tiles0 + (uint32_t)s * a.stage_stride;
-                    const uint32_t b_src = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * w_chunk_bytes : a_src + kLcABytes;
-#pragma unroll
-                    for (int j = 0; j < kLcChunk / 8; ++j)
-                        lc_mma_tf32(tmem_d, lc_operand_desc(a_src + 32u * j), lc_operand_desc(b_src + 32u * j), idesc,
-                                    (kc | j) != 0);
-                    lc_mma_commit(empty_bar(s));  // the stage is free once these MMAs have read it
-                    if (++s == a.stages) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+        const uint32_t idesc = lc_instr_desc(a.hidden);
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = !a.w_resident || lc_wait_warp(w_bar, 0, abort_flag, a.error, a.spin_limit);
+        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++it) {
+            const int buf = it & 1;
+            const uint32_t acc_ph = (uint32_t)(it >> 1) & 1u;
+            if (!lc_wait_warp(acc_empty_bar(buf), acc_ph ^ 1u, abort_flag, a.error, a.spin_limit)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcMaxHidden;
+            for (int kc = 0; kc < a.k_chunks; ++kc) {
+                if (!lc_wait_warp(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
+                    ok = false;
+                    break;
                 }
-                if (ok) lc_mma_commit(acc_full_bar(buf));
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies, seen by the tensor core
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t a_src = tiles0 + (uint32_t)s * a.stage_stride;
+                const uint32_t b_src = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * w_chunk_bytes : a_src + kLcABytes;
+                const uint64_t a_desc = lc_operand_desc(a_src), b_desc = lc_operand_desc(b_src);
+#pragma unroll
+                for (int j = 0; j < kLcChunk / 8; ++j)  // 32 bytes of a row, two units of a descriptor's address, per K-step
+                    lc_mma_tf32(tmem_d, a_desc + 2 * j, b_desc + 2 * j, idesc, (kc | j) != 0);
+                lc_mma_commit(empty_bar(s));  // the stage is free once these MMAs have read it
+                if (++s == a.stages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            // tensor memory may only be freed once the tensor core is idle
-            lc_mma_commit(drain_bar);
-            for (uint32_t i = 0; i < kLcSpinLimit; ++i)
-                if (lc_mbar_try_wait(drain_bar, 0)) break;
+            if (ok) lc_mma_commit(acc_full_bar(buf));
         }
+        // tensor memory may only be freed once the tensor core is idle
+        lc_mma_commit(drain_bar);
+        for (uint32_t i = 0; i < kLcSpinLimit; ++i)
+            if (lc_mbar_try_wait(drain_bar, 0)) break;
         __syncwarp();
     } else {
         // ---------------------------------------------------------------- epilogue
@@ -757,46 +771,41 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
         asm volatile("cp.async.wait_all;" ::: "memory");  // nothing may land after this CTA has left
     } else if (warp == kLcMmaWarp) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = lc_instr_desc(a.n_half, (int)tile_rows);
-            const uint32_t quarter = (uint32_t)(a.n_half / 2) * 128u;  // a pair: from the first accumulator's weight rows to the second's
+            // a pair: from the first accumulator's weight rows to the second's, in a descriptor's units
+            const uint32_t quarter = (uint32_t)(a.n_half / 2) * (128u >> 4);
             int s = 0, it = 0;  // it: accumulators taken so far
             uint32_t ph = 0;
-            bool ok = !a.w_resident || lc_wait<PAIR>(w_bar, 0, abort_flag, a.error, a.spin_limit);
+            bool ok = !a.w_resident || lc_wait_warp<PAIR>(w_bar, 0, abort_flag, a.error, a.spin_limit);
             for (int t = first; t < total_tiles && ok; t += step, it += kCtas) {
                 for (int kc = 0; kc < a.k_chunks && ok; ++kc) {
-                    if (!lc_wait<PAIR>(full_bar(s), ph, abort_flag, a.error, a.spin_limit)) {
-                        ok = false;
-                        break;
-                    }
-                    // the copies, seen by the tensor core (a pair: either CTA's splitters have seen to that)
-                    if (!PAIR) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
-                    const uint32_t xh = base, xl = tmem_low(s);
                     const int steps = k_steps(kc);
 #pragma unroll
                     for (int part = 0; part < kCtas; ++part) {
                         const int buf = (it + part) % kAccs;
-                        if (kc == 0 && !lc_wait<PAIR>(acc_empty_bar(buf), ((uint32_t)((it + part) / kAccs) & 1u) ^ 1u, abort_flag,
-                                                      a.error, a.spin_limit)) {
-                            ok = false;
-                            break;
-                        }
+                        if (kc == 0) ok = lc_wait_warp<PAIR>(acc_empty_bar(buf), ((uint32_t)((it + part) / kAccs) & 1u) ^ 1u, abort_flag, a.error, a.spin_limit);
+                        if (part == 0) ok = ok && lc_wait_warp<PAIR>(full_bar(s), ph, abort_flag, a.error, a.spin_limit);
+                        if (!ok) break;
+                        // the copies, seen by the tensor core (a pair: either CTA's splitters have seen to that)
+                        if (!PAIR) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcX3MaxCols;
-                        const uint32_t wh = (a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart) + part * quarter;
-                        const uint32_t wl = wh + w_part;
-                        for (int j = 0; j < steps; ++j) {
-                            const uint32_t o = 32u * j;
+                        const uint32_t base = tiles0 + (uint32_t)s * a.stage_stride;
+                        const uint32_t tmem_d = tmem_base + (uint32_t)buf * kLcX3MaxCols, xl = tmem_low(s);
+                        const uint32_t w_src = a.w_resident ? tiles0 + a.w_off + (uint32_t)kc * 2u * w_part : base + kPart;
+                        const uint64_t xh = lc_operand_desc(base), wh = lc_operand_desc(w_src) + part * quarter,
+                                       wl = lc_operand_desc(w_src + w_part) + part * quarter;
+#pragma unroll
+                        for (int j = 0; j < kLcChunk / 8; ++j) {
+                            if (j >= steps) break;
                             // small terms first, the leading term last
-                            lc_mma_tf32_ta<PAIR>(tmem_d, xl + 8u * j, lc_operand_desc(wh + o), idesc, (kc | j) != 0);
-                            lc_mma_tf32<PAIR>(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wl + o), idesc, 1u);
-                            lc_mma_tf32<PAIR>(tmem_d, lc_operand_desc(xh + o), lc_operand_desc(wh + o), idesc, 1u);
+                            lc_mma_tf32_ta<PAIR>(tmem_d, xl + 8u * j, wh + 2 * j, idesc, (kc | j) != 0);
+                            lc_mma_tf32<PAIR>(tmem_d, xh + 2 * j, wl + 2 * j, idesc, 1u);
+                            lc_mma_tf32<PAIR>(tmem_d, xh + 2 * j, wh + 2 * j, idesc, 1u);
                         }
+                        if (part == kCtas - 1) lc_mma_commit<PAIR>(empty_bar(s));
                         if (kc == a.k_chunks - 1) lc_mma_commit<PAIR>(acc_full_bar(buf));
                     }
-                    if (!ok) break;
-                    lc_mma_commit<PAIR>(empty_bar(s));
                     if (++s == a.stages) {
                         s = 0;
                         ph ^= 1u;
