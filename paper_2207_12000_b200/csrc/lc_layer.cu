@@ -221,8 +221,10 @@ __device__ __forceinline__ uint32_t lc_instr_desc(int n, int m = kLcTileM) {
 }
 
 // MMAs and commits are called by the whole MMA warp and issued by one elected lane (always the same): in code that all lanes
-// share the compiler keeps descriptors and addresses in uniform registers, which is where the instruction wants them; in a branch
-// of one lane it moved each of them there, MMA by MMA.
+// share the compiler can keep descriptors and addresses in uniform registers, which is where the instruction wants them; issued
+// from a branch of one lane, with descriptors built for each, an MMA took some 150 cycles, twice what the tensor core needs.
+// Split operands, 2.4 M rows x 3 hops, F = 100, hidden 256: 3130 us so / 2870 now; 600,000 rows, F = 256 519 / 487, F = 602
+// 1172 / 1090 (the clock falls to 1520..1620 MHz under the power cap); plain tf32 2030 / 2004.
 // PAIR: both CTAs' rows (their own operand A) by both CTAs' columns (half of operand B each); either CTA's tensor memory gets
 // its own rows of D.  Shared and tensor memory addresses mean the same place in both.
 template <bool PAIR = false>
@@ -598,9 +600,8 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // 256, random order, under load: 4630 us when the copying threads split into a second half of two stages (and their proxy
 // fence waited for all their copies in flight), 3379 us now (single passes on a cool device: 3550 us with splitter warps and two
 // buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the latency of a
-// tile's chain over those four stages and, in long runs, by the power that all its parts draw: pairs of CTAs 3250 -> 3130 us,
-// F = 256 990 -> 882; of those, without two of the three products 2450 us, without the stores 2545, without the copies 2640,
-// without the low parts 3050.
+// tile's chain over those four stages and, in long runs, by the power that all its parts draw (3250 us in halves, 3130 in
+// pairs of CTAs, 2870 with MMAs issued from uniform registers).
 // K-steps of the last chunk beyond the features are neither copied nor multiplied.
 //
 // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
@@ -961,11 +962,11 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
         // Hidden > 128, many tiles: pairs of CTAs that gather each row once (and stream the weight half as often) instead of CTAs
-        // that take a column half each.  A tile of a pair takes longer, so a few tiles are slower.  us, halves / pairs: F = 100
-        // (resident weight), hidden 256, tiles of 128 rows x hops 1250 75 / 78, 4692 265 / 255, 13596 752 / 722, 57408
-        // 3265 / 3130; F = 160 (streamed) 626 57 / 59, 1250 105 / 100, 4692 388 / 355; F = 256 157 32 / 39, 626 82 / 82, 1250
-        // 157 / 146, 4692 587 / 516; F = 602 1250 373 / 329, 4692 1378 / 1172.
-        pair = halves == 2 && std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m >= (resident ? 28 : 8) * (int64_t)num_sms;
+        // that take a column half each.  A tile of a pair takes longer, so a few tiles are slower.  us, halves / pairs, hidden
+        // 256, at 157 / 626 / 1250 tiles of 128 rows x hops: F = 100 (resident weight) 20.1 / 24.8, 43.3 / 45.2, 75.7 / 73.0;
+        // F = 160 (streamed) 23.4 / 26.7, 55.5 / 52.9, 107 / 96; F = 256 31.1 / 34.8, 82.8 / 73.6, 160 / 137; F = 602
+        // 61.5 / 65.6, 191 / 162, 379 / 310.
+        pair = halves == 2 && std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m >= (resident ? 8 : 4) * (int64_t)num_sms;
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + 2u * w_part;
         stages = (int32_t)std::min<int64_t>(pair ? kLcPairStages : kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     }
@@ -1015,17 +1016,22 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.spin_limit = selftest_polls > 0 ? selftest_polls : kLcSpinLimit;
         const int64_t total = (int64_t)kn * a.tiles_m;
         const unsigned grid = (unsigned)(std::min<int64_t>(num_sms / halves, total) * halves);
+        if (!pair) {
+            kernel<<<grid, x3 ? kLcX3Threads : kLcThreads, smem, st>>>(maps, a);
+            GNNPRE_CUDA(cudaGetLastError());
+            continue;
+        }
         cudaLaunchAttribute two{};
         two.id = cudaLaunchAttributeClusterDimension;
         two.val.clusterDim.x = 2;
         two.val.clusterDim.y = two.val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(x3 ? kLcX3Threads : kLcThreads);
+        cfg.blockDim = dim3(kLcX3Threads);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
         cfg.attrs = &two;
-        cfg.numAttrs = pair ? 1 : 0;
+        cfg.numAttrs = 1;
         GNNPRE_CUDA(cudaLaunchKernelEx(&cfg, kernel, maps, a));
     }
     return GNNPRE_OK;

@@ -102,11 +102,11 @@ def test_normal_inputs_within_the_bound_of_the_precision(B, n, F, H, bs, K, prec
         assert np.abs(got - want).max() < 0.01 * np.abs(want).max()
 
 
-PAIR_SHAPES = [  # split operands, hidden > 128, enough tiles of 128 rows (8 times the SMs, 28 times with a resident weight) for pairs of CTAs
+PAIR_SHAPES = [  # split operands, hidden > 128, enough tiles of 128 rows (4 times the SMs, 8 times with a resident weight) for pairs of CTAs
     (3000, 200, 192, 592 * 128 + 1, 2),  # accumulators of 96 columns; the last tile has one row, its second CTA none
     (900, 300, 256, 50600, 3),           # the second CTA of the last tile has 40 rows
-    (66400, 104, 256, None, 8),          # no batch; resident weight
-    (3000, 33, 192, 518 * 128 + 1, 8),   # resident weight, a last chunk of one feature
+    (66400, 104, 256, None, 3),          # no batch; resident weight
+    (3000, 33, 192, 518 * 128 + 1, 3),   # resident weight, a last chunk of one feature
 ]
 
 
@@ -116,7 +116,7 @@ def test_pairs_of_ctas_on_one_tile(B, n, F, H, bs, K):
     precision on normal inputs (as above)."""
     rng = np.random.default_rng(n + F)
     rows = n if bs is None else bs
-    assert K * -(-rows // 128) >= (28 if F <= 128 else 8) * torch.cuda.get_device_properties(0).multi_processor_count
+    assert K * -(-rows // 128) >= (8 if F <= 128 else 4) * torch.cuda.get_device_properties(0).multi_processor_count
     batch_np = None if bs is None else rng.integers(0, n, size=bs)
     batch = None if bs is None else torch.from_numpy(batch_np.astype(np.int32)).cuda()
     hops_np, Wt_np = [integer_matrix(n, F, 500 + k, -7, 7) for k in range(K)], integer_matrix(H, F, 17, -5, 5)
