@@ -205,7 +205,8 @@ namespace {
 // register kernel's 90 KB do not; everywhere else its copy engine, about 33 ps per row whatever the row's width, is the
 // slower path.  us per hop, bulk copy / register: 2.4 M nodes of mean degree 51, mean operator, 72 columns 3634 / 3845,
 // 100 columns 4085 / 4509, 124 columns 4670 / 5150, but 128 columns, rows of whole cache lines, 4641 / 4461; degree 34,
-// 100 columns 3187 / 3368.  With a weight per edge the rows wait for their weights instead: GCN, degree 51, 72 / 100 / 128
+// 100 columns 3187 / 3368.  (In the order of the edge list; in that of the sources 100 columns 3637 / 3870, in long runs three hops
+// 12.7 / 13.0 ms.)  With a weight per edge the rows wait for their weights instead: GCN, degree 51, 72 / 100 / 128
 // columns 4583 / 4243, 4971 / 4927, 5519 / 4792; GIN, whose few weighted edges are marked, in turn on one device 4239 / 4039,
 // 4874 / 4887, 5226 / 4739.  800 K nodes of degree 63, mean, 100 columns (2.4 x L2): register; 1.7 M nodes of degree 15 as well.  What the rule gives away: rows of equal length
 // and sources without hubs, X about as large as the L2 - 200,000 nodes of degree 160, 100 columns 898 / 1006, degree 96 523 / 571 -
