@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "gnnpre_internal.cuh"
+#include "segment_rules.h"
 
 namespace gnnpre {
 
@@ -416,15 +417,13 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
 // 1386 / 1378; 1 M nodes, 30 M edges, GCN, 128 columns 1072 / 1029; 400 K nodes, 40 M edges, sum, 256 columns 2200 / 2090;
 // about the L2's size: 300 K nodes, 40 M edges, GCN, 128 columns 1115 / 1068, 96 columns 997 / 990; well inside it: 169 K
 // nodes, 2.5 M edges, GCN, 128 columns 99 / 102.  Four or eight coarse ranges of columns instead: 3 to 6 % slower.
-constexpr int kOrderBuckets = 1024;  // by the middle column; one more for the segments of several rows and the empty ones
-
 __device__ __forceinline__ int order_bucket(const Segment* __restrict__ segs, int64_t s, int64_t nseg,
                                             const uint32_t* __restrict__ colx, int64_t n) {
     if (s + 1 >= nseg) return kOrderBuckets;
     const Segment g = segs[s], nx = segs[s + 1];
     const bool one_row = nx.rank == g.rank || (nx.rank == g.rank + 1 && nx.slot_head < 0);
     if (g.len == 0 || !one_row) return kOrderBuckets;
-    return (int)((int64_t)(colx[g.start + g.len / 2] & ~kRowEndBit) * kOrderBuckets / n);
+    return column_bucket(colx[g.start + g.len / 2] & ~kRowEndBit, n);
 }
 
 // SCATTER false: counts[b] = segments of bucket b.  true: counts[b] holds where the bucket begins; copies the segments there.

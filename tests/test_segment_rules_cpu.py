@@ -1,0 +1,36 @@
+"""The rules of plan construction in csrc/segment_rules.h, compiled for the CPU."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SHIM = r"""
+#include "segment_rules.h"
+extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
+extern "C" int order_buckets() { return gnnpre::kOrderBuckets; }
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-fPIC", "-shared", "-I", os.path.join(ROOT, "paper_2207_12000_b200", "csrc"),
+                    "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
+    lib = ctypes.CDLL(str(d / "shim.so"))
+    lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
+    return lib
+
+
+@pytest.mark.parametrize("n", [1, 2, 1000, 1024, 2449029, 2 ** 31 - 2])
+def test_buckets_of_columns_stay_in_range_whatever_the_column(rules, n):
+    """Columns are not checked with GNNPRE_FLAG_SKIP_VALIDATION, and the bucket is an index of the plan's tables."""
+    B = rules.order_buckets()
+    inside = sorted({0, n // 3, n // 2, n - 1})
+    for col in inside:
+        assert rules.column_bucket(col, n) == col * B // n < B
+    for col in (n, n + 1, 2 * n, 2 ** 31 - 1):
+        assert rules.column_bucket(min(col, 2 ** 31 - 1), n) == B - 1
