@@ -179,6 +179,10 @@ int gnnpre_plan_scales(const gnnpre_plan_t* plan, int32_t* deg_out, float* rscal
 /* Host copy of the support's CSR: rowptr_out int64[n+1], colidx_out int32[nnz_tilde].  Either may be NULL. */
 int gnnpre_plan_support(const gnnpre_plan_t* plan, int64_t* rowptr_out, int32_t* colidx_out);
 
+/* The order in which a launch over all segments takes them: first_edges_out int64[num_segments], the first edge of each.  It
+ * ascends, except where the matrix is larger than the L2: there segments inside one row come first, by their columns. */
+int gnnpre_plan_hop_order(const gnnpre_plan_t* plan, int64_t* first_edges_out);
+
 /*
  * Algorithm 1: out[k-1] <- A^ applied k times to X, for k = 1..K (X itself is not repeated); with a
  * teleport term in the plan, out[k-1] <- (1 - alpha) A^ out[k-2] + alpha X instead.

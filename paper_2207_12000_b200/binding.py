@@ -85,6 +85,7 @@ def _load() -> ctypes.CDLL:
     lib.gnnpre_plan_block.argtypes = [p, i32, ctypes.POINTER(gnnpre_block_info_t)]
     lib.gnnpre_plan_scales.argtypes = [p, p, p, p]
     lib.gnnpre_plan_support.argtypes = [p, p, p]
+    lib.gnnpre_plan_hop_order.argtypes = [p, p]
     lib.gnnpre_propagate.argtypes = [p, p, i64, i32, i32, ctypes.POINTER(p), i64, i32, p,
                                      ctypes.POINTER(gnnpre_stats_t)]
     lib.gnnpre_hop_static.argtypes = [ctypes.POINTER(gnnpre_csr_t), i32, ctypes.c_float, i64, p, i64, p, i64, p]
@@ -227,6 +228,13 @@ def gnnpre_plan_support(plan: Plan):
     ci = torch.empty(info["nnz_tilde"], dtype=torch.int32)
     _check(_lib.gnnpre_plan_support(plan.handle, rp.data_ptr(), ci.data_ptr()), "gnnpre_plan_support")
     return rp, ci
+
+
+def gnnpre_plan_hop_order(plan: Plan):
+    """int64 [num_segments] on the host: the first edge of each segment, in the order a whole hop takes them."""
+    first = torch.empty(gnnpre_plan_info(plan)["num_segments"], dtype=torch.int64)
+    _check(_lib.gnnpre_plan_hop_order(plan.handle, first.data_ptr()), "gnnpre_plan_hop_order")
+    return first
 
 
 def gnnpre_propagate(plan: Plan, X: torch.Tensor, K: int, out: Sequence[torch.Tensor] | None = None, *,
@@ -438,7 +446,7 @@ def gnnpre_status_string(status: int) -> str:
 
 def exported_symbols():
     return ["gnnpre_degrees", "gnnpre_build_plan", "gnnpre_plan_info", "gnnpre_plan_block", "gnnpre_plan_scales",
-            "gnnpre_plan_support", "gnnpre_propagate", "gnnpre_propagate_weighted", "gnnpre_hop_static", "gnnpre_lc_first_layer", "gnnpre_lc_selftest_wait_timeout", "gnnpre_normalize",
+            "gnnpre_plan_support", "gnnpre_plan_hop_order", "gnnpre_propagate", "gnnpre_propagate_weighted", "gnnpre_hop_static", "gnnpre_lc_first_layer", "gnnpre_lc_selftest_wait_timeout", "gnnpre_normalize",
             "gnnpre_solve_normalisation_blocks", "gnnpre_selftest_wait_timeout", "gnnpre_selftest_wait_timeout_async",
             "gnnpre_plan_status", "gnnpre_inject_alloc_failure", "gnnpre_gather_ceiling", "gnnpre_describe_panels", "gnnpre_plan_destroy", "gnnpre_release_cached_memory", "gnnpre_solve_budget",
             "gnnpre_status_string", "gnnpre_last_cuda_error"]

@@ -352,11 +352,18 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     segs[s] = g;
 }
 
+// Whether all edges of segment s belong to one row (never the last segment: the sentinel has no row); nx_head: the segment
+// after it begins inside a row.
+__device__ __forceinline__ bool inside_one_row(int64_t s, int64_t nseg, const Segment& g, const Segment& nx, bool nx_head) {
+    return s + 1 < nseg && nx.start > g.start && (nx.rank == g.rank || (nx.rank == g.rank + 1 && !nx_head));
+}
+
 // What segment s accounts for: a scratch row if its first row began earlier (head), one if the row of its last edge
 // goes on and began in it (tail), a fix-up if the row that began earlier ends in it.  first[s] = the segment that row
-// began in.
+// began in.  in_edge_order (or nullptr): whether a hop takes the segment in the order of the edge list (see k_segment_order).
 __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs, const int64_t* __restrict__ rowptr_t,
-                                 int32_t hub_parts, SegCounts* __restrict__ counts, int32_t* __restrict__ first) {
+                                 int32_t hub_parts, SegCounts* __restrict__ counts, int32_t* __restrict__ first,
+                                 int32_t* __restrict__ in_edge_order) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     const Segment g = segs[s], nx = segs[s + 1];
@@ -380,11 +387,15 @@ __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs,
         hub = s - lo + 1 > hub_parts;
     }
     counts[s] = {head + tail, emit, hub};
+    if (in_edge_order) in_edge_order[s] = !inside_one_row(s, nseg, g, nx, nx.slot_head);
 }
 
+// by_source (or nullptr): the segments that a hop takes in the order of the edge list go to its end; edge_before[s] of them come
+// before segment s.
 __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, const SegCounts* __restrict__ counts,
                                    const SegCounts* __restrict__ before, const int32_t* __restrict__ first,
-                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs, const int* err) {
+                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs,
+                                   const int32_t* __restrict__ edge_before, Segment* __restrict__ by_source, const int* err) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s > nseg || *err) return;
     if (s < nseg) {
@@ -404,6 +415,7 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
         segs[s].slot_tail = c.slots > head ? b.slots + head : -1;
     }
     segs[s].len = s < nseg ? (int32_t)(segs[s + 1].start - segs[s].start) : 0;
+    if (by_source && s < nseg && edge_before[s] < edge_before[s + 1]) by_source[nseg - edge_before[nseg] + edge_before[s]] = segs[s];
 }
 
 // ---------------------------------------------------------------- the order in which a hop takes its segments
@@ -417,27 +429,45 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
 // 1386 / 1378; 1 M nodes, 30 M edges, GCN, 128 columns 1072 / 1029; 400 K nodes, 40 M edges, sum, 256 columns 2200 / 2090;
 // about the L2's size: 300 K nodes, 40 M edges, GCN, 128 columns 1115 / 1068, 96 columns 997 / 990; well inside it: 169 K
 // nodes, 2.5 M edges, GCN, 128 columns 99 / 102.  Four or eight coarse ranges of columns instead: 3 to 6 % slower.
-__device__ __forceinline__ int order_bucket(const Segment* __restrict__ segs, int64_t s, int64_t nseg,
-                                            const uint32_t* __restrict__ colx, int64_t n) {
-    if (s + 1 >= nseg) return kOrderBuckets;
-    const Segment g = segs[s], nx = segs[s + 1];
-    const bool one_row = nx.rank == g.rank || (nx.rank == g.rank + 1 && nx.slot_head < 0);
-    if (g.len == 0 || !one_row) return kOrderBuckets;
-    return column_bucket(colx[g.start + g.len / 2] & ~kRowEndBit, n);
-}
+//
+// Segments of several rows follow in the order of the edge list: where the caller's numbering has locality (communities, meshes)
+// neighbours read the same part of the matrix.  Where hardly any segment lies in one row, or most that do lie near the
+// diagonal, the table is left out, as they come.  2 M nodes, GCN, 128 columns, us per hop, edge order / several-row segments in
+// order of arrival / so: communities of 20,000, degree 24, 1810 / 3370 / 1790; the same with hubs in each, degree 34, 2280 / 3480 /
+// 2285 (2514 with the one-row segments first); a 27-point mesh 1720 / 2080 / 1700; no locality: R-MAT 3260 / 3060 / 3070,
+// Erdos-Renyi 3770 / 3765 / 3765.
+constexpr int64_t kFewSegments = 64;  // one in so many
 
-// SCATTER false: counts[b] = segments of bucket b.  true: counts[b] holds where the bucket begins; copies the segments there.
+// SCATTER false: counts[b] = segments of bucket b, *near = those whose row lies near their columns.  true: counts[b] holds where
+// the bucket begins; copies the segments there.
 template <bool SCATTER>
-__global__ void k_segment_order(int64_t nseg, const Segment* __restrict__ segs, const uint32_t* __restrict__ colx, int64_t n,
-                                int32_t* __restrict__ counts, Segment* __restrict__ ordered) {
+__global__ void k_segment_order(int64_t nseg, const Segment* __restrict__ segs, const uint32_t* __restrict__ colx,
+                                const int32_t* __restrict__ nzrows, int64_t n, int32_t* __restrict__ counts, int32_t* near,
+                                Segment* __restrict__ ordered, const int* err) {
+    if (*err) return;  // then there is neither a table nor an edge list
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int bucket = s < nseg ? order_bucket(segs, s, nseg, colx, n) : -1;
+    int bucket = -1;
+    bool local = false;
+    Segment g;
+    if (s < nseg) {
+        g = segs[s];
+        const Segment nx = segs[s + 1];
+        if (inside_one_row(s, nseg, g, nx, nx.slot_head >= 0)) {
+            const uint32_t col = colx[g.start + g.len / 2] & ~kRowEndBit;
+            bucket = column_bucket(col, n);
+            if (!SCATTER) local = near_diagonal((uint32_t)(nzrows ? nzrows[g.rank] : g.rank), col, n);
+        }
+    }
     const unsigned same = __match_any_sync(0xffffffffu, bucket);  // one addition per bucket and warp
     const int lane = threadIdx.x & 31, first = __ffs(same) - 1;
     int at = 0;
     if (lane == first && bucket >= 0) at = atomicAdd(&counts[bucket], __popc(same));
     at = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
-    if (SCATTER && bucket >= 0) ordered[at] = segs[s];
+    if (SCATTER && bucket >= 0) ordered[at] = g;
+    if (!SCATTER) {
+        const int locals = __popc(__ballot_sync(0xffffffffu, local));
+        if (lane == 0 && locals > 0) atomicAdd(near, locals);
+    }
 }
 
 // Parts beyond which a cut row counts as a hub and gets a whole CTA of the finishing kernel (64 chains) instead of a
@@ -826,9 +856,11 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // driver mostly has at hand, about 1 us.)  The temporaries of the build live where E goes at the very end,
     // if there is room.
     struct Report {  // followed by BlockRows[b] and SegCounts[b + 1]
-        int32_t err, nonempty, longest_row, unused;
+        int32_t err, nonempty, longest_row;
+        int32_t in_edge_order, near;  // of the segments: see k_segment_order
+        int32_t unused;
     };
-    static_assert(sizeof(Report) == 16 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
+    static_assert(sizeof(Report) % 8 == 0 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
     // (the report has a place of its own: E overwrites the temporaries before the host reads it)
     DevBuf<char> report;
     const size_t report_bytes = sizeof(Report) + sizeof(BlockRows) * (size_t)b + sizeof(SegCounts) * (size_t)(b + 1);
@@ -845,7 +877,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         if (small_report) carve.want(report, report_bytes);
         if (by_source) {
             carve.want(P->by_source, (size_t)nseg);
-            carve.want(P->by_source_counts, 2 * (kOrderBuckets + 1) + 1);
+            carve.want(P->by_source_counts, 2 * kOrderBuckets + 1);
         }
         if (!e_host) carve.want(P->colx, (size_t)m);
     };
@@ -890,7 +922,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
     DevBuf<char> temp_arena;
     if (!small_report) GNNPRE_TRY(report.alloc(report_bytes));
-    DevBuf<int32_t> flag, rank, rank_temp, first;
+    DevBuf<int32_t> flag, rank, rank_temp, first, in_edge_order, edge_before, edge_temp;
     DevBuf<SegCounts> counts, before, counts_temp;
     DevBuf<int64_t> offsets;
     Carve temps;
@@ -904,6 +936,11 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     temps.want(counts, (size_t)nseg);
     temps.want(before, (size_t)nseg + 1);
     temps.want(counts_temp, scan_temp_items(nseg));
+    if (by_source) {
+        temps.want(in_edge_order, (size_t)nseg);
+        temps.want(edge_before, (size_t)nseg + 1);
+        temps.want(edge_temp, scan_temp_items(nseg));
+    }
     if (temps.bytes() <= colx.bytes()) GNNPRE_TRY(temps.place(reinterpret_cast<char*>(colx.p)));
     else GNNPRE_TRY(temps.place(temp_arena));
     Report* d_report = reinterpret_cast<Report*>(report.p);
@@ -959,9 +996,14 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap, uncut,
                                                                   &d_report->longest_row, P->rowptr_t.p, n, rank.p, P->segments.p);
         GNNPRE_CUDA(cudaGetLastError());
-        k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);
+        k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p,
+                                                                in_edge_order.p);
         GNNPRE_CUDA(cudaGetLastError());
         GNNPRE_TRY(exclusive_scan(counts.p, nseg, before.p, counts_temp.p, st));
+        if (by_source) {
+            GNNPRE_TRY(exclusive_scan(in_edge_order.p, nseg, edge_before.p, edge_temp.p, st));
+            GNNPRE_CUDA(cudaMemcpyAsync(&d_report->in_edge_order, edge_before.p + nseg, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        }
         k_block_report<<<grid_for(b + 1, kTB / 32), kTB, 0, st>>>((int)b, d_e_off, d_seg_base, before.p, P->rowptr_t.p, n, d_rows, d_at);
         GNNPRE_CUDA(cudaGetLastError());
     }
@@ -1006,7 +1048,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         return GNNPRE_OK;
     }
     k_segment_finalize<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, P->segments.p, counts.p, before.p, first.p, P->fixups.p,
-                                                                P->hubs.p, &d_report->err);
+                                                                P->hubs.p, edge_before.p, P->by_source.p, &d_report->err);
     GNNPRE_CUDA(cudaGetLastError());
 
     // ---- E, the support's edge list: overwrites the temporaries
@@ -1018,6 +1060,14 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         const int64_t row_blocks = diag ? (n + kTB - 1) / kTB : 0;
         k_support<<<(unsigned)(edge_blocks + row_blocks), kTB, 0, st>>>(diag ? 1 : 0, check ? 1 : 0, n, nnz, per_warp, edge_blocks,
                                                                        d_rowptr, d_colidx, colx.p, &d_report->err);
+        GNNPRE_CUDA(cudaGetLastError());
+    }
+    int32_t *bucket_counts = P->by_source_counts.p, *bucket_begins = bucket_counts + kOrderBuckets;
+    const int32_t* row_of_rank = diag ? nullptr : P->nzrows.p;  // (nullptr as well where every row has edges)
+    if (by_source) {
+        GNNPRE_CUDA(cudaMemsetAsync(bucket_counts, 0, sizeof(int32_t) * kOrderBuckets, st));
+        k_segment_order<false><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, bucket_counts,
+                                                                    &d_report->near, nullptr, &d_report->err);
         GNNPRE_CUDA(cudaGetLastError());
     }
     GNNPRE_TRY(read_report());  // everything is in place
@@ -1040,15 +1090,17 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         B.done_row_hi = l == b - 1 ? n : r.done_row_hi;
     }
     if (by_source) {
-        int32_t *counts = P->by_source_counts.p, *begins = counts + kOrderBuckets + 1;
-        GNNPRE_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * (kOrderBuckets + 1), st));
-        k_segment_order<false><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, n, counts, nullptr);
-        GNNPRE_CUDA(cudaGetLastError());
-        static_assert(kOrderBuckets + 1 <= kScanTile, "the scan needs no temporary memory");
-        GNNPRE_TRY(exclusive_scan<int32_t>(counts, kOrderBuckets + 1, begins, nullptr, st));
-        k_segment_order<true><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, n, begins, P->by_source.p);
-        GNNPRE_CUDA(cudaGetLastError());
-        GNNPRE_CUDA(cudaStreamSynchronize(st));
+        const int64_t one_row = nseg - rep->in_edge_order;
+        if (one_row * kFewSegments >= nseg && 2 * (int64_t)rep->near <= one_row) {
+            static_assert(kOrderBuckets <= kScanTile, "the scan needs no temporary memory");
+            GNNPRE_TRY(exclusive_scan<int32_t>(bucket_counts, kOrderBuckets, bucket_begins, nullptr, st));
+            k_segment_order<true><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, bucket_begins,
+                                                                       nullptr, P->by_source.p, &d_report->err);
+            GNNPRE_CUDA(cudaGetLastError());
+            GNNPRE_CUDA(cudaStreamSynchronize(st));
+        } else {
+            P->by_source.reset();  // the segments stay as they are
+        }
     }
 
     // ---- a host-resident structure keeps E in pinned memory and streams it block by block
@@ -1162,6 +1214,15 @@ extern "C" int gnnpre_plan_block(const gnnpre_plan_t* P, int32_t l, gnnpre_block
     o->row_hi = B.row_hi;
     o->first_row_partial = B.first_partial;
     o->last_row_partial = B.last_partial;
+    return GNNPRE_OK;
+}
+
+extern "C" int gnnpre_plan_hop_order(const gnnpre_plan_t* P, int64_t* first_edges_out) {
+    if (!P || !first_edges_out) return GNNPRE_ERR_INVALID_ARG;
+    if (P->num_segments == 0) return GNNPRE_OK;
+    const Segment* segments = P->by_source.p ? P->by_source.p : P->segments.p;
+    GNNPRE_CUDA(cudaMemcpy2D(first_edges_out, sizeof(int64_t), &segments->start, sizeof(Segment), sizeof(int64_t),
+                             (size_t)P->num_segments, cudaMemcpyDeviceToHost));
     return GNNPRE_OK;
 }
 

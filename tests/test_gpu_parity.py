@@ -436,6 +436,36 @@ def test_segments_in_the_order_of_their_sources_give_the_same_bits(B, op, graph,
 
 
 @pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("seg", [32, 200])
+@pytest.mark.parametrize("graph", ["hubs", "no hubs", "numbered"])
+def test_segments_of_several_rows_stay_in_the_order_of_the_edge_list(B, op, graph, seg):
+    """Over a matrix beyond the L2 a hop takes the segments inside one row first, by their middle columns, and the others as the
+    edge list has them; all of them so where hardly any lies in one row (no hubs) or those that do read rows numbered like
+    their own (hubs of their neighbours): a caller's numbering keeps its locality."""
+    n, F = 300000, 128
+    g = {"hubs": lambda: gi.rmat(n, 3000000, 41, directed_candidates=False, device="cuda"), "no hubs": lambda: gi.erdos_renyi(n, 700000, 42, device="cuda"),
+         "numbered": lambda: gi.from_edge_list(n, [(i - i % 1000, i) for i in range(n) if i % 1000], device="cuda")}[graph]()
+    plan = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, gin_eps=EPS, segment_edges=seg, force_blocks=1, force_col_slabs=1)
+    order = B.gnnpre_plan_hop_order(plan).numpy()
+    rp, ci = (t.numpy() for t in B.gnnpre_plan_support(plan))
+    plan.close()
+    lo = np.sort(order)
+    if graph != "hubs":
+        assert np.array_equal(order, lo)
+        return
+    hi = np.append(lo[1:], len(ci))
+    row_of = lambda e: np.searchsorted(rp, e, side="right") - 1
+    one_row = (hi > lo) & (hi < len(ci)) & (row_of(lo) == row_of(np.maximum(hi - 1, 0)))
+    first = int(one_row.sum())
+    assert len(lo) // 64 < first < len(lo)
+    assert np.array_equal(order[first:], lo[~one_row])
+    assert np.array_equal(np.sort(order[:first]), lo[one_row])
+    middle = dict(zip(lo[one_row], ci[(lo + (hi - lo) // 2)[one_row]]))
+    buckets = np.array([int(middle[e]) * 1024 // n for e in order[:first]])
+    assert (np.diff(buckets) >= 0).all() and buckets[-1] > buckets[0]
+
+
+@pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("F", [16, 32, 64, 128])
 @pytest.mark.parametrize("m", [3000, 80000, 330000])
 def test_segments_of_a_small_graph_fill_whole_waves(B, op, F, m):

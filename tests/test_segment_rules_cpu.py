@@ -10,6 +10,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SHIM = r"""
 #include "segment_rules.h"
 extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
+extern "C" int near_diagonal(uint32_t row, uint32_t col, int64_t n) { return gnnpre::near_diagonal(row, col, n); }
 extern "C" int order_buckets() { return gnnpre::kOrderBuckets; }
 """
 
@@ -22,6 +23,7 @@ def rules(tmp_path_factory):
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
+    lib.near_diagonal.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int64]
     return lib
 
 
@@ -34,3 +36,12 @@ def test_buckets_of_columns_stay_in_range_whatever_the_column(rules, n):
         assert rules.column_bucket(col, n) == col * B // n < B
     for col in (n, n + 1, 2 * n, 2 ** 31 - 1):
         assert rules.column_bucket(min(col, 2 ** 31 - 1), n) == B - 1
+
+
+def test_near_the_diagonal_is_a_thirty_second_of_all_rows(rules):
+    n = 1024 * 100
+    for row in (0, 50000, n - 1):
+        for apart, near in ((0, 1), (3199, 1), (3400, 0), (60000, 0)):
+            for col in (row - apart, row + apart):
+                if 0 <= col < n:
+                    assert rules.near_diagonal(row, col, n) == near
