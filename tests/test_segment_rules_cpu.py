@@ -11,6 +11,9 @@ SHIM = r"""
 #include "segment_rules.h"
 extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
 extern "C" int near_diagonal(uint32_t row, uint32_t col, int64_t n) { return gnnpre::near_diagonal(row, col, n); }
+extern "C" int auto_segment_edges(int64_t width, int64_t m, int bulk_copy, int beyond, int whole_hops, int num_sms) {
+    return gnnpre::auto_segment_edges(width, m, bulk_copy, beyond, whole_hops, num_sms);
+}
 extern "C" int order_buckets() { return gnnpre::kOrderBuckets; }
 """
 
@@ -23,6 +26,7 @@ def rules(tmp_path_factory):
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
+    lib.auto_segment_edges.argtypes = [ctypes.c_int64, ctypes.c_int64] + [ctypes.c_int] * 4
     lib.near_diagonal.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int64]
     return lib
 
@@ -45,3 +49,15 @@ def test_near_the_diagonal_is_a_thirty_second_of_all_rows(rules):
             for col in (row - apart, row + apart):
                 if 0 <= col < n:
                     assert rules.near_diagonal(row, col, n) == near
+
+
+SMS = 148
+
+
+@pytest.mark.parametrize("width,m,want", [
+    (500, 13264, 16), (500, 10556, 16), (256, 7000, 16), (132, 28000, 16),  # all tiles' segments of 16 edges at once
+    (500, 24400, 32), (1433, 13264, 32), (3703, 13264, 32),                 # several waves of them
+])
+def test_small_graphs_of_several_column_tiles(rules, width, m, want):
+    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 0, 0, 1, SMS) == want
+    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 0, 0, 0, SMS) == 32  # a launch of one block
