@@ -789,7 +789,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const int64_t m_launch = per_block ? m / b : m;
     P->segment_edges = opts->segment_edges > 0
                            ? opts->segment_edges
-                           : auto_segment_edges(P->slab_width, m_launch, uses_bulk_copy(P, (int32_t)P->slab_width),
+                           : auto_segment_edges(P->slab_width, m_launch, per_block ? 1 : b, uses_bulk_copy(P, (int32_t)P->slab_width),
                                                 beyond_cache(P, (int32_t)P->slab_width), !per_block, P->num_sms);
     if (P->segment_edges < 1) return GNNPRE_ERR_INVALID_ARG;
 

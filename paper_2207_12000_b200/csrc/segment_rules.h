@@ -28,9 +28,16 @@ GNNPRE_HOST_DEVICE inline bool near_diagonal(uint32_t row, uint32_t col, int64_t
     return apart <= kOrderBuckets / 32 && apart >= -kOrderBuckets / 32;
 }
 
-// Edges per segment of a plan that was not given any.  m: edges that one launch covers; bulk_copy: summed by the bulk-copy kernel;
+// Segments of `edges` edges in m edges cut into `blocks` blocks: block l holds the edges [floor(l m / blocks),
+// floor((l + 1) m / blocks)), that is, m mod blocks of them one more than the others.
+inline int64_t count_segments(int64_t m, int64_t blocks, int64_t edges) {
+    const int64_t q = m / blocks, longer = m % blocks;
+    return (blocks - longer) * ((q + edges - 1) / edges) + longer * ((q + edges) / edges);
+}
+
+// Edges per segment of a plan that was not given any.  m: edges that one launch covers, in how many blocks; bulk_copy: summed by the bulk-copy kernel;
 // beyond: the rows gathered from are more than the L2 holds; whole_hops: one launch covers a hop.
-inline int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy, bool beyond, bool whole_hops, int num_sms) {
+inline int32_t auto_segment_edges(int64_t slab_width, int64_t m, int64_t blocks, bool bulk_copy, bool beyond, bool whole_hops, int num_sms) {
     if (bulk_copy) {
         // persistent warps walk whole segments with a two-stage pipeline that drains at every segment end: long segments, but
         // at least ~4 per resident warp so the tail stays short, and short enough that half the edges lie in segments of a
@@ -53,10 +60,14 @@ inline int32_t auto_segment_edges(int64_t slab_width, int64_t m, bool bulk_copy,
     // 132.3 / 125.8 (four); 24 M, 16 columns 209 / 198 (four).  Where the epilogue reads rows too, long segments are uneven: 64
     // columns, 2.4 M edges, ten hops with a teleport term and their sum 1155 at 80 edges, 1241 in one wave; 128 columns, 1.2 M
     // edges 843 at 64, 888 at 160, and without the epilogue 170 / 162; so those stay at 96 edges, and at one wave of 160.
+    // Every edge block ends with a segment of its own, so the segments are counted: where a longer one makes the wave whole it is
+    // taken, else one more wave.  GCN, 256 blocks, us for two hops, blocks not counted / counted: 150,000 nodes, 2.3 M edges, 32 columns
+    // 90.4 / 81.9; 56,000 nodes, 870,000 edges, 32 columns 40.7 / 38.9, 64 columns 56.5 / 57.0.
     if (whole_hops && !beyond && slab_width <= 128) {
-        const int64_t most = lanes == 4 ? 192 : lanes == 16 ? 96 : 160, waves = per_group / most + 1;
-        const int64_t whole = waves <= (lanes == 32 ? 1 : 4) ? waves : 0;
-        if (whole > 0) return (int32_t)std::max<int64_t>(16, (m / (groups * whole) + 8) / 8 * 8);
+        const int64_t most = lanes == 4 ? 192 : lanes == 16 ? 96 : 160;
+        for (int64_t waves = per_group / most + 1; waves <= (lanes == 32 ? 1 : 4); ++waves)
+            for (int64_t L = std::max<int64_t>(16, (m / (groups * waves) + 8) / 8 * 8); L <= most; L += 8)
+                if (count_segments(m, blocks, L) <= groups * waves) return (int32_t)L;
     }
     // Wider rows are several column tiles in one launch.  Where all tiles' segments of 16 edges run at once the hop is a chain of
     // latencies, and it takes those; else 32 at least.  us per hop at 16 / 32 edges, GCN and mean: 2,700 nodes, 10,600 edges, 500

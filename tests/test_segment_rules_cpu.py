@@ -11,9 +11,10 @@ SHIM = r"""
 #include "segment_rules.h"
 extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
 extern "C" int near_diagonal(uint32_t row, uint32_t col, int64_t n) { return gnnpre::near_diagonal(row, col, n); }
-extern "C" int auto_segment_edges(int64_t width, int64_t m, int bulk_copy, int beyond, int whole_hops, int num_sms) {
-    return gnnpre::auto_segment_edges(width, m, bulk_copy, beyond, whole_hops, num_sms);
+extern "C" int auto_segment_edges(int64_t width, int64_t m, int64_t blocks, int bulk_copy, int beyond, int whole_hops, int num_sms) {
+    return gnnpre::auto_segment_edges(width, m, blocks, bulk_copy, beyond, whole_hops, num_sms);
 }
+extern "C" int64_t count_segments(int64_t m, int64_t blocks, int64_t edges) { return gnnpre::count_segments(m, blocks, edges); }
 extern "C" int order_buckets() { return gnnpre::kOrderBuckets; }
 """
 
@@ -26,7 +27,8 @@ def rules(tmp_path_factory):
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
-    lib.auto_segment_edges.argtypes = [ctypes.c_int64, ctypes.c_int64] + [ctypes.c_int] * 4
+    lib.auto_segment_edges.argtypes = [ctypes.c_int64] * 3 + [ctypes.c_int] * 4
+    lib.count_segments.argtypes, lib.count_segments.restype = [ctypes.c_int64] * 3, ctypes.c_int64
     lib.near_diagonal.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int64]
     return lib
 
@@ -59,5 +61,25 @@ SMS = 148
     (500, 24400, 32), (1433, 13264, 32), (3703, 13264, 32),                 # several waves of them
 ])
 def test_small_graphs_of_several_column_tiles(rules, width, m, want):
-    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 0, 0, 1, SMS) == want
-    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 0, 0, 0, SMS) == 32  # a launch of one block
+    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 1, 0, 0, 1, SMS) == want
+    assert rules.auto_segment_edges((width + 3) // 4 * 4, m, 1, 0, 0, 0, SMS) == 32  # a launch of one block
+
+
+@pytest.mark.parametrize("m,blocks,edges", [(1, 1, 16), (100, 7, 16), (1000, 32, 31), (1000, 1000, 8), (123457, 256, 40)])
+def test_segments_of_all_blocks_are_counted(rules, m, blocks, edges):
+    ends = [l * m // blocks for l in range(blocks + 1)]
+    assert rules.count_segments(m, blocks, edges) == sum(-(-(hi - lo) // edges) for lo, hi in zip(ends, ends[1:]))
+
+
+@pytest.mark.parametrize("blocks", [1, 4, 32, 256])
+@pytest.mark.parametrize("width,most_edges,most_waves", [(16, 192, 4), (32, 160, 4), (64, 96, 4), (128, 160, 1)])
+def test_whole_waves_count_the_blocks(rules, width, most_edges, most_waves, blocks):
+    """Segments of a whole hop over few waves: as many waves as the longest segments need, none nearly empty, the shortest such."""
+    groups = SMS * 28 * 32 // (width // 4)
+    for m in range(50_000, groups * most_edges * most_waves, 7919):
+        got = rules.auto_segment_edges(width, m, blocks, 0, 0, 1, SMS)
+        waves = -(-rules.count_segments(m, blocks, got) // groups)
+        fewest = next((w for w in range(1, most_waves + 1) if rules.count_segments(m, blocks, most_edges) <= groups * w), None)
+        if fewest is not None:
+            assert got % 8 == 0 and 16 <= got <= most_edges and waves == fewest, m
+            assert got == 16 or rules.count_segments(m, blocks, got - 8) > groups * waves or m >= groups * waves * (got - 8), m
