@@ -36,16 +36,18 @@ inline int64_t count_segments(int64_t m, int64_t blocks, int64_t edges) {
 }
 
 // Edges per segment of a plan that was not given any.  m: edges that one launch covers, in how many blocks; bulk_copy: summed by the bulk-copy kernel;
-// beyond: the rows gathered from are more than the L2 holds; whole_hops: one launch covers a hop.
+// beyond: the rows gathered from are on the device and more than the L2 holds (a streamed plan waits for the host's link and keeps
+// the longer segments, which need fewer scratch rows); whole_hops: one launch covers a hop.
 inline int32_t auto_segment_edges(int64_t slab_width, int64_t m, int64_t blocks, bool bulk_copy, bool beyond, bool whole_hops, int num_sms) {
     if (bulk_copy) {
         // persistent warps walk whole segments with a two-stage pipeline that drains at every segment end: long segments, but
         // at least ~4 per resident warp so the tail stays short, and short enough that half the edges lie in segments of a
         // single row (k_segment_order; 124 M edges, 100 columns, us per hop at 256 / 512 / 1024 / 2048 edges
-        // 3843 / 3651 / 3637 / 3745)
+        // 3843 / 3651 / 3637 / 3745; without such rows, 90 M edges, 6365 at 1024 and 6260 at 4096).  Blocks launched singly gain
+        // as much by the shorter tail (124 M edges in one block 4410 at 4096 and 4425 at 1024, in two 4890 and 4445).
         const int64_t per_warp = m / ((int64_t)std::max(num_sms, 1) * 16 * 4);
         int32_t p = 256;
-        while ((int64_t)p * 2 <= per_warp && p < 1024) p *= 2;
+        while ((int64_t)p * 2 <= per_warp && p < (beyond ? 1024 : 4096)) p *= 2;
         return p;
     }
     const int64_t f4 = std::min<int64_t>(std::max<int64_t>(slab_width, 4), 128) / 4;
@@ -81,7 +83,8 @@ inline int32_t auto_segment_edges(int64_t slab_width, int64_t m, int64_t blocks,
     // group remain (23 M edges, 128 columns: 829 / 744 / 702 us at 64 / 128 / 256, as fast at 1024; 12.8 M edges: 531 at 256,
     // 583 at 1024): what longer segments save there is tables and scratch rows.  Up to 512 for a matrix beyond the L2, where
     // segments of a single row are the better ones (124 M edges, 100 columns, at 128 / 256 / 512 / 1024 edges
-    // 4008 / 3898 / 3870 / 3950; GCN, 128 columns 4434 / 4331 / 4295).
+    // 4008 / 3898 / 3870 / 3950; GCN, 128 columns 4434 / 4331 / 4295), and blocks launched singly end sooner (GCN, 128 columns, two
+    // blocks, 124 M edges 5460 at 1024 and 5330 at 512).
     const int64_t L = std::max(std::min<int64_t>(per_group / (lanes <= 8 ? 2 : 3), 256), per_group / 8);
     int32_t p = 32;
     while ((int64_t)p * 2 <= L && p < (beyond ? 512 : 1024)) p *= 2;

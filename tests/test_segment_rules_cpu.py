@@ -83,3 +83,12 @@ def test_whole_waves_count_the_blocks(rules, width, most_edges, most_waves, bloc
         if fewest is not None:
             assert got % 8 == 0 and 16 <= got <= most_edges and waves == fewest, m
             assert got == 16 or rules.count_segments(m, blocks, got - 8) > groups * waves or m >= groups * waves * (got - 8), m
+
+
+@pytest.mark.parametrize("bulk_copy", [0, 1])
+def test_long_segments_where_the_order_of_the_sources_is_not_used(rules, bulk_copy):
+    """124 M edges in one launch over a matrix beyond the L2: shorter segments where more of them then lie in one row; streamed
+    plans (for which the rule is told that nothing is beyond the L2) keep the long ones."""
+    for width in (72, 100, 124):
+        assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 1, 1, SMS) == (1024 if bulk_copy else 512)
+        assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 0, 0, SMS) == (4096 if bulk_copy else 1024)
