@@ -43,6 +43,7 @@
 #include <cuda.h>
 
 #include "gnnpre_internal.cuh"
+#include "lc_rules.h"
 
 namespace gnnpre {
 namespace {
@@ -621,7 +622,7 @@ __device__ __forceinline__ void lc_store_low_part(const uint32_t (&v)[4], uint32
                  : "memory");
 }
 
-template <bool PAIR>
+template <bool PAIR, bool AHEAD>
 __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __grid_constant__ LcMaps maps, const LcArgs a) {
     extern __shared__ unsigned char lc_smem[];
     __shared__ __align__(8) unsigned long long bars[3 * kLcMaxStages + 8];
@@ -744,6 +745,16 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
+        // AHEAD: a tile's rows of the hop matrix (-1: none) are asked for while the tile before it is copied.
+        int row_of[8];
+        auto ask_rows = [&](int t) {
+            const int64_t pos0 = (int64_t)(t % a.tiles_m) * tile_rows + rank_row + row0;
+            const int left = (int)min(a.batch_size - pos0, (int64_t)32);
+            const int32_t* const at = a.batch + pos0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) row_of[i] = 4 * i >= left ? -1 : a.batch ? __ldg(at + 4 * i) : (int)pos0 + 4 * i;
+        };
+        if (AHEAD) ask_rows(first);
         for (int t = first; t < total_tiles && ok; t += step) {
             const int hop = t / a.tiles_m, mt = t - hop * a.tiles_m;
             const float* src_row[8];
@@ -751,9 +762,11 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
             for (int i = 0; i < 8; ++i) {
                 const int64_t pos = mt * tile_rows + rank_row + row0 + 4 * i;
                 int64_t r = -1;
-                if (pos < a.batch_size) r = a.batch ? (int64_t)__ldg(a.batch + pos) : pos;
+                if (AHEAD) r = row_of[i];
+                else if (pos < a.batch_size) r = a.batch ? (int64_t)__ldg(a.batch + pos) : pos;
                 src_row[i] = (r >= 0 && r < a.n) ? a.hop[hop] + r * a.ldh : nullptr;
             }
+            if (AHEAD && t + step < total_tiles) ask_rows(t + step);
             for (int kc = 0; kc < a.k_chunks; ++kc) {
                 if (!lc_wait(empty_bar(s), ph ^ 1u, abort_flag, a.error, a.spin_limit)) {
                     ok = false;
@@ -973,13 +986,15 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     w_off = (uint32_t)stages * stage_stride;
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
     const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
-    auto kernel = pair ? k_lc_first_layer_x3<true> : x3 ? k_lc_first_layer_x3<false> : k_lc_first_layer;
+    const bool ahead = x3 && !pair && rows_asked_ahead(k_chunks, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms / halves);
+    auto kernel = pair ? k_lc_first_layer_x3<true, false> : ahead ? k_lc_first_layer_x3<false, true> : x3 ? k_lc_first_layer_x3<false, false> : k_lc_first_layer;
+    const int which = pair ? 3 : ahead ? 2 : x3 ? 1 : 0;
     // the opt-in to large dynamic shared memory, per kernel and device: always the most a launch can want, so once is enough
     constexpr int kMostSmem = 1024 + kLcPipeBytes + 8 * kLcEpiBytes;
-    static std::atomic<bool> opted_in[3][kLcMaxDevices];
-    if (dev >= kLcMaxDevices || !opted_in[x3 + pair][dev].load(std::memory_order_relaxed)) {
+    static std::atomic<bool> opted_in[4][kLcMaxDevices];
+    if (dev >= kLcMaxDevices || !opted_in[which][dev].load(std::memory_order_relaxed)) {
         GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
-        if (dev < kLcMaxDevices) opted_in[x3 + pair][dev].store(true, std::memory_order_relaxed);
+        if (dev < kLcMaxDevices) opted_in[which][dev].store(true, std::memory_order_relaxed);
     }
 
     LcMaps maps;

@@ -1,4 +1,4 @@
-"""The rules of plan construction in csrc/segment_rules.h, compiled for the CPU."""
+"""The rules of plan construction (csrc/segment_rules.h) and of the first dense stage (csrc/lc_rules.h), compiled for the CPU."""
 import ctypes
 import os
 import subprocess
@@ -9,6 +9,8 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 SHIM = r"""
 #include "segment_rules.h"
+#include "lc_rules.h"
+extern "C" int rows_asked_ahead(int k_chunks, int64_t tiles, int64_t ctas) { return gnnpre::rows_asked_ahead(k_chunks, tiles, ctas); }
 extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
 extern "C" int near_diagonal(uint32_t row, uint32_t col, int64_t n) { return gnnpre::near_diagonal(row, col, n); }
 extern "C" int auto_segment_edges(int64_t width, int64_t m, int64_t blocks, int bulk_copy, int beyond, int whole_hops, int num_sms) {
@@ -28,6 +30,7 @@ def rules(tmp_path_factory):
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
     lib.auto_segment_edges.argtypes = [ctypes.c_int64] * 3 + [ctypes.c_int] * 4
+    lib.rows_asked_ahead.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int64]
     lib.count_segments.argtypes, lib.count_segments.restype = [ctypes.c_int64] * 3, ctypes.c_int64
     lib.near_diagonal.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int64]
     return lib
@@ -92,3 +95,9 @@ def test_long_segments_where_the_order_of_the_sources_is_not_used(rules, bulk_co
     for width in (72, 100, 124):
         assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 1, 1, SMS) == (1024 if bulk_copy else 512)
         assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 0, 0, SMS) == (4096 if bulk_copy else 1024)
+
+
+@pytest.mark.parametrize("k_chunks,per_cta", [(1, 4), (3, 4), (4, 8), (19, 8)])
+def test_row_numbers_are_asked_for_ahead_where_a_cta_has_many_tiles(rules, k_chunks, per_cta):
+    for ctas in (74, 148):
+        assert rules.rows_asked_ahead(k_chunks, per_cta * ctas, ctas) and not rules.rows_asked_ahead(k_chunks, per_cta * ctas - 1, ctas)
