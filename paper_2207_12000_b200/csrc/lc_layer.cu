@@ -974,12 +974,7 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         const uint32_t w_part = (uint32_t)n_half * 128u;
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
-        // Hidden > 128, many tiles: pairs of CTAs that gather each row once (and stream the weight half as often) instead of CTAs
-        // that take a column half each.  A tile of a pair takes longer, so a few tiles are slower.  us, halves / pairs, hidden
-        // 256, at 157 / 626 / 1250 tiles of 128 rows x hops: F = 100 (resident weight) 20.1 / 24.8, 43.3 / 45.2, 75.7 / 73.0;
-        // F = 160 (streamed) 23.4 / 26.7, 55.5 / 52.9, 107 / 96; F = 256 31.1 / 34.8, 82.8 / 73.6, 160 / 137; F = 602
-        // 61.5 / 65.6, 191 / 162, 379 / 310.
-        pair = halves == 2 && std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m >= (resident ? 8 : 4) * (int64_t)num_sms;
+        pair = pairs_of_ctas(hidden, k_chunks, resident, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms);
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + 2u * w_part;
         stages = (int32_t)std::min<int64_t>(pair ? kLcPairStages : kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     }

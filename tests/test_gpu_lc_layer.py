@@ -102,21 +102,29 @@ def test_normal_inputs_within_the_bound_of_the_precision(B, n, F, H, bs, K, prec
         assert np.abs(got - want).max() < 0.01 * np.abs(want).max()
 
 
-PAIR_SHAPES = [  # split operands, hidden > 128, enough tiles of 128 rows (4 times the SMs, 8 times with a resident weight) for pairs of CTAs
-    (3000, 200, 192, 592 * 128 + 1, 2),  # accumulators of 96 columns; the last tile has one row, its second CTA none
-    (900, 300, 256, 50600, 3),           # the second CTA of the last tile has 40 rows
-    (66400, 104, 256, None, 3),          # no batch; resident weight
-    (3000, 33, 192, 518 * 128 + 1, 3),   # resident weight, a last chunk of one feature
+PAIR_SHAPES = [  # split operands, hidden > 128, enough features and tiles of 128 rows for pairs of CTAs (see tiles_for_pairs)
+    (3000, 200, 192, 592 * 128 + 1, 2),   # accumulators of 96 columns; the last tile has one row, its second CTA none
+    (900, 300, 256, 50600, 3),            # the second CTA of the last tile has 40 rows
+    (75900, 104, 256, None, 3),           # no batch; resident weight
+    (3000, 65, 192, 1184 * 128 + 1, 3),   # resident weight, a last chunk of one feature; three chunks, four
+    (3000, 97, 192, 518 * 128 + 1, 3),
 ]
+HALVES_SHAPES = [(3000, 33, 192, 518 * 128 + 1, 3), (3000, 66, 256, 592 * 128 + 1, 3), (66400, 104, 256, None, 3)]  # and too few for them
 
 
-@pytest.mark.parametrize("n,F,H,bs,K", PAIR_SHAPES)
+def tiles_for_pairs(F, H):
+    """Tiles times hops from which pairs of CTAs are the faster form, per SM."""
+    return float("inf") if F <= 64 or (F <= 96 and H > 192) else 24 if F <= 96 else 4 if F > 160 or (F > 128 and H > 192) else 12 if H > 192 else 8
+
+
+@pytest.mark.parametrize("n,F,H,bs,K", PAIR_SHAPES + HALVES_SHAPES)
 def test_pairs_of_ctas_on_one_tile(B, n, F, H, bs, K):
-    """Exact on integers (every hop against plain tf32, which is exact there too, two against the oracle), and the bound of the
-    precision on normal inputs (as above)."""
+    """Many tiles of hidden > 128, by pairs of CTAs and by column halves.  Exact on integers (every hop against plain tf32, which is
+    exact there too, two against the oracle), and the bound of the precision on normal inputs (as above)."""
     rng = np.random.default_rng(n + F)
     rows = n if bs is None else bs
-    assert K * -(-rows // 128) >= (8 if F <= 128 else 4) * torch.cuda.get_device_properties(0).multi_processor_count
+    pairs = K * -(-rows // 128) >= tiles_for_pairs(F, H) * torch.cuda.get_device_properties(0).multi_processor_count
+    assert pairs == ((n, F, H, bs, K) in PAIR_SHAPES)
     batch_np = None if bs is None else rng.integers(0, n, size=bs)
     batch = None if bs is None else torch.from_numpy(batch_np.astype(np.int32)).cuda()
     hops_np, Wt_np = [integer_matrix(n, F, 500 + k, -7, 7) for k in range(K)], integer_matrix(H, F, 17, -5, 5)

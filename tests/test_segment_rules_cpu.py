@@ -11,6 +11,9 @@ SHIM = r"""
 #include "segment_rules.h"
 #include "lc_rules.h"
 extern "C" int rows_asked_ahead(int k_chunks, int64_t tiles, int64_t ctas) { return gnnpre::rows_asked_ahead(k_chunks, tiles, ctas); }
+extern "C" int pairs_of_ctas(int64_t hidden, int k_chunks, int resident, int64_t tiles, int num_sms) {
+    return gnnpre::pairs_of_ctas(hidden, k_chunks, resident, tiles, num_sms);
+}
 extern "C" int column_bucket(uint32_t col, int64_t n) { return gnnpre::column_bucket(col, n); }
 extern "C" int near_diagonal(uint32_t row, uint32_t col, int64_t n) { return gnnpre::near_diagonal(row, col, n); }
 extern "C" int auto_segment_edges(int64_t width, int64_t m, int64_t blocks, int bulk_copy, int beyond, int whole_hops, int num_sms) {
@@ -30,6 +33,7 @@ def rules(tmp_path_factory):
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.column_bucket.argtypes = [ctypes.c_uint32, ctypes.c_int64]
     lib.auto_segment_edges.argtypes = [ctypes.c_int64] * 3 + [ctypes.c_int] * 4
+    lib.pairs_of_ctas.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int64, ctypes.c_int]
     lib.rows_asked_ahead.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int64]
     lib.count_segments.argtypes, lib.count_segments.restype = [ctypes.c_int64] * 3, ctypes.c_int64
     lib.near_diagonal.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int64]
@@ -95,6 +99,19 @@ def test_long_segments_where_the_order_of_the_sources_is_not_used(rules, bulk_co
     for width in (72, 100, 124):
         assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 1, 1, SMS) == (1024 if bulk_copy else 512)
         assert rules.auto_segment_edges(width, 123718280, 1, bulk_copy, 0, 0, SMS) == (4096 if bulk_copy else 1024)
+
+
+@pytest.mark.parametrize("hidden,features,resident,per_sm", [
+    (256, 16, 1, None), (192, 64, 1, None), (256, 96, 1, None), (128, 256, 1, None),  # never: few features; one half only
+    (192, 65, 1, 24), (192, 96, 1, 24), (256, 97, 1, 12), (192, 97, 1, 8), (192, 160, 1, 8),
+    (256, 129, 0, 4), (192, 161, 0, 4), (256, 602, 0, 4),
+])
+def test_pairs_of_ctas_from_as_many_tiles_as_make_them_faster(rules, hidden, features, resident, per_sm):
+    pairs = lambda tiles: rules.pairs_of_ctas(hidden, -(-features // 32), resident, tiles, SMS)
+    if per_sm is None:
+        assert not pairs(SMS * 10_000)
+    else:
+        assert pairs(SMS * per_sm) and not pairs(SMS * per_sm - 1)
 
 
 @pytest.mark.parametrize("k_chunks,per_cta", [(1, 4), (3, 4), (4, 8), (19, 8)])
