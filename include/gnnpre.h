@@ -383,11 +383,12 @@ int gnnpre_lc_first_layer(const float* const* hops, int32_t num_hops, int64_t n,
                           int32_t* error_flag, void* stream);
 
 /*
- * Failure-detection self-test of gnnpre_lc_first_layer's kernel: one launch (one tile of up to 128 rows of `hop`,
- * tf32 mode) in which the producer warps never announce a chunk, so that every bounded wait of the kernel gives up
- * after `polls` polls (1..100000; a poll parks the warp for at most 20 us).  The kernel must raise the error word,
+ * Failure-detection self-test of gnnpre_lc_first_layer's kernels: launches (one tile of up to 128 rows of `hop`) of every
+ * form that `hidden` allows - tf32; split operands; pairs of CTAs, too - in which nobody hears of the copies that have landed
+ * (of a pair: neither CTA, the first, the second), so that every bounded wait of the kernel gives up
+ * after `polls` polls (1..100000; a poll parks the warp for at most 20 us).  A kernel must raise the error word,
  * let its copies land, free its tensor memory and return; the call synchronises the stream and returns
- * GNNPRE_ERR_TIMEOUT when the error word was raised (the expected outcome), GNNPRE_OK otherwise.  No wait is
+ * GNNPRE_ERR_TIMEOUT when each launch raised the error word (the expected outcome), GNNPRE_OK otherwise.  No wait is
  * unbounded and nothing faults: the device stays usable and a following gnnpre_lc_first_layer call must succeed.
  * Arguments as for gnnpre_lc_first_layer (device pointers; error_flag required; Y receives nothing meaningful).
  */

@@ -35,7 +35,9 @@
 //
 // Every wait is bounded.  A wait that runs out raises the CTA's abort flag and the caller's error
 // word; every role then leaves its loop, the producers wait for the copies they still have in
-// flight, the MMA lane waits (bounded) for the tensor core to drain, and tensor memory is freed.
+// flight, the MMA warp waits (bounded) for the tensor core to drain, and tensor memory is freed.  Of a pair of
+// CTAs each has its flag and learns by its own limits that the other has given up; the cluster barrier before
+// they leave has no limit of its own, but all that its arrivals wait for has.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
@@ -100,7 +102,7 @@ struct LcArgs {
     int64_t ldw;
     int32_t halves;        // column parts: CTAs with blockIdx.x % halves == h compute columns [h n_half, (h + 1) n_half)
     int32_t n_half;
-    // failure-detection self-test: the producers never announce a chunk, so every wait runs out
+    // failure-detection self-test: copies that have landed are not announced, so every wait runs out (see LcSelfTest)
     int32_t drop_announcements;
     uint32_t spin_limit;   // polls before a wait gives up
 };
@@ -650,7 +652,8 @@ __global__ void __launch_bounds__(kLcX3Threads, 1) k_lc_first_layer_x3(const __g
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kLcMaxStages; ++s) {
-            lc_mbar_init(copied_bar(s), kLcProducerThreads);
+            // (the self-test: one arrival that never comes)
+            lc_mbar_init(copied_bar(s), kLcProducerThreads + (a.drop_announcements == 1 || a.drop_announcements == 2 + rank ? 1 : 0));
             lc_mbar_init(full_bar(s), kCtas * kLcX3SplitWarps);  // a stage's low parts are there as well
             lc_mbar_init(empty_bar(s), 1);
         }
@@ -920,11 +923,19 @@ int encode_map_2d(const float* base, int64_t inner, int64_t outer, int64_t ld, i
 
 using namespace gnnpre;
 
-// selftest_polls > 0: the producers announce nothing and every wait gives up after that many polls.
+enum : int32_t { kLcFormTf32, kLcFormX3, kLcFormX3Ahead, kLcFormX3Pair, kLcForms };
+
+// What a self-test changes: the form of the kernel, which CTAs learn nothing of copies that have landed (1: all, 2 / 3: of a pair the
+// first / second) and after how many polls every wait gives up.
+struct LcSelfTest {
+    int32_t form, drop;
+    uint32_t polls;
+};
+
 static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int64_t feat_dim, int64_t ldh,
                      const int32_t* batch, int64_t batch_size, const float* Wt, int64_t hidden, int64_t ldw, uint64_t relu_mask,
                      int32_t precision, float* Y, int64_t ldy, int64_t y_hop_stride, int32_t* error_flag, void* stream,
-                     uint32_t selftest_polls) {
+                     const LcSelfTest* test = nullptr) {
     if (!hops || num_hops < 1 || num_hops > GNNPRE_MAX_HOPS || !Wt || (!Y && batch_size != 0)) return GNNPRE_ERR_INVALID_ARG;
     if (n < 1 || n > INT32_MAX || feat_dim < 1 || feat_dim > INT32_MAX - kLcChunk || batch_size < 0) return GNNPRE_ERR_INVALID_ARG;
     if (precision != GNNPRE_LC_TF32 && precision != GNNPRE_LC_TF32X3) return GNNPRE_ERR_INVALID_ARG;
@@ -974,22 +985,24 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         const uint32_t w_part = (uint32_t)n_half * 128u;
         w_bytes = (int64_t)k_chunks * 2 * w_part;
         resident = w_bytes <= kLcResidentMax;
-        pair = pairs_of_ctas(hidden, k_chunks, resident, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms);
+        pair = test ? test->form == kLcFormX3Pair
+                    : pairs_of_ctas(hidden, k_chunks, resident, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms);
         stage_stride = resident ? (uint32_t)kLcABytes : (uint32_t)kLcABytes + 2u * w_part;
         stages = (int32_t)std::min<int64_t>(pair ? kLcPairStages : kLcMaxStages, (kLcPipeBytes - (resident ? w_bytes : 0)) / stage_stride);
     }
     w_off = (uint32_t)stages * stage_stride;
     const uint32_t epi_off = w_off + (resident ? (uint32_t)w_bytes : 0u);
     const size_t smem = 1024 + (size_t)epi_off + 8 * kLcEpiBytes;
-    const bool ahead = x3 && !pair && rows_asked_ahead(k_chunks, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms / halves);
+    const bool ahead = test ? test->form == kLcFormX3Ahead
+                            : x3 && !pair && rows_asked_ahead(k_chunks, std::min<int64_t>(num_hops, kLcMaxHops) * tiles_m, num_sms / halves);
     auto kernel = pair ? k_lc_first_layer_x3<true, false> : ahead ? k_lc_first_layer_x3<false, true> : x3 ? k_lc_first_layer_x3<false, false> : k_lc_first_layer;
-    const int which = pair ? 3 : ahead ? 2 : x3 ? 1 : 0;
+    const int32_t form = pair ? kLcFormX3Pair : ahead ? kLcFormX3Ahead : x3 ? kLcFormX3 : kLcFormTf32;
     // the opt-in to large dynamic shared memory, per kernel and device: always the most a launch can want, so once is enough
     constexpr int kMostSmem = 1024 + kLcPipeBytes + 8 * kLcEpiBytes;
-    static std::atomic<bool> opted_in[4][kLcMaxDevices];
-    if (dev >= kLcMaxDevices || !opted_in[which][dev].load(std::memory_order_relaxed)) {
+    static std::atomic<bool> opted_in[kLcForms][kLcMaxDevices];
+    if (dev >= kLcMaxDevices || !opted_in[form][dev].load(std::memory_order_relaxed)) {
         GNNPRE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
-        if (dev < kLcMaxDevices) opted_in[which][dev].store(true, std::memory_order_relaxed);
+        if (dev < kLcMaxDevices) opted_in[form][dev].store(true, std::memory_order_relaxed);
     }
 
     LcMaps maps;
@@ -1022,8 +1035,8 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
         a.ldw = ldw;
         a.halves = halves;
         a.n_half = n_half;
-        a.drop_announcements = selftest_polls > 0 ? 1 : 0;
-        a.spin_limit = selftest_polls > 0 ? selftest_polls : kLcSpinLimit;
+        a.drop_announcements = test ? test->drop : 0;
+        a.spin_limit = test ? test->polls : kLcSpinLimit;
         const int64_t total = (int64_t)kn * a.tiles_m;
         const unsigned grid = (unsigned)(std::min<int64_t>(num_sms / halves, total) * halves);
         if (!pair) {
@@ -1052,7 +1065,7 @@ extern "C" int gnnpre_lc_first_layer(const float* const* hops, int32_t num_hops,
                                      uint64_t relu_mask, int32_t precision, float* Y, int64_t ldy, int64_t y_hop_stride,
                                      int32_t* error_flag, void* stream) {
     return lc_launch(hops, num_hops, n, feat_dim, ldh, batch, batch_size, Wt, hidden, ldw, relu_mask, precision, Y, ldy,
-                     y_hop_stride, error_flag, stream, 0);
+                     y_hop_stride, error_flag, stream);
 }
 
 // Failure-detection self-test: see include/gnnpre.h.
@@ -1061,13 +1074,22 @@ extern "C" int gnnpre_lc_selftest_wait_timeout(const float* hop, int64_t n, int6
                                                uint32_t polls, void* stream) {
     if (!error_flag || polls == 0 || polls > 100000u) return GNNPRE_ERR_INVALID_ARG;
     const float* hops[1] = {hop};
-    const int64_t rows = n < kLcTileM ? n : kLcTileM;  // one tile, one CTA
-    GNNPRE_CUDA(cudaMemsetAsync(error_flag, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream)));
-    const int rc = lc_launch(hops, 1, n, feat_dim, ldh, nullptr, rows, Wt, hidden, ldw, 0, GNNPRE_LC_TF32, Y, ldy, 0, error_flag,
-                             stream, polls);
-    if (rc != GNNPRE_OK) return rc;
-    GNNPRE_CUDA(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
-    int32_t flag = 0;
-    GNNPRE_CUDA(cudaMemcpy(&flag, error_flag, sizeof(flag), cudaMemcpyDeviceToHost));
-    return flag ? GNNPRE_ERR_TIMEOUT : GNNPRE_OK;
+    const int64_t rows = n < kLcTileM ? n : kLcTileM;  // one tile: one CTA, two column halves or one pair
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const bool split = hidden <= 128 || hidden % 64 == 0;
+    for (int32_t form = kLcFormTf32; form < kLcForms; ++form) {
+        if (form != kLcFormTf32 && !split) continue;
+        if (form == kLcFormX3Pair && hidden <= 128) continue;
+        for (int32_t drop = 1; drop <= (form == kLcFormX3Pair ? 3 : 1); ++drop) {
+            const LcSelfTest test{form, drop, polls};
+            GNNPRE_CUDA(cudaMemsetAsync(error_flag, 0, sizeof(int32_t), st));
+            GNNPRE_TRY(lc_launch(hops, 1, n, feat_dim, ldh, nullptr, rows, Wt, hidden, ldw, 0,
+                                 form == kLcFormTf32 ? GNNPRE_LC_TF32 : GNNPRE_LC_TF32X3, Y, ldy, 0, error_flag, stream, &test));
+            GNNPRE_CUDA(cudaStreamSynchronize(st));
+            int32_t flag = 0;
+            GNNPRE_CUDA(cudaMemcpy(&flag, error_flag, sizeof(flag), cudaMemcpyDeviceToHost));
+            if (!flag) return GNNPRE_OK;
+        }
+    }
+    return GNNPRE_ERR_TIMEOUT;
 }

@@ -242,3 +242,19 @@ def test_waits_that_run_out_are_reported_and_the_device_stays_usable(B):
         assert B.gnnpre_lc_selftest_wait_timeout(hop, Wt, polls=200) == -8
         Y = B.gnnpre_lc_first_layer([hop], None, Wt)
         assert np.array_equal(to_np(Y[0]).astype(np.float64), orc.lc_first_layer(hop_np, None, Wt_np, relu=False))
+
+
+@pytest.mark.parametrize("n,F,H,bs,K", [(1500, 200, 128, 700, 2), (600, 100, 256, 300, 1), PAIR_SHAPES[2], PAIR_SHAPES[4]])
+def test_waits_of_the_split_operand_kernels_that_run_out_are_reported(B, n, F, H, bs, K):
+    """The same for split operands, a streamed weight, column halves and pairs of CTAs (either CTA of a pair alone included): the
+    next call of the form that these sizes take is exact."""
+    hops_np = [integer_matrix(n, F, 700 + k, -4, 4) for k in range(K)]
+    Wt_np = integer_matrix(H, F, 2, -4, 4)
+    batch = None if bs is None else torch.from_numpy(np.random.default_rng(n).integers(0, n, size=bs).astype(np.int32)).cuda()
+    hops, Wt = [padded_cuda(h, 2) for h in hops_np], padded_cuda(Wt_np, 5)
+    for _ in range(2):
+        assert B.gnnpre_lc_selftest_wait_timeout(hops[0], Wt, polls=200) == -8
+        for precision in PRECISIONS:
+            Y = B.gnnpre_lc_first_layer(hops, batch, Wt, precision=precision)
+            want = orc.lc_first_layer(hops_np[0], None if bs is None else batch.cpu().numpy(), Wt_np, relu=False)
+            assert np.array_equal(to_np(Y[0]).astype(np.float64), want)
