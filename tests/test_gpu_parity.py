@@ -420,15 +420,18 @@ def test_bulk_copy_kernel_on_a_dense_graph_far_larger_than_the_cache(B, op, F):
 @pytest.mark.parametrize("F,seg", [(128, 32), (200, 200)])
 def test_segments_in_the_order_of_their_sources_give_the_same_bits(B, op, graph, F, seg):
     """A whole hop over a matrix beyond the L2 takes its segments in the order of their columns, hops launched block by block in
-    that of the edge list: segments of one row, of several, empty ones, one segment only (the star's centre has all edges)."""
+    that of the edge list: segments of one row, of several, empty ones, those of one row only (the star's centre)."""
     n = 300000
     g = {"hubs": lambda: gi.rmat(n, 900000, 41, directed_candidates=False, device="cuda"), "no hubs": lambda: gi.erdos_renyi(n, 700000, 42, device="cuda"),
-         "one row": lambda: gi.from_edge_list(n, [(3, j) for j in range(5, 405)], device="cuda")}[graph]()
+         "one row": lambda: gi.from_edge_list(n, [(n - 1000, 700 * j) for j in range(1, 401)], device="cuda")}[graph]()
     X = gi.normal_matrix(n, F, 43, device="cuda")
     kw = dict(gin_eps=EPS, segment_edges=seg, force_blocks=1, force_col_slabs=1)
     a = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, **kw)
     b = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, flags=B.GNNPRE_FLAG_LAUNCH_PER_BLOCK, **kw)
     assert a.info()["num_segments"] == b.info()["num_segments"]
+    ascending = [bool((first[1:] >= first[:-1]).all()) for first in map(B.gnnpre_plan_hop_order, (a, b))]
+    # (self-loops: hardly any segment lies in one row; segments of 200: no row is cut, and the centre's is the last one)
+    assert ascending == [graph == "no hubs" or (graph == "one row" and (op != 1 or seg == 200)), True]
     for x, y in zip(B.gnnpre_propagate(a, X, 2)[0], B.gnnpre_propagate(b, X, 2)[0]):
         assert torch.equal(x, y)
     a.close()
@@ -796,10 +799,14 @@ def test_weighted_hop_sum_behind_cut_rows_takes_its_own_operands(B, F, alpha):
             assert bool((hops[-1][1:].abs() < 1e20).all())
 
 
-@pytest.mark.parametrize("op,n,F", [(0, 140000, 64), (2, 140000, 64), (1, 70000, 128), (0, 70000, 100), (2, 70000, 128), (0, 50000, 200)])
+@pytest.mark.parametrize("op,n,F", [(0, 140000, 64), (2, 140000, 64), (1, 70000, 128), (1, 90000, 100), (0, 90000, 100), (2, 70000, 128), (0, 50000, 200)])
 def test_epilogues_whose_rows_are_fetched_ahead_give_the_bits_of_narrow_ones(B, op, n, F):
-    """Matrices that together exceed the L2: wide tiles ask for X_0, Z and X_{k-1} ahead, tiles of 32 columns do not."""
+    """Matrices that together exceed the L2: wide tiles ask for X_0, Z and X_{k-1} ahead, tiles of 32 columns do not; the mean
+    operator's on a graph that has rows without edges, where a row is not its rank."""
+    L2 = torch.cuda.get_device_properties(0).L2_cache_size
+    assert n * F * 16 > L2 > n * 32 * 16 and n * min(F, 128) * 4 <= L2 * 4 // 5  # asked for ahead; not at 32 columns; X itself fits
     g = gi.rmat(n, 1300000, 51, directed_candidates=True, device="cuda")  # (so many segments that their cuts do not depend on the width)
+    assert bool((g.rowptr[1:] == g.rowptr[:-1]).any())
     X = gi.normal_matrix(n, F, 52, device="cuda")
     gamma, kw = [0.3, -0.5, 0.25, 0.125], dict(gin_eps=EPS, segment_edges=64, force_blocks=1, force_col_slabs=1, teleport_alpha=0.2)
     wide = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, **kw)
