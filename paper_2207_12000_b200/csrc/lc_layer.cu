@@ -14,8 +14,8 @@
 //            first: at 128 bytes per gathered row the copy engine's per-row rate, about 95 rows per
 //            microsecond and SM, capped the kernel at 60 % of what the output stores alone sustain.)
 //            The weight travels by tiled tensor copies, counted in bytes on an mbarrier.
-//   warp 4   one lane issues tcgen05.mma (kind::tf32, M = 128, N = hidden, K = 8 per instruction,
-//            operands read from shared memory through swizzled K-major descriptors, fp32 accumulator
+//   warp 4   runs the loop as a whole; one elected lane issues tcgen05.mma (kind::tf32, M = 128, N = hidden, K = 8 per
+//            instruction, operands read from shared memory through swizzled K-major descriptors, fp32 accumulator
 //            in tensor memory) and hands stages back with tcgen05.commit on the `empty` mbarrier.
 //   warps 5-12  epilogue.  Two warps share each quarter of the accumulator's 128 lanes (even and odd
 //            column boxes); a warp pulls its part out of tensor memory with tcgen05.ld 32 columns at a
@@ -602,9 +602,10 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lc_first_layer(const __grid_c
 // stages, and shared memory holds four stages of copied rows beside 128 KB of weight.  2.4 M rows x 3 hops, F = 100, hidden
 // 256, random order, under load: 4630 us when the copying threads split into a second half of two stages (and their proxy
 // fence waited for all their copies in flight), 3379 us now (single passes on a cool device: 3550 us with splitter warps and two
-// buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Bound by the latency of a
-// tile's chain over those four stages and, in long runs, by the power that all its parts draw (3250 us in halves, 3130 in
-// pairs of CTAs, 2870 with MMAs issued from uniform registers).
+// buffers of low parts in shared memory, 2816 us now); 500 K rows x 2, F = 256: 1540 / 908 / 856.  Of 100 features and more it is
+// bound by no part alone (612,257 rows x 3 hops, F = 100, hidden 256, one launch at 1965 MHz: 630 us, tensor pipe 45 % active, DRAM
+// 4.3 TB/s, two thirds of the copy rate) and, in long runs, by the power that all its parts draw (3250 us in halves, 3130 in
+// pairs of CTAs, 2870 with MMAs issued from uniform registers); of fewer features by its stores and the hand-offs of a tile.
 // K-steps of the last chunk beyond the features are neither copied nor multiplied.
 //
 // The tensor core ignores the low 13 mantissa bits of an fp32 operand (checked on the device: 1 + 7 * 2^-13
@@ -941,10 +942,8 @@ static int lc_launch(const float* const* hops, int32_t num_hops, int64_t n, int6
     if (precision != GNNPRE_LC_TF32 && precision != GNNPRE_LC_TF32X3) return GNNPRE_ERR_INVALID_ARG;
     if (hidden < 16 || hidden > kLcMaxHidden || hidden % 16 != 0) return GNNPRE_ERR_INVALID_ARG;
     const bool x3 = precision == GNNPRE_LC_TF32X3;
-    // Split operands: both parts of a CTA's weight columns must fit in shared memory, so a CTA computes at most 128
-    // output columns; each part is a whole number of 32-column boxes.  (Parts of 64 columns leave room for four
-    // operand stages instead of two but were measured slower, 8.4 against 4.5 ms on the 2.4 M-row workload: the
-    // per-tile hand-offs, not the stage count, set the pace.)
+    // Split operands: both parts of a CTA's weight rows must fit in shared memory, so a CTA holds at most 128 of them; each
+    // column half is a whole number of 32-column boxes.
     const int32_t halves = x3 && hidden > 128 ? 2 : 1;
     if (halves == 2 && hidden % 64 != 0) return GNNPRE_ERR_INVALID_ARG;
     if (ldh < feat_dim || ldw < feat_dim || ldy < hidden) return GNNPRE_ERR_INVALID_ARG;
