@@ -352,18 +352,11 @@ __global__ void k_segment_starts(int64_t nseg, int b, const int64_t* __restrict_
     segs[s] = g;
 }
 
-// Whether all edges of segment s belong to one row (never the last segment: the sentinel has no row); nx_head: the segment
-// after it begins inside a row.
-__device__ __forceinline__ bool inside_one_row(int64_t s, int64_t nseg, const Segment& g, const Segment& nx, bool nx_head) {
-    return s + 1 < nseg && nx.start > g.start && (nx.rank == g.rank || (nx.rank == g.rank + 1 && !nx_head));
-}
-
 // What segment s accounts for: a scratch row if its first row began earlier (head), one if the row of its last edge
 // goes on and began in it (tail), a fix-up if the row that began earlier ends in it.  first[s] = the segment that row
-// began in.  in_edge_order (or nullptr): whether a hop takes the segment in the order of the edge list (see k_segment_order).
+// began in.
 __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs, const int64_t* __restrict__ rowptr_t,
-                                 int32_t hub_parts, SegCounts* __restrict__ counts, int32_t* __restrict__ first,
-                                 int32_t* __restrict__ in_edge_order) {
+                                 int32_t hub_parts, SegCounts* __restrict__ counts, int32_t* __restrict__ first) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     const Segment g = segs[s], nx = segs[s + 1];
@@ -387,15 +380,11 @@ __global__ void k_segment_counts(int64_t nseg, const Segment* __restrict__ segs,
         hub = s - lo + 1 > hub_parts;
     }
     counts[s] = {head + tail, emit, hub};
-    if (in_edge_order) in_edge_order[s] = !inside_one_row(s, nseg, g, nx, nx.slot_head);
 }
 
-// by_source (or nullptr): the segments that a hop takes in the order of the edge list go to its end; edge_before[s] of them come
-// before segment s.
 __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, const SegCounts* __restrict__ counts,
                                    const SegCounts* __restrict__ before, const int32_t* __restrict__ first,
-                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs,
-                                   const int32_t* __restrict__ edge_before, Segment* __restrict__ by_source, const int* err) {
+                                   RowFixup* __restrict__ fixups, int32_t* __restrict__ hubs, const int* err) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s > nseg || *err) return;
     if (s < nseg) {
@@ -415,7 +404,6 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
         segs[s].slot_tail = c.slots > head ? b.slots + head : -1;
     }
     segs[s].len = s < nseg ? (int32_t)(segs[s + 1].start - segs[s].start) : 0;
-    if (by_source && s < nseg && edge_before[s] < edge_before[s + 1]) by_source[nseg - edge_before[nseg] + edge_before[s]] = segs[s];
 }
 
 // ---------------------------------------------------------------- the order in which a hop takes its segments
@@ -438,35 +426,59 @@ __global__ void k_segment_finalize(int64_t nseg, Segment* __restrict__ segs, con
 // Erdos-Renyi 3770 / 3765 / 3765.
 constexpr int64_t kFewSegments = 64;  // one in so many
 
-// SCATTER false: counts[b] = segments of bucket b, *near = those whose row lies near their columns.  true: counts[b] holds where
-// the bucket begins; copies the segments there.
+// What the host decides by: segments inside one row, and those of them whose row lies near their columns.
+struct OrderCounts {
+    int32_t one_row, near;
+};
+
+// SCATTER false: places[0 .. kOrderBuckets) += segments of the buckets, places[kOrderBuckets + block] = the other segments of the
+// block's.  true: places holds the exclusive prefix sums of that, that is, where each bucket and each block's other segments
+// begin; copies the segments there.
 template <bool SCATTER>
-__global__ void k_segment_order(int64_t nseg, const Segment* __restrict__ segs, const uint32_t* __restrict__ colx,
-                                const int32_t* __restrict__ nzrows, int64_t n, int32_t* __restrict__ counts, int32_t* near,
-                                Segment* __restrict__ ordered, const int* err) {
+__global__ void __launch_bounds__(kTB) k_segment_order(int64_t nseg, const Segment* __restrict__ segs, const uint32_t* __restrict__ colx,
+                                                       const int32_t* __restrict__ nzrows, int64_t n, int32_t* __restrict__ places,
+                                                       OrderCounts* report, Segment* __restrict__ ordered, const int* err) {
+    constexpr unsigned kFull = 0xffffffffu;
+    __shared__ int others[kTB / 32];
     if (*err) return;  // then there is neither a table nor an edge list
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t s = (int64_t)blockIdx.x * kTB + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int bucket = -1;
-    bool local = false;
+    bool near = false;
     Segment g;
     if (s < nseg) {
         g = segs[s];
         const Segment nx = segs[s + 1];
-        if (inside_one_row(s, nseg, g, nx, nx.slot_head >= 0)) {
+        // all edges in one row (never the last segment: the sentinel has no row)
+        if (s + 1 < nseg && g.len > 0 && (nx.rank == g.rank || (nx.rank == g.rank + 1 && nx.slot_head < 0))) {
             const uint32_t col = colx[g.start + g.len / 2] & ~kRowEndBit;
             bucket = column_bucket(col, n);
-            if (!SCATTER) local = near_diagonal((uint32_t)(nzrows ? nzrows[g.rank] : g.rank), col, n);
+            if (!SCATTER) near = near_diagonal((uint32_t)(nzrows ? nzrows[g.rank] : g.rank), col, n);
         }
     }
-    const unsigned same = __match_any_sync(0xffffffffu, bucket);  // one addition per bucket and warp
-    const int lane = threadIdx.x & 31, first = __ffs(same) - 1;
+    const unsigned same = __match_any_sync(kFull, bucket);  // one addition per bucket and warp
+    const int first = __ffs(same) - 1;
     int at = 0;
-    if (lane == first && bucket >= 0) at = atomicAdd(&counts[bucket], __popc(same));
-    at = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
-    if (SCATTER && bucket >= 0) ordered[at] = g;
+    if (lane == first && bucket >= 0) at = atomicAdd(&places[bucket], __popc(same));
+    at = __shfl_sync(kFull, at, first) + __popc(same & ((1u << lane) - 1u));
+    const unsigned other = __ballot_sync(kFull, s < nseg && bucket < 0);
+    if (lane == 0) others[warp] = __popc(other);
     if (!SCATTER) {
-        const int locals = __popc(__ballot_sync(0xffffffffu, local));
-        if (lane == 0 && locals > 0) atomicAdd(near, locals);
+        const unsigned one_row = __ballot_sync(kFull, bucket >= 0), nears = __ballot_sync(kFull, near);
+        if (lane == 0 && one_row) atomicAdd(&report->one_row, __popc(one_row));
+        if (lane == 0 && nears) atomicAdd(&report->near, __popc(nears));
+    }
+    __syncthreads();
+    if (SCATTER) {
+        if (s < nseg && bucket < 0) {
+            at = places[kOrderBuckets + blockIdx.x] + __popc(other & ((1u << lane) - 1u));
+            for (int w = 0; w < warp; ++w) at += others[w];
+        }
+        if (s < nseg) ordered[at] = g;
+    } else if (threadIdx.x == 0) {
+        int sum = 0;
+        for (int w = 0; w < kTB / 32; ++w) sum += others[w];
+        places[kOrderBuckets + blockIdx.x] = sum;
     }
 }
 
@@ -817,8 +829,8 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // if there is room.
     struct Report {  // followed by BlockRows[b] and SegCounts[b + 1]
         int32_t err, nonempty, longest_row;
-        int32_t in_edge_order, near;  // of the segments: see k_segment_order
         int32_t unused;
+        OrderCounts order;
     };
     static_assert(sizeof(Report) % 8 == 0 && sizeof(BlockRows) % 8 == 0, "the report's parts stay aligned");
     // (the report has a place of its own: E overwrites the temporaries before the host reads it)
@@ -827,6 +839,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     DevBuf<uint32_t> e_temp;
     DevBuf<uint32_t>& colx = e_host ? e_temp : P->colx;  // E of a host-resident structure is on the device for the build only
     const bool small_report = b <= 4096;
+    const int64_t places = kOrderBuckets + (nseg + kTB - 1) / kTB;  // see k_segment_order
     auto want_fixed = [&](Carve& carve) {
         carve.want(P->deg, (size_t)n);
         carve.want(P->rscale, (size_t)n);
@@ -837,7 +850,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         if (small_report) carve.want(report, report_bytes);
         if (by_source) {
             carve.want(P->by_source, (size_t)nseg);
-            carve.want(P->by_source_counts, 2 * kOrderBuckets + 1);
+            carve.want(P->by_source_counts, 2 * (size_t)places + 1 + scan_temp_items(places));
         }
         if (!e_host) carve.want(P->colx, (size_t)m);
     };
@@ -882,7 +895,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     if (e_host) GNNPRE_TRY(e_temp.alloc((size_t)m));
     DevBuf<char> temp_arena;
     if (!small_report) GNNPRE_TRY(report.alloc(report_bytes));
-    DevBuf<int32_t> flag, rank, rank_temp, first, in_edge_order, edge_before, edge_temp;
+    DevBuf<int32_t> flag, rank, rank_temp, first;
     DevBuf<SegCounts> counts, before, counts_temp;
     DevBuf<int64_t> offsets;
     Carve temps;
@@ -896,11 +909,6 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     temps.want(counts, (size_t)nseg);
     temps.want(before, (size_t)nseg + 1);
     temps.want(counts_temp, scan_temp_items(nseg));
-    if (by_source) {
-        temps.want(in_edge_order, (size_t)nseg);
-        temps.want(edge_before, (size_t)nseg + 1);
-        temps.want(edge_temp, scan_temp_items(nseg));
-    }
     if (temps.bytes() <= colx.bytes()) GNNPRE_TRY(temps.place(reinterpret_cast<char*>(colx.p)));
     else GNNPRE_TRY(temps.place(temp_arena));
     Report* d_report = reinterpret_cast<Report*>(report.p);
@@ -956,14 +964,9 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         k_segment_starts<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, (int)b, d_seg_base, d_e_off, L, snap, uncut,
                                                                   &d_report->longest_row, P->rowptr_t.p, n, rank.p, P->segments.p);
         GNNPRE_CUDA(cudaGetLastError());
-        k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p,
-                                                                in_edge_order.p);
+        k_segment_counts<<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->rowptr_t.p, P->hub_parts, counts.p, first.p);
         GNNPRE_CUDA(cudaGetLastError());
         GNNPRE_TRY(exclusive_scan(counts.p, nseg, before.p, counts_temp.p, st));
-        if (by_source) {
-            GNNPRE_TRY(exclusive_scan(in_edge_order.p, nseg, edge_before.p, edge_temp.p, st));
-            GNNPRE_CUDA(cudaMemcpyAsync(&d_report->in_edge_order, edge_before.p + nseg, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-        }
         k_block_report<<<grid_for(b + 1, kTB / 32), kTB, 0, st>>>((int)b, d_e_off, d_seg_base, before.p, P->rowptr_t.p, n, d_rows, d_at);
         GNNPRE_CUDA(cudaGetLastError());
     }
@@ -1008,7 +1011,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         return GNNPRE_OK;
     }
     k_segment_finalize<<<grid_for(nseg + 1, kTB), kTB, 0, st>>>(nseg, P->segments.p, counts.p, before.p, first.p, P->fixups.p,
-                                                                P->hubs.p, edge_before.p, P->by_source.p, &d_report->err);
+                                                                P->hubs.p, &d_report->err);
     GNNPRE_CUDA(cudaGetLastError());
 
     // ---- E, the support's edge list: overwrites the temporaries
@@ -1022,12 +1025,12 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
                                                                        d_rowptr, d_colidx, colx.p, &d_report->err);
         GNNPRE_CUDA(cudaGetLastError());
     }
-    int32_t *bucket_counts = P->by_source_counts.p, *bucket_begins = bucket_counts + kOrderBuckets;
+    int32_t *counted = P->by_source_counts.p, *begins = counted + places;
     const int32_t* row_of_rank = diag ? nullptr : P->nzrows.p;  // (nullptr as well where every row has edges)
     if (by_source) {
-        GNNPRE_CUDA(cudaMemsetAsync(bucket_counts, 0, sizeof(int32_t) * kOrderBuckets, st));
-        k_segment_order<false><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, bucket_counts,
-                                                                    &d_report->near, nullptr, &d_report->err);
+        GNNPRE_CUDA(cudaMemsetAsync(counted, 0, sizeof(int32_t) * kOrderBuckets, st));
+        k_segment_order<false><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, counted,
+                                                                    &d_report->order, nullptr, &d_report->err);
         GNNPRE_CUDA(cudaGetLastError());
     }
     GNNPRE_TRY(read_report());  // everything is in place
@@ -1050,12 +1053,10 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         B.done_row_hi = l == b - 1 ? n : r.done_row_hi;
     }
     if (by_source) {
-        const int64_t one_row = nseg - rep->in_edge_order;
-        if (one_row * kFewSegments >= nseg && 2 * (int64_t)rep->near <= one_row) {
-            static_assert(kOrderBuckets <= kScanTile, "the scan needs no temporary memory");
-            GNNPRE_TRY(exclusive_scan<int32_t>(bucket_counts, kOrderBuckets, bucket_begins, nullptr, st));
-            k_segment_order<true><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, bucket_begins,
-                                                                       nullptr, P->by_source.p, &d_report->err);
+        if (rep->order.one_row * kFewSegments >= nseg && 2 * (int64_t)rep->order.near <= rep->order.one_row) {
+            GNNPRE_TRY(exclusive_scan<int32_t>(counted, places, begins, begins + places + 1, st));
+            k_segment_order<true><<<grid_for(nseg, kTB), kTB, 0, st>>>(nseg, P->segments.p, P->colx.p, row_of_rank, n, begins, nullptr,
+                                                                       P->by_source.p, &d_report->err);
             GNNPRE_CUDA(cudaGetLastError());
             GNNPRE_CUDA(cudaStreamSynchronize(st));
         } else {
