@@ -869,8 +869,10 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     // a segment has at most a head and a tail part and ends at most one cut row, a hub has more than kHubParts parts
     const int64_t most_rows = diag ? 0 : n;
     const int64_t most_bytes = 16 * nseg + 12 * most_rows + 2 * nseg * P->slab_width * 4;
-    bool one_allocation = !ask && opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE && most_bytes <= (128 << 20) &&
-                          fixed.bytes() > (1 << 20);
+    // (a plan over a matrix beyond the L2 has up to twice the segments, and as much room for them: 2 M nodes, 80 M edges, GCN, 128
+    // columns, us for a build with two allocations / one 2550 / 1950; one hop with its plan 5310 / 4710)
+    bool one_allocation = !ask && opts->budget_bytes <= 0 && opts->operands_mem == GNNPRE_MEM_DEVICE &&
+                          most_bytes <= (by_source ? 256 << 20 : 128 << 20) && fixed.bytes() > (1 << 20);
     if (one_allocation) want_sized(fixed, nseg, nseg / kHubParts, most_rows, most_rows, 2 * nseg);
     const int64_t refused = refused_allocations();
     int placed;
