@@ -956,7 +956,14 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
     const int64_t lanes = f4_slab <= 4 ? 4 : f4_slab <= 8 ? 8 : f4_slab <= 16 ? 16 : 32;
     const bool one_wave = nseg * lanes <= (int64_t)P->num_sms * 768;
     const int32_t snap = one_wave ? L - 1 : L / 2;
-    const int64_t uncut = longest_uncut_row(m_launch, lanes, L, one_wave);
+    // Segments of 16 or 24 edges that fill one wave (of 28 warps an SM) cut nearly every row of a uniform graph whose rows are a
+    // little longer: rows of up to 72 edges are not cut there (96 in groups of whole warps, which wait for nobody's longer
+    // segment).  us for two hops, segments of 32 edges / cut / so: degree 24, mean operator, 480,000 edges, 16 columns 16.5 / 25.5 / 16.1,
+    // 240,000, 32 columns 13.1 / 17.4 / 12.6, 120,000, 64 columns 11.6 / 15.6 / 11.6; degree 36 16.7 / 22.9 / 18.3, 14.1 / 16.3 / 15.0,
+    // 13.0 / 13.9 / 14.0; degree 60, 128 columns, 60,000 edges 10.6 / 13.7 / 12.0; not cut in narrower groups, degree 60 is slower
+    // (240,000 edges, 32 columns 15.0 / 13.9 / 19.6).
+    const int64_t uncut = std::max<int64_t>(longest_uncut_row(m_launch, lanes, L, one_wave),
+                                            one_wave || L >= 32 || opts->segment_edges > 0 ? 0 : lanes == 32 ? 96 : 72);
     if (m > 0) {
         std::vector<int64_t> h_off(e_off);
         h_off.insert(h_off.end(), seg_base.begin(), seg_base.end());

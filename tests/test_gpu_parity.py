@@ -486,6 +486,23 @@ def test_segments_of_a_small_graph_fill_whole_waves(B, op, F, m):
 
 
 @pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("b", [1, 3, 32])
+@pytest.mark.parametrize("F,m", [(16, 480000), (32, 240000), (64, 120000), (64, 180000), (128, 60000)])
+def test_rows_longer_than_short_segments_are_not_cut(B, op, F, m, b):
+    """Uniform graphs whose segments of 16 or 24 edges fill one wave: rows of fewer than 72 edges are not cut, whichever block they
+    lie in, but for those that a block's end cuts."""
+    g = gi.erdos_renyi(m // 30, m // 2, 46)
+    assert 3 * 16 <= int((g.rowptr[1:] - g.rowptr[:-1]).max()) < 71
+    X = gi.normal_matrix(g.n, F, 45)
+    plan = B.gnnpre_build_plan(*dev(g), op, F, gin_eps=EPS, force_blocks=b)
+    info = plan.info()
+    assert info["segment_edges"] in (16, 24) and info["num_row_fixups"] <= b - 1
+    outs, _ = B.gnnpre_propagate(plan, X.cuda(), 2)
+    check_all_hops(op, EPS, g.rowptr.numpy(), g.colidx.numpy(), X.numpy(), outs, single_hop=single_hop_of(B, plan))
+    plan.close()
+
+
+@pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("F", [4, 16, 20, 32, 36, 64, 68, 132, 260])
 @pytest.mark.parametrize("seg", [1, 7, 8, 9, 31, 33])
 def test_register_kernel_tile_and_segment_edges(B, op, F, seg):
