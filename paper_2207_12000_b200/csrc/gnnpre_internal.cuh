@@ -233,6 +233,7 @@ struct gnnpre_plan {
     int64_t num_hubs = 0;
     int32_t hub_parts = 0;
     int64_t num_segments = 0, num_fixups = 0, num_slots = 0;
+    bool short_rows = false;  // rows are few edges long on average, or most of them are much shorter than the longest
     gnnpre::DevBuf<float> scratch;  // num_slots rows of slab_width floats
     gnnpre::DevBuf<int> dev_error;  // set by a kernel whose bounded wait ran out
     int num_sms = 0;

@@ -992,6 +992,7 @@ int build_plan_impl(const gnnpre_csr_t* csr, const int32_t* degrees, const gnnpr
         P->num_nonempty = diag ? n : rep->nonempty;
         P->num_empty = n - P->num_nonempty;
         P->rows_all_nonempty = P->num_empty == 0;
+        P->short_rows = m <= 8 * n || rep->longest_row * n > 4 * m;
         if (m > 0) {
             P->num_slots = at[b].slots;
             P->num_fixups = at[b].fixups;

@@ -41,17 +41,26 @@ __global__ void k_wait_that_runs_out(int* error, uint32_t polls) {
 #include "fixups.cuh"
 #include "ceiling.cuh"
 
+template <int G, int OP, bool HAS_EMPTY, int EP, bool FAR>
+int launch_segments_epilogue(const SegArgs& a, dim3 grid, cudaStream_t st) {
+    if constexpr (!FAR && kFetchesAhead<G, OP, EP>) {
+        // the two that gain on long rows of equal length too
+        constexpr int kFrom = EP == kEpTeleport && ((G == 16 && OP == GNNPRE_OP_GCN_SYM) || (G == 32 && OP == GNNPRE_OP_GIN_SUM)) ? 1 : 2;
+        if (a.tp.ahead >= kFrom) return launch_dependent(k_segments<G, OP, HAS_EMPTY, EP, FAR, true>, grid, kSegThreads, 0, a.back_to_back, st, a);
+    }
+    return launch_dependent(k_segments<G, OP, HAS_EMPTY, EP, FAR, false>, grid, kSegThreads, 0, a.back_to_back, st, a);
+}
+
 template <int G, bool FAR = false>
 int launch_segments_shape(const gnnpre_plan* P, const SegArgs& a, cudaStream_t st) {
     const int64_t groups = a.seg_hi - a.seg_lo;
     const dim3 grid((unsigned)((groups * G + kSegThreads - 1) / kSegThreads), (unsigned)((a.f4 + a.tile_f4 - 1) / a.tile_f4));
     const int ep = epilogue_of(a.tp);
-#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                                                    \
-    do {                                                                                                                       \
-        if (ep == kEpSum) return launch_dependent(k_segments<G, OP_, EMPTY_, kEpSum, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a); \
-        if (ep == kEpTeleport)                                                                                                 \
-            return launch_dependent(k_segments<G, OP_, EMPTY_, kEpTeleport, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a);     \
-        return launch_dependent(k_segments<G, OP_, EMPTY_, kEpPlain, FAR>, grid, kSegThreads, 0, a.back_to_back, st, a);            \
+#define GNNPRE_LAUNCH_SEGMENTS(OP_, EMPTY_)                                                             \
+    do {                                                                                                \
+        if (ep == kEpSum) return launch_segments_epilogue<G, OP_, EMPTY_, kEpSum, FAR>(a, grid, st);       \
+        if (ep == kEpTeleport) return launch_segments_epilogue<G, OP_, EMPTY_, kEpTeleport, FAR>(a, grid, st); \
+        return launch_segments_epilogue<G, OP_, EMPTY_, kEpPlain, FAR>(a, grid, st);                      \
     } while (0)
     switch (P->op) {
     case GNNPRE_OP_GCN_SYM: GNNPRE_LAUNCH_SEGMENTS(GNNPRE_OP_GCN_SYM, false);
@@ -192,7 +201,8 @@ Teleport teleport_of(const gnnpre_plan* P, const HopArgs& h, int32_t f0) {
     tp.zsum_first = h.zsum_first ? 1 : 0;
     // with X_0 and Z a hop has three to five matrices; tiles of more than 64 columns that exceed the L2 alone gain nothing
     // (600 K nodes, 128 columns: 10.3 ms without, 10.5 with; 1 M nodes, 64 columns 6.1 / 5.8)
-    tp.ahead = P->n * h.width * 16 > l2_cache_bytes() && (h.width <= 64 || !beyond_cache(P, h.width));
+    const bool from_memory = P->n * h.width * 16 > l2_cache_bytes() && (h.width <= 64 || !beyond_cache(P, h.width));
+    tp.ahead = !from_memory ? 0 : P->short_rows ? 2 : 1;  // 1: long rows of equal length (see kFetchesAhead)
     return tp;
 }
 

@@ -78,7 +78,21 @@ struct __align__(16) SegStage {  // read in 16-byte pieces
     }
 };
 
-template <int G, int OP, bool HAS_EMPTY, int EP, bool FAR>
+// AHEAD: epilogue operands come from memory where the hop's matrices together exceed the L2, and one row ahead is too late for that:
+// each lane asks for the pieces that belong to its row end when the chunk is staged.  169 K nodes, without / with, us a
+// call: teleport term, three hops, GCN, 64 columns 302 / 270, 128 394 / 385, sum operator, 100 columns 386 / 359; with
+// the sum of ten hops GCN, 64 columns 1125 / 1035, 100 1517 / 1458, sum operator, 64 columns 1042 / 996, mean, 128
+// 1315 / 1283.  Not the mean operator's 64 columns (889 / 918) nor narrower rows (16 columns 15 % slower).  A kernel of its own: the
+// code alone, not taken, cost 2 to 3 % (ten hops and their sum, GCN, 60,000 nodes of degree 20, 128 columns 638 / 655).  Those are
+// R-MAT graphs, whose many short rows end soon after one another.  Long rows of equal length leave the time that one row ahead
+// needs, and the requests cost: Erdos-Renyi graphs of 1.3 times the L2, ten hops and their sum, degree 6 / 12 / 16 / 32, with against
+// without: GCN, 64 columns 0.98 / 1.00 / 1.03 / 1.02, 128 1.01 / 1.04 / 1.01 / 1.06, sum operator, 64 columns 1.00 / 1.06 / 1.07 / 1.07; with
+// a teleport term only 0.92 / 0.95 / 0.94 / 0.92, 0.97 / 1.02 / 1.03 / 1.04, 0.96 / 1.02 / 1.03 / 1.02, sum operator, 128 columns 0.95 / 0.98 /
+// 0.98 / 0.99.  Hence where rows are short, or uneven, and in the two kernels that gain anyway.
+template <int G, int OP, int EP>
+constexpr bool kFetchesAhead = EP != kEpPlain && (G == 32 || (G == 16 && OP != GNNPRE_OP_SAGE_MEAN));
+
+template <int G, int OP, bool HAS_EMPTY, int EP, bool FAR, bool AHEAD>
 __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegArgs a) {
     constexpr unsigned kFull = 0xffffffffu;
     // GIN's weights are 1 but for the self-loops': groups of 16 lanes and more mark those in a bit mask and add the rest
@@ -89,12 +103,6 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
     // and the piece in shared memory: 3144, 100).
     constexpr bool kDiagonal = OP == GNNPRE_OP_GIN_SUM && G >= 16 && EP != kEpTeleport;
     constexpr bool kWeighted = OP != GNNPRE_OP_SAGE_MEAN && !kDiagonal;
-    // Epilogue operands come from memory where the hop's matrices together exceed the L2, and one row ahead is too late for that:
-    // each lane asks for the pieces that belong to its row end when the chunk is staged.  169 K nodes, without / with, us a
-    // call: teleport term, three hops, GCN, 64 columns 302 / 270, 128 394 / 385, sum operator, 100 columns 386 / 359; with
-    // the sum of ten hops GCN, 64 columns 1125 / 1035, 100 1517 / 1458, sum operator, 64 columns 1042 / 996, mean, 128
-    // 1315 / 1283.  Not the mean operator's 64 columns (889 / 918) nor narrower rows (16 columns 15 % slower).
-    constexpr bool kAhead = EP != kEpPlain && (G == 32 || (G == 16 && OP != GNNPRE_OP_SAGE_MEAN));
     constexpr bool kShort = G == 4 || (G == 32 && EP == kEpPlain);
     using RowOut = std::conditional_t<kShort, RowOutShort, RowOutLong>;
     using Stage = SegStage<G, kWeighted, RowOut>;
@@ -190,8 +198,8 @@ __global__ void __launch_bounds__(kSegThreads, kSegBlocks) k_segments(const SegA
             if constexpr (kShort) o.row = slot >= 0 ? ~slot : row[m];
             else o.row = slot >= 0 ? -1 : row[m];
             stage.out[i] = o;
-            if constexpr (kAhead) {
-                if (a.tp.ahead && i <= last && slot < 0) {
+            if constexpr (AHEAD) {
+                if (a.tp.ahead && i <= last && slot < 0) {  // (always ahead here; without the look the compiler spills more: 1 %)
                     constexpr int kLines = G / 8;
                     const int tile_w = min(a.tile_f4, a.f4 - q0);
                     if (EP == kEpTeleport || a.tp.alpha != 0.f || a.tp.zsum_first)

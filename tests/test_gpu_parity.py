@@ -817,13 +817,16 @@ def test_weighted_hop_sum_behind_cut_rows_takes_its_own_operands(B, F, alpha):
 
 
 @pytest.mark.parametrize("op,n,F", [(0, 140000, 64), (2, 140000, 64), (1, 70000, 128), (1, 90000, 100), (0, 90000, 100), (2, 70000, 128), (0, 50000, 200)])
-def test_epilogues_whose_rows_are_fetched_ahead_give_the_bits_of_narrow_ones(B, op, n, F):
+@pytest.mark.parametrize("rows", ["uneven", "even"])
+def test_epilogues_whose_rows_are_fetched_ahead_give_the_bits_of_narrow_ones(B, op, n, F, rows):
     """Matrices that together exceed the L2: wide tiles ask for X_0, Z and X_{k-1} ahead, tiles of 32 columns do not; the mean
-    operator's on a graph that has rows without edges, where a row is not its rank."""
+    operator's on a graph that has rows without edges, where a row is not its rank.  Where rows are long and even only some do."""
     L2 = torch.cuda.get_device_properties(0).L2_cache_size
     assert n * F * 16 > L2 > n * 32 * 16 and n * min(F, 128) * 4 <= L2 * 4 // 5  # asked for ahead; not at 32 columns; X itself fits
-    g = gi.rmat(n, 1300000, 51, directed_candidates=True, device="cuda")  # (so many segments that their cuts do not depend on the width)
-    assert bool((g.rowptr[1:] == g.rowptr[:-1]).any())
+    g = (gi.rmat(n, 1300000, 51, directed_candidates=True, device="cuda") if rows == "uneven" else  # (so many segments that their cuts do not
+         gi.erdos_renyi(n, 10 * n, 52, device="cuda"))                                              # depend on the width; here: no cut rows)
+    deg = g.rowptr[1:] - g.rowptr[:-1]
+    assert (int(deg.min()) == 0 and int(deg.max()) * n > 4 * g.nnz) if rows == "uneven" else (g.nnz > 9 * n and int(deg.max()) * n < 3 * g.nnz)
     X = gi.normal_matrix(n, F, 52, device="cuda")
     gamma, kw = [0.3, -0.5, 0.25, 0.125], dict(gin_eps=EPS, segment_edges=64, force_blocks=1, force_col_slabs=1, teleport_alpha=0.2)
     wide = B.gnnpre_build_plan(g.rowptr, g.colidx, op, F, **kw)
